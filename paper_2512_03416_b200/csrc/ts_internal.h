@@ -131,9 +131,14 @@ struct CtxView {
   int max_tokens;           // most tokens a step may hold
 };
 int ctx_view(ts_ctx* c, cudaStream_t stream, CtxView* out);
-// Tile height (128 or 256 rows per CTA) that finishes an M x N product in the fewest tile-waves.
-int gemm_tile_m(int M, int N, int n_sms);
-cudaError_t launch_gemm(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, int tile_m, int n_sms,
+// How a product is laid over the chip: tile height (128 or 256 rows per CTA), and the number of CTAs
+// that share a 128-row tile's K range (split > 1: clusters of that size).
+struct GemmPlan {
+  int tile_m, split;
+};
+// The plan for an M x N x K product; `tall` = 256-row tiles may be used. The device is the current one.
+GemmPlan gemm_plan(int M, int N, int K, int n_sms, bool tall);
+cudaError_t launch_gemm(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, GemmPlan plan, int n_sms,
                         cudaStream_t stream);
 // out[row] = x[row] / sqrt(mean(x[row]^2) + eps) * gain, bf16 in and out, fp32 inside; width % 8 == 0
 cudaError_t launch_rmsnorm(const uint16_t* x, const uint16_t* gain, uint16_t* out, int rows, int width, float eps,

@@ -227,7 +227,7 @@ int ts_layer_step(ts_layer* l, const ts_step* st, const void* x_in, void* x_out,
   g.N = qd + 2 * kvd; g.K = hidden; g.epi = ts::GEMM_EPI_ROPE;
   g.C = q; g.C2 = k; g.C3 = v; g.q_cols = qd; g.kv_cols = kvd; g.pos = pos_dev;
   g.rope_table = (const float2*)(ws + l->L.off_table);
-  TSL_CUDA(l, ts::launch_gemm(g, l->a_h, l->w_qkv, 128, l->view.n_sms, stream));
+  TSL_CUDA(l, ts::launch_gemm(g, l->a_h, l->w_qkv, ts::gemm_plan(N, g.N, g.K, l->view.n_sms, false), l->view.n_sms, stream));
   // attention over the paged KV cache, with the append of the new K/V
   ts_step inner = *st;
   inner.q = q; inner.k_new = k; inner.v_new = v; inner.out = attn;
@@ -235,14 +235,14 @@ int ts_layer_step(ts_layer* l, const ts_step* st, const void* x_in, void* x_out,
   if (rc != TS_OK) return rc;
   // y = x + attn . W_o^T
   g.N = hidden; g.K = qd; g.epi = ts::GEMM_EPI_STORE; g.C = y; g.R = (const uint16_t*)x_in; g.ldc = hidden;
-  TSL_CUDA(l, ts::launch_gemm(g, l->a_attn, l->w_o, ts::gemm_tile_m(N, hidden, l->view.n_sms), l->view.n_sms, stream));
+  TSL_CUDA(l, ts::launch_gemm(g, l->a_attn, l->w_o, ts::gemm_plan(N, g.N, g.K, l->view.n_sms, true), l->view.n_sms, stream));
   // h2 = rmsnorm(y); z = silu(h2 . W_gate^T) * (h2 . W_up^T)
   TSL_CUDA(l, ts::launch_rmsnorm(y, (const uint16_t*)l->cfg.w_norm2, h, N, hidden, l->eps, stream));
   g.N = 2 * inter; g.K = hidden; g.epi = ts::GEMM_EPI_SILU_MUL; g.C = z; g.R = nullptr; g.ldc = inter;
-  TSL_CUDA(l, ts::launch_gemm(g, l->a_h, l->w_gu, ts::gemm_tile_m(N, 2 * inter, l->view.n_sms), l->view.n_sms, stream));
+  TSL_CUDA(l, ts::launch_gemm(g, l->a_h, l->w_gu, ts::gemm_plan(N, g.N, g.K, l->view.n_sms, true), l->view.n_sms, stream));
   // out = y + z . W_down^T
   g.N = hidden; g.K = inter; g.epi = ts::GEMM_EPI_STORE; g.C = (uint16_t*)x_out; g.R = y; g.ldc = hidden;
-  TSL_CUDA(l, ts::launch_gemm(g, l->a_z, l->w_down, ts::gemm_tile_m(N, hidden, l->view.n_sms), l->view.n_sms, stream));
+  TSL_CUDA(l, ts::launch_gemm(g, l->a_z, l->w_down, ts::gemm_plan(N, g.N, g.K, l->view.n_sms, true), l->view.n_sms, stream));
   return TS_OK;
 }
 
@@ -268,8 +268,8 @@ int ts_gemm_bf16(int32_t device, int32_t M, int32_t N, int32_t K, const void* A,
   g.C = (uint16_t*)C; g.R = (const uint16_t*)R; g.ldc = N;
   g.status = device_status;
   g.wait_cycles = ts::kWaitCycles;
-  const int tm = tile_m ? tile_m : ts::gemm_tile_m(M, N, n_sms);
-  return ts::launch_gemm(g, a_map, b_map, tm, n_sms, (cudaStream_t)cuda_stream) == cudaSuccess ? TS_OK : TS_ERR_CUDA;
+  const ts::GemmPlan plan = tile_m ? ts::GemmPlan{tile_m, 1} : ts::gemm_plan(M, N, K, n_sms, true);
+  return ts::launch_gemm(g, a_map, b_map, plan, n_sms, (cudaStream_t)cuda_stream) == cudaSuccess ? TS_OK : TS_ERR_CUDA;
 }
 
 int ts_layer_last_cuda_error(const ts_layer* l) { return l ? l->last_cuda_error : 0; }

@@ -71,6 +71,14 @@ def test_gemm_matches_the_oracle(case, tile_m):
     assert_close_bf16(from_dev(dc), want, f"gemm {case} tile_m {tile_m}")
 
 
+@pytest.mark.parametrize("case", [(1, 256, 1024, False), (64, 512, 4096, True), (127, 264, 1032, False), (129, 1024, 2056, True),
+                                  (256, 4096, 4096, False)], ids=lambda c: f"{c[0]}x{c[1]}x{c[2]}")
+def test_gemm_of_few_tiles_matches_the_oracle(case):
+    """The default plan on products whose K range is shared by a cluster: one row, ragged row blocks,
+    ragged last columns and K blocks, K blocks that do not divide by the cluster."""
+    test_gemm_matches_the_oracle(case, 0)
+
+
 def test_gemm_rejects_bad_arguments():
     t = torch.zeros(64, dtype=torch.int16, device="cuda")
     s = torch.zeros(1, dtype=torch.int32, device="cuda")
@@ -92,7 +100,8 @@ def make_weights(rng, s, hidden, inter):
 @pytest.mark.parametrize("shape,hidden,inter,ctx,ql", [
     (wl.Shape(4, 2, 128), 256, 384, [40, 0, 7], [1, 150, 1]),
     (wl.Shape(8, 2, 128), 512, 1024, [300, 17, 33], [1, 1, 200]),
-], ids=["4-2-128", "8-2-128"])
+    (wl.Shape(8, 2, 128), 2048, 1024, [40, 0, 7], [1, 33, 1]),      # deep, few tokens: every projection is split over K
+], ids=["4-2-128", "8-2-128", "8-2-128-deep"])
 def test_layer_step_matches_the_oracle(shape, hidden, inter, ctx, ql):
     """One layer iteration over decode rows and a prefill chunk: output and KV pages against the fp64
     layer oracle, whose attention is the paged-attention oracle on the oracle's own pool."""
