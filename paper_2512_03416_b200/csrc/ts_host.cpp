@@ -239,6 +239,24 @@ int make_q_map(ts_ctx* c, const void* q, int64_t n_tokens, CUtensorMap* out) {
   return TS_OK;
 }
 
+// The step's new K/V viewed as (head_dim, KV head, token); box = 64 elements of one head x 16 tokens
+// (a page's worth).
+int make_new_kv_maps(ts_ctx* c, const ts_step* st, int64_t n_tokens, ts::NewKvMaps* out) {
+  const cuuint64_t D = c->cfg.head_dim, H = c->cfg.n_kv_heads;
+  const cuuint64_t dims[3] = {D, H, (cuuint64_t)n_tokens};
+  const cuuint64_t strides[2] = {D * 2, H * D * 2};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  const cuuint32_t box[3] = {64, 1, (cuuint32_t)ts::kPageSize};
+  for (int kv = 0; kv < 2; ++kv) {
+    const CUresult r = ((EncodeFn)c->encode_fn)(kv ? &out->v : &out->k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
+                                                const_cast<void*>(kv ? st->v_new : st->k_new), dims, strides, box, estr,
+                                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return cuda_fail(c, cudaErrorInvalidValue);
+  }
+  return TS_OK;
+}
+
 int ensure_cuda(ts_ctx* c, cudaStream_t stream) {
   if (!c->cfg.kv_pool || !c->cfg.workspace) return cuda_fail(c, cudaErrorInvalidDevicePointer);
   TS_CUDA(c, cudaSetDevice(c->cfg.device));
@@ -510,8 +528,8 @@ void fill_device(ts_ctx* c, const ts_step* st, int64_t n_tokens, ts::StepDevice*
   d->scale_log2 = c->scale * 1.4426950408889634f;
   d->append_in_decode = 0;
   d->wait_cycles = c->cfg.wait_limit_cycles > 0 ? (long long)c->cfg.wait_limit_cycles : ts::kWaitCycles;
-  d->append_ctas = 0;          // both set by the mixed launch
-  d->append_arrivals = 0;
+  d->append_wide = 0;          // both set by the mixed launch
+  d->debug_arrivals = 0;
 }
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
@@ -526,16 +544,13 @@ bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 //           at no more than 6.1 TB/s; the step time is flat over a range of splits, of which the
 //           middle is taken (its ends are the sensitive ones).
 //   G >  4: measured fraction of the full-chip rate by SM count, linear in between:
-//           48 0.475, 64 0.62, 74 0.715, 84 0.78, 100 0.85, 116 0.92, 132 0.95, 148 1
-// A prefill CTA starts on its first unit once the prefill rows' new tokens are in their pages,
-// which next to the decode streams takes ~8 us plus ~11 ns per token.
+//           48 0.43, 64 0.62, 74 0.715, 84 0.78, 100 0.85, 116 0.92, 132 0.95, 148 1
 int choose_prefill_ctas(const ts_ctx* c, int n_ctas, double prefill_block_pairs, double prefill_units,
-                        double decode_bytes, double decode_units, double prefill_tokens) {
+                        double decode_bytes, double decode_units) {
   static const double kSm8[] = {0, 48, 64, 74, 84, 100, 116, 132, 148};
-  static const double kRate8[] = {0, 0.475, 0.62, 0.715, 0.78, 0.85, 0.92, 0.95, 1.0};
+  static const double kRate8[] = {0, 0.43, 0.62, 0.715, 0.78, 0.85, 0.92, 0.95, 1.0};
   const bool wide = c->G > 4;
   const double w_pf = prefill_block_pairs * 2.1 + prefill_units * 2.0;
-  const double t_append = 8.0 + 0.011 * prefill_tokens;
   const double t_dec_full = decode_bytes / 6.1e6;   // us at 6.1 TB/s
   const double unit_bytes = decode_bytes / std::max(1.0, decode_units);
   const double sm_rate = unit_bytes / (unit_bytes / 70e3 + 2.0);   // bytes per us and SM
@@ -551,7 +566,7 @@ int choose_prefill_ctas(const ts_ctx* c, int n_ctas, double prefill_block_pairs,
     } else {
       td = std::max(t_dec_full, decode_bytes / ((double)(n_ctas - p) * sm_rate));
     }
-    return std::max(td, (w_pf + (double)p * t_append + (double)(n_ctas - p) * td) / n_ctas);
+    return std::max(td, (w_pf + (double)(n_ctas - p) * td) / n_ctas);
   };
   int best = 0;
   double best_t = 1e30;
@@ -631,6 +646,9 @@ int run_step(ts_ctx* c, const ts_step* st, void* cuda_stream, bool attention) {
         CUtensorMap q_map;
         rc = make_q_map(c, st->q, n_tokens, &q_map);
         if (rc != TS_OK) return rc;
+        ts::NewKvMaps new_maps;
+        rc = make_new_kv_maps(c, st, n_tokens, &new_maps);
+        if (rc != TS_OK) return rc;
         // One persistent launch: CTAs [0, p) take prefill tiles, the others run the decode
         // splits first and then help with the tiles (decode rows ride along when G <= 8).
         const long long pf_units = (long long)c->n_prefill_items * c->cfg.n_kv_heads;
@@ -638,17 +656,18 @@ int run_step(ts_ctx* c, const ts_step* st, void* cuda_stream, bool attention) {
         const bool fuse = dec_units > 0 && c->G <= 8 && c->cfg.mixed_prefill_ctas >= 0;
         int n_ctas = (int)std::min<long long>(c->n_sms, pf_units + (fuse ? dec_units : 0));
         int p = n_ctas;
+        double pairs = 0.0;                                    // 128-key block pairs of the prefill units
+        for (int i = 0; i < c->n_prefill_items; ++i) pairs += ceil_div(c->items[i].k_end, 128);
+        pairs *= c->cfg.n_kv_heads;
         if (fuse) {
           if (c->cfg.mixed_prefill_ctas > 0) {
             p = c->cfg.mixed_prefill_ctas;
           } else {
-            double pairs = 0.0, bytes = 0.0;
-            for (int i = 0; i < c->n_prefill_items; ++i) pairs += ceil_div(c->items[i].k_end, 128);
+            double bytes = 0.0;
             for (int i = c->n_prefill_items; i < n_items; ++i)
               bytes += (double)(c->items[i].k_end - c->items[i].k_begin);
             bytes *= 2.0 * c->cfg.n_kv_heads * c->cfg.head_dim * 2.0;
-            p = choose_prefill_ctas(c, n_ctas, pairs * c->cfg.n_kv_heads, (double)pf_units, bytes, (double)dec_units,
-                                    (double)n_prefill);
+            p = choose_prefill_ctas(c, n_ctas, pairs, (double)pf_units, bytes, (double)dec_units);
           }
           p = (int)std::min<long long>(p, pf_units);
           p = std::min(p, n_ctas - 1);                         // at least one CTA runs the decode splits
@@ -656,12 +675,15 @@ int run_step(ts_ctx* c, const ts_step* st, void* cuda_stream, bool attention) {
           decode_launched = true;
         }
         if (pe) c->prof_mixed.back() = decode_launched;
-        // every CTA appends a share of the prefill rows' tokens (in a CTA that streams decode rows
-        // first its loader warpgroup does, so the page stream starts with the kernel), but only a
-        // CTA about to start on prefill work waits for all of them
-        d.append_ctas = n_ctas;
-        d.append_arrivals = d.append_ctas + ((c->cfg.debug_flags & TS_DEBUG_LOSE_APPEND_ARRIVAL) ? 1 : 0);
-        TS_CUDA(c, ts::launch_mixed(d, q_map, c->kv_map, c->kv_tile_map, n_ctas, p, stream));
+        // A CTA that starts on prefill units appends its share of the new tokens with one warp next
+        // to the tiles (~2 us per 4 KB of K/V, the latency of two rounds of loads and stores). Where
+        // that takes longer than the tiles themselves (~2 us per block pair, and a launch with fewer
+        // units than SMs gives every CTA one), the sixteen softmax warps do it before their first scores.
+        const double append_us = 2.0 * (double)n_prefill / (p + 4.0 * (n_ctas - p)) *
+                                 ceil_div(4 * c->cfg.n_kv_heads * c->cfg.head_dim, 4096);
+        d.append_wide = append_us > 2.0 * pairs / n_ctas;
+        d.debug_arrivals = (c->cfg.debug_flags & TS_DEBUG_LOSE_APPEND_ARRIVAL) ? n_ctas + 1 : 0;
+        TS_CUDA(c, ts::launch_mixed(d, q_map, c->kv_map, c->kv_tile_map, new_maps, n_ctas, p, stream));
       } else {
         ts::StepDevice dp = d;
         dp.n_items = c->n_prefill_items;

@@ -76,9 +76,8 @@ struct StepDevice {
   int32_t Hq, Hkv, D, n_pages, max_pages_per_req, max_requests;
   float scale_log2;        // softmax scale * log2(e)
   long long wait_cycles;   // limit of every bounded wait of the step's kernels, in clock cycles
-  int32_t append_ctas;     // CTAs of the mixed kernel that append the new tokens of the prefill rows: all of them
-  int32_t append_arrivals; // what the mixed kernel's CTAs wait for before their first prefill unit:
-                           // append_ctas, or one more when ts_config.debug_flags asks for a wait that runs out
+  int32_t append_wide;     // mixed kernel: CTAs that start on prefill units append with their softmax warps first
+  int32_t debug_arrivals;  // > 0: the mixed kernel waits for that many arrivals, which nothing sends (TS_DEBUG_LOSE_APPEND_ARRIVAL)
 };
 
 // Launchers. Each enqueues on `stream` and returns the launch's cudaError_t.
@@ -96,9 +95,13 @@ cudaError_t launch_combine(const StepDevice& s, cudaStream_t stream);
 // n_prefill_ctas == n_ctas the decode splits are left to launch_decode. When it runs the decode
 // splits it also merges them (no launch_combine needed).
 // q_map views q as (head_dim, G, KV head, token), box 64 x G x 1 x 128/G. kv_tile_map is the pool
-// view of kv_map with a box of one operand only (64 x 16 x 1 x 1 x 1): the prefill tiles' K/V copies.
+// view of kv_map with a box of one operand only (64 x 16 x 1 x 1 x 1): the prefill tiles' copies of
+// cached K/V; new_maps view the step's own K/V.
+struct NewKvMaps {          // k_new / v_new as (head_dim, KV head, token), box 64 x 1 x 16
+  CUtensorMap k, v;
+};
 cudaError_t launch_mixed(const StepDevice& s, const CUtensorMap& q_map, const CUtensorMap& kv_map,
-                         const CUtensorMap& kv_tile_map, int n_ctas, int n_prefill_ctas, cudaStream_t stream);
+                         const CUtensorMap& kv_tile_map, const NewKvMaps& new_maps, int n_ctas, int n_prefill_ctas, cudaStream_t stream);
 cudaError_t launch_decode(const StepDevice& s, const CUtensorMap& kv_map, int n_sms, cudaStream_t stream);
 
 // ---- the decoder layer around the attention step: GEMMs and small kernels (ts_gemm.cu, ts_layer_kernels.cu)
@@ -241,19 +244,6 @@ __device__ __forceinline__ void append_tokens(const StepDevice& s, const int32_t
     }
     if (s.append_in_decode && row_start[lo + 1] - row_start[lo] == 1) continue;
     append_one(s, tok, rows[n + lo] + (tok - row_start[lo]), rows[2 * n + lo], lane);
-  }
-}
-// The same for the tokens of the prefill work items only (they cover every token of every row with
-// more than one new token exactly once, `tokens_per_item` at most each): nothing to stage and no
-// search, the item names the row and the position. Warps `first_warp`, `first_warp + n_warps`, ...
-__device__ __forceinline__ void append_prefill_items(const StepDevice& s, int tokens_per_item, int first_warp, int n_warps,
-                                                     int lane) {
-  const int total = s.n_prefill_items * tokens_per_item;
-  for (int w = first_warp; w < total; w += n_warps) {
-    const WorkItem it = s.items[w / tokens_per_item];
-    const int j = w % tokens_per_item;
-    if (j >= it.q_count) continue;
-    append_one(s, s.row_tok0[it.row] + it.q_begin + j, it.k_end - it.q_count + j, s.row_slot[it.row], lane);
   }
 }
 // Log-sum-exp merge of the splits of one (token, head) for head_dim element d: the exact merge

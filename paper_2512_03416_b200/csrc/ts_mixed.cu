@@ -33,9 +33,9 @@
 // The O rescale is lazy: a row's reference maximum only moves when a block's maximum exceeds it by
 // more than 2^8, so most blocks never touch O.
 // The kernel appends the step's new K/V to the pages itself, which saves a launch in front of it:
-// every CTA copies a share of the prefill rows' tokens (in a CTA that streams decode rows first, the
-// loader warpgroup does, next to the stream), and only the CTAs about to start on prefill work wait
-// for all of them; the decode units write their rows' own tokens.
+// every CTA copies a share of the prefill rows' tokens next to its other work, and nothing waits for
+// the copies, because the tiles take a chunk's own tokens from the step's tensors; the decode units
+// write their rows' own tokens.
 // Every wait is bounded; a wait that runs out raises TS_DEV_TIMEOUT and the CTA drains.
 #include <cuda_bf16.h>
 #include <math_constants.h>
@@ -87,7 +87,8 @@ enum {
   BAR_Q_EMPTY = BAR_O_EMPTY + 2,          // the last Q K^T of a work unit has consumed the Q tiles
   BAR_PAIR = BAR_Q_EMPTY + 1,             // [8] per tile and row quarter: the two warps that share the rows
   BAR_V_LANDED = BAR_PAIR + 8,            // [kVStages] the copies of a V tile are in shared memory
-  BAR_COUNT = BAR_V_LANDED + kVStages
+  BAR_K_LANDED = BAR_V_LANDED + kVStages, // the same for a K tile that needs a touch-up before it is announced
+  BAR_COUNT = BAR_K_LANDED + 1
 };
 // misc words: [0] TMEM base address, [1] failure flag, [2] work units published so far;
 // then a ring of the published units' records (8 words each)
@@ -210,12 +211,83 @@ __device__ __forceinline__ PfUnit unit_shape(const UnitRec& r, int tile_tokens) 
   return u;
 }
 
+// The append of the prefill rows' new tokens (Sec. 2.1). The prefill work items cover those tokens
+// exactly once, `per_item` at most each; warp i of n appends tokens i, i + n, ... of that list. A lane
+// looks up one of the warp's next 32 tokens (item -> row -> block table: three dependent loads, paid
+// once per 32 tokens instead of once per token, 5 us each), then the warp copies them one by one, U
+// 16-byte loads in flight per lane.
+struct AppendCursor {
+  __device__ __forceinline__ AppendCursor(int first, int n, int warps) : next(first), end(n), stride(warps) {}
+  int next, end, stride;       // list position of the next token, end of the list, warps that share it
+  int left = 0, at = 0;        // looked-up tokens not yet copied, lane that holds the next one
+  int tok = -1;                // this lane's token in the step's tensors (-1: nothing to copy)
+  uint32_t dst = 0;            // its page * 16 + slot
+
+  __device__ __forceinline__ bool done() const { return left == 0 && next >= end; }
+  __device__ __forceinline__ void look_up(const StepDevice& s, int per_item, int lane) {
+    const int w = next + lane * stride;
+    tok = -1;
+    if (w < end) {
+      const WorkItem it = s.items[w / per_item];
+      const int j = w % per_item;
+      if (j < it.q_count) {
+        const int slot = s.row_slot[it.row], t = it.k_end - it.q_count + j;
+        if ((unsigned)slot >= (unsigned)s.max_requests || (unsigned)(t >> 4) >= (unsigned)s.max_pages_per_req) {
+          atomicOr(s.status, TS_DEV_BAD_INDEX);
+        } else {
+          const int page = s.table[(size_t)slot * s.max_pages_per_req + (t >> 4)];
+          if ((unsigned)page >= (unsigned)s.n_pages) {
+            atomicOr(s.status, TS_DEV_BAD_PAGE);
+          } else {
+            tok = s.row_tok0[it.row] + it.q_begin + j;
+            dst = (uint32_t)page * kPageSize + (uint32_t)(t & 15);
+          }
+        }
+      }
+    }
+    left = min(32, (end - next + stride - 1) / stride);
+    at = 0;
+    next += 32 * stride;
+  }
+  // Copies one token (call only while !done()).
+  template <int U>
+  __device__ __forceinline__ void step(const StepDevice& s, int per_item, int lane) {
+    if (left == 0) look_up(s, per_item, lane);
+    const int token = __shfl_sync(0xffffffffu, tok, at);
+    const uint32_t d = __shfl_sync(0xffffffffu, dst, at);
+    ++at;
+    --left;
+    if (token < 0) return;
+    const int half = s.Hkv * (kD / 8);             // 16-byte chunks of the token's K (and of its V)
+    const size_t src = (size_t)token * s.Hkv * kD, page0 = (size_t)(d / kPageSize) * 2 * s.Hkv;
+#pragma unroll 1
+    for (int c0 = lane; c0 < 2 * half; c0 += U * 32) {
+      uint4 v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int c = c0 + u * 32;
+        if (c < 2 * half) v[u] = *reinterpret_cast<const uint4*>(c < half ? s.k_new + src + c * 8 : s.v_new + src + (c - half) * 8);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {                // chunk c: K|V and head = c / 16 counted through, c % 16 of that head's row
+        const int c = c0 + u * 32;
+        if (c < 2 * half)
+          *reinterpret_cast<uint4*>(s.pool + ((page0 + c / 16) * kPageSize + d % kPageSize) * kD + (c & 15) * 8) = v[u];
+      }
+    }
+  }
+  template <int U>
+  __device__ __forceinline__ void run(const StepDevice& s, int per_item, int lane) {
+    while (!done()) step<U>(s, per_item, lane);
+  }
+};
+
 __device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 0;\n" ::: "memory"); }
 
 __global__ void __launch_bounds__(kPfThreads, 1)
 mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
              const __grid_constant__ CUtensorMap kv_map, const __grid_constant__ CUtensorMap kv_tile_map,
-             const int n_prefill_ctas) {
+             const __grid_constant__ NewKvMaps new_maps, const int n_prefill_ctas) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
@@ -269,16 +341,15 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
     if (tid == 0) {
       misc[1] = 0;
       misc[2] = 0;
-      {   // the prefill rows' new K/V must be in their pages before the first tile is read
+      if (s.debug_arrivals > 0) {   // a wait that nothing ends, asked for by ts_config.debug_flags
         const volatile int32_t* arrived = s.pf_queue + 2;
         const long long t0 = clock64();
-        while (*arrived < s.append_arrivals) {
+        while (*arrived < s.debug_arrivals) {
           if (clock64() - t0 > s.wait_cycles) {
             atomicOr(s.status, TS_DEV_TIMEOUT);
             break;
           }
         }
-        __threadfence();
       }
       for (int i = 0; i < BAR_COUNT; ++i) {
         const bool softmax_arrives = (i >= BAR_P_FULL && i < BAR_P_FULL + 2) || (i >= BAR_O_EMPTY && i < BAR_O_EMPTY + 2);
@@ -305,38 +376,32 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
     tc_fence_after();
   };
   // ---------------------------------------------------------------- KV append (Sec. 2.1)
-  // Every CTA copies a share of the new tokens of the prefill rows into their pages, straight from
-  // the prefill work items (which cover those tokens exactly once), and counts itself; a CTA waits
-  // for that count only before its first prefill unit (prefill_setup). In a CTA that takes prefill
-  // units from the start all twenty warps copy. In a CTA that streams decode rows first only the
-  // fifth warpgroup copies (aux_setup) while warps 0-7 are already on their decode units: nothing
-  // those read depends on this append (the new token of a decode row is written by the decode unit
-  // that reads the row's last page), so the page stream starts with the kernel.
-  constexpr int kWarpsAll = kPfThreads / 32, kWarpsAux = 4;
-  const int append_warps = n_prefill_ctas * kWarpsAll + ((int)gridDim.x - n_prefill_ctas) * kWarpsAux;
+  // The new tokens of the prefill rows are copied into their pages straight from the prefill work
+  // items (which cover those tokens exactly once), and nothing in this launch waits for the copies:
+  // the K/V loaders read a chunk's own tokens from the step's tensors. In a CTA that streams decode
+  // rows first the fifth warpgroup copies a share while warps 0-7 are on their decode units. In a CTA
+  // that takes prefill units from the start the Q loader copies one between its Q tiles; where the
+  // units are too short to hide that (s.append_wide, decided on the host) the sixteen softmax warps
+  // copy before their first scores arrive. The new token of a decode row is written by the decode
+  // unit that reads the row's last page.
+  constexpr int kWarpsAux = 4;
+  const int warps_first = s.append_wide ? kSoftmaxWarps : 1;     // appending warps of a CTA that starts on prefill units
+  const int append_end = s.n_prefill_items * 2 * tile_tokens;
+  const int append_warps = n_prefill_ctas * warps_first + ((int)gridDim.x - n_prefill_ctas) * kWarpsAux;
   // The fifth warpgroup (loaders, MMA issuer, Q loader): gives registers to the softmax warpgroups
   // and, in a decode-first CTA, appends and then waits while warps 0-7 run the CTA's decode units.
   auto aux_setup = [&]() {
     reg_dec<kRegsAux>();
     if (decode_first) {
-      append_prefill_items(s, 2 * tile_tokens,
-                           n_prefill_ctas * kWarpsAll + ((int)blockIdx.x - n_prefill_ctas) * kWarpsAux + (warp - kSoftmaxWarps),
-                           append_warps, lane);
-      __threadfence();         // this thread's page writes are visible before the CTA counts itself
-      asm volatile("bar.sync 2, 128;\n" ::: "memory");
-      if (tid == kSoftmaxWarps * 32) atomicAdd(s.pf_queue + 2, 1);
+      AppendCursor{n_prefill_ctas * warps_first + ((int)blockIdx.x - n_prefill_ctas) * kWarpsAux + (warp - kSoftmaxWarps),
+                   append_end, append_warps}
+          .run<8>(s, 2 * tile_tokens, lane);
       cta_sync();
     }
     prefill_setup();
   };
 
   pdl_wait();                  // the previous step's kernels are done with the pool and the counters
-  if (!decode_first) {
-    append_prefill_items(s, 2 * tile_tokens, (int)blockIdx.x * kWarpsAll + warp, append_warps, lane);
-    __threadfence();
-    cta_sync();
-    if (tid == 0) atomicAdd(s.pf_queue + 2, 1);
-  }
 
   if (warp < kSoftmaxWarps) {
     // ------------------ softmax + epilogue: thread = half of a query row of tile x (64 of the 128
@@ -362,6 +427,8 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
       reg_inc<kRegsSoftmax>();
     }
     prefill_setup();
+    if (!decode_first && s.append_wide)
+      AppendCursor{(int)blockIdx.x * kSoftmaxWarps + warp, append_end, append_warps}.run<8>(s, 2 * tile_tokens, lane);
     const uint32_t tmem = misc[0];
     const int x = (warp >> 2) & 1;          // tile
     const int hf = warp >> 3;               // which half of the keys / of the head_dim columns
@@ -567,20 +634,32 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
     aux_setup();
     if (warp < kWarpLoader0 + 2) {
       // ------------------------------------------------------------------ K/V loaders
-      // One warp per operand. A 128-key tile is sixteen tensor copies of 2 KB (one page of one KV
-      // head, 64 head_dim columns each; the page id is a coordinate of the copy, so scattered pages
-      // cost nothing extra), issued by sixteen lanes at once and landing in the 128-byte-swizzled
-      // operand layout the MMA reads. K tiles complete their "full" barrier by transaction bytes.
-      // V tiles complete a "landed" barrier first: the warp then clears, in shared memory, the V
-      // rows of a ragged last page (slots past the last key may hold anything, and 0 * NaN would
-      // poison O; the same rows of K only produce scores that are masked) and announces the tile.
+      // One warp per operand. A 128-key tile of cached tokens is sixteen tensor copies of 2 KB (one
+      // page of one KV head, 64 head_dim columns each; the page id is a coordinate of the copy, so
+      // scattered pages cost nothing extra), issued by sixteen lanes at once and landing in the
+      // 128-byte-swizzled operand layout the MMA reads. The tokens of the chunk itself come from the
+      // step's K/V tensors, sixteen at a time, not from the pages they are appended to; where the
+      // chunk starts inside a page the cached rows of that page are laid over the copy by plain
+      // loads. (Reading the chunk back from its pages meant that every CTA waited for the whole
+      // launch's append: 11 us in front of the first tile on a 2048-token chunk alone, ~30 us next
+      // to decode streams. 2048-token chunk alone, 8B shape: 54.3 -> 52.0 us with the step's tensors
+      // cold, 52.5 -> 48.6 us repeated. One copy of 128 tokens instead of eight measured the same.)
+      // K tiles complete their "full" barrier by transaction bytes. V tiles complete a "landed"
+      // barrier first: the warp then clears, in shared memory, the V rows past the unit's last key
+      // (they may hold anything, and 0 * NaN would poison O; the same rows of K only produce scores
+      // that are masked) and announces the tile. A K tile with cached rows to lay over does the same.
       // The loaders run up to a ring of stages ahead of the tensor pipe.
       const int kv = warp - kWarpLoader0;                      // 0: K, 1: V
       const int stages = kv ? kVStages : kKStages;
       const int lag = stages - 1;                              // V tiles in flight besides the announced one
       const int full = kv ? BAR_V_FULL : BAR_K_FULL, empty = kv ? BAR_V_EMPTY : BAR_K_EMPTY;
       const uint32_t tile0 = base + (kv ? kOffV : kOffK);
-      if (lane == 0) tma_prefetch_desc(&kv_tile_map);
+      const CUtensorMap* new_map = kv ? &new_maps.v : &new_maps.k;
+      if (lane == 0) {
+        tma_prefetch_desc(new_map);
+        tma_prefetch_desc(&kv_tile_map);
+      }
+      int n_touched = 0;                                       // K tiles that went through BAR_K_LANDED
       // The K loader's first thread takes work units off the global queue, one at a time and only
       // when the K loader is ready for it (it runs a few key blocks ahead of the tensor pipe, which
       // hides the round trip), and publishes each to the other roles through a small ring.
@@ -616,11 +695,12 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
         PfUnit u;
         if (!get_work(k, u)) break;
         const int32_t* table_row = s.table + (size_t)u.table_slot * s.max_pages_per_req;
-        // lane i < 16 copies page i / 2 of the tile, head_dim columns [64 (i % 2), +64)
+        // lane i < 16 copies page i / 2 of the tile, head_dim columns [64 (i % 2), +64): page id of a
+        // page that only holds cached tokens (others: not needed)
         auto fetch_page = [&](int j) {
           const int key = j * kBlockKeys + (lane >> 1) * kPageSize;
           int page = s.n_pages;                                // out of range on purpose: the copy delivers zeros
-          if (lane < 16 && key < u.k_end) {
+          if (lane < 16 && key < u.k_end && key + kPageSize <= u.ctx) {
             page = table_row[key >> 4];
             if ((unsigned)page >= (unsigned)s.n_pages) {
               atomicOr(s.status, TS_DEV_BAD_PAGE);
@@ -629,19 +709,34 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
           }
           return page;
         };
+        // does the chunk start inside a page of this tile?
+        const int start_tile = (u.ctx & 15) ? u.ctx / kBlockKeys : -1;
+        // ... then the page's cached rows are laid over the copy of the new tokens
+        auto lay_cached = [&](unsigned char* tile_smem) {
+          const int r0 = (u.ctx & ~15) % kBlockKeys, n_rows = u.ctx & 15;
+          const int page = table_row[u.ctx >> 4];
+          const bool ok = (unsigned)page < (unsigned)s.n_pages;
+          if (!ok && lane == 0) atomicOr(s.status, TS_DEV_BAD_PAGE);
+          const uint16_t* src = s.pool + (((size_t)(ok ? page : 0) * 2 + kv) * s.Hkv + u.kv_head) * kPageSize * kD;
+          for (int i = lane; i < n_rows * 16; i += 32) {
+            const int r = i >> 4, c = i & 15;                  // a row is 8 chunks of 16 bytes in each 64-column half
+            const uint4 val = ok ? *reinterpret_cast<const uint4*>(src + r * kD + c * 8) : make_uint4(0, 0, 0, 0);
+            *reinterpret_cast<uint4*>(tile_smem + (c >> 3) * kHalfBytes + (r0 + r) * 128 + (((c ^ r) & 7) << 4)) = val;
+          }
+        };
         auto announce = [&](int tile) {                        // V only; tile = block index within the unit
           const int gt = g0 + tile, st = gt % stages;
           wait(BAR_V_LANDED + st, (gt / stages) & 1);
+          unsigned char* vt = smem + kOffV + st * kTileBytes;
           const int first_bad = u.k_end - tile * kBlockKeys;   // rows from here on hold no key of the unit
-          if (first_bad < kBlockKeys && (first_bad & 15)) {
-            const int n_rows = 16 - (first_bad & 15);          // up to the end of that page; later pages were not copied
-            unsigned char* vt = smem + kOffV + st * kTileBytes;
-            for (int i = lane; i < n_rows * 16; i += 32) {
-              const int r = first_bad + (i >> 4), c = i & 15;  // a row is 8 chunks of 16 bytes in each 64-column half
+          if (tile == start_tile) lay_cached(vt);
+          if (first_bad < kBlockKeys) {
+            for (int i = lane; i < (kBlockKeys - first_bad) * 16; i += 32) {
+              const int r = first_bad + (i >> 4), c = i & 15;
               *reinterpret_cast<uint4*>(vt + (c >> 3) * kHalfBytes + r * 128 + ((c & 7) << 4)) = make_uint4(0, 0, 0, 0);
             }
-            fence_proxy_async();
           }
+          if (tile == start_tile || first_bad < kBlockKeys) fence_proxy_async();
           __syncwarp();
           if (lane == 0) mbar_arrive(bar(full + st));
         };
@@ -652,14 +747,31 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
           if (kv && j >= lag) announce(j - lag);
           const int page_next = j + 1 < u.nb ? fetch_page(j + 1) : 0;   // the table load flies while this tile is issued
           if (g >= stages) wait(empty + st, ((g / stages) & 1) ^ 1);
-          const uint32_t landed = bar(kv ? BAR_V_LANDED + st : full + st);
+          const bool touch = kv == 0 && j == start_tile;
+          const uint32_t landed = bar(kv ? BAR_V_LANDED + st : touch ? BAR_K_LANDED : full + st);
           if (misc[1] == 0) {                                  // after a failure no new copies are started
             if (lane == 0) mbar_expect_tx(landed, kTileBytes);
             __syncwarp();
-            if (lane < 16)
-              tma_load_5d(tile0 + st * kTileBytes + (lane & 1) * kHalfBytes + (lane >> 1) * 2048, &kv_tile_map, landed,
-                          (lane & 1) * 64, 0, u.kv_head, kv, page);
+            const uint32_t dst = tile0 + st * kTileBytes;
+            const int first_tok = u.tok0 + j * kBlockKeys - u.ctx;      // token of the tile's first key, if it is a new one
+            if (lane < 16) {
+              const int key = j * kBlockKeys + (lane >> 1) * kPageSize;
+              const uint32_t page_dst = dst + (lane & 1) * kHalfBytes + (lane >> 1) * 2048;
+              if (key + kPageSize > u.ctx && key < u.k_end)
+                tma_load_3d(page_dst, new_map, landed, (lane & 1) * 64, u.kv_head, first_tok + (lane >> 1) * kPageSize);
+              else
+                tma_load_5d(page_dst, &kv_tile_map, landed, (lane & 1) * 64, 0, u.kv_head, kv, page);
+            }
+            if (touch) {
+              __syncwarp();
+              wait(BAR_K_LANDED, n_touched & 1);
+              lay_cached(smem + kOffK + st * kTileBytes);
+              fence_proxy_async();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(bar(full + st));
+            }
           }
+          n_touched += touch;
           page = page_next;
         }
         // the last `lag` V tiles (fewer when the unit is short) have not been announced yet
@@ -757,24 +869,37 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
           }
         }
       }
-      if (warp == kWarpSched && lane == 0) {
+      if (warp == kWarpSched) {
         // ------------------------------------------------------------------ Q loader
         // Brings in each work unit's Q tiles by TMA once the previous unit's last Q K^T is done.
-        tma_prefetch_desc(&q_map);
+        // Between two units it appends, a token at a time, this CTA's share of the new K/V.
+        if (lane == 0) tma_prefetch_desc(&q_map);
+        AppendCursor app{decode_first || s.append_wide ? append_end : (int)blockIdx.x, append_end, append_warps};
+        auto append_until = [&](auto&& ready) {
+          while (!app.done() && !__any_sync(0xffffffffu, ready())) app.step<4>(s, 2 * tile_tokens, lane);   // 4: 64 registers here
+        };
         for (int k = 0;; ++k) {
           PfUnit u;
+          append_until([&]() { return (int)misc[2] > k; });
           if (!get_work(k, u)) break;
           const int ta = u.tok0 + u.q_begin;
-          if (k > 0) wait(BAR_Q_EMPTY, (k - 1) & 1);
-          // a box delivers 64 columns of tile_tokens * G packed rows (all 128 only when G divides 128)
-          mbar_expect_tx(bar(BAR_Q), (u.cnt_b > 0 ? 2 : 1) * 2 * (tile_tokens * G * 128));
-          tma_load_4d(base + kOffQ, &q_map, bar(BAR_Q), 0, 0, u.kv_head, ta);
-          tma_load_4d(base + kOffQ + kHalfBytes, &q_map, bar(BAR_Q), 64, 0, u.kv_head, ta);
-          if (u.cnt_b > 0) {
-            tma_load_4d(base + kOffQ + kTileBytes, &q_map, bar(BAR_Q), 0, 0, u.kv_head, ta + tile_tokens);
-            tma_load_4d(base + kOffQ + kTileBytes + kHalfBytes, &q_map, bar(BAR_Q), 64, 0, u.kv_head, ta + tile_tokens);
+          if (k > 0) {
+            append_until([&]() { return mbar_test(bar(BAR_Q_EMPTY), (k - 1) & 1); });
+            wait(BAR_Q_EMPTY, (k - 1) & 1);
           }
+          // a box delivers 64 columns of tile_tokens * G packed rows (all 128 only when G divides 128)
+          if (lane == 0) {
+            mbar_expect_tx(bar(BAR_Q), (u.cnt_b > 0 ? 2 : 1) * 2 * (tile_tokens * G * 128));
+            tma_load_4d(base + kOffQ, &q_map, bar(BAR_Q), 0, 0, u.kv_head, ta);
+            tma_load_4d(base + kOffQ + kHalfBytes, &q_map, bar(BAR_Q), 64, 0, u.kv_head, ta);
+            if (u.cnt_b > 0) {
+              tma_load_4d(base + kOffQ + kTileBytes, &q_map, bar(BAR_Q), 0, 0, u.kv_head, ta + tile_tokens);
+              tma_load_4d(base + kOffQ + kTileBytes + kHalfBytes, &q_map, bar(BAR_Q), 64, 0, u.kv_head, ta + tile_tokens);
+            }
+          }
+          __syncwarp();
         }
+        append_until([]() { return false; });
       }
       __syncwarp();
     }
@@ -797,7 +922,7 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
 }  // namespace
 
 cudaError_t launch_mixed(const StepDevice& s, const CUtensorMap& q_map, const CUtensorMap& kv_map,
-                         const CUtensorMap& kv_tile_map, int n_ctas, int n_prefill_ctas, cudaStream_t stream) {
+                         const CUtensorMap& kv_tile_map, const NewKvMaps& new_maps, int n_ctas, int n_prefill_ctas, cudaStream_t stream) {
   if (s.n_prefill_items <= 0 || n_ctas <= 0) return cudaSuccess;
   const int G = s.Hq / s.Hkv;
   size_t smem = kSmemBytes;
@@ -807,7 +932,7 @@ cudaError_t launch_mixed(const StepDevice& s, const CUtensorMap& q_map, const CU
   }
   cudaError_t e = cudaFuncSetAttribute(mixed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(mixed_kernel, dim3(n_ctas), dim3(kPfThreads), smem, stream, s, q_map, kv_map, kv_tile_map, n_prefill_ctas);
+  return launch_pdl(mixed_kernel, dim3(n_ctas), dim3(kPfThreads), smem, stream, s, q_map, kv_map, kv_tile_map, new_maps, n_prefill_ctas);
 }
 
 }  // namespace ts

@@ -194,3 +194,39 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_step_is_clean():
     assert_parity(got, want, "peaked", "step after a timed-out one")
     assert np.array_equal(ok.pool(), pool_want)
 
+
+
+@pytest.mark.parametrize("shape", [wl.LLAMA8B, wl.Shape(64, 8, 128), wl.Shape(2, 2, 128)], ids=["32-8", "64-8", "2-2"])
+@pytest.mark.parametrize("rows", [
+    # (cached tokens, chunk) per row: the chunk starts on and around page and key-tile boundaries, and
+    # ends inside a page, at its end, one past a key tile
+    [(0, 128), (15, 2), (16, 16), (17, 15)],
+    [(127, 129), (128, 127), (129, 40), (1, 255)],
+    [(300, 200), (113, 15), (271, 17), (0, 2), (50, 1)],
+    [(143, 300), (640, 33), (1000, 1)],
+], ids=["starts", "tiles", "mixed", "long"])
+def test_chunk_tokens_are_read_from_the_step_tensors(shape, rows):
+    """Key tiles of cached tokens, of the chunk's own tokens, and of both, several chunks in one step,
+    without decode rows, next to a few, and in a launch of few and of many work units."""
+    b = wl.make_batch("own", shape, [c for c, _ in rows], [t for _, t in rows], seed=len(rows) + shape.Hq, profile="peaked")
+    want, pool_want = oracle_step(b)
+    run = GpuRun(b, chunk_size=0)
+    assert_parity(run.step(keep_len=True), want, "peaked", f"{rows}")
+    assert np.array_equal(run.pool(), pool_want)
+    assert_parity(run.step(), want, "peaked", f"{rows}, repeated")
+
+
+def test_another_rows_values_cannot_reach_a_chunk():
+    """A key tile of a chunk is copied with whatever tokens follow the chunk in the step's tensors;
+    infinities and NaN there must not reach the chunk's output, nor its pages anything but its own tokens."""
+    b = wl.make_batch("nan", wl.LLAMA8B, [37, 5, 0], [90, 60, 20], seed=77, profile="peaked")
+    want, _ = oracle_step(b)
+    b.k_new[90:150] = wl.BF16_NAN
+    b.v_new[90:150:2] = 0x7F80
+    b.v_new[91:150:2] = wl.BF16_NAN
+    _, pool_want = oracle_step(b)
+    run = GpuRun(b, chunk_size=0)
+    got = run.step()
+    clean = np.r_[0:90, 150:170]
+    assert_parity(got[clean], want[clean], "peaked", "rows around a row of NaN")
+    assert np.array_equal(run.pool(), pool_want)
