@@ -30,8 +30,9 @@
 namespace ts {
 namespace {
 
-constexpr int kGemmThreads = 192;
+constexpr int kGemmThreads = 320;               // producer warp, MMA warp, eight epilogue warps
 constexpr int kBN = 256, kBK = 64;
+constexpr int kTileStages = 4;                  // of gemm_kernel
 constexpr int kMaxSplit = 8;                    // portable cluster size
 constexpr int kABytes = 128 * kBK * 2;          // one 128-row operand block: 16 KB
 constexpr int kBBytes = kBN * kBK * 2;          // the 256-row weight block: 32 KB
@@ -42,10 +43,16 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
       : "memory");
 }
-// The box at (c0, c1) into L2.
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int c0, int c1) {
-  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];\n" ::"l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1)
-               : "memory");
+// Asks for `bytes` bytes of weight row `row`, from byte `at` on, in L2. The weights do not come from the
+// kernel in front of this one, so a launch asks for the first part of what it will read before it waits
+// for that kernel: HBM then works while the chip drains and refills, and it is asked for runs of
+// kilobytes instead of the 128-byte pieces of a K block.
+constexpr int kPrefetchBytes = 512;             // about what the stages hold; 2 KB or more per row got in the way of the copies themselves
+__device__ __forceinline__ void prefetch_weights(const GemmArgs& g, int row, int k0, int k1) {
+  if (row >= g.N) return;
+  const int bytes = min(kPrefetchBytes, (min(k1, g.K) - k0) * 2);
+  const uint16_t* src = g.B + (size_t)row * g.K + k0;
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(src), "r"(bytes) : "memory");
 }
 // bf16 x bf16 -> fp32, M = 128, N = 256, both operands K-major
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
@@ -96,12 +103,109 @@ __device__ __forceinline__ void silu_mul8(float* gate, const float* up) {
   }
 }
 
-template <int TILE_M, int EPI>
+// Epilogue of one accumulator (TMEM lanes = 128 rows, 256 columns): half `hf` of this thread's row of
+// the tile whose columns start at n0 (two warps share a quarter of the lanes; the epilogue of a
+// launch's last tiles is not hidden behind anything). `release` is called once that half is in registers.
+template <int EPI, typename Release>
+__device__ __forceinline__ void epilogue_row(const GemmArgs& g, uint32_t tacc, int row, int n0, int hf, Release&& release) {
+  const bool row_ok = row < g.M;
+  if (EPI == GEMM_EPI_STORE) {
+    uint16_t* crow = g.C + (size_t)row * g.ldc + n0;
+    const uint16_t* rrow = g.R ? g.R + (size_t)row * g.ldc + n0 : nullptr;
+#pragma unroll 1
+    for (int c = hf * 4; c < hf * 4 + 4; ++c) {
+      float v[32];
+      uint4 r[4];
+      const bool with_r = rrow && row_ok;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)                          // the residual's loads fly while TMEM is read
+        if (with_r && n0 + c * 32 + i * 8 < g.N) r[i] = *reinterpret_cast<const uint4*>(rrow + c * 32 + i * 8);
+      tmem_ld32(v, tacc + c * 32);
+      tmem_ld_wait();
+      if (c == hf * 4 + 3) release();
+      if (row_ok) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (n0 + c * 32 + i * 8 < g.N) {
+            if (with_r) {
+              float x[8];
+              unpack8(r[i], x);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) v[i * 8 + e] += x[e];
+            }
+            *reinterpret_cast<uint4*>(crow + c * 32 + i * 8) = pack8(v + i * 8);
+          }
+        }
+      }
+    }
+  } else if (EPI == GEMM_EPI_ROPE) {
+    // A tile holds two heads of 128 columns. Query and key heads are rotated: column i < 64 of a
+    // head pairs with column i + 64, angle table[pos][i]. Each head goes to its own tensor.
+    const float2* cs = g.rope_table + (size_t)(row_ok ? g.pos[row] : 0) * 64;
+    const int col0 = n0 + hf * 128;
+    const bool rotate = col0 < g.q_cols + g.kv_cols;
+    uint16_t* dst = col0 < g.q_cols ? g.C + (size_t)row * g.q_cols + col0
+                    : rotate        ? g.C2 + (size_t)row * g.kv_cols + (col0 - g.q_cols)
+                                    : g.C3 + (size_t)row * g.kv_cols + (col0 - g.q_cols - g.kv_cols);
+#pragma unroll 1
+    for (int c = 0; c < 2; ++c) {
+      float lo[32], hi[32];
+      float2 t2[32];                                      // (cos, sin); the loads fly while TMEM is read
+      if (rotate) {
+#pragma unroll
+        for (int i = 0; i < 32; i += 2) {
+          const float4 w = *reinterpret_cast<const float4*>(cs + c * 32 + i);
+          t2[i] = make_float2(w.x, w.y);
+          t2[i + 1] = make_float2(w.z, w.w);
+        }
+      }
+      tmem_ld32(lo, tacc + hf * 128 + c * 32);
+      tmem_ld32(hi, tacc + hf * 128 + 64 + c * 32);
+      tmem_ld_wait();
+      if (c == 1) release();
+      if (row_ok && col0 < g.N) {
+        if (rotate) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const float a = lo[i], b = hi[i];
+            lo[i] = a * t2[i].x - b * t2[i].y;
+            hi[i] = b * t2[i].x + a * t2[i].y;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          *reinterpret_cast<uint4*>(dst + c * 32 + i * 8) = pack8(lo + i * 8);
+          *reinterpret_cast<uint4*>(dst + 64 + c * 32 + i * 8) = pack8(hi + i * 8);
+        }
+      }
+    }
+  } else {
+    // GEMM_EPI_SILU_MUL: the weight rows of a tile are 128 gate rows followed by the 128 up rows of
+    // the same intermediate features; out[row][n0 / 2 + i] = silu(gate_i) * up_i.
+    uint16_t* crow = g.C + (size_t)row * g.ldc + n0 / 2;
+#pragma unroll 1
+    for (int c = hf * 2; c < hf * 2 + 2; ++c) {
+      float gt[32], up[32];
+      tmem_ld32(gt, tacc + c * 32);
+      tmem_ld32(up, tacc + 128 + c * 32);
+      tmem_ld_wait();
+      if (c == hf * 2 + 1) release();
+      if (row_ok && n0 < g.N) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          silu_mul8(gt + i * 8, up + i * 8);
+          *reinterpret_cast<uint4*>(crow + c * 32 + i * 8) = pack8(gt + i * 8);
+        }
+      }
+    }
+  }
+}
+
+// One CTA per 128 x 256 tile, persistent; the two accumulators alternate between tiles.
+template <int EPI>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, const __grid_constant__ CUtensorMap b_map) {
-  constexpr int kMB = TILE_M / 128;                       // accumulators (and M = 128 MMAs per K step) of a tile
-  constexpr int kStageBytes = kMB * kABytes + kBBytes;    // 48 KB or 64 KB
-  constexpr int kStages = TILE_M == 128 ? 4 : 3;
+  constexpr int kStages = kTileStages, kStageBytes = kABytes + kBBytes;
   constexpr int kOffBar = kStages * kStageBytes;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -115,8 +219,8 @@ gemm_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, const _
   if (tid == 0) {
     misc[1] = 0;
     for (int i = 0; i < 2 * kStages + 2; ++i) mbar_init(bar(i), 1);
-    mbar_init(bar(BAR_ACC_EMPTY), 128);
-    mbar_init(bar(BAR_ACC_EMPTY + 1), 128);
+    mbar_init(bar(BAR_ACC_EMPTY), 256);
+    mbar_init(bar(BAR_ACC_EMPTY + 1), 256);
     mbar_init_fence();
   }
   if (warp == 1) tmem_alloc(base + kOffBar + (2 * kStages + 4) * 8, 512);
@@ -133,28 +237,28 @@ gemm_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, const _
   auto wait = [&](int i, uint32_t parity) {
     if (!mbar_wait(bar(i), parity, misc[1] ? 2000 : g.wait_cycles)) give_up();
   };
-  const int m_tiles = (g.M + TILE_M - 1) / TILE_M, n_tiles = (g.N + kBN - 1) / kBN;
+  const int m_tiles = (g.M + 127) / 128, n_tiles = (g.N + kBN - 1) / kBN;
   const int n_work = m_tiles * n_tiles;
   const int k_blocks = (g.K + kBK - 1) / kBK;
-  pdl_wait();                      // the operands may come from the kernel in front of this one
 
   if (warp == 0) {
     // ---------------------------------------------------------------------- TMA producer
     if (lane == 0) {
       tma_prefetch_desc(&a_map);
       tma_prefetch_desc(&b_map);
+      pdl_wait();                  // the activations come from the kernel in front of this one
       int it = 0;                                          // K blocks issued so far (ring position)
       for (int t = blockIdx.x; t < n_work; t += gridDim.x) {
-        const int m0 = (t % m_tiles) * TILE_M, n0 = (t / m_tiles) * kBN;
+        const int m0 = (t % m_tiles) * 128, n0 = (t / m_tiles) * kBN;
         for (int kb = 0; kb < k_blocks; ++kb, ++it) {
           const int st = it % kStages;
           if (it >= kStages) wait(BAR_EMPTY + st, ((it / kStages) & 1) ^ 1);
           if (misc[1]) continue;                           // after a failure no new copies are started
           const uint32_t dst = base + st * kStageBytes;
           mbar_expect_tx(bar(BAR_FULL + st), kStageBytes);
-#pragma unroll
-          for (int mb = 0; mb < kMB; ++mb) tma_load_2d(dst + mb * kABytes, &a_map, bar(BAR_FULL + st), kb * kBK, m0 + mb * 128);
-          tma_load_2d(dst + kMB * kABytes, &b_map, bar(BAR_FULL + st), kb * kBK, n0);
+          tma_load_2d(dst, &a_map, bar(BAR_FULL + st), kb * kBK, m0);
+          tma_load_2d(dst + kABytes, &b_map, bar(BAR_FULL + st), kb * kBK, n0);
+          tma_load_2d(dst + kABytes + kBBytes / 2, &b_map, bar(BAR_FULL + st), kb * kBK, n0 + 128);
         }
       }
     }
@@ -170,144 +274,40 @@ gemm_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, const _
     };
     int it = 0, n_done = 0;                                // K blocks consumed, tiles issued
     for (int t = blockIdx.x; t < n_work; t += gridDim.x, ++n_done) {
-      // TILE_M = 128: tile n uses accumulator n % 2; TILE_M = 256: both, so every tile waits for the epilogue
-      const int buf = kMB == 1 ? (n_done & 1) : 0;
-      const int uses = kMB == 1 ? (n_done >> 1) : n_done;  // earlier tiles that used this accumulator
-      if (uses > 0) {
-        iwait(BAR_ACC_EMPTY + buf, (uses - 1) & 1);
-        if (kMB == 2) iwait(BAR_ACC_EMPTY + 1, (uses - 1) & 1);
-      }
+      const int buf = n_done & 1, uses = n_done >> 1;      // accumulator, earlier tiles that used it
+      if (uses > 0) iwait(BAR_ACC_EMPTY + buf, (uses - 1) & 1);
       tc_fence_after();
       for (int kb = 0; kb < k_blocks; ++kb, ++it) {
         const int st = it % kStages;
         iwait(BAR_FULL + st, (it / kStages) & 1);
         tc_fence_after();
         if (!dead) {
-          const uint64_t b_desc = smem_desc(base + st * kStageBytes + kMB * kABytes, 0, 1024);
+          const uint64_t a_desc = smem_desc(base + st * kStageBytes, 0, 1024);
+          const uint64_t b_desc = smem_desc(base + st * kStageBytes + kABytes, 0, 1024);
 #pragma unroll
-          for (int mb = 0; mb < kMB; ++mb) {
-            const uint64_t a_desc = smem_desc(base + st * kStageBytes + mb * kABytes, 0, 1024);
-#pragma unroll
-            for (int ks = 0; ks < kBK / 16; ++ks)          // 16 of K = 32 bytes along the swizzled row
-              mma_ss(tmem + (kMB == 1 ? buf : mb) * 256, a_desc + (uint64_t)(ks * 2), b_desc + (uint64_t)(ks * 2), kIdesc,
-                     (kb > 0 || ks > 0) ? 1u : 0u, issue);
-          }
+          for (int ks = 0; ks < kBK / 16; ++ks)            // 16 of K = 32 bytes along the swizzled row
+            mma_ss(tmem + buf * 256, a_desc + (uint64_t)(ks * 2), b_desc + (uint64_t)(ks * 2), kIdesc,
+                   (kb > 0 || ks > 0) ? 1u : 0u, issue);
           tc_commit(bar(BAR_EMPTY + st), issue);           // the stage is free once these MMAs have read it
         }
       }
-      if (!dead) {
-        tc_commit(bar(BAR_ACC_FULL + buf), issue);
-        if (kMB == 2) tc_commit(bar(BAR_ACC_FULL + 1), issue);
-      }
+      if (!dead) tc_commit(bar(BAR_ACC_FULL + buf), issue);
     }
   } else {
     // --------------------------------------------------------------------------- epilogue
-    const int q = warp & 3;                                // the TMEM lanes this warp can reach
-    const int row_in_blk = q * 32 + lane;
+    const int q = warp & 3, hf = (warp - 2) >> 2;          // the TMEM lanes this warp can reach, its half of the columns
+    prefetch_weights(g, ((int)blockIdx.x / m_tiles) * kBN + tid - 64, 0, g.K);
+    pdl_wait();                    // the residual or the positions may come from the kernel in front of this one
     int n_done = 0;
     for (int t = blockIdx.x; t < n_work; t += gridDim.x, ++n_done) {
-      const int m0 = (t % m_tiles) * TILE_M, n0 = (t / m_tiles) * kBN;
-#pragma unroll 1
-      for (int mb = 0; mb < kMB; ++mb) {
-        const int buf = kMB == 1 ? (n_done & 1) : mb;
-        const int uses = kMB == 1 ? (n_done >> 1) : n_done;
-        wait(BAR_ACC_FULL + buf, uses & 1);
-        tc_fence_after();
-        const int row = m0 + mb * 128 + row_in_blk;
-        const bool row_ok = row < g.M;
-        const uint32_t tacc = tmem + buf * 256 + ((uint32_t)(q * 32) << 16);
-        if (EPI == GEMM_EPI_STORE) {
-          uint16_t* crow = g.C + (size_t)row * g.ldc + n0;
-          const uint16_t* rrow = g.R ? g.R + (size_t)row * g.ldc + n0 : nullptr;
-#pragma unroll 1
-          for (int c = 0; c < kBN / 32; ++c) {
-            float v[32];
-            tmem_ld32(v, tacc + c * 32);
-            tmem_ld_wait();
-            if (c == kBN / 32 - 1) {
-              tc_fence_before();
-              mbar_arrive(bar(BAR_ACC_EMPTY + buf));       // the accumulator is in registers
-            }
-            if (row_ok) {
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const int col = n0 + c * 32 + i * 8;
-                if (col < g.N) {
-                  if (rrow) {
-                    float r[8];
-                    unpack8(*reinterpret_cast<const uint4*>(rrow + c * 32 + i * 8), r);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) v[i * 8 + e] += r[e];
-                  }
-                  *reinterpret_cast<uint4*>(crow + c * 32 + i * 8) = pack8(v + i * 8);
-                }
-              }
-            }
-          }
-        } else if (EPI == GEMM_EPI_ROPE) {
-          // A tile holds two heads of 128 columns. Query and key heads are rotated: column i < 64 of a
-          // head pairs with column i + 64, angle table[pos][i]. Each head goes to its own tensor.
-          const float2* cs = g.rope_table + (size_t)(row_ok ? g.pos[row] : 0) * 64;
-#pragma unroll 1
-          for (int h = 0; h < 2; ++h) {
-            const int col0 = n0 + h * 128;
-            const bool rotate = col0 < g.q_cols + g.kv_cols;
-            uint16_t* dst = col0 < g.q_cols ? g.C + (size_t)row * g.q_cols + col0
-                            : rotate        ? g.C2 + (size_t)row * g.kv_cols + (col0 - g.q_cols)
-                                            : g.C3 + (size_t)row * g.kv_cols + (col0 - g.q_cols - g.kv_cols);
-#pragma unroll 1
-            for (int c = 0; c < 2; ++c) {
-              float lo[32], hi[32];
-              tmem_ld32(lo, tacc + h * 128 + c * 32);
-              tmem_ld32(hi, tacc + h * 128 + 64 + c * 32);
-              tmem_ld_wait();
-              if (h == 1 && c == 1) {
-                tc_fence_before();
-                mbar_arrive(bar(BAR_ACC_EMPTY + buf));
-              }
-              if (row_ok && col0 < g.N) {
-                if (rotate) {
-#pragma unroll
-                  for (int i = 0; i < 32; ++i) {
-                    const float2 t2 = cs[c * 32 + i];     // (cos, sin)
-                    const float a = lo[i], b = hi[i];
-                    lo[i] = a * t2.x - b * t2.y;
-                    hi[i] = b * t2.x + a * t2.y;
-                  }
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  *reinterpret_cast<uint4*>(dst + c * 32 + i * 8) = pack8(lo + i * 8);
-                  *reinterpret_cast<uint4*>(dst + 64 + c * 32 + i * 8) = pack8(hi + i * 8);
-                }
-              }
-            }
-          }
-        } else {
-          // GEMM_EPI_SILU_MUL: the weight rows of a tile are 128 gate rows followed by the 128 up rows of
-          // the same intermediate features; out[row][n0 / 2 + i] = silu(gate_i) * up_i, both
-          // rounded to bf16 first (they are bf16 tensors of the layer's definition).
-          uint16_t* crow = g.C + (size_t)row * g.ldc + n0 / 2;
-#pragma unroll 1
-          for (int c = 0; c < 4; ++c) {
-            float gt[32], up[32];
-            tmem_ld32(gt, tacc + c * 32);
-            tmem_ld32(up, tacc + 128 + c * 32);
-            tmem_ld_wait();
-            if (c == 3) {
-              tc_fence_before();
-              mbar_arrive(bar(BAR_ACC_EMPTY + buf));
-            }
-            if (row_ok && n0 < g.N) {
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                silu_mul8(gt + i * 8, up + i * 8);
-                *reinterpret_cast<uint4*>(crow + c * 32 + i * 8) = pack8(gt + i * 8);
-              }
-            }
-          }
-        }
-      }
+      const int m0 = (t % m_tiles) * 128, n0 = (t / m_tiles) * kBN;
+      const int buf = n_done & 1;
+      wait(BAR_ACC_FULL + buf, (n_done >> 1) & 1);
+      tc_fence_after();
+      epilogue_row<EPI>(g, tmem + buf * 256 + ((uint32_t)(q * 32) << 16), m0 + q * 32 + lane, n0, hf, [&]() {
+        tc_fence_before();
+        mbar_arrive(bar(BAR_ACC_EMPTY + buf));             // the accumulator is in registers
+      });
     }
   }
   tc_fence_before();
@@ -315,34 +315,195 @@ gemm_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, const _
   if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-// ---------------------------------------------------------------------------------- split-K kernel
-// For products with few tiles (a decode batch: one 128-row block of tokens). Such a product is bound
-// by the HBM traffic of its weights, but with one CTA per 128 x 256 tile only 16-24 of the 148 SMs
-// pull on HBM (hidden 4096: 37 us for the 50 MB of QKV weights, 1.35 TB/s). Here a cluster of S
-// CTAs shares a tile: CTA r multiplies K blocks [kb r / S, kb (r+1) / S), lays its fp32 accumulator
-// into its own shared memory (the operand stages are free by then), and after a cluster barrier the
-// S CTAs add up the S accumulators, each a share of the elements, in the order r = 0 .. S-1
-// (through distributed shared memory: nothing goes to global memory, no workspace, and the result
-// does not depend on timing), apply the epilogue and write it.
+// ------------------------------------------------------------------------------------ pair kernel
+// For products with many rows. Two CTAs of a cluster share a 256 x 256 tile (cta_group::2): CTA r
+// fetches rows [128 r, 128 r + 128) of both operand blocks and holds that half of the accumulator's
+// rows; one MMA of M = 256, N = 256 reads the B halves of both CTAs. Per CTA and 64 of K that is 32 KB
+// fetched and 32 KB read for 512 cycles of tensor work, where a CTA on its own moves 48 KB + 48 KB
+// for a 128 x 256 tile (shared memory gives 128 bytes per clock: its limit, not the tensor pipe's).
+// CTA 0 issues all MMAs. Every CTA's copies complete CTA 0's "full" barrier; the commits arrive at
+// both CTAs' "empty" and "accumulator full" barriers; both epilogues release the accumulator to CTA 0.
 __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-  return v;
-}
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;\n" ::: "memory");
 }
+// `bar` may lie in the other CTA of the pair
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
+      : "memory");
+}
+__device__ __forceinline__ void mma_ss_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate, uint32_t issue) {
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.u32 p, %4, 0;\nsetp.ne.u32 q, %5, 0;\n"
+      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(issue)
+      : "memory");
+}
+// Arrives at this barrier of both CTAs once the MMAs issued so far are done.
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint32_t issue) {
+  asm volatile(
+      "{\n.reg .pred q;\nsetp.ne.u32 q, %1, 0;\n"
+      "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %2;\n}\n" ::"r"(bar),
+      "r"(issue), "h"((uint16_t)3)
+      : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
 
-constexpr int kSplitStages = 4, kSplitStageBytes = kABytes + kBBytes;
+constexpr int kPairStages = 6, kPairStageBytes = 2 * kABytes;
+constexpr int kPairBars = 2 * kPairStages + 4;
+constexpr int kPairSmem = kPairStages * kPairStageBytes + kPairBars * 8 + 16 + 1024;
+constexpr uint32_t kIdescPair = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3) << 17) | ((256u >> 4) << 24);
+
+template <int EPI>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+gemm_pair_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, const __grid_constant__ CUtensorMap b_map) {
+  extern __shared__ unsigned char smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t rank = blockIdx.x & 1;                    // in the cluster
+  constexpr int kOffBar = kPairStages * kPairStageBytes, kOffMisc = kOffBar + kPairBars * 8;
+  pdl_launch_dependents();
+  auto bar = [&](int i) { return base + kOffBar + (uint32_t)i * 8u; };
+  constexpr int BAR_FULL = 0, BAR_EMPTY = kPairStages, BAR_ACC_FULL = 2 * kPairStages, BAR_ACC_EMPTY = 2 * kPairStages + 2;
+  volatile uint32_t* misc = reinterpret_cast<volatile uint32_t*>(smem + kOffMisc);   // [0] TMEM base, [1] failure flag
+  if (tid == 0) {
+    misc[1] = 0;
+    for (int i = 0; i < BAR_ACC_EMPTY; ++i) mbar_init(bar(i), 1);
+    mbar_init(bar(BAR_ACC_EMPTY), 16);                     // eight epilogue warps of each CTA (CTA 0's barrier is the one used)
+    mbar_init(bar(BAR_ACC_EMPTY + 1), 16);
+    mbar_init_fence();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(base + kOffMisc) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();                  // the other CTA's barriers are initialised too
+  tc_fence_after();
+  const uint32_t tmem = misc[0];
+  auto give_up = [&]() {
+    if (misc[1] == 0) {
+      atomicOr(g.status, TS_DEV_TIMEOUT);
+      misc[1] = 1;
+    }
+  };
+  auto wait = [&](int i, uint32_t parity) {
+    if (!mbar_wait(bar(i), parity, misc[1] ? 2000 : g.wait_cycles)) give_up();
+  };
+  const int m_tiles = (g.M + 255) / 256, n_tiles = (g.N + kBN - 1) / kBN;
+  const int n_work = m_tiles * n_tiles, first = blockIdx.x >> 1, stride = gridDim.x >> 1;
+  const int k_blocks = (g.K + kBK - 1) / kBK;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      tma_prefetch_desc(&a_map);
+      tma_prefetch_desc(&b_map);
+      pdl_wait();
+      int it = 0;
+      for (int t = first; t < n_work; t += stride) {
+        const int m0 = (t % m_tiles) * 256 + (int)rank * 128, n0 = (t / m_tiles) * kBN + (int)rank * 128;
+        for (int kb = 0; kb < k_blocks; ++kb, ++it) {
+          const int st = it % kPairStages;
+          if (it >= kPairStages) wait(BAR_EMPTY + st, ((it / kPairStages) & 1) ^ 1);
+          if (misc[1]) continue;                           // after a failure no new copies are started
+          const uint32_t dst = base + st * kPairStageBytes, full = mapa(bar(BAR_FULL + st), 0);
+          if (rank == 0) mbar_expect_tx(bar(BAR_FULL + st), 2 * kPairStageBytes);
+          tma_load_2d_pair(dst, &a_map, full, kb * kBK, m0);
+          tma_load_2d_pair(dst + kABytes, &b_map, full, kb * kBK, n0);
+        }
+      }
+      // the commits that free the last stages arrive here too: they must have before this CTA may leave
+      for (int i = max(0, it - kPairStages); i < it; ++i) wait(BAR_EMPTY + i % kPairStages, (i / kPairStages) & 1);
+    }
+  } else if (warp == 1) {
+    if (rank == 0) {
+      const uint32_t issue = elect_one();
+      bool dead = false;
+      auto iwait = [&](int i, uint32_t parity) {
+        if (!mbar_poll(bar(i), parity, dead ? 2000 : g.wait_cycles)) {
+          dead = true;
+          give_up();
+        }
+      };
+      int it = 0, n_done = 0;
+      for (int t = first; t < n_work; t += stride, ++n_done) {
+        const int buf = n_done & 1, uses = n_done >> 1;
+        if (uses > 0) iwait(BAR_ACC_EMPTY + buf, (uses - 1) & 1);
+        tc_fence_after();
+        for (int kb = 0; kb < k_blocks; ++kb, ++it) {
+          const int st = it % kPairStages;
+          iwait(BAR_FULL + st, (it / kPairStages) & 1);
+          tc_fence_after();
+          if (!dead) {
+            const uint64_t a_desc = smem_desc(base + st * kPairStageBytes, 0, 1024);
+            const uint64_t b_desc = smem_desc(base + st * kPairStageBytes + kABytes, 0, 1024);
+#pragma unroll
+            for (int ks = 0; ks < kBK / 16; ++ks)
+              mma_ss_pair(tmem + buf * 256, a_desc + (uint64_t)(ks * 2), b_desc + (uint64_t)(ks * 2), kIdescPair,
+                          (kb > 0 || ks > 0) ? 1u : 0u, issue);
+            tc_commit_pair(bar(BAR_EMPTY + st), issue);
+          }
+        }
+        if (!dead) tc_commit_pair(bar(BAR_ACC_FULL + buf), issue);
+      }
+    }
+  } else {
+    if (tid - 64 < 128) prefetch_weights(g, (first / m_tiles) * kBN + (int)rank * 128 + tid - 64, 0, g.K);
+    pdl_wait();                    // the residual or the positions may come from the kernel in front of this one
+    const int q = warp & 3, hf = (warp - 2) >> 2;
+    int n_done = 0;
+    for (int t = first; t < n_work; t += stride, ++n_done) {
+      const int m0 = (t % m_tiles) * 256 + (int)rank * 128, n0 = (t / m_tiles) * kBN;
+      const int buf = n_done & 1;
+      wait(BAR_ACC_FULL + buf, (n_done >> 1) & 1);
+      tc_fence_after();
+      epilogue_row<EPI>(g, tmem + buf * 256 + ((uint32_t)(q * 32) << 16), m0 + q * 32 + lane, n0, hf, [&]() {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(mapa(bar(BAR_ACC_EMPTY + buf), 0));
+      });
+    }
+  }
+  tc_fence_before();
+  __syncwarp();
+  cluster_sync();                  // no CTA leaves while the other one's copies, commits or arrivals may still reach it
+  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;\n" ::"r"(tmem) : "memory");
+}
+
+// ---------------------------------------------------------------------------------- split-K kernel
+// For products with few tiles (a decode batch: one 128-row block of tokens). Such a product is bound
+// by the HBM traffic of its weights, but with one CTA per 128 x 256 tile only 16-24 of the 148 SMs
+// pull on HBM (hidden 4096: 37 us for the 50 MB of QKV weights, 1.35 TB/s). Here a cluster of S
+// CTAs shares a 128 x 128 tile: CTA r multiplies K blocks [kb r / S, kb (r+1) / S), lays its fp32
+// accumulator into its own shared memory (the operand stages are free by then), and after a cluster
+// barrier the S CTAs add up the S accumulators, each a share of the elements, in the order r = 0 ..
+// S-1 (through distributed shared memory: nothing goes to global memory, no workspace, and the
+// result does not depend on timing), apply the epilogue and write it. The merge is bound by the
+// distributed reads (~8 bytes per clock and SM); half the tile width with half the split halves them
+// twice over: 128 x 256 tiles in clusters of 6-8 took 18.2 / 15.8 / 31.5 us at 64 rows (QKV / output /
+// down), 128 x 128 tiles in clusters of 3-4 take
+// 15.3 / 11.6 / 25.5 us.
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  return v;
+}
+constexpr int kSplitN = 128;
+constexpr int kSplitStages = 6, kSplitStageBytes = kABytes + kBBytes / 2;
 constexpr int kSplitSmem = kSplitStages * kSplitStageBytes + (2 * kSplitStages + 1) * 8 + 16 + 1024;
-static_assert(128 * kBN * 4 <= kSplitStages * kSplitStageBytes, "the accumulator image takes the place of the operand stages");
+static_assert(128 * kSplitN * 4 <= kSplitStages * kSplitStageBytes, "the accumulator image takes the place of the operand stages");
 // 16-byte chunk `c` of row `row` of the accumulator image; the XOR spreads a column of rows over the banks
-__device__ __forceinline__ uint32_t image_off(int row, int c) { return (uint32_t)(row * (kBN * 4) + ((c ^ (row & 7)) << 4)); }
+__device__ __forceinline__ uint32_t image_off(int row, int c) { return (uint32_t)(row * (kSplitN * 4) + ((c ^ (row & 7)) << 4)); }
 
 template <int EPI>
 __global__ void __launch_bounds__(kGemmThreads, 1)
@@ -363,7 +524,7 @@ gemm_split_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, c
     for (int i = 0; i < 2 * kSplitStages + 1; ++i) mbar_init(bar(i), 1);
     mbar_init_fence();
   }
-  if (warp == 1) tmem_alloc(base + kOffMisc, 256);
+  if (warp == 1) tmem_alloc(base + kOffMisc, kSplitN);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -376,7 +537,7 @@ gemm_split_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, c
   };
   const int m_tiles = (g.M + 127) / 128;
   const int t = blockIdx.x / split, rank = blockIdx.x % split;     // the cluster's CTAs are consecutive blocks
-  const int m0 = (t % m_tiles) * 128, n0 = (t / m_tiles) * kBN;
+  const int m0 = (t % m_tiles) * 128, n0 = (t / m_tiles) * kSplitN;
   const int rows = min(128, g.M - m0);
   const int k_blocks = (g.K + kBK - 1) / kBK;
   const int kb0 = k_blocks * rank / split, kb1 = k_blocks * (rank + 1) / split;   // never empty: split <= k_blocks
@@ -385,8 +546,6 @@ gemm_split_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, c
     if (lane == 0) {
       tma_prefetch_desc(&a_map);
       tma_prefetch_desc(&b_map);
-      // the weights do not come from the kernel in front of this one: bring the first of them into L2 meanwhile
-      for (int kb = kb0; kb < min(kb1, kb0 + 2 * kSplitStages); ++kb) tma_prefetch_2d(&b_map, kb * kBK, n0);
       pdl_wait();
       for (int kb = kb0, it = 0; kb < kb1; ++kb, ++it) {
         const int st = it % kSplitStages;
@@ -413,19 +572,20 @@ gemm_split_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, c
       const uint64_t b_desc = smem_desc(base + st * kSplitStageBytes + kABytes, 0, 1024);
 #pragma unroll
       for (int ks = 0; ks < kBK / 16; ++ks)
-        mma_ss(tmem, a_desc + (uint64_t)(ks * 2), b_desc + (uint64_t)(ks * 2), kIdesc, (it > 0 || ks > 0) ? 1u : 0u, issue);
+        mma_ss(tmem, a_desc + (uint64_t)(ks * 2), b_desc + (uint64_t)(ks * 2), instr_desc(false), (it > 0 || ks > 0) ? 1u : 0u, issue);
       tc_commit(bar(BAR_EMPTY + st), issue);
     }
     if (!dead) tc_commit(bar(BAR_ACC), issue);
   } else {
+    if (tid - 64 < kSplitN) prefetch_weights(g, n0 + tid - 64, kb0 * kBK, kb1 * kBK);
     // accumulator -> image in shared memory; every operand stage has been read once the barrier completes
     if (!mbar_wait(bar(BAR_ACC), 0, misc[1] ? 2000 : g.wait_cycles)) give_up();
     tc_fence_after();
-    const int q = warp & 3;                                // the TMEM lanes this warp can reach
+    const int q = warp & 3, hf = (warp - 2) >> 2;          // the TMEM lanes this warp can reach, its half of the columns
     const int row = q * 32 + lane;
     if (q * 32 < rows && misc[1] == 0) {
 #pragma unroll 1
-      for (int c = 0; c < kBN / 32; ++c) {
+      for (int c = hf * 2; c < hf * 2 + 2; ++c) {
         float v[32];
         tmem_ld32(v, tmem + ((uint32_t)(q * 32) << 16) + c * 32);
         tmem_ld_wait();
@@ -440,17 +600,25 @@ gemm_split_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, c
   __syncwarp();
   cluster_sync();                  // the images are complete
   pdl_wait();                      // every thread reads the residual or the positions below
-  // one item = 8 columns of a row (STORE), or 8 columns and their partners 64 (ROPE) or 128 (SILU_MUL) further on
-  constexpr int kItems = EPI == GEMM_EPI_STORE ? 32 : 16;
+  // one item = 8 columns of a row, for ROPE with their partners 64 further on
+  constexpr int kItems = EPI == GEMM_EPI_STORE ? 16 : 8;
   auto sum8 = [&](int row, int col, float (&v)[8]) {
+    float4 x[kMaxSplit], y[kMaxSplit];                     // all loads fly at once
 #pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = 0.f;
-#pragma unroll 4
-    for (int r = 0; r < split; ++r) {
-      const uint32_t img = mapa(base, (uint32_t)r);
-      const float4 x = ld_cluster4(img + image_off(row, col / 4)), y = ld_cluster4(img + image_off(row, col / 4 + 1));
-      v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
-      v[4] += y.x; v[5] += y.y; v[6] += y.z; v[7] += y.w;
+    for (int r = 0; r < kMaxSplit; ++r) {
+      x[r] = y[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r < split) {
+        const uint32_t img = mapa(base, (uint32_t)r);
+        x[r] = ld_cluster4(img + image_off(row, col / 4));
+        y[r] = ld_cluster4(img + image_off(row, col / 4 + 1));
+      }
+    }
+    v[0] = x[0].x; v[1] = x[0].y; v[2] = x[0].z; v[3] = x[0].w;
+    v[4] = y[0].x; v[5] = y[0].y; v[6] = y[0].z; v[7] = y[0].w;
+#pragma unroll
+    for (int r = 1; r < kMaxSplit; ++r) {                  // a rank that is not there adds zeros
+      v[0] += x[r].x; v[1] += x[r].y; v[2] += x[r].z; v[3] += x[r].w;
+      v[4] += y[r].x; v[5] += y[r].y; v[6] += y[r].z; v[7] += y[r].w;
     }
   };
   for (int i = rank * kGemmThreads + tid; i < rows * kItems; i += split * kGemmThreads) {
@@ -459,53 +627,53 @@ gemm_split_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, c
       const int col = n0 + ch * 8;
       if (col >= g.N) continue;
       float v[8];
+      uint4 res;
+      if (g.R) res = *reinterpret_cast<const uint4*>(g.R + (size_t)row * g.ldc + col);
       sum8(r, ch * 8, v);
       if (g.R) {
         float x[8];
-        unpack8(*reinterpret_cast<const uint4*>(g.R + (size_t)row * g.ldc + col), x);
+        unpack8(res, x);
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] += x[e];
       }
       *reinterpret_cast<uint4*>(g.C + (size_t)row * g.ldc + col) = pack8(v);
-    } else if (EPI == GEMM_EPI_ROPE) {
-      const int h = ch / 8, c = (ch % 8) * 8, col0 = n0 + h * 128;
-      if (col0 >= g.N) continue;
-      float lo[8], hi[8];
-      sum8(r, h * 128 + c, lo);
-      sum8(r, h * 128 + 64 + c, hi);
-      rope8(g, row, col0, c, lo, hi);
     } else {
-      if (n0 >= g.N) continue;
-      float gt[8], up[8];
-      sum8(r, ch * 8, gt);
-      sum8(r, 128 + ch * 8, up);
-      silu_mul8(gt, up);
-      *reinterpret_cast<uint4*>(g.C + (size_t)row * g.ldc + n0 / 2 + ch * 8) = pack8(gt);
+      float lo[8], hi[8];
+      sum8(r, ch * 8, lo);
+      sum8(r, 64 + ch * 8, hi);
+      rope8(g, row, n0, ch * 8, lo, hi);
     }
   }
   tc_fence_before();
   cluster_sync();                  // no CTA leaves while another one reads its image
-  if (warp == 1) tmem_dealloc(tmem, 256);
+  if (warp == 1) tmem_dealloc(tmem, kSplitN);
+}
+
+// launch_pdl for a grid of clusters of `cluster` CTAs.
+template <typename... Params, typename... Args>
+cudaError_t launch_cluster(void (*kernel)(Params...), int ctas, int cluster, int smem, cudaStream_t stream, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(kGemmThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
 template <int EPI>
 cudaError_t launch_split_t(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, int split, cudaStream_t stream) {
   cudaError_t e = cudaFuncSetAttribute(gemm_split_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem);
   if (e != cudaSuccess) return e;
-  const int tiles = ((g.M + 127) / 128) * ((g.N + kBN - 1) / kBN);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(tiles * split);
-  cfg.blockDim = dim3(kGemmThreads);
-  cfg.dynamicSmemBytes = kSplitSmem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim = {(unsigned)split, 1, 1};
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, gemm_split_kernel<EPI>, g, a_map, b_map, split);
+  const int tiles = ((g.M + 127) / 128) * ((g.N + kSplitN - 1) / kSplitN);
+  return launch_cluster(gemm_split_kernel<EPI>, tiles * split, split, kSplitSmem, stream, g, a_map, b_map, split);
 }
 
 // CTAs of gemm_split_kernel that the device runs at once in clusters of `split` (a hardware figure;
@@ -524,7 +692,8 @@ int split_slots(int split) {
   cfg.dynamicSmemBytes = kSplitSmem;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim = {(unsigned)split, 1, 1};
+  attr[0].val.clusterDim.x = (unsigned)split;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int clusters = 0;
@@ -536,49 +705,63 @@ int split_slots(int split) {
   return clusters * split;
 }
 
-template <int TILE_M, int EPI>
-cudaError_t launch_t(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, int n_sms, cudaStream_t stream) {
-  constexpr int kStageBytes = (TILE_M / 128) * kABytes + kBBytes;
-  constexpr int kStages = TILE_M == 128 ? 4 : 3;
-  const size_t smem = (size_t)kStages * kStageBytes + (2 * kStages + 4) * 8 + 16 + 1024;
-  cudaError_t e = cudaFuncSetAttribute(gemm_kernel<TILE_M, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int EPI>
+cudaError_t launch_tile_t(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, int n_sms, cudaStream_t stream) {
+  const size_t smem = (size_t)kTileStages * (kABytes + kBBytes) + (2 * kTileStages + 4) * 8 + 16 + 1024;
+  cudaError_t e = cudaFuncSetAttribute(gemm_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int m_tiles = (g.M + TILE_M - 1) / TILE_M, n_tiles = (g.N + kBN - 1) / kBN;
-  const int grid = std::min(n_sms, m_tiles * n_tiles);
-  return launch_pdl(gemm_kernel<TILE_M, EPI>, dim3(grid), dim3(kGemmThreads), smem, stream, g, a_map, b_map);
+  const int tiles = ((g.M + 127) / 128) * ((g.N + kBN - 1) / kBN);
+  return launch_pdl(gemm_kernel<EPI>, dim3(std::min(n_sms, tiles)), dim3(kGemmThreads), smem, stream, g, a_map, b_map);
+}
+
+template <int EPI>
+cudaError_t launch_pair_t(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, int n_sms, cudaStream_t stream) {
+  cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
+  if (e != cudaSuccess) return e;
+  const int tiles = ((g.M + 255) / 256) * ((g.N + kBN - 1) / kBN);
+  return launch_cluster(gemm_pair_kernel<EPI>, 2 * std::min(n_sms / 2, tiles), 2, kPairSmem, stream, g, a_map, b_map);
+}
+
+template <int EPI>
+cudaError_t launch_epi(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, GemmPlan plan, int n_sms,
+                       cudaStream_t stream) {
+  if constexpr (EPI != GEMM_EPI_SILU_MUL)                // a gate and its up column are 128 columns apart: no tile of 128 holds both
+    if (plan.split > 0) return launch_split_t<EPI>(g, a_map, b_map, plan.split, stream);
+  if (plan.tile_m == 256) return launch_pair_t<EPI>(g, a_map, b_map, n_sms, stream);
+  return launch_tile_t<EPI>(g, a_map, b_map, n_sms, stream);
 }
 
 }  // namespace
 
-// Cost of a launch in us. Without a split: waves x K blocks, the 256-row tile being cheaper per flop
-// (it fetches a third fewer operand bytes) but coarser in the wave count. With a split: the K blocks
-// of the longest share and the merge; only where all clusters run at once. A K block takes a CTA
-// kBlockUs, or as long as HBM needs for the weight blocks that are in flight at that moment. Measured
-// (8B-shaped projections, weights not in L2, one CTA per tile -> split): 64 rows QKV 35.2 -> 18.5 us,
-// output 34.6 -> 17.2, down 96.7 -> 35.2; 256 rows QKV 36.8 -> 32.9, output 35.5 -> 22.4, down 96.5
-// -> 42.0; 512 rows output 35.3 -> 31.7, down 96.2 -> 66.9. The merge takes 2-3 us for one row and
-// ~8 us for 128 rows. Gate/up (112 tiles) is not split: its tiles already fill three quarters of the SMs.
-GemmPlan gemm_plan(int M, int N, int K, int n_sms, bool tall) {
-  constexpr double kBlockUs = 0.42, kHbmBytesPerUs = 6.2e6;
-  const double merge_us = 2.5 + 0.045 * std::min(M, 128);
-  const int n_tiles = (N + kBN - 1) / kBN, m128 = (M + 127) / 128, m256 = (M + 255) / 256;
-  const int kb = (K + kBK - 1) / kBK;
-  auto block_us = [&](int ctas, int m_tiles, double tile_cost) {
-    return std::max(kBlockUs * tile_cost, (double)std::min(ctas, n_sms) / m_tiles * kBBytes / kHbmBytesPerUs);
+// Cost of a launch in us besides what every launch pays: waves x K blocks x the time of a K block, which
+// is what the tensor pipe and shared memory take (0.37 us for a CTA's 128 x 256 tile, 0.30 us for a
+// pair's 256 x 256 tile, 0.33 us for a 128 x 128 tile) or what HBM needs for the weight blocks in flight
+// at that moment; for the split kernel also the merge, and only where all clusters run at once.
+// Measured (8B-shaped projections, weights not in L2, us; 128 x 256 tile / pair / split kernel): 64 rows
+// QKV 30.4 / 26.8 / 15.3, output 29.7 / 26.3 / 11.6, down 88.8 / 71.8 / 25.5; 256 rows output 32.0 /
+// 29.1 / 17.3, down 90.9 / 75.0 / 40.3; 1024 rows (tile / pair) QKV 58.6 / 50.9, gate/up 212 / 180, down
+// 106 / 90; 2112 rows 89.3 / 82.5, output 60.5 / 56.1, gate/up 390 / 360, down 199 / 181.
+GemmPlan gemm_plan(const GemmArgs& g, int n_sms) {
+  constexpr double kTileUs = 0.37, kPairUs = 0.30, kSplitUs = 0.33, kHbmBytesPerUs = 6.2e6;
+  const double merge_us = 2.5 + 0.03 * std::min(g.M, 128);
+  const int n_tiles = (g.N + kBN - 1) / kBN, m128 = (g.M + 127) / 128, m256 = (g.M + 255) / 256;
+  const int kb = (g.K + kBK - 1) / kBK;
+  // `at_once` workers on weight blocks of `width` rows, each on another one unless m_tiles row blocks share it
+  auto cost_of = [&](double us, int tiles, int workers, int m_tiles, int width, int blocks) {
+    const double hbm = (double)std::min(tiles, workers) / m_tiles * width * kBK * 2 / kHbmBytesPerUs;
+    return (double)((tiles + workers - 1) / workers) * blocks * std::max(us, hbm);
   };
-  auto waves = [&](int tiles) { return (tiles + n_sms - 1) / n_sms; };
-  GemmPlan best = {128, 1};
-  double cost = (double)waves(m128 * n_tiles) * kb * block_us(m128 * n_tiles, m128, 1.0);
-  if (tall) {
-    const double c = (double)waves(m256 * n_tiles) * kb * block_us(m256 * n_tiles, m256, 2.0 * 0.9);
-    if (c < cost) {
-      cost = c;
-      best = {256, 1};
-    }
+  GemmPlan best = {128, 0};
+  double cost = cost_of(kTileUs, m128 * n_tiles, n_sms, m128, kBN, kb);
+  const double pair_cost = cost_of(kPairUs, m256 * n_tiles, n_sms / 2, m256, kBN, kb);
+  if (pair_cost < cost) {
+    cost = pair_cost;
+    best = {256, 0};
   }
-  for (int s = 2; s <= std::min(kMaxSplit, kb); ++s) {
-    if (m128 * n_tiles * s > n_sms || m128 * n_tiles * s > split_slots(s)) break;
-    const double c = (double)((kb + s - 1) / s) * block_us(m128 * n_tiles * s, m128, 1.0) + merge_us;
+  const int split_tiles = m128 * ((g.N + kSplitN - 1) / kSplitN);
+  for (int s = 2; s <= std::min(kMaxSplit, kb) && g.epi != GEMM_EPI_SILU_MUL; ++s) {
+    if (split_tiles * s > n_sms || split_tiles * s > split_slots(s)) break;
+    const double c = cost_of(kSplitUs, split_tiles * s, split_tiles * s, m128, kSplitN, (kb + s - 1) / s) + merge_us;
     if (c < cost * 0.98) {
       cost = c;
       best = {128, s};
@@ -590,17 +773,11 @@ GemmPlan gemm_plan(int M, int N, int K, int n_sms, bool tall) {
 cudaError_t launch_gemm(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, GemmPlan plan, int n_sms,
                         cudaStream_t stream) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
-  if (plan.split > 1) {
-    if (g.epi == GEMM_EPI_ROPE) return launch_split_t<GEMM_EPI_ROPE>(g, a_map, b_map, plan.split, stream);
-    if (g.epi == GEMM_EPI_SILU_MUL) return launch_split_t<GEMM_EPI_SILU_MUL>(g, a_map, b_map, plan.split, stream);
-    return launch_split_t<GEMM_EPI_STORE>(g, a_map, b_map, plan.split, stream);
+  switch (g.epi) {
+    case GEMM_EPI_ROPE: return launch_epi<GEMM_EPI_ROPE>(g, a_map, b_map, plan, n_sms, stream);
+    case GEMM_EPI_SILU_MUL: return launch_epi<GEMM_EPI_SILU_MUL>(g, a_map, b_map, plan, n_sms, stream);
+    default: return launch_epi<GEMM_EPI_STORE>(g, a_map, b_map, plan, n_sms, stream);
   }
-  if (g.epi == GEMM_EPI_ROPE) return launch_t<128, GEMM_EPI_ROPE>(g, a_map, b_map, n_sms, stream);
-  if (g.epi == GEMM_EPI_SILU_MUL)
-    return plan.tile_m == 256 ? launch_t<256, GEMM_EPI_SILU_MUL>(g, a_map, b_map, n_sms, stream)
-                              : launch_t<128, GEMM_EPI_SILU_MUL>(g, a_map, b_map, n_sms, stream);
-  return plan.tile_m == 256 ? launch_t<256, GEMM_EPI_STORE>(g, a_map, b_map, n_sms, stream)
-                            : launch_t<128, GEMM_EPI_STORE>(g, a_map, b_map, n_sms, stream);
 }
 
 }  // namespace ts

@@ -110,6 +110,7 @@ enum { GEMM_EPI_STORE = 0, GEMM_EPI_ROPE = 1, GEMM_EPI_SILU_MUL = 2 };
 struct GemmArgs {
   int32_t M, N, K;
   int32_t epi;              // GEMM_EPI_*
+  const uint16_t* B;        // the weights themselves (prefetches)
   uint16_t* C;              // STORE: [M][ldc]; ROPE: the query heads [M][q_cols]; SILU_MUL: [M][ldc], ldc = N / 2
   const uint16_t* R;        // STORE: residual [M][ldc] added before rounding, or null
   int32_t ldc;
@@ -134,13 +135,15 @@ struct CtxView {
   int max_tokens;           // most tokens a step may hold
 };
 int ctx_view(ts_ctx* c, cudaStream_t stream, CtxView* out);
-// How a product is laid over the chip: tile height (128 or 256 rows per CTA), and the number of CTAs
-// that share a 128-row tile's K range (split > 1: clusters of that size).
+// How a product is laid over the chip. split = 0: 128 x 256 tiles, one CTA each, or (tile_m = 256)
+// 256 x 256 tiles, a pair of CTAs each; split > 0: 128 x 128 tiles whose K range a cluster of `split`
+// CTAs shares.
 struct GemmPlan {
   int tile_m, split;
 };
-// The plan for an M x N x K product; `tall` = 256-row tiles may be used. The device is the current one.
-GemmPlan gemm_plan(int M, int N, int K, int n_sms, bool tall);
+// The plan for a product (M, N, K and epi are read). The device is the current one.
+GemmPlan gemm_plan(const GemmArgs& g, int n_sms);
+// Both maps view an operand as (K, row), box 64 x 128.
 cudaError_t launch_gemm(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, GemmPlan plan, int n_sms,
                         cudaStream_t stream);
 // out[row] = x[row] / sqrt(mean(x[row]^2) + eps) * gain, bf16 in and out, fp32 inside; width % 8 == 0

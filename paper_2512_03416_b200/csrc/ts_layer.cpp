@@ -20,11 +20,11 @@ typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void
                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// 2-D view of a K-major bf16 matrix [rows][k]: box = 64 of K (128 bytes, the swizzle span) x box_rows.
-bool make_operand_map(void* encode_fn, const void* ptr, int64_t rows, int64_t k, int box_rows, CUtensorMap* out) {
+// 2-D view of a K-major bf16 matrix [rows][k]: box = 64 of K (128 bytes, the swizzle span) x 128 rows.
+bool make_operand_map(void* encode_fn, const void* ptr, int64_t rows, int64_t k, CUtensorMap* out) {
   const cuuint64_t dims[2] = {(cuuint64_t)k, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)k * 2};
-  const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
+  const cuuint32_t box[2] = {64, 128};
   const cuuint32_t estr[2] = {1, 1};
   return ((EncodeFn)encode_fn)(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -67,8 +67,8 @@ struct ts_layer {
   LayerLayout L;
   int max_tokens = 0;
   float eps = 0.f, theta = 0.f;
-  CUtensorMap w_qkv, w_o, w_gu, w_down;        // weights: box 64 x 256
-  CUtensorMap a_h, a_attn, a_z;                // activations in the workspace: box 64 x 128
+  CUtensorMap w_qkv, w_o, w_gu, w_down;        // weights
+  CUtensorMap a_h, a_attn, a_z;                // activations in the workspace
   void* pos_host[kPosRing] = {};
   cudaEvent_t pos_ev[kPosRing] = {};
   bool pos_busy[kPosRing] = {};
@@ -136,13 +136,13 @@ int ts_layer_create(ts_ctx* ctx, const ts_layer_config* cfg, void* cuda_stream, 
   const ts_config* c = view.cfg;
   const int64_t qd = (int64_t)c->n_q_heads * c->head_dim, kvd = (int64_t)c->n_kv_heads * c->head_dim;
   char* ws = (char*)cfg->workspace;
-  bool ok = make_operand_map(view.encode_fn, cfg->w_qkv, qd + 2 * kvd, cfg->hidden, 256, &l->w_qkv) &&
-            make_operand_map(view.encode_fn, cfg->w_o, cfg->hidden, qd, 256, &l->w_o) &&
-            make_operand_map(view.encode_fn, cfg->w_gate_up, 2 * (int64_t)cfg->intermediate, cfg->hidden, 256, &l->w_gu) &&
-            make_operand_map(view.encode_fn, cfg->w_down, cfg->hidden, cfg->intermediate, 256, &l->w_down) &&
-            make_operand_map(view.encode_fn, ws + l->L.off_h, l->max_tokens, cfg->hidden, 128, &l->a_h) &&
-            make_operand_map(view.encode_fn, ws + l->L.off_attn, l->max_tokens, qd, 128, &l->a_attn) &&
-            make_operand_map(view.encode_fn, ws + l->L.off_z, l->max_tokens, cfg->intermediate, 128, &l->a_z);
+  bool ok = make_operand_map(view.encode_fn, cfg->w_qkv, qd + 2 * kvd, cfg->hidden, &l->w_qkv) &&
+            make_operand_map(view.encode_fn, cfg->w_o, cfg->hidden, qd, &l->w_o) &&
+            make_operand_map(view.encode_fn, cfg->w_gate_up, 2 * (int64_t)cfg->intermediate, cfg->hidden, &l->w_gu) &&
+            make_operand_map(view.encode_fn, cfg->w_down, cfg->hidden, cfg->intermediate, &l->w_down) &&
+            make_operand_map(view.encode_fn, ws + l->L.off_h, l->max_tokens, cfg->hidden, &l->a_h) &&
+            make_operand_map(view.encode_fn, ws + l->L.off_attn, l->max_tokens, qd, &l->a_attn) &&
+            make_operand_map(view.encode_fn, ws + l->L.off_z, l->max_tokens, cfg->intermediate, &l->a_z);
   if (!ok) {
     delete l;
     return TS_ERR_CUDA;
@@ -224,25 +224,25 @@ int ts_layer_step(ts_layer* l, const ts_step* st, const void* x_in, void* x_out,
 
   // h = rmsnorm(x); (q, k, v) = rope(h . W_qkv^T)
   TSL_CUDA(l, ts::launch_rmsnorm((const uint16_t*)x_in, (const uint16_t*)l->cfg.w_norm1, h, N, hidden, l->eps, stream));
-  g.N = qd + 2 * kvd; g.K = hidden; g.epi = ts::GEMM_EPI_ROPE;
+  g.N = qd + 2 * kvd; g.K = hidden; g.epi = ts::GEMM_EPI_ROPE; g.B = (const uint16_t*)l->cfg.w_qkv;
   g.C = q; g.C2 = k; g.C3 = v; g.q_cols = qd; g.kv_cols = kvd; g.pos = pos_dev;
   g.rope_table = (const float2*)(ws + l->L.off_table);
-  TSL_CUDA(l, ts::launch_gemm(g, l->a_h, l->w_qkv, ts::gemm_plan(N, g.N, g.K, l->view.n_sms, false), l->view.n_sms, stream));
+  TSL_CUDA(l, ts::launch_gemm(g, l->a_h, l->w_qkv, ts::gemm_plan(g, l->view.n_sms), l->view.n_sms, stream));
   // attention over the paged KV cache, with the append of the new K/V
   ts_step inner = *st;
   inner.q = q; inner.k_new = k; inner.v_new = v; inner.out = attn;
   rc = ts_mixed_step(l->ctx, &inner, cuda_stream);
   if (rc != TS_OK) return rc;
   // y = x + attn . W_o^T
-  g.N = hidden; g.K = qd; g.epi = ts::GEMM_EPI_STORE; g.C = y; g.R = (const uint16_t*)x_in; g.ldc = hidden;
-  TSL_CUDA(l, ts::launch_gemm(g, l->a_attn, l->w_o, ts::gemm_plan(N, g.N, g.K, l->view.n_sms, true), l->view.n_sms, stream));
+  g.N = hidden; g.K = qd; g.epi = ts::GEMM_EPI_STORE; g.B = (const uint16_t*)l->cfg.w_o; g.C = y; g.R = (const uint16_t*)x_in; g.ldc = hidden;
+  TSL_CUDA(l, ts::launch_gemm(g, l->a_attn, l->w_o, ts::gemm_plan(g, l->view.n_sms), l->view.n_sms, stream));
   // h2 = rmsnorm(y); z = silu(h2 . W_gate^T) * (h2 . W_up^T)
   TSL_CUDA(l, ts::launch_rmsnorm(y, (const uint16_t*)l->cfg.w_norm2, h, N, hidden, l->eps, stream));
-  g.N = 2 * inter; g.K = hidden; g.epi = ts::GEMM_EPI_SILU_MUL; g.C = z; g.R = nullptr; g.ldc = inter;
-  TSL_CUDA(l, ts::launch_gemm(g, l->a_h, l->w_gu, ts::gemm_plan(N, g.N, g.K, l->view.n_sms, true), l->view.n_sms, stream));
+  g.N = 2 * inter; g.K = hidden; g.epi = ts::GEMM_EPI_SILU_MUL; g.B = (const uint16_t*)l->cfg.w_gate_up; g.C = z; g.R = nullptr; g.ldc = inter;
+  TSL_CUDA(l, ts::launch_gemm(g, l->a_h, l->w_gu, ts::gemm_plan(g, l->view.n_sms), l->view.n_sms, stream));
   // out = y + z . W_down^T
-  g.N = hidden; g.K = inter; g.epi = ts::GEMM_EPI_STORE; g.C = (uint16_t*)x_out; g.R = y; g.ldc = hidden;
-  TSL_CUDA(l, ts::launch_gemm(g, l->a_z, l->w_down, ts::gemm_plan(N, g.N, g.K, l->view.n_sms, true), l->view.n_sms, stream));
+  g.N = hidden; g.K = inter; g.epi = ts::GEMM_EPI_STORE; g.B = (const uint16_t*)l->cfg.w_down; g.C = (uint16_t*)x_out; g.R = y; g.ldc = hidden;
+  TSL_CUDA(l, ts::launch_gemm(g, l->a_z, l->w_down, ts::gemm_plan(g, l->view.n_sms), l->view.n_sms, stream));
   return TS_OK;
 }
 
@@ -261,14 +261,14 @@ int ts_gemm_bf16(int32_t device, int32_t M, int32_t N, int32_t K, const void* A,
   int n_sms = 0;
   if (cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return TS_ERR_CUDA;
   CUtensorMap a_map, b_map;
-  if (!make_operand_map(encode_fn, A, M, K, 128, &a_map) || !make_operand_map(encode_fn, B, N, K, 256, &b_map)) return TS_ERR_CUDA;
+  if (!make_operand_map(encode_fn, A, M, K, &a_map) || !make_operand_map(encode_fn, B, N, K, &b_map)) return TS_ERR_CUDA;
   ts::GemmArgs g;
   std::memset(&g, 0, sizeof g);
-  g.M = M; g.N = N; g.K = K; g.epi = ts::GEMM_EPI_STORE;
+  g.M = M; g.N = N; g.K = K; g.epi = ts::GEMM_EPI_STORE; g.B = (const uint16_t*)B;
   g.C = (uint16_t*)C; g.R = (const uint16_t*)R; g.ldc = N;
   g.status = device_status;
   g.wait_cycles = ts::kWaitCycles;
-  const ts::GemmPlan plan = tile_m ? ts::GemmPlan{tile_m, 1} : ts::gemm_plan(M, N, K, n_sms, true);
+  const ts::GemmPlan plan = tile_m ? ts::GemmPlan{tile_m, 0} : ts::gemm_plan(g, n_sms);
   return ts::launch_gemm(g, a_map, b_map, plan, n_sms, (cudaStream_t)cuda_stream) == cudaSuccess ? TS_OK : TS_ERR_CUDA;
 }
 

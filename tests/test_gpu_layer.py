@@ -72,10 +72,10 @@ def test_gemm_matches_the_oracle(case, tile_m):
 
 
 @pytest.mark.parametrize("case", [(1, 256, 1024, False), (64, 512, 4096, True), (127, 264, 1032, False), (129, 1024, 2056, True),
-                                  (256, 4096, 4096, False)], ids=lambda c: f"{c[0]}x{c[1]}x{c[2]}")
+                                  (256, 4096, 4096, False), (500, 1032, 1544, True)], ids=lambda c: f"{c[0]}x{c[1]}x{c[2]}")
 def test_gemm_of_few_tiles_matches_the_oracle(case):
-    """The default plan on products whose K range is shared by a cluster: one row, ragged row blocks,
-    ragged last columns and K blocks, K blocks that do not divide by the cluster."""
+    """The default plan on products of few tiles, whose K range a cluster shares: one row, ragged row
+    blocks, ragged last columns and K blocks, K blocks that do not divide by the cluster."""
     test_gemm_matches_the_oracle(case, 0)
 
 
