@@ -1,5 +1,5 @@
 // Stand-alone split-KV flash-decode kernel for the 1-token rows (sm_100a): one persistent CTA
-// per SM running dec::decode_units (ts_decode_body.h) over all decode units of the step.
+// per SM running dec::decode_units and its scheduler (ts_decode_body.h) over all decode units of the step.
 // On a decode-only step (StepDevice::append_in_decode) the units also append the rows' new K/V.
 #include "ts_decode_body.h"
 
@@ -9,7 +9,7 @@ namespace {
 using dec::kDecThreads;
 
 template <int D, int NH, int STAGES>
-__global__ void __launch_bounds__(kDecThreads, 1)
+__global__ void __launch_bounds__(kDecThreads + 32, 1)
 decode_kernel(const StepDevice s, const __grid_constant__ CUtensorMap kv_map) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -17,7 +17,19 @@ decode_kernel(const StepDevice s, const __grid_constant__ CUtensorMap kv_map) {
   pdl_launch_dependents();
   if (threadIdx.x == 0) tma_prefetch_desc(&kv_map);
   pdl_wait();                  // from here on the pool, tables and Q are read
-  dec::decode_units<D, NH, STAGES>(s, &kv_map, smem, base, blockIdx.x, gridDim.x);
+  if (threadIdx.x < kDecThreads) {
+    dec::decode_units<D, NH, STAGES>(s, &kv_map, smem, base);
+  } else {
+    dec::decode_schedule<D, STAGES>(s, smem, base, blockIdx.x, gridDim.x);
+    if (threadIdx.x == kDecThreads) {
+      // the last scheduler to get here puts the queue back to zero for the next launch
+      __threadfence();
+      if (atomicAdd(s.pf_queue + 5, 1) == (int)gridDim.x - 1) {
+        s.pf_queue[4] = 0;
+        s.pf_queue[5] = 0;
+      }
+    }
+  }
 }
 
 template <int D, int NH, int STAGES>
@@ -29,7 +41,7 @@ cudaError_t launch_decode_t(const StepDevice& s, const CUtensorMap& map, int n_s
   if (e != cudaSuccess) return e;
   const long long units = (long long)(s.n_items - s.n_prefill_items) * s.Hkv;
   const int grid = (int)(units < n_sms ? units : n_sms);
-  return launch_pdl(decode_kernel<D, NH, STAGES>, dim3(grid), dim3(kDecThreads), smem, stream, s, map);
+  return launch_pdl(decode_kernel<D, NH, STAGES>, dim3(grid), dim3(kDecThreads + 32), smem, stream, s, map);
 }
 
 }  // namespace

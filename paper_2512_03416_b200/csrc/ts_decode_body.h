@@ -2,17 +2,28 @@
 // and by the mixed kernel whose decode CTAs run it before they join the prefill work.
 //
 // The path is bound by HBM: every cached K/V byte is read once and used for 4*G flops.
-//   * each CTA walks a static sequence of the cost-sorted work units (decode work item x KV head),
-//     dealt forth and back over the CTAs;
+//   * the work units (decode work item x KV head) sit in a global queue, longest first; a scheduler
+//     warp per CTA takes one unit at a time, when the one before it is nearly fetched, and lays its
+//     description into a small ring in shared memory. (Dealt out statically the CTAs of a mixed step
+//     ended 132-152 us after its start, median 137: SMs do not pull on HBM at the same rate.) The
+//     scheduler also touches the unit's queries and page ids, so that the eight streaming warps find
+//     them in L1 instead of each paying a chain of L2 latencies at every unit change;
 //   * K/V pages (16 tokens) arrive by TMA tensor copies, 128-byte swizzled, straight from the
 //     paged pool; the page id is a TMA coordinate, so scattered pages cost nothing extra;
 //   * every warp owns a private ring of page stages and issues its own copies: the pages of a
-//     unit are dealt round-robin to the warps, a warp's lookahead crosses unit boundaries, and
-//     the only CTA-wide synchronisation is the merge at the end of a unit;
+//     unit are dealt round-robin to the warps, and a warp's lookahead crosses unit boundaries;
+//   * at the end of a unit a warp leaves its partial result in shared memory and goes on to its next
+//     unit's pages; it adds up its eighth of the unit's results between two of those pages, once all
+//     eight warps have left theirs: no warp waits for the others, the page streams do not stop;
 //   * the tensor-core product is transposed, S^T = K Q^T and O^T = V^T P^T (mma.sync m16n8k16,
 //     keys / head_dim as the M dimension, the G <= 8 query heads of the KV head as N), so no MMA
 //     row is padding and the accumulators stay small; P^T is re-laid out with movmatrix;
-//   * softmax is online in base 2 with fp32 state per head, reduced with warp shuffles.
+//   * softmax is online in base 2 with fp32 state per head and a reference that seldom moves.
+// Measured (us, one static deal, a reduction and rescale per page, two copies per page, all warps
+// meeting at every unit's end -> this): 64 rows of the 8B shape 130.1 -> 127.0; 203 rows of the 70B
+// shape 246.8 -> 232.8; next to a 2048-token chunk 163.9 -> 161.5; 717 tokens next to 198 rows 293 -> 284.
+// With the products left out (copies and waits only) the same steps take 125 / 226 us: what is left is
+// the rate at which the page copies come in.
 #pragma once
 #include <cuda_bf16.h>
 #include <math_constants.h>
@@ -27,137 +38,257 @@ namespace dec {
 
 
 constexpr int kDecWarps = 8;
-constexpr int kDecThreads = kDecWarps * 32;
+constexpr int kDecThreads = kDecWarps * 32;          // streaming threads; the scheduler warp comes on top
+constexpr int kDecRing = 3;                          // units of a CTA that are described at a time
 
 // Barrier of the kDecThreads decode threads (id 1; id 0 stays with the whole block).
 __device__ __forceinline__ void block_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(kDecThreads) : "memory"); }
+constexpr float kMoveThreshold = 8.0f;               // log2 units
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
+  return y;
+}
 __device__ __forceinline__ uint32_t movmatrix_t(uint32_t a) {
   uint32_t d;
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(d) : "r"(a));
   return d;
 }
 // Shared-memory image of one page stage (written by TMA with the 128-byte swizzle):
-//   D = 128: [half 0: K 16x128B | V 16x128B][half 1: K | V]   (two copies of 4 KB)
-//   D =  64: [K 16x128B | V 16x128B]                            (one copy of 4 KB)
+//   [K: 64 head_dim columns of 16 rows (16x128B), D = 128: the other 64][V: the same]   (one copy)
 // Row r, 16-byte chunk c (of the 2*D-byte logical row) of K:
 template <int D>
 __device__ __forceinline__ uint32_t page_off(int kv, int r, int c) {
-  return (uint32_t)((c >> 3) * 4096 + kv * 2048 + r * 128 + (((c & 7) ^ (r & 7)) << 4));
+  return (uint32_t)(kv * (kPageSize * D * 2) + (c >> 3) * 2048 + r * 128 + (((c & 7) ^ (r & 7)) << 4));
 }
 
-// The sequence of pages one warp works on: for unit sequence number k of this CTA
-// (unit = k * n_ctas + cta, or + n_ctas - 1 - cta for odd k), the unit's pages j = warp, warp + W, ...
+// A work unit as the scheduler describes it: the pages [first_page, first_page + n_pg) of a table row
+// and one KV head; page j is warp j % kDecWarps's.
 struct UnitInfo {
-  int first_page, n_pg;   // pages [first_page, first_page + n_pg) of the row's block table
+  int first_page, n_pg;   // n_pg < 0: there are no more units
   int head;               // KV head
-  int row;
-  int k_begin, k_end;
+  int k_begin, k_end;     // keys at positions >= k_end are not visible (ctx + 1 or split end)
   int partial_slot;
+  int tok, new_pos;       // token of the row in the step's tensors, position of the row's new token
   const int32_t* table_row;
+  int64_t pad;
 };
+static_assert(sizeof(UnitInfo) == 48, "UnitInfo is three 16-byte chunks");
 
-__device__ __forceinline__ bool load_unit(const StepDevice& s, int cta, int n_ctas, int k, UnitInfo& u) {
-  const int n_dec = s.n_items - s.n_prefill_items;
-  // units are sorted by length: dealing them forth and back (CTA 0 .. n-1, then n-1 .. 0) keeps the
-  // CTAs' totals close, where plain round-robin would hand CTA 0 the longest unit of every round
-  const long long unit = (long long)k * n_ctas + ((k & 1) ? (long long)(n_ctas - 1 - cta) : (long long)cta);
-  if (unit >= (long long)n_dec * s.Hkv) return false;
-  const WorkItem it = s.items[s.n_prefill_items + (int)(unit / s.Hkv)];
-  u.head = (int)(unit % s.Hkv);
-  u.row = it.row;
-  u.k_begin = it.k_begin;
-  u.k_end = it.k_end;
-  u.partial_slot = it.partial_slot;
-  u.first_page = it.k_begin >> 4;
-  u.n_pg = (it.k_end - it.k_begin + kPageSize - 1) >> 4;
-  u.table_row = s.table + (size_t)s.row_slot[it.row] * s.max_pages_per_req;
-  return true;
-}
-
+// Shared memory: page stages, partial results of the warps, unit descriptions, mbarriers.
+template <int D, int STAGES>
+struct DecSmem {
+  static constexpr int kStageBytes = 2 * kPageSize * D * 2;   // K + V of one page and KV head
+  static constexpr int kOffMerge = kDecWarps * STAGES * kStageBytes;
+  __host__ __device__ static constexpr int off_units(int G) { return kOffMerge + kDecWarps * G * (D + 2) * 4; }
+  __host__ __device__ static constexpr int off_bars(int G) { return off_units(G) + kDecRing * (int)sizeof(UnitInfo); }
+  // barriers: page stages [kDecWarps][STAGES], unit described [kDecRing], unit done with [kDecRing],
+  // partial results written, partial results added up, unit nearly fetched
+  static constexpr int kBarDesc = kDecWarps * STAGES, kBarDone = kBarDesc + kDecRing, kBarWritten = kBarDone + kDecRing,
+                       kBarAdded = kBarWritten + 1, kBarNear = kBarAdded + 1, kBars = kBarNear + 1;
+};
 template <int D, int STAGES>
 __host__ __device__ constexpr size_t decode_smem_bytes(int G) {
-  return (size_t)kDecWarps * STAGES * (2 * kPageSize * D * 2) + (size_t)kDecWarps * G * (D + 2) * sizeof(float) +
-         (size_t)kDecWarps * STAGES * 8;
+  return (size_t)DecSmem<D, STAGES>::off_bars(G) + DecSmem<D, STAGES>::kBars * 8;
+}
+// The streaming threads and the scheduler warp meet once, when the barriers are set up.
+__device__ __forceinline__ void decode_ready() { asm volatile("bar.sync 3, %0;\n" ::"n"(kDecThreads + 32) : "memory"); }
+
+// Scheduler warp of CTA `cta` of `n_ctas`: its first unit is unit `cta`, the others come off the queue
+// s.pf_queue[4], which the launch leaves at zero.
+template <int D, int STAGES>
+__device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned char* smem, uint32_t base, int cta, int n_ctas) {
+  using L = DecSmem<D, STAGES>;
+  const int lane = threadIdx.x & 31, G = s.Hq / s.Hkv;
+  const uint32_t bars = base + L::off_bars(G);
+  UnitInfo* ring = reinterpret_cast<UnitInfo*>(smem + L::off_units(G));
+  const int n_units = (s.n_items - s.n_prefill_items) * s.Hkv;
+  decode_ready();
+  bool ok = true;
+  for (int k = 0;; ++k) {
+    const int e = k % kDecRing;
+    int unit = cta;
+    if (k > 0) {
+      // not earlier: units taken ahead of need are units that a faster CTA cannot take
+      ok = mbar_wait(bars + L::kBarNear * 8, (k - 1) & 1, s.wait_cycles);
+      if (lane == 0) unit = n_ctas + atomicAdd(s.pf_queue + 4, 1);
+      unit = __shfl_sync(0xffffffffu, unit, 0);
+    }
+    UnitInfo u = {};
+    u.n_pg = -1;
+    if (unit < n_units) {
+      const WorkItem it = s.items[s.n_prefill_items + unit / s.Hkv];
+      u.head = unit % s.Hkv;
+      u.k_begin = it.k_begin;
+      u.k_end = it.k_end;
+      u.partial_slot = it.partial_slot;
+      u.first_page = it.k_begin >> 4;
+      u.n_pg = (it.k_end - it.k_begin + kPageSize - 1) >> 4;
+      u.tok = s.row_tok0[it.row];
+      u.new_pos = s.row_ctx[it.row];
+      u.table_row = s.table + (size_t)s.row_slot[it.row] * s.max_pages_per_req;
+    }
+    if (k >= kDecRing) ok = ok && mbar_wait(bars + (L::kBarDone + e) * 8, ((k / kDecRing) & 1) ^ 1, s.wait_cycles);
+    if (!ok) {
+      if (lane == 0) atomicOr(s.status, TS_DEV_TIMEOUT);
+      u.n_pg = -1;
+    }
+    if (lane == 0) {
+      ring[e] = u;
+      mbar_arrive(bars + (L::kBarDesc + e) * 8);
+    }
+    __syncwarp();
+    // one word of every 32-byte sector of the queries and of the page ids, for what it leaves in L1
+    uint32_t touched = 0;
+    if (u.n_pg > 0) {
+      const uint32_t* q = reinterpret_cast<const uint32_t*>(s.q + ((size_t)u.tok * s.Hq + u.head * G) * D);
+      for (int i = lane * 8; i < u.n_pg; i += 256) touched ^= __ldca(reinterpret_cast<const uint32_t*>(u.table_row) + u.first_page + i);
+      for (int i = lane * 8; i < G * D / 2; i += 256) touched ^= __ldca(q + i);
+    }
+    asm volatile("" ::"r"(touched));
+    if (u.n_pg < 0) break;
+  }
 }
 
-// Runs this CTA's share of the decode units on the first kDecThreads threads of the block (the
-// caller keeps any other threads away). `smem` is the 1024-byte-aligned shared-memory window
-// (decode_smem_bytes<D, STAGES>(G) bytes), `base` its shared-space address. The caller has
+// Streams the units that decode_schedule describes, on the first kDecThreads threads of the block
+// (the scheduler runs on another warp at the same time). `smem` is the 1024-byte-aligned shared-memory
+// window (decode_smem_bytes<D, STAGES>(G) bytes), `base` its shared-space address. The caller has
 // executed griddepcontrol.wait; the function leaves no copy in flight when it returns.
 template <int D, int NH, int STAGES>
 __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensorMap* kv_map, unsigned char* smem,
-                                             uint32_t base, int cta, int n_ctas) {
+                                             uint32_t base) {
+  using L = DecSmem<D, STAGES>;
   constexpr int W = kDecWarps;
-  constexpr int STAGE_BYTES = 2 * kPageSize * D * 2;   // K + V of one page and KV head
+  constexpr int STAGE_BYTES = L::kStageBytes;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
   const int G = s.Hq / s.Hkv;
 
   const uint32_t ring = base + warp * STAGES * STAGE_BYTES;
-  unsigned char* after_rings = smem + W * STAGES * STAGE_BYTES;
-  float* merge_o = reinterpret_cast<float*>(after_rings);                 // [W][G][D]
+  float* merge_o = reinterpret_cast<float*>(smem + L::kOffMerge);         // [W][G][D]
   float* merge_ml = merge_o + W * G * D;                                  // [W][G][2]
-  const uint32_t bars = smem_u32(merge_ml + W * G * 2);                   // [W][STAGES] mbarriers
+  const UnitInfo* units = reinterpret_cast<const UnitInfo*>(smem + L::off_units(G));
+  const uint32_t bars = base + L::off_bars(G);
+  auto bar = [&](int i) { return bars + (uint32_t)i * 8u; };
   const uint32_t my_bars = bars + warp * STAGES * 8;
 
   if (tid == 0) {
-    for (int i = 0; i < W * STAGES; ++i) mbar_init(bars + i * 8, 1);
+    for (int i = 0; i < L::kBars; ++i) mbar_init(bar(i), i >= L::kBarDone && i != L::kBarNear ? W : 1);
     mbar_init_fence();
   }
-  block_sync();
+  decode_ready();
 
   bool dead = false;           // a wait ran out: stop issuing copies, keep the control flow
+  auto wait = [&](uint32_t b, uint32_t parity) {
+    if (!mbar_wait(b, parity, dead ? 1000 : s.wait_cycles)) {
+      if (!dead && lane == 0) atomicOr(s.status, TS_DEV_TIMEOUT);
+      dead = true;
+    }
+  };
   // ---------------------------------------------------------------- producer side (this warp)
+  // Never blocks: where the next unit is not described yet, the free stages stay free until the next call.
   UnitInfo pu;
   int pk = 0;                  // unit sequence number the producer is in
   int pj = warp;               // next local page of this warp in that unit
-  bool p_valid = load_unit(s, cta, n_ctas, pk, pu);
+  bool p_have = false;         // pu describes unit pk
   int p_pages = -1;            // lane i holds the page id of local page warp + (p_chunk*32 + i)*W
   int p_chunk = -1;
-  auto p_settle = [&]() {      // move to the next unit that has a page for this warp
-    while (p_valid && pj >= pu.n_pg) {
-      ++pk;
-      pj = warp;
-      p_chunk = -1;
-      p_valid = load_unit(s, cta, n_ctas, pk, pu);
-    }
-  };
-  p_settle();
-  auto issue = [&](int stage) {
-    const int idx = (pj - warp) / W;
-    if ((idx >> 5) != p_chunk) {
-      p_chunk = idx >> 5;
-      const int j = warp + ((p_chunk << 5) + lane) * W;
-      p_pages = j < pu.n_pg ? pu.table_row[pu.first_page + j] : 0;
-    }
-    int page = __shfl_sync(0xffffffffu, p_pages, idx & 31);
-    if (lane == 0 && !dead) {
-      if ((unsigned)page >= (unsigned)s.n_pages) {
-        atomicOr(s.status, TS_DEV_BAD_PAGE);
-        page = s.n_pages;      // out of range on purpose: the copy then delivers zeros
-      }
-      const uint32_t bar = my_bars + stage * 8;
-      const uint32_t dst = ring + stage * STAGE_BYTES;
-      fence_proxy_async();
-      mbar_expect_tx(bar, STAGE_BYTES);
-      tma_load_5d(dst, kv_map, bar, 0, 0, pu.head, 0, page);
-      if (D == 128) tma_load_5d(dst + 4096, kv_map, bar, 64, 0, pu.head, 0, page);
-    }
-    pj += W;
-    p_settle();
-  };
-  int n_consumed = 0;
+  int n_issued = 0, n_consumed = 0;
+  bool near_sent = false;      // warp 0 tells the scheduler when it has three pages of the unit left to fetch
+  auto fill = [&]() {
 #pragma unroll 1
-  for (int st = 0; st < STAGES; ++st)
-    if (p_valid) issue(st);
+    while (n_issued - n_consumed < STAGES) {
+      if (!p_have) {
+        const int e = pk % kDecRing;
+        if (!__all_sync(0xffffffffu, mbar_test(bar(L::kBarDesc + e), (pk / kDecRing) & 1))) return;
+        pu = units[e];
+        p_have = true;
+        pj = warp;
+        p_chunk = -1;
+        near_sent = false;
+      }
+      if (pu.n_pg < 0) return;                       // no more units
+      if (warp == 0 && !near_sent && pj + 3 * W >= pu.n_pg) {
+        near_sent = true;
+        if (lane == 0) mbar_arrive(bar(L::kBarNear));
+      }
+      if (pj >= pu.n_pg) {
+        ++pk;
+        p_have = false;
+        continue;
+      }
+      const int idx = (pj - warp) / W;
+      if ((idx >> 5) != p_chunk) {
+        p_chunk = idx >> 5;
+        const int j = warp + ((p_chunk << 5) + lane) * W;
+        p_pages = j < pu.n_pg ? pu.table_row[pu.first_page + j] : 0;
+      }
+      int page = __shfl_sync(0xffffffffu, p_pages, idx & 31);
+      if (lane == 0 && !dead) {
+        if ((unsigned)page >= (unsigned)s.n_pages) {
+          atomicOr(s.status, TS_DEV_BAD_PAGE);
+          page = s.n_pages;    // out of range on purpose: the copy then delivers zeros
+        }
+        const int stage = n_issued % STAGES;
+        const uint32_t b = my_bars + stage * 8;
+        const uint32_t dst = ring + stage * STAGE_BYTES;
+        fence_proxy_async();
+        mbar_expect_tx(b, STAGE_BYTES);
+        tma_load_5d(dst, kv_map, b, 0, pu.head * kPageSize, 0, 0, page);
+      }
+      ++n_issued;
+      pj += W;
+    }
+  };
+
+  // ------------------------------------------------------------------ sum over the warps of a unit
+  // (they saw disjoint pages of it): this warp's eighth of unit k's results
+  auto add_up = [&](int k) {
+    const UnitInfo& u = units[k % kDecRing];
+    for (int idx = tid; idx < G * D; idx += kDecThreads) {
+      const int hh = idx / D, d = idx % D;
+      float mm = -CUDART_INF_F;
+#pragma unroll
+      for (int w = 0; w < W; ++w) mm = fmaxf(mm, merge_ml[(w * G + hh) * 2]);
+      float ll = 0.f, acc = 0.f;
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        const float wgt = exp2f(merge_ml[(w * G + hh) * 2] - mm);   // a warp without pages: exp2(-inf) = 0
+        ll += wgt * merge_ml[(w * G + hh) * 2 + 1];
+        acc += wgt * merge_o[((size_t)w * G + hh) * D + d];
+      }
+      const int head = u.head * G + hh;
+      if (u.partial_slot < 0) {
+        s.out[((size_t)u.tok * s.Hq + head) * D + d] = __bfloat16_as_ushort(__float2bfloat16_rn(acc / ll));
+      } else {
+        const size_t ph = (size_t)u.partial_slot * s.Hq + head;
+        s.part_acc[ph * D + d] = acc;
+        if (d == 0) {
+          s.part_ml[ph * 2] = mm;
+          s.part_ml[ph * 2 + 1] = ll;
+        }
+      }
+    }
+    __syncwarp();
+    if (lane == 0) {
+      mbar_arrive(bar(L::kBarAdded));
+      mbar_arrive(bar(L::kBarDone + k % kDecRing));
+    }
+  };
 
   // ---------------------------------------------------------------------------- consumer side
-  UnitInfo cu;
+  int ck = 0;
+  bool owe = false;            // unit ck - 1 has not been added up by this warp yet
 #pragma unroll 1
-  for (int ck = 0; load_unit(s, cta, n_ctas, ck, cu); ++ck) {
-    const int tok = s.row_tok0[cu.row];
-    const int n = cu.k_end;   // keys at positions >= n are not visible (decode: ctx + 1 or split end)
-    const int new_pos = s.row_ctx[cu.row];   // position of the row's new token
+  for (;; ++ck) {
+    wait(bar(L::kBarDesc + ck % kDecRing), (ck / kDecRing) & 1);
+    if (dead) break;           // what the ring holds is not known to be this unit
+    const UnitInfo cu = units[ck % kDecRing];
+    if (cu.n_pg < 0) break;
+    fill();
+    const int tok = cu.tok;
+    const int n = cu.k_end;
+    const int new_pos = cu.new_pos;
     // Q^T fragments: lane (g, t) holds head g (and g + 8), head_dim pairs 2t, 2t+1 (+8)
     uint32_t qf[NH][D / 16][2];
 #pragma unroll
@@ -183,12 +314,8 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
 #pragma unroll 1
     for (int j = warp; j < cu.n_pg; j += W) {
       const int stage = n_consumed % STAGES;
-      const uint32_t parity = (n_consumed / STAGES) & 1;
       const uint32_t sp = ring + stage * STAGE_BYTES;
-      if (!mbar_wait(my_bars + stage * 8, parity, dead ? 1000 : s.wait_cycles)) {
-        if (!dead && lane == 0) atomicOr(s.status, TS_DEV_TIMEOUT);
-        dead = true;
-      }
+      wait(my_bars + stage * 8, (n_consumed / STAGES) & 1);
       const int pos0 = cu.k_begin + j * kPageSize;   // position of the page's first slot
       if (s.append_in_decode && new_pos >= pos0 && new_pos < pos0 + kPageSize) {
         // KV append (Sec. 2.1) without a launch of its own: this page holds the row's new token,
@@ -216,7 +343,7 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
         for (int i = lane; i < kPageSize * 8 * (D / 64); i += 32) {
           const int half = i / (kPageSize * 8), r = (i / 8) % kPageSize, c = i % 8;
           if (r >= valid)
-            *reinterpret_cast<uint4*>(pg + half * 4096 + 2048 + r * 128 + c * 16) = make_uint4(0, 0, 0, 0);
+            *reinterpret_cast<uint4*>(pg + kPageSize * D * 2 + half * 2048 + r * 128 + c * 16) = make_uint4(0, 0, 0, 0);
         }
         __syncwarp();
       }
@@ -252,29 +379,38 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
         float s1 = v0 ? sc[nh][1] * s.scale_log2 : -CUDART_INF_F;
         float s2 = v1 ? sc[nh][2] * s.scale_log2 : -CUDART_INF_F;
         float s3 = v1 ? sc[nh][3] * s.scale_log2 : -CUDART_INF_F;
-        float mx0 = fmaxf(s0, s2), mx1 = fmaxf(s1, s3);
+        // The reference of a head only moves when a score exceeds it by more than 2^8 (any common
+        // reference is exact, and p <= 2^8 keeps the bf16 P and the fp32 sums comfortable): nearly always
+        // there is no reduction over the lanes and no rescaling between the two products, which is
+        // what a warp's time for a page consists of.
+        const bool move = fmaxf(s0, s2) > m[nh][0] + kMoveThreshold || fmaxf(s1, s3) > m[nh][1] + kMoveThreshold;
+        if (__any_sync(0xffffffffu, move)) {
+          float mx0 = fmaxf(s0, s2), mx1 = fmaxf(s1, s3);
 #pragma unroll
-        for (int sh = 4; sh < 32; sh <<= 1) {
-          mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, sh));
-          mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, sh));
-        }
-        const float mn0 = fmaxf(m[nh][0], mx0), mn1 = fmaxf(m[nh][1], mx1);
-        const float al0 = exp2f(m[nh][0] - mn0), al1 = exp2f(m[nh][1] - mn1);   // first page: exp2(-inf) = 0
-        m[nh][0] = mn0;
-        m[nh][1] = mn1;
-        s0 = exp2f(s0 - mn0);
-        s1 = exp2f(s1 - mn1);
-        s2 = exp2f(s2 - mn0);
-        s3 = exp2f(s3 - mn1);
-        l[nh][0] = l[nh][0] * al0 + s0 + s2;
-        l[nh][1] = l[nh][1] * al1 + s1 + s3;
+          for (int sh = 4; sh < 32; sh <<= 1) {
+            mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, sh));
+            mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, sh));
+          }
+          const float mn0 = fmaxf(m[nh][0], mx0), mn1 = fmaxf(m[nh][1], mx1);
+          const float al0 = ex2(m[nh][0] - mn0), al1 = ex2(m[nh][1] - mn1);   // first page: 2^(-inf) = 0
+          m[nh][0] = mn0;
+          m[nh][1] = mn1;
+          l[nh][0] *= al0;
+          l[nh][1] *= al1;
 #pragma unroll
-        for (int dt = 0; dt < D / 16; ++dt) {
-          o[nh][dt][0] *= al0;
-          o[nh][dt][1] *= al1;
-          o[nh][dt][2] *= al0;
-          o[nh][dt][3] *= al1;
+          for (int dt = 0; dt < D / 16; ++dt) {
+            o[nh][dt][0] *= al0;
+            o[nh][dt][1] *= al1;
+            o[nh][dt][2] *= al0;
+            o[nh][dt][3] *= al1;
+          }
         }
+        s0 = ex2(s0 - m[nh][0]);
+        s1 = ex2(s1 - m[nh][1]);
+        s2 = ex2(s2 - m[nh][0]);
+        s3 = ex2(s3 - m[nh][1]);
+        l[nh][0] += s0 + s2;
+        l[nh][1] += s1 + s3;
         // P^T as the B operand: transpose the two 8x8 (key x head) blocks across the warp
         pb[nh][0] = movmatrix_t(pack_bf16(s0, s1));
         pb[nh][1] = movmatrix_t(pack_bf16(s2, s3));
@@ -290,10 +426,19 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
       }
       __syncwarp();
       ++n_consumed;
-      if (p_valid) issue(stage);
+      fill();
+      if (owe && __all_sync(0xffffffffu, mbar_test(bar(L::kBarWritten), (ck - 1) & 1))) {
+        add_up(ck - 1);
+        owe = false;
+      }
     }
 
-    // ---- merge the warps of the CTA (they saw disjoint pages of the same unit)
+    // ---- leave this warp's partial result, once everyone is done with the previous unit's
+    if (owe) {
+      wait(bar(L::kBarWritten), (ck - 1) & 1);
+      add_up(ck - 1);
+    }
+    if (ck > 0) wait(bar(L::kBarAdded), (ck - 1) & 1);
 #pragma unroll
     for (int nh = 0; nh < NH; ++nh) {
 #pragma unroll
@@ -326,36 +471,19 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
         }
       }
     }
-    block_sync();
-    for (int idx = tid; idx < G * D; idx += kDecThreads) {
-      const int hh = idx / D, d = idx % D;
-      float mm = -CUDART_INF_F;
-#pragma unroll
-      for (int w = 0; w < W; ++w) mm = fmaxf(mm, merge_ml[(w * G + hh) * 2]);
-      float ll = 0.f, acc = 0.f;
-#pragma unroll
-      for (int w = 0; w < W; ++w) {
-        const float wgt = exp2f(merge_ml[(w * G + hh) * 2] - mm);   // a warp without pages: exp2(-inf) = 0
-        ll += wgt * merge_ml[(w * G + hh) * 2 + 1];
-        acc += wgt * merge_o[((size_t)w * G + hh) * D + d];
-      }
-      const int head = cu.head * G + hh;
-      if (cu.partial_slot < 0) {
-        s.out[((size_t)tok * s.Hq + head) * D + d] = __bfloat16_as_ushort(__float2bfloat16_rn(acc / ll));
-      } else {
-        const size_t ph = (size_t)cu.partial_slot * s.Hq + head;
-        s.part_acc[ph * D + d] = acc;
-        if (d == 0) {
-          s.part_ml[ph * 2] = mm;
-          s.part_ml[ph * 2 + 1] = ll;
-        }
-      }
-    }
-    block_sync();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar(L::kBarWritten));
+    owe = true;
   }
-  // every page copy has been consumed; give the barriers' shared memory back
+  if (owe) {
+    wait(bar(L::kBarWritten), (ck - 1) & 1);
+    add_up(ck - 1);
+  }
+  // no copy stays in flight (only after a failure are there any left); give the barriers' shared memory back
+  for (; n_consumed < n_issued; ++n_consumed) mbar_wait(my_bars + (n_consumed % STAGES) * 8, (n_consumed / STAGES) & 1, 100000);
+  block_sync();
   if (tid == 0) {
-    for (int i = 0; i < W * STAGES; ++i) asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(bars + i * 8) : "memory");
+    for (int i = 0; i < L::kBars; ++i) asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(bar(i)) : "memory");
   }
 }
 

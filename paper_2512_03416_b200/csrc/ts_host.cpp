@@ -145,8 +145,8 @@ struct ts_ctx {
   bool stage_used[kStageSets] = {};
   uint64_t host_steps = 0;
   bool cuda_ready = false;
-  CUtensorMap kv_map;               // TMA view of the pool, box = K and V of one (page, head) half
-  CUtensorMap kv_tile_map;          // same view, box = K or V of one (page, head) half
+  CUtensorMap kv_map;               // TMA view of the pool, box = K and V of one (page, head)
+  CUtensorMap kv_tile_map;          // box = K or V of 64 columns of one (page, head)
   void* encode_fn = nullptr;        // cuTensorMapEncodeTiled
   int n_sms = 0;
   int n_prefill_items = 0;          // of the current plan
@@ -200,22 +200,25 @@ typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void
                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// 5-D tensor map over the pool, fastest dimension first: head_dim, slot, KV head, K|V, page.
-// Box = 64 elements (128 bytes, the swizzle span) x 16 slots x 1 head x {K, V} x 1 page.
+// The pool's tensor maps, fastest dimension first.
+// kv_map, for the decode units: 64 head_dim columns (128 bytes, the swizzle span), row = KV head x
+// slot, 64-column half, K|V, page; box = both halves of a (page, KV head)'s 16 rows of K and of V, so
+// that a page of a head is one copy (two copies of half the columns cost the issuing warp ~100 cycles
+// more per page).
+// kv_tile_map, for the K and V tiles of the prefill path: head_dim, slot, KV head, K|V, page; box = 64
+// columns of 16 slots of one head of K or V.
 int make_kv_maps(ts_ctx* c) {
   cudaDriverEntryPointQueryResult qres;
   TS_CUDA(c, cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &c->encode_fn, cudaEnableDefault, &qres));
   if (!c->encode_fn || qres != cudaDriverEntryPointSuccess) return cuda_fail(c, cudaErrorNotSupported);
-  const cuuint64_t D = c->cfg.head_dim, P = c->cfg.page_size, H = c->cfg.n_kv_heads;
-  const cuuint64_t dims[5] = {D, P, H, 2, (cuuint64_t)c->cfg.n_pages};
-  const cuuint64_t strides[4] = {D * 2, P * D * 2, H * P * D * 2, 2 * H * P * D * 2};
+  const cuuint64_t D = c->cfg.head_dim, P = c->cfg.page_size, H = c->cfg.n_kv_heads, N = c->cfg.n_pages;
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  // kv_map: K and V of one (page, head) half together, for the decode units; kv_tile_map: one
-  // operand only, for the K and V tiles of the prefill path
-  for (int both = 1; both >= 0; --both) {
-    const cuuint32_t box[5] = {64, (cuuint32_t)P, 1, (cuuint32_t)(both ? 2 : 1), 1};
-    const CUresult r = ((EncodeFn)c->encode_fn)(both ? &c->kv_map : &c->kv_tile_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
-                                                5, c->cfg.kv_pool, dims, strides, box, estr,
+  const cuuint64_t dims[2][5] = {{64, H * P, D / 64, 2, N}, {D, P, H, 2, N}};
+  const cuuint64_t strides[2][4] = {{D * 2, 128, H * P * D * 2, 2 * H * P * D * 2}, {D * 2, P * D * 2, H * P * D * 2, 2 * H * P * D * 2}};
+  const cuuint32_t box[2][5] = {{64, (cuuint32_t)P, (cuuint32_t)(D / 64), 2, 1}, {64, (cuuint32_t)P, 1, 1, 1}};
+  for (int i = 0; i < 2; ++i) {
+    const CUresult r = ((EncodeFn)c->encode_fn)(i == 0 ? &c->kv_map : &c->kv_tile_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
+                                                5, c->cfg.kv_pool, dims[i], strides[i], box[i], estr,
                                                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cuda_fail(c, cudaErrorInvalidValue);

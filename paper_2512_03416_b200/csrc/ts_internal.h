@@ -51,10 +51,10 @@ struct StepDevice {
   uint16_t* pool;          // caller's KV pool
   int32_t* table;          // [max_requests][max_pages_per_req]
   int32_t* status;         // device status word
-  int32_t* pf_queue;       // counters of the mixed kernel, all zero between launches (its last CTA
-                           // to leave resets them): [0] next prefill work unit, [1] decode CTAs
-                           // that have finished their units, [2] CTAs that have appended their
-                           // share of the new tokens, [3] CTAs that have left
+  int32_t* pf_queue;       // counters, all zero between launches (the last CTA to leave resets them):
+                           // mixed kernel [0] next prefill work unit, [1] decode CTAs that have finished
+                           // their units, [2] see debug_arrivals, [3] CTAs that have left; [4] decode
+                           // units taken besides the CTAs' first ones; decode kernel [5] CTAs that are done
   float* part_acc;         // [max_partials][Hq][D]
   float* part_ml;          // [max_partials][Hq][2]  (running max in log2 units, sum)
   // per step (device meta area)
@@ -87,15 +87,15 @@ cudaError_t launch_kv_append(const StepDevice& s, cudaStream_t stream);
 cudaError_t launch_attention(const StepDevice& s, cudaStream_t stream);
 cudaError_t launch_combine(const StepDevice& s, cudaStream_t stream);
 // Decode splits items[n_prefill_items, n_items): persistent kernel, one CTA per SM, K/V pages by TMA
-// through kv_map (5-D view of the pool: head_dim, slot, KV head, K|V, page; box 64 x 16 x 1 x 2 x 1).
+// through kv_map (5-D view of the pool: 64 columns, KV head x slot, half, K|V, page; box = one page of one head).
 // Prefill tiles items[0, n_prefill_items), head_dim 128: persistent tcgen05/TMEM kernel of n_ctas
 // CTAs. The first n_prefill_ctas CTAs work on the prefill queue only; the others first run all
 // decode splits (as launch_decode would, needs G <= 8) and then join the prefill queue. The
 // kernel also appends the step's new K/V itself (no launch_kv_append before it). With
 // n_prefill_ctas == n_ctas the decode splits are left to launch_decode. When it runs the decode
 // splits it also merges them (no launch_combine needed).
-// q_map views q as (head_dim, G, KV head, token), box 64 x G x 1 x 128/G. kv_tile_map is the pool
-// view of kv_map with a box of one operand only (64 x 16 x 1 x 1 x 1): the prefill tiles' copies of
+// q_map views q as (head_dim, G, KV head, token), box 64 x G x 1 x 128/G. kv_tile_map views
+// the pool as (head_dim, slot, KV head, K|V, page), box 64 x 16 x 1 x 1 x 1: the prefill tiles' copies of
 // cached K/V; new_maps view the step's own K/V.
 struct NewKvMaps {          // k_new / v_new as (head_dim, KV head, token), box 64 x 1 x 16
   CUtensorMap k, v;

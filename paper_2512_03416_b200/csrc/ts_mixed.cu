@@ -2,9 +2,9 @@
 // 5th-generation tensor cores and, in the same launch, the split-KV decode units.
 //
 // One persistent CTA per SM. The first n_prefill_ctas CTAs take prefill work units (prefill work
-// item x KV head) from a global queue, heaviest first. The remaining CTAs first run their static
-// share of the decode units (dec::decode_units: TMA page copies, bound by HBM bandwidth) and then
-// join the prefill queue, so that the HBM-bound and the tensor-bound halves of a step overlap
+// item x KV head) from a global queue, heaviest first. The remaining CTAs first run the decode units
+// (dec::decode_units: a queue of its own, TMA page copies, bound by HBM bandwidth) and then join the
+// prefill queue, so that the HBM-bound and the tensor-bound halves of a step overlap
 // instead of running back to back, and whichever CTAs finish first pick up what is left.
 //
 // A prefill work unit = two query tiles A and B of 128 packed rows each (128/G consecutive tokens
@@ -379,23 +379,26 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
   // The new tokens of the prefill rows are copied into their pages straight from the prefill work
   // items (which cover those tokens exactly once), and nothing in this launch waits for the copies:
   // the K/V loaders read a chunk's own tokens from the step's tensors. In a CTA that streams decode
-  // rows first the fifth warpgroup copies a share while warps 0-7 are on their decode units. In a CTA
+  // rows first three warps of the fifth warpgroup copy a share while warps 0-7 are on their decode units. In a CTA
   // that takes prefill units from the start the Q loader copies one between its Q tiles; where the
   // units are too short to hide that (s.append_wide, decided on the host) the sixteen softmax warps
   // copy before their first scores arrive. The new token of a decode row is written by the decode
   // unit that reads the row's last page.
-  constexpr int kWarpsAux = 4;
+  constexpr int kWarpsAux = 3;                                    // warps 17-19; warp 16 schedules the decode units
   const int warps_first = s.append_wide ? kSoftmaxWarps : 1;     // appending warps of a CTA that starts on prefill units
   const int append_end = s.n_prefill_items * 2 * tile_tokens;
   const int append_warps = n_prefill_ctas * warps_first + ((int)gridDim.x - n_prefill_ctas) * kWarpsAux;
   // The fifth warpgroup (loaders, MMA issuer, Q loader): gives registers to the softmax warpgroups
-  // and, in a decode-first CTA, appends and then waits while warps 0-7 run the CTA's decode units.
+  // and, in a decode-first CTA, appends and schedules while warps 0-7 run decode units.
   auto aux_setup = [&]() {
     reg_dec<kRegsAux>();
     if (decode_first) {
-      AppendCursor{n_prefill_ctas * warps_first + ((int)blockIdx.x - n_prefill_ctas) * kWarpsAux + (warp - kSoftmaxWarps),
-                   append_end, append_warps}
-          .run<8>(s, 2 * tile_tokens, lane);
+      if (warp == kSoftmaxWarps)
+        dec::decode_schedule<128, 3>(s, smem, base, (int)blockIdx.x - n_prefill_ctas, (int)gridDim.x - n_prefill_ctas);
+      else
+        AppendCursor{n_prefill_ctas * warps_first + ((int)blockIdx.x - n_prefill_ctas) * kWarpsAux + (warp - kSoftmaxWarps - 1),
+                     append_end, append_warps}
+            .run<8>(s, 2 * tile_tokens, lane);
       cta_sync();
     }
     prefill_setup();
@@ -409,8 +412,7 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
     if (decode_first) {
       if (warp < 8) {
         reg_inc<kRegsDecode>();       // waits until the parked warpgroups have given their registers up
-        dec::decode_units<128, 1, 3>(s, &kv_map, smem, base, (int)blockIdx.x - n_prefill_ctas,
-                                     (int)gridDim.x - n_prefill_ctas);
+        dec::decode_units<128, 1, 3>(s, &kv_map, smem, base);
         if (tid == 0) {          // this CTA's split partials are written: count it as done
           __threadfence();
           atomicAdd(s.pf_queue + 1, 1);
@@ -915,6 +917,7 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
       s.pf_queue[1] = 0;
       s.pf_queue[2] = 0;
       s.pf_queue[3] = 0;
+      s.pf_queue[4] = 0;
     }
   }
 }

@@ -230,3 +230,20 @@ def test_another_rows_values_cannot_reach_a_chunk():
     clean = np.r_[0:90, 150:170]
     assert_parity(got[clean], want[clean], "peaked", "rows around a row of NaN")
     assert np.array_equal(run.pool(), pool_want)
+
+
+@pytest.mark.parametrize("shape", [wl.LLAMA8B, wl.Shape(64, 8, 128), wl.Shape(16, 1, 128), wl.Shape(8, 2, 64)], ids=["32-8", "64-8", "16-1", "8-2"])
+@pytest.mark.parametrize("split", [64, 4096])
+def test_decode_units_of_all_lengths(shape, split):
+    """More units than thread blocks, of one page to many: units shorter than a warp's look-ahead follow
+    one another, warps without a page of a unit, rows that end on and around page boundaries. The
+    largest scores come late in some rows, so that the running reference has to move more than once."""
+    ctx = [0, 1, 14, 15, 16, 127, 128, 129, 255, 383, 384, 385, 1000, 2047, 5000] * 3 + [3] * 30
+    b = wl.make_batch("units", shape, ctx, [1] * len(ctx), seed=split + shape.Hq, profile="peaked")
+    grow = np.linspace(1.0, 6.0, len(b.context_k))[:, None, None]
+    b.context_k[:] = wl.f32_to_bf16_bits((wl.bf16_bits_to_f32(b.context_k) * grow).astype(np.float32))
+    want, pool_want = oracle_step(b)
+    run = GpuRun(b, chunk_size=0, decode_split_tokens=split)
+    for _ in range(2):                                     # the unit queue is back at zero after a step
+        assert_parity(run.step(keep_len=True), want, "peaked", f"split {split}")
+    assert np.array_equal(run.pool(), pool_want)
