@@ -1,6 +1,6 @@
 // Stand-alone split-KV flash-decode kernel for the 1-token rows (sm_100a): one persistent CTA
 // per SM running dec::decode_units and its scheduler (ts_decode_body.h) over all decode units of the step.
-// On a decode-only step (StepDevice::append_in_decode) the units also append the rows' new K/V.
+// The units also append the rows' new K/V.
 #include "ts_decode_body.h"
 
 namespace ts {
@@ -10,7 +10,7 @@ using dec::kDecThreads;
 
 template <int D, int NH, int STAGES>
 __global__ void __launch_bounds__(kDecThreads + 32, 1)
-decode_kernel(const StepDevice s, const __grid_constant__ CUtensorMap kv_map) {
+decode_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUtensorMap kv_map) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));

@@ -117,16 +117,16 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
     UnitInfo u = {};
     u.n_pg = -1;
     if (unit < n_units) {
-      const WorkItem it = s.items[s.n_prefill_items + unit / s.Hkv];
+      const WorkItem it = s.item(s.n_prefill_items + unit / s.Hkv);
       u.head = unit % s.Hkv;
       u.k_begin = it.k_begin;
       u.k_end = it.k_end;
       u.partial_slot = it.partial_slot;
       u.first_page = it.k_begin >> 4;
       u.n_pg = (it.k_end - it.k_begin + kPageSize - 1) >> 4;
-      u.tok = s.row_tok0[it.row];
-      u.new_pos = s.row_ctx[it.row];
-      u.table_row = s.table + (size_t)s.row_slot[it.row] * s.max_pages_per_req;
+      u.tok = s.row_tok0(it.row);
+      u.new_pos = s.row_ctx(it.row);
+      u.table_row = s.table + (size_t)s.row_slot(it.row) * s.max_pages_per_req;
     }
     if (k >= kDecRing) ok = ok && mbar_wait(bars + (L::kBarDone + e) * 8, ((k / kDecRing) & 1) ^ 1, s.wait_cycles);
     if (!ok) {
@@ -317,7 +317,7 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
       const uint32_t sp = ring + stage * STAGE_BYTES;
       wait(my_bars + stage * 8, (n_consumed / STAGES) & 1);
       const int pos0 = cu.k_begin + j * kPageSize;   // position of the page's first slot
-      if (s.append_in_decode && new_pos >= pos0 && new_pos < pos0 + kPageSize) {
+      if (new_pos >= pos0 && new_pos < pos0 + kPageSize) {
         // KV append (Sec. 2.1) without a launch of its own: this page holds the row's new token,
         // which is not in the pool yet. Lay its K and V over the page image in shared memory and
         // write them to the pool page; a lane moves one 16-byte chunk of K or V.

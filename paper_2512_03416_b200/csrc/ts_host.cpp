@@ -35,7 +35,6 @@ struct Layout {
   size_t off_status, off_table, off_meta, off_delta, off_part_acc, off_part_ml, off_stage;
   size_t meta_bytes, slot_bytes, delta_bytes, stage_q_bytes, stage_kv_bytes, stage_set_bytes, total;
   // int32 offsets inside the meta area
-  size_t m_row_slot, m_row_ctx, m_row_qlen, m_row_tok0, m_items, m_combines, m_end;
 };
 
 bool shape_ok(const ts_config* c) {
@@ -56,15 +55,8 @@ void compute_layout(const ts_config* c, Layout* L) {
   L->max_tokens = c->chunk_size > 0 ? c->chunk_size : kDefaultMaxTokens;
   L->max_partials = 2048 + 2 * R;
   L->max_items = L->max_partials + R + ceil_div(L->max_tokens, std::max(1, ts::kPackedRowsPerTile / G)) + R;
-  size_t m = 0;
-  L->m_row_slot = m; m += R;
-  L->m_row_ctx = m; m += R;
-  L->m_row_qlen = m; m += R;
-  L->m_row_tok0 = m; m += R + 1;
-  m = (m + 7) / 8 * 8;                       // items start 32-byte aligned
-  L->m_items = m; m += (size_t)L->max_items * 8;
-  L->m_combines = m; m += (size_t)R * 4;
-  L->m_end = m;
+  // row arrays, work items (32-byte aligned), combine list; a step packs only what it has
+  const size_t m = ((size_t)3 * R + 1 + 7) / 8 * 8 + (size_t)L->max_items * 8 + (size_t)R * 4;
   L->meta_bytes = align_up(m * sizeof(int32_t));
   L->delta_bytes = align_up((size_t)kDeltaCapacity * sizeof(TableDelta));
   size_t off = 0;
@@ -413,7 +405,7 @@ int sync_tables(ts_ctx* c, const ts_step* st, cudaStream_t stream, int* n_slot_d
   }
   if (c->deltas.size() <= (size_t)kSlotDeltas) {
     // the usual case (a few rows crossed a page boundary): the entries travel with the step's
-    // metadata over the copy stream, see upload_meta
+    // metadata, see send_meta
     *n_slot_deltas = (int)c->deltas.size();
     return TS_OK;
   }
@@ -442,56 +434,83 @@ void commit_table_sync(ts_ctx* c) {
   c->sync_marks.clear();
 }
 
-// Sends the step's metadata to the next device slot. The copy goes over the context's copy stream:
-// it only has to wait for the step that last read this slot (kRing steps ago), so it runs while
-// the previous step's kernels are still busy, and the caller's stream just waits for its event.
-int upload_meta(ts_ctx* c, const ts_step* st, int n_items, int n_combines, int n_slot_deltas, cudaStream_t stream) {
-  const int slot = c->meta_next;
-  c->meta_next = (c->meta_next + 1) % kRing;
-  c->meta_cur = slot;
-  MetaSlot& ms = c->meta[slot];
-  if (ms.copy_in_flight) {                 // the pinned buffer is free once its last upload is done
-    TS_CUDA(c, cudaEventSynchronize(ms.copied));
-    ms.copy_in_flight = false;
-  }
-  int32_t* m = (int32_t*)ms.host;
+// Word offsets of the step's row arrays and work list, packed one after the other; returns the total.
+size_t meta_offsets(int n_rows, int n_items, int n_combines, ts::StepDevice* d) {
+  size_t at = 0;
+  d->o_slot = 0; at += n_rows;
+  d->o_ctx = (uint32_t)at; at += n_rows;
+  d->o_tok0 = (uint32_t)at; at += n_rows + 1;
+  at = (at + 7) / 8 * 8;                     // items start 32-byte aligned
+  d->o_items = (uint32_t)at; at += (size_t)n_items * 8;
+  d->o_combines = (uint32_t)at; at += (size_t)n_combines * 4;
+  return at;
+}
+void pack_meta(const ts_ctx* c, const ts_step* st, const ts::StepDevice& d, int n_items, int n_combines, int32_t* dst) {
   const int R = st->n_rows;
-  std::memcpy(m + c->L.m_row_slot, st->slot, sizeof(int32_t) * R);
-  std::memcpy(m + c->L.m_row_ctx, st->ctx_len, sizeof(int32_t) * R);
-  std::memcpy(m + c->L.m_row_qlen, st->q_len, sizeof(int32_t) * R);
-  std::memcpy(m + c->L.m_row_tok0, c->tok0.data(), sizeof(int32_t) * (R + 1));
-  size_t used = c->L.m_row_tok0 + R + 1;
-  if (n_items > 0) {
-    std::memcpy(m + c->L.m_items, c->items.data(), sizeof(WorkItem) * n_items);
-    used = c->L.m_items + (size_t)n_items * 8;
+  std::memcpy(dst + d.o_slot, st->slot, sizeof(int32_t) * R);
+  std::memcpy(dst + d.o_ctx, st->ctx_len, sizeof(int32_t) * R);
+  std::memcpy(dst + d.o_tok0, c->tok0.data(), sizeof(int32_t) * (R + 1));
+  if (n_items > 0) std::memcpy(dst + d.o_items, c->items.data(), sizeof(WorkItem) * n_items);
+  if (n_combines > 0) std::memcpy(dst + d.o_combines, c->combines.data(), sizeof(CombineItem) * n_combines);
+}
+
+// Brings the step's metadata and its block-table entries to the kernels. Small metadata (at most
+// ts::kInlineWords words) travels inside the step's launch parameters, few table entries inside the
+// parameters of the launch that applies them; what is larger goes to the next device slot over the
+// context's copy stream: that copy only has to wait for the step that last read the slot (kRing steps
+// ago), so it runs while the previous step's kernels are still busy, and the caller's stream just
+// waits for its event.
+int send_meta(ts_ctx* c, const ts_step* st, int n_items, int n_combines, int n_slot_deltas, cudaStream_t stream, ts::StepDevice* d) {
+  const size_t used = meta_offsets(st->n_rows, n_items, n_combines, d);
+  const bool inline_meta = used <= (size_t)ts::kInlineWords;
+  const bool inline_deltas = n_slot_deltas <= ts::kInlineDeltas;
+  char* ws = (char*)c->cfg.workspace;
+  c->meta_cur = -1;
+  d->meta = nullptr;
+  if (inline_meta) pack_meta(c, st, *d, n_items, n_combines, d->words);
+  if (!inline_meta || !inline_deltas) {
+    const int slot = c->meta_next;
+    c->meta_next = (c->meta_next + 1) % kRing;
+    c->meta_cur = slot;
+    MetaSlot& ms = c->meta[slot];
+    if (ms.copy_in_flight) {                 // the pinned buffer is free once its last upload is done
+      TS_CUDA(c, cudaEventSynchronize(ms.copied));
+      ms.copy_in_flight = false;
+    }
+    char* dev_slot = ws + c->L.off_meta + (size_t)slot * c->L.slot_bytes;
+    if (ms.read_in_flight) TS_CUDA(c, cudaStreamWaitEvent(c->copy_stream, ms.consumed, 0));
+    if (!inline_meta) {
+      pack_meta(c, st, *d, n_items, n_combines, (int32_t*)ms.host);
+      d->meta = (const int32_t*)dev_slot;
+      TS_CUDA(c, cudaMemcpyAsync(dev_slot, ms.host, used * sizeof(int32_t), cudaMemcpyHostToDevice, c->copy_stream));
+    }
+    if (!inline_deltas) {
+      std::memcpy((char*)ms.host + c->L.meta_bytes, c->deltas.data(), (size_t)n_slot_deltas * sizeof(TableDelta));
+      TS_CUDA(c, cudaMemcpyAsync(dev_slot + c->L.meta_bytes, (char*)ms.host + c->L.meta_bytes,
+                                 (size_t)n_slot_deltas * sizeof(TableDelta), cudaMemcpyHostToDevice, c->copy_stream));
+    }
+    TS_CUDA(c, cudaEventRecord(ms.copied, c->copy_stream));
+    ms.copy_in_flight = true;
+    TS_CUDA(c, cudaStreamWaitEvent(stream, ms.copied, 0));
+    if (!inline_deltas)
+      TS_CUDA(c, ts::launch_table_update((int32_t*)(ws + c->L.off_table), c->cfg.max_pages_per_req, c->cfg.max_requests,
+                                         (int32_t*)(ws + c->L.off_status), (const TableDelta*)(dev_slot + c->L.meta_bytes),
+                                         n_slot_deltas, stream));
   }
-  if (n_combines > 0) {
-    std::memcpy(m + c->L.m_combines, c->combines.data(), sizeof(CombineItem) * n_combines);
-    used = c->L.m_combines + (size_t)n_combines * 4;
+  if (inline_deltas && n_slot_deltas > 0) {
+    ts::InlineDeltas in;
+    in.n = n_slot_deltas;
+    std::memcpy(in.d, c->deltas.data(), (size_t)n_slot_deltas * sizeof(TableDelta));
+    TS_CUDA(c, ts::launch_table_update((int32_t*)(ws + c->L.off_table), c->cfg.max_pages_per_req, c->cfg.max_requests,
+                                       (int32_t*)(ws + c->L.off_status), in, stream));
   }
-  char* dev_slot = (char*)c->cfg.workspace + c->L.off_meta + (size_t)slot * c->L.slot_bytes;
-  if (n_slot_deltas > 0)
-    std::memcpy((char*)ms.host + c->L.meta_bytes, c->deltas.data(), (size_t)n_slot_deltas * sizeof(TableDelta));
-  if (ms.read_in_flight) TS_CUDA(c, cudaStreamWaitEvent(c->copy_stream, ms.consumed, 0));
-  TS_CUDA(c, cudaMemcpyAsync(dev_slot, ms.host, used * sizeof(int32_t), cudaMemcpyHostToDevice, c->copy_stream));
-  if (n_slot_deltas > 0)
-    TS_CUDA(c, cudaMemcpyAsync(dev_slot + c->L.meta_bytes, (char*)ms.host + c->L.meta_bytes,
-                               (size_t)n_slot_deltas * sizeof(TableDelta), cudaMemcpyHostToDevice, c->copy_stream));
-  TS_CUDA(c, cudaEventRecord(ms.copied, c->copy_stream));
-  ms.copy_in_flight = true;
-  TS_CUDA(c, cudaStreamWaitEvent(stream, ms.copied, 0));
-  if (n_slot_deltas > 0) {
-    char* ws = (char*)c->cfg.workspace;
-    TS_CUDA(c, ts::launch_table_update((int32_t*)(ws + c->L.off_table), c->cfg.max_pages_per_req,
-                                       c->cfg.max_requests, (int32_t*)(ws + c->L.off_status),
-                                       (const TableDelta*)(dev_slot + c->L.meta_bytes), n_slot_deltas, stream));
-    ++c->cnt.kernel_launches;
-  }
+  if (n_slot_deltas > 0) ++c->cnt.kernel_launches;
   return TS_OK;
 }
 
 // After the step's kernels: marks the slot as read once the caller's stream gets here.
 int release_meta(ts_ctx* c, cudaStream_t stream) {
+  if (c->meta_cur < 0) return TS_OK;         // the step took no slot
   MetaSlot& ms = c->meta[c->meta_cur];
   TS_CUDA(c, cudaEventRecord(ms.consumed, stream));
   ms.read_in_flight = true;
@@ -500,19 +519,12 @@ int release_meta(ts_ctx* c, cudaStream_t stream) {
 
 void fill_device(ts_ctx* c, const ts_step* st, int64_t n_tokens, ts::StepDevice* d) {
   char* ws = (char*)c->cfg.workspace;
-  const int32_t* meta = (const int32_t*)(ws + c->L.off_meta + (size_t)c->meta_cur * c->L.slot_bytes);
   d->pool = (uint16_t*)c->cfg.kv_pool;
   d->table = (int32_t*)(ws + c->L.off_table);
   d->status = (int32_t*)(ws + c->L.off_status);
   d->pf_queue = d->status + 1;
   d->part_acc = (float*)(ws + c->L.off_part_acc);
   d->part_ml = (float*)(ws + c->L.off_part_ml);
-  d->row_slot = meta + c->L.m_row_slot;
-  d->row_ctx = meta + c->L.m_row_ctx;
-  d->row_qlen = meta + c->L.m_row_qlen;
-  d->row_tok0 = meta + c->L.m_row_tok0;
-  d->items = (const WorkItem*)(meta + c->L.m_items);
-  d->combines = (const CombineItem*)(meta + c->L.m_combines);
   d->q = (const uint16_t*)st->q;
   d->k_new = (const uint16_t*)st->k_new;
   d->v_new = (const uint16_t*)st->v_new;
@@ -529,7 +541,6 @@ void fill_device(ts_ctx* c, const ts_step* st, int64_t n_tokens, ts::StepDevice*
   d->max_pages_per_req = c->cfg.max_pages_per_req;
   d->max_requests = c->cfg.max_requests;
   d->scale_log2 = c->scale * 1.4426950408889634f;
-  d->append_in_decode = 0;
   d->wait_cycles = c->cfg.wait_limit_cycles > 0 ? (long long)c->cfg.wait_limit_cycles : ts::kWaitCycles;
   d->append_wide = 0;          // both set by the mixed launch
   d->debug_arrivals = 0;
@@ -608,11 +619,11 @@ int run_step(ts_ctx* c, const ts_step* st, void* cuda_stream, bool attention) {
   if (rc != TS_OK) return rc;
   const int n_items = attention ? (int)c->items.size() : 0;
   const int n_combines = attention ? (int)c->combines.size() : 0;
-  rc = upload_meta(c, st, n_items, n_combines, n_slot_deltas, stream);
-  if (rc != TS_OK) return rc;
-  commit_table_sync(c);
   ts::StepDevice d;
   fill_device(c, st, n_tokens, &d);
+  rc = send_meta(c, st, n_items, n_combines, n_slot_deltas, stream, &d);
+  if (rc != TS_OK) return rc;
+  commit_table_sync(c);
   d.n_items = n_items;
   d.n_combines = n_combines;
   cudaEvent_t* pe = nullptr;
@@ -629,14 +640,9 @@ int run_step(ts_ctx* c, const ts_step* st, void* cuda_stream, bool attention) {
     c->prof_mixed.push_back(0);
     TS_CUDA(c, cudaEventRecord(pe[0], stream));
   }
-  // head_dim 128 steps with prefill tiles: the mixed kernel appends the new K/V itself
-  const bool append_in_kernel = attention && c->n_prefill_items > 0 && c->cfg.head_dim == 128;
-  // decode rows of decode-only steps and of head_dim 128 steps: the unit that reads a row's last
-  // page writes the row's new token into it
-  const bool append_in_decode =
-      attention && n_items > c->n_prefill_items && (c->n_prefill_items == 0 || append_in_kernel);
-  d.append_in_decode = append_in_decode;
-  if (!append_in_kernel && !append_in_decode) {
+  // A step's kernels append the new K/V themselves: the tiles' kernel the prefill rows' tokens, the
+  // decode unit that reads a row's last page that row's token. ts_kv_append is a launch of its own.
+  if (!attention) {
     TS_CUDA(c, ts::launch_kv_append(d, stream));
     ++c->cnt.kernel_launches;
   }

@@ -45,7 +45,8 @@ struct TableDelta {
   int32_t slot, index, page;
 };
 
-// Device pointers of one step, all inside the caller's workspace unless noted.
+constexpr int kInlineWords = 768;   // 3 KB: with the tensor maps the mixed kernel's parameters stay within 4 KB
+// One step as its kernels see it; device pointers lie in the caller's workspace unless noted.
 struct StepDevice {
   // static
   uint16_t* pool;          // caller's KV pool
@@ -57,13 +58,6 @@ struct StepDevice {
                            // units taken besides the CTAs' first ones; decode kernel [5] CTAs that are done
   float* part_acc;         // [max_partials][Hq][D]
   float* part_ml;          // [max_partials][Hq][2]  (running max in log2 units, sum)
-  // per step (device meta area)
-  const int32_t* row_slot;
-  const int32_t* row_ctx;
-  const int32_t* row_qlen;
-  const int32_t* row_tok0; // [n_rows + 1] prefix sums of q_len
-  const WorkItem* items;
-  const CombineItem* combines;
   // step tensors
   const uint16_t* q;
   const uint16_t* k_new;
@@ -72,18 +66,40 @@ struct StepDevice {
   // shape
   int32_t n_rows, n_tokens, n_items, n_combines;
   int32_t n_prefill_items;  // items[0, n_prefill_items) are prefill tiles, the rest decode splits
-  int32_t append_in_decode; // != 0: the decode units append their rows' new K/V themselves
   int32_t Hq, Hkv, D, n_pages, max_pages_per_req, max_requests;
   float scale_log2;        // softmax scale * log2(e)
   long long wait_cycles;   // limit of every bounded wait of the step's kernels, in clock cycles
   int32_t append_wide;     // mixed kernel: CTAs that start on prefill units append with their softmax warps first
   int32_t debug_arrivals;  // > 0: the mixed kernel waits for that many arrivals, which nothing sends (TS_DEBUG_LOSE_APPEND_ARRIVAL)
+  // The step's row arrays and work list: word offsets from `meta`, a device address, or, where they
+  // are small, from `words`: they then travel as launch parameters, without an upload of their own (a copy
+  // on another stream, two event records and two waits: ~6 us of host time and a dependency per step).
+  const int32_t* meta;     // null: `words`
+  uint32_t o_slot, o_ctx, o_tok0, o_items, o_combines;
+  int32_t words[kInlineWords];
+#ifdef __CUDACC__
+  __device__ __forceinline__ const int32_t* at(uint32_t o) const { return (meta ? meta : words) + o; }
+  __device__ __forceinline__ int32_t row_slot(int r) const { return at(o_slot)[r]; }
+  __device__ __forceinline__ int32_t row_ctx(int r) const { return at(o_ctx)[r]; }
+  __device__ __forceinline__ int32_t row_tok0(int r) const { return at(o_tok0)[r]; }   // [n_rows + 1] prefix sums of the new tokens
+  __device__ __forceinline__ WorkItem item(int i) const { return reinterpret_cast<const WorkItem*>(at(o_items))[i]; }
+  __device__ __forceinline__ CombineItem combine(int i) const { return reinterpret_cast<const CombineItem*>(at(o_combines))[i]; }
+#endif
 };
 
 // Launchers. Each enqueues on `stream` and returns the launch's cudaError_t.
 cudaError_t launch_table_update(int32_t* table, int max_pages_per_req, int max_requests, int32_t* status,
                                 const TableDelta* deltas, int n_deltas, cudaStream_t stream);
+// The same for up to kInlineDeltas entries, which travel as launch parameters.
+constexpr int kInlineDeltas = 64;
+struct InlineDeltas {
+  int32_t n;
+  TableDelta d[kInlineDeltas];
+};
+cudaError_t launch_table_update(int32_t* table, int max_pages_per_req, int max_requests, int32_t* status,
+                                const InlineDeltas& deltas, cudaStream_t stream);
 cudaError_t launch_kv_append(const StepDevice& s, cudaStream_t stream);
+// Work items [0, n_items); prefill items read their chunk's own K/V from the step's tensors and append them.
 cudaError_t launch_attention(const StepDevice& s, cudaStream_t stream);
 cudaError_t launch_combine(const StepDevice& s, cudaStream_t stream);
 // Decode splits items[n_prefill_items, n_items): persistent kernel, one CTA per SM, K/V pages by TMA
@@ -185,10 +201,10 @@ inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, 
 __device__ __forceinline__ void stage_rows(const StepDevice& s, int32_t* rows, int tid, int n_threads) {
   const int n = s.n_rows + 1;                  // rows[0..n): first-token prefix sums, then ctx, then slot
   for (int i = tid; i < n; i += n_threads) {
-    rows[i] = s.row_tok0[i];
+    rows[i] = s.row_tok0(i);
     if (i < s.n_rows) {
-      rows[n + i] = s.row_ctx[i];
-      rows[2 * n + i] = s.row_slot[i];
+      rows[n + i] = s.row_ctx(i);
+      rows[2 * n + i] = s.row_slot(i);
     }
   }
 }
@@ -245,7 +261,6 @@ __device__ __forceinline__ void append_tokens(const StepDevice& s, const int32_t
       const int mid = (lo + hi) >> 1;
       if (row_start[mid] <= tok) lo = mid; else hi = mid;
     }
-    if (s.append_in_decode && row_start[lo + 1] - row_start[lo] == 1) continue;
     append_one(s, tok, rows[n + lo] + (tok - row_start[lo]), rows[2 * n + lo], lane);
   }
 }

@@ -10,6 +10,8 @@
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
+#include <cstddef>
+
 #include "../../include/tokenscale.h"
 #include "ts_internal.h"
 #include "ts_ptx.h"
@@ -36,9 +38,22 @@ __global__ void table_update_kernel(int32_t* table, int width, int max_requests,
   table[(size_t)d.slot * width + d.index] = d.page;
 }
 
-// KV append as a launch of its own (ts_kv_append, and steps whose attention kernel does not
-// append itself): one warp per new token at a time, see append_tokens.
-__global__ void kv_append_kernel(StepDevice s) {
+__global__ void table_update_inline_kernel(int32_t* table, int width, int max_requests, int32_t* status,
+                                           const __grid_constant__ InlineDeltas deltas) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int i = threadIdx.x;
+  if (i >= deltas.n) return;
+  const TableDelta d = deltas.d[i];
+  if ((unsigned)d.slot >= (unsigned)max_requests || (unsigned)d.index >= (unsigned)width) {
+    atomicOr(status, TS_DEV_BAD_INDEX);        // never expected: the host builds these records
+    return;
+  }
+  table[(size_t)d.slot * width + d.index] = d.page;
+}
+
+// KV append as a launch of its own (ts_kv_append): one warp per new token at a time, see append_tokens.
+__global__ void kv_append_kernel(const __grid_constant__ StepDevice s) {
   extern __shared__ int32_t rows[];             // staged row arrays, see stage_rows
   pdl_launch_dependents();
   pdl_wait();
@@ -49,10 +64,10 @@ __global__ void kv_append_kernel(StepDevice s) {
 }
 
 // Merge of the splits of one token: grid (n_combines, Hq), block D threads.
-__global__ void combine_kernel(StepDevice s) {
+__global__ void combine_kernel(const __grid_constant__ StepDevice s) {
   pdl_launch_dependents();
   pdl_wait();
-  const CombineItem c = s.combines[blockIdx.x];
+  const CombineItem c = s.combine(blockIdx.x);
   const int h = blockIdx.y, d = threadIdx.x;
   const float o = merge_splits(s, c.first_partial, c.n_splits, h, d);
   s.out[((size_t)c.token * s.Hq + h) * s.D + d] = __bfloat16_as_ushort(__float2bfloat16_rn(o));
@@ -69,7 +84,7 @@ __device__ __forceinline__ uint32_t tile_off(int row, int chunk) {
 template <int D>
 __device__ __forceinline__ void load_tile(uint32_t sK, uint32_t sV, const StepDevice& s,
                                           const int32_t* __restrict__ table_row, int kv_head, int kt,
-                                          int k_end, int tid) {
+                                          int k_end, int new_from, int tok_new, int tid) {
   constexpr int CH = D / 8;
   const size_t v_off = (size_t)s.Hkv * kPageSize * D;  // K tile -> V tile of the same page
 #pragma unroll
@@ -77,8 +92,14 @@ __device__ __forceinline__ void load_tile(uint32_t sK, uint32_t sV, const StepDe
     const int row = c / CH, ch = c % CH;
     const int j = kt + row;
     const uint16_t* src = s.pool;
+    const uint16_t* src_v = nullptr;
     int bytes = 0;
-    if (j < k_end) {
+    if (j >= new_from && j < k_end) {        // a token of this chunk: from the step's tensors
+      const size_t off = ((size_t)(tok_new + j - new_from) * s.Hkv + kv_head) * D + ch * 8;
+      src = s.k_new + off;
+      src_v = s.v_new + off;
+      bytes = 16;
+    } else if (j < k_end) {
       const int page = table_row[j >> 4];
       if ((unsigned)page < (unsigned)s.n_pages) {
         src = s.pool + ((((size_t)page * 2) * s.Hkv + kv_head) * kPageSize + (j & 15)) * D + ch * 8;
@@ -89,7 +110,7 @@ __device__ __forceinline__ void load_tile(uint32_t sK, uint32_t sV, const StepDe
     }
     const uint32_t off = tile_off<D>(row, ch);
     cp_async16(sK + off, src, bytes);
-    cp_async16(sV + off, bytes ? src + v_off : src, bytes);
+    cp_async16(sV + off, src_v ? src_v : bytes ? src + v_off : src, bytes);
   }
 }
 
@@ -178,20 +199,21 @@ __device__ __forceinline__ void warp_tile(uint32_t sK, uint32_t sV, int key_row0
 }
 
 template <int D>
-__global__ void __launch_bounds__(kThreads, 2) attention_kernel(StepDevice s) {
+__global__ void __launch_bounds__(kThreads, 2) attention_kernel(const __grid_constant__ StepDevice s) {
   extern __shared__ __align__(128) unsigned char smem[];
   pdl_launch_dependents();
   pdl_wait();
   constexpr int kTileBytes = kKeysPerTile * D * 2;
   const uint32_t smem_base = smem_u32(smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const WorkItem it = s.items[blockIdx.x];
+  const WorkItem it = s.item(blockIdx.x);
   const int kv_head = blockIdx.y;
   const int G = s.Hq / s.Hkv;
-  const int ctx = s.row_ctx[it.row];
-  const int tok0 = s.row_tok0[it.row];
-  const int32_t* table_row = s.table + (size_t)s.row_slot[it.row] * s.max_pages_per_req;
+  const int ctx = s.row_ctx(it.row);
+  const int tok0 = s.row_tok0(it.row);
+  const int32_t* table_row = s.table + (size_t)s.row_slot(it.row) * s.max_pages_per_req;
   const bool decode = it.kind == 0;
+  const int new_from = decode ? 0x7fffffff : ctx;       // keys from here on are the chunk's own tokens
 
   // The 16 packed rows of this warp: decode -> all warps share rows 0..15; prefill -> 16 each.
   const int row_base = decode ? 0 : warp * 16;
@@ -233,8 +255,22 @@ __global__ void __launch_bounds__(kThreads, 2) attention_kernel(StepDevice s) {
   for (int st = 0; st < kStages - 1; ++st) {
     if (st < n_tiles)
       load_tile<D>(smem_base + st * 2 * kTileBytes, smem_base + st * 2 * kTileBytes + kTileBytes, s,
-                   table_row, kv_head, it.k_begin + st * kKeysPerTile, it.k_end, tid);
+                   table_row, kv_head, it.k_begin + st * kKeysPerTile, it.k_end, new_from, tok0, tid);
     cp_async_commit();
+  }
+  // KV append (Sec. 2.1): this item's tokens of this head, next to the tiles (which do not read them back)
+  if (!decode) {
+    constexpr int CH = D / 8;
+    for (int i = tid; i < it.q_count * 2 * CH; i += kThreads) {
+      const int c = i % CH, kv = (i / CH) & 1, tk = it.q_begin + i / (2 * CH);
+      const int page = table_row[(ctx + tk) >> 4];
+      if ((unsigned)page >= (unsigned)s.n_pages) {
+        atomicOr(s.status, TS_DEV_BAD_PAGE);
+        continue;
+      }
+      *reinterpret_cast<uint4*>(s.pool + ((((size_t)page * 2 + kv) * s.Hkv + kv_head) * kPageSize + ((ctx + tk) & 15)) * D + c * 8) =
+          *reinterpret_cast<const uint4*>((kv ? s.v_new : s.k_new) + ((size_t)(tok0 + tk) * s.Hkv + kv_head) * D + c * 8);
+    }
   }
   for (int t = 0; t < n_tiles; ++t) {
     cp_async_wait<kStages - 2>();
@@ -243,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, 2) attention_kernel(StepDevice s) {
     if (nxt < n_tiles) {
       const int st = nxt % kStages;
       load_tile<D>(smem_base + st * 2 * kTileBytes, smem_base + st * 2 * kTileBytes + kTileBytes, s,
-                   table_row, kv_head, it.k_begin + nxt * kKeysPerTile, it.k_end, tid);
+                   table_row, kv_head, it.k_begin + nxt * kKeysPerTile, it.k_end, new_from, tok0, tid);
     }
     cp_async_commit();
     const int st = t % kStages;
@@ -347,6 +383,13 @@ cudaError_t launch_table_update(int32_t* table, int max_pages_per_req, int max_r
   if (n_deltas <= 0) return cudaSuccess;
   return launch_pdl(table_update_kernel, dim3((n_deltas + 255) / 256), dim3(256), 0, stream, table, max_pages_per_req,
                     max_requests, status, deltas, n_deltas);
+}
+
+cudaError_t launch_table_update(int32_t* table, int max_pages_per_req, int max_requests, int32_t* status,
+                                const InlineDeltas& deltas, cudaStream_t stream) {
+  if (deltas.n <= 0) return cudaSuccess;
+  return launch_pdl(table_update_inline_kernel, dim3(1), dim3(kInlineDeltas), 0, stream, table, max_pages_per_req,
+                    max_requests, status, deltas);
 }
 
 cudaError_t launch_kv_append(const StepDevice& s, cudaStream_t stream) {
@@ -489,15 +532,14 @@ extern "C" int ts_decode_attention_static(int32_t device, int32_t n_q_heads, int
   d.table = (int32_t*)block_tables;       // only read
   d.status = &sc->status;
   d.pf_queue = nullptr;
-  d.append_in_decode = 0;
   d.part_acc = sc->part_acc;
   d.part_ml = sc->part_ml;
-  d.row_slot = sc->row_slot;
-  d.row_ctx = sc->row_ctx;
-  d.row_qlen = nullptr;                   // not read by attention / combine
-  d.row_tok0 = sc->row_tok0;
-  d.items = sc->items;
-  d.combines = sc->combines;
+  d.meta = (const int32_t*)sc;
+  d.o_slot = offsetof(StaticScratch, row_slot) / 4;
+  d.o_ctx = offsetof(StaticScratch, row_ctx) / 4;
+  d.o_tok0 = offsetof(StaticScratch, row_tok0) / 4;
+  d.o_items = offsetof(StaticScratch, items) / 4;
+  d.o_combines = offsetof(StaticScratch, combines) / 4;
   d.q = (const uint16_t*)q;
   d.k_new = nullptr;
   d.v_new = nullptr;

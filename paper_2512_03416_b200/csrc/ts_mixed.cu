@@ -228,10 +228,10 @@ struct AppendCursor {
     const int w = next + lane * stride;
     tok = -1;
     if (w < end) {
-      const WorkItem it = s.items[w / per_item];
+      const WorkItem it = s.item(w / per_item);
       const int j = w % per_item;
       if (j < it.q_count) {
-        const int slot = s.row_slot[it.row], t = it.k_end - it.q_count + j;
+        const int slot = s.row_slot(it.row), t = it.k_end - it.q_count + j;
         if ((unsigned)slot >= (unsigned)s.max_requests || (unsigned)(t >> 4) >= (unsigned)s.max_pages_per_req) {
           atomicOr(s.status, TS_DEV_BAD_INDEX);
         } else {
@@ -239,7 +239,7 @@ struct AppendCursor {
           if ((unsigned)page >= (unsigned)s.n_pages) {
             atomicOr(s.status, TS_DEV_BAD_PAGE);
           } else {
-            tok = s.row_tok0[it.row] + it.q_begin + j;
+            tok = s.row_tok0(it.row) + it.q_begin + j;
             dst = (uint32_t)page * kPageSize + (uint32_t)(t & 15);
           }
         }
@@ -285,7 +285,7 @@ struct AppendCursor {
 __device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 0;\n" ::: "memory"); }
 
 __global__ void __launch_bounds__(kPfThreads, 1)
-mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
+mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUtensorMap q_map,
              const __grid_constant__ CUtensorMap kv_map, const __grid_constant__ CUtensorMap kv_tile_map,
              const __grid_constant__ NewKvMaps new_maps, const int n_prefill_ctas) {
   extern __shared__ unsigned char smem_raw[];
@@ -593,7 +593,7 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
       // a lane merges four head_dim elements
       const int n_pairs = s.n_combines * s.Hq;
       for (int pi = (int)blockIdx.x * 8 + warp; pi < n_pairs; pi += (int)gridDim.x * 8) {
-        const CombineItem c = s.combines[pi / s.Hq];
+        const CombineItem c = s.combine(pi / s.Hq);
         const int h = pi % s.Hq;
         const float* ml = s.part_ml + ((size_t)c.first_partial * s.Hq + h) * 2;
         const float* pa = s.part_acc + ((size_t)c.first_partial * s.Hq + h) * kD + lane * 4;
@@ -671,14 +671,14 @@ mixed_kernel(const StepDevice s, const __grid_constant__ CUtensorMap q_map,
         UnitRec r = {};
         r.w = -1;
         if (w < n_units) {
-          const WorkItem it = s.items[w / s.Hkv];
+          const WorkItem it = s.item(w / s.Hkv);
           r.w = w;
-          r.table_slot = s.row_slot[it.row];
+          r.table_slot = s.row_slot(it.row);
           r.kv_head = w % s.Hkv;
           r.q_begin = it.q_begin;
           r.q_count = it.q_count;
           r.ctx = it.k_end - it.q_begin - it.q_count;
-          r.tok0 = s.row_tok0[it.row];
+          r.tok0 = s.row_tok0(it.row);
           if ((unsigned)r.table_slot >= (unsigned)s.max_requests) {
             atomicOr(s.status, TS_DEV_BAD_INDEX);
             r.w = -1;

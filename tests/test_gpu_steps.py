@@ -275,3 +275,38 @@ def test_chunked_replay_with_several_prefill_tasks_sampled_parity():
 
     run = _replay_sampled_parity(wl.TraceReplay(chunk_size=2304, max_prefill_tasks=4), extra, 6)
     assert max(ps.n_tokens for ps in run.steps) <= 2304
+
+
+@pytest.mark.parametrize("rows", [1, 60, 90, 240])
+@pytest.mark.parametrize("shape", [wl.Shape(4, 2, 64), wl.Shape(8, 2, 128)], ids=["d64", "d128"])
+def test_metadata_inside_and_outside_the_launch_parameters(rows, shape):
+    """Steps whose row arrays and work list fit the launch parameters (up to 768 words) and steps for
+    which they are uploaded, and, over page boundaries, table entries of both kinds (up to 64, and
+    more), in turn on one context: a chunk next to `rows` decode rows, then further tokens for all."""
+    ctx = [13 + (r % 3) for r in range(rows)] + [0]
+    b = wl.make_batch("meta", shape, ctx, [1] * rows + [40], seed=rows, profile="peaked", chunk_size=rows + 40, n_pages=4 * rows + 16)
+    want, pool_want = oracle_step(b)
+    lb = LoadedBatch(b, extra_pages=2)
+    lb.step()
+    assert lb.dec.device_status() == 0
+    assert_parity(lb.output(), want, "peaked", f"{rows} rows")
+    assert np.array_equal(lb.pool(), pool_want)
+    s = shape
+    bank = wl.ValueBank(rows, 1.0, 20)
+    lens = [c + 1 for c in ctx[:-1]] + [40]
+    pool = pool_want
+    n = rows + 1
+    for _ in range(4):                                       # every row crosses into a new page
+        for slot, c in zip(lb.slots, lens):
+            lb.dec.alloc_pages(slot, c + 1)
+        q = bank.take(n * s.Hq * s.D).reshape(n, s.Hq, s.D)
+        k = bank.take(n * s.Hkv * s.D).reshape(n, s.Hkv, s.D)
+        v = bank.take(n * s.Hkv * s.D).reshape(n, s.Hkv, s.D)
+        out = torch.full((n, s.Hq, s.D), 0x7FC0, dtype=torch.int16, device="cuda")
+        lb.dec.mixed_step(lb.slots, [1] * n, lens, to_dev(q), to_dev(k), to_dev(v), out)
+        want = oracle.mixed_step(pool, s.Hq, s.Hkv, s.D, s.P, 1 / math.sqrt(s.D), _oracle_tables(lb.dec, lb.slots, 64),
+                                 lens, [1] * n, q, k, v)
+        assert_parity(wl.bf16_bits_to_f32(from_dev(out)), want, "peaked", f"{rows} rows, lengths {lens[0]}")
+        lens = [c + 1 for c in lens]
+    assert lb.dec.device_status() == 0
+    assert np.array_equal(lb.pool(), pool)
