@@ -80,8 +80,9 @@ typedef struct {
   int32_t chunk_size;         /* Sec. 4.4: largest allowed (prefill tokens + decode batch size)
                                  of one step; 0 disables the check                             */
   int32_t reserved_pages;     /* Eq. 6: pages only ts_alloc_pages(..., for_prefill=1) may take */
-  int32_t decode_split_tokens;/* keys per split of a decode row; 0 = library default; rounded
-                                 up to a multiple of 64                                        */
+  int32_t decode_split_tokens;/* keys per split of a decode row, rounded up to a multiple of
+                                 64; 0 = the library decides per step (512 to 4096, by how many
+                                 keys the step's decode rows have per SM)                      */
   int32_t mixed_prefill_ctas; /* CTAs of the mixed attention kernel that only take prefill tiles
                                  while the other CTAs stream the decode rows first (Sec. 3.4:
                                  the decoder absorbs prefill work next to its decode batch);

@@ -20,7 +20,8 @@ using ts::WorkItem;
 constexpr int kRing = 4;                  // pinned metadata buffers in flight
 constexpr int kDeltaCapacity = 32768;     // table entries per upload batch (bulk loads)
 constexpr int kSlotDeltas = 4096;         // table entries that ride along with a step's metadata
-constexpr int kDefaultSplit = 4096;       // keys per decode split (measured: 2048 and 8192 are both a few percent slower)
+constexpr int kMinDefaultSplit = 512, kMaxDefaultSplit = 4096;   // keys per decode split, see plan()
+constexpr int kSmsB200 = 148;             // for plans made before the device is known
 constexpr int kDefaultMaxTokens = 16384;  // step size bound when chunk_size == 0
 constexpr size_t kAlign = 256;
 
@@ -343,7 +344,20 @@ int validate(ts_ctx* c, const ts_step* st, bool attention, bool need_tensors, in
 // Builds c->items / c->combines for a validated step.
 void plan(ts_ctx* c, const ts_step* st) {
   const int G = c->G;
-  int split = c->cfg.decode_split_tokens > 0 ? c->cfg.decode_split_tokens : kDefaultSplit;
+  int split = c->cfg.decode_split_tokens;
+  if (split <= 0) {
+    // An SM's share of the step's (key, KV head) pairs, so that a small batch's long rows spread over
+    // the chip; not below 512 (a unit costs ~2 us besides its keys), not above kMaxDefaultSplit. Measured
+    // with the pages of 8 KV heads, G = 4, us at splits of 512 / 1024 / 2048 / 4096: 4 rows of ~1300 keys
+    // (share 286) 13.4 / 16.6 / 22.2 / 20.8; 16 rows of ~1700 (1468) 31.0 / 27.2 / 28.0 / 33.0; 32 rows
+    // (2234) 41.3 / 39.1 / 38.3 / 39.0; 64 rows (7864) 109 / 101.5 / 99.0 / 100.9; with G = 8, 203 rows
+    // (16579) 248 / 209 / 201 / 196.
+    int64_t keys = 0;
+    for (int r = 0; r < st->n_rows; ++r)
+      if (st->q_len[r] == 1) keys += st->ctx_len[r] + 1;
+    const int64_t share = keys * c->cfg.n_kv_heads / (c->n_sms > 0 ? c->n_sms : kSmsB200);
+    split = (int)std::min<int64_t>(std::max<int64_t>(share, kMinDefaultSplit), kMaxDefaultSplit);
+  }
   split = ceil_div(split, ts::kKeysPerTile) * ts::kKeysPerTile;
   for (;;) {
     c->items.clear();

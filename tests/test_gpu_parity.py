@@ -247,3 +247,16 @@ def test_decode_units_of_all_lengths(shape, split):
     for _ in range(2):                                     # the unit queue is back at zero after a step
         assert_parity(run.step(keep_len=True), want, "peaked", f"split {split}")
     assert np.array_equal(run.pool(), pool_want)
+
+
+@pytest.mark.parametrize("rows", [[0], [511, 512], [513, 40, 1500], [8191], [1500] * 20, [700, 3000, 150] * 9], ids=lambda r: f"{len(r)}x{r[0]}")
+def test_default_splits_of_small_batches(rows):
+    """The default split follows the batch: rows around the shortest split, one long row, batches whose
+    share per SM lies between the limits; next to a chunk as well."""
+    for extra in ([], [(0, 33)]):
+        b = wl.make_batch("few", wl.LLAMA8B, rows + [c for c, _ in extra], [1] * len(rows) + [t for _, t in extra], seed=len(rows),
+                          profile="peaked")
+        want, pool_want = oracle_step(b)
+        run = GpuRun(b, chunk_size=0)
+        assert_parity(run.step(), want, "peaked", f"{rows} {extra}")
+        assert np.array_equal(run.pool(), pool_want)
