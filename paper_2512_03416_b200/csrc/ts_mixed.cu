@@ -85,8 +85,7 @@ enum {
   BAR_O_FULL = BAR_P_FULL + 2,            // [2] per tile
   BAR_O_EMPTY = BAR_O_FULL + 2,           // [2] per tile: the epilogue has read O out of TMEM
   BAR_Q_EMPTY = BAR_O_EMPTY + 2,          // the last Q K^T of a work unit has consumed the Q tiles
-  BAR_PAIR = BAR_Q_EMPTY + 1,             // [8] per tile and row quarter: the two warps that share the rows
-  BAR_V_LANDED = BAR_PAIR + 8,            // [kVStages] the copies of a V tile are in shared memory
+  BAR_V_LANDED = BAR_Q_EMPTY + 1,         // [kVStages] the copies of a V tile are in shared memory
   BAR_K_LANDED = BAR_V_LANDED + kVStages, // the same for a K tile that needs a touch-up before it is announced
   BAR_COUNT = BAR_K_LANDED + 1
 };
@@ -316,6 +315,17 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
   };
   // k-th work unit of this CTA (w = -1 after the last one), published by the K loaders' first thread
   volatile int4* ring = reinterpret_cast<volatile int4*>(smem + kOffRing);
+  auto read_unit = [&](int k, PfUnit& u) -> bool {           // of a published unit
+    UnitRec r;
+    const int e = (k & (kSchedRing - 1)) * 2;
+    const int4 lo = make_int4(ring[e].x, ring[e].y, ring[e].z, ring[e].w);
+    const int4 hi = make_int4(ring[e + 1].x, ring[e + 1].y, ring[e + 1].z, ring[e + 1].w);
+    r.w = lo.x; r.table_slot = lo.y; r.kv_head = lo.z; r.q_begin = lo.w;
+    r.q_count = hi.x; r.ctx = hi.y; r.tok0 = hi.z;
+    if (r.w < 0) return false;
+    u = unit_shape(r, tile_tokens);
+    return true;
+  };
   auto get_work = [&](int k, PfUnit& u) -> bool {
     if ((int)misc[2] <= k) {
       const long long t0 = clock64();
@@ -326,15 +336,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
         }
       }
     }
-    UnitRec r;
-    const int e = (k & (kSchedRing - 1)) * 2;
-    const int4 lo = make_int4(ring[e].x, ring[e].y, ring[e].z, ring[e].w);
-    const int4 hi = make_int4(ring[e + 1].x, ring[e + 1].y, ring[e + 1].z, ring[e + 1].w);
-    r.w = lo.x; r.table_slot = lo.y; r.kv_head = lo.z; r.q_begin = lo.w;
-    r.q_count = hi.x; r.ctx = hi.y; r.tok0 = hi.z;
-    if (r.w < 0) return false;
-    u = unit_shape(r, tile_tokens);
-    return true;
+    return read_unit(k, u);
   };
   // The set-up every warp class runs between the decode phase and the prefill phase.
   auto prefill_setup = [&]() {
@@ -353,8 +355,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
       }
       for (int i = 0; i < BAR_COUNT; ++i) {
         const bool softmax_arrives = (i >= BAR_P_FULL && i < BAR_P_FULL + 2) || (i >= BAR_O_EMPTY && i < BAR_O_EMPTY + 2);
-        const bool pair = i >= BAR_PAIR && i < BAR_PAIR + 8;
-        mbar_init(bar(i), softmax_arrives ? 256 : pair ? 64 : 1);
+        mbar_init(bar(i), softmax_arrives ? 256 : 1);
       }
       mbar_init_fence();
     }
@@ -438,31 +439,33 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t tS = tmem + x * 128 + hf * 64 + lane_addr;         // my 64 score columns; P goes to the first 32
     const uint32_t tO = tmem + 256 + x * 128 + hf * 64 + lane_addr;   // my 64 columns of O
-    // The two warps that share a quarter of a tile's rows meet on an mbarrier (a bounded wait, like
-    // every other one here) around each exchange through shared memory.
-    const int pair_bar = BAR_PAIR + x * 4 + (warp & 3);
-    int n_pair = 0;
-    auto pair_arrive = [&]() { mbar_arrive(bar(pair_bar)); };
-    auto pair_wait = [&]() {
-      wait(pair_bar, n_pair & 1);
-      ++n_pair;
-    };
-    auto pair_sync = [&]() {
-      pair_arrive();
-      pair_wait();
-    };
+    // The two warps that share a quarter of a tile's rows meet on a hardware barrier (ids 4-11) around
+    // each exchange through shared memory; it wakes them sooner than an mbarrier (8192-token chunk
+    // next to 190 rows 1274 -> 1238 us, 2048 tokens alone 50.7 -> 48.4 us). It has no time limit, so
+    // the two must never disagree about how often they meet: all their other waits are limited and end
+    // in the same control flow, and whether there is another work unit is for the first of them to say.
+    auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;\n" ::"r"(4 + x * 4 + (warp & 3)) : "memory"); };
     float* xchg = reinterpret_cast<float*>(smem + kOffXchg) + x * 256;   // [half][row] of my tile
     float* xchg_mine = xchg + hf * 128 + row;
-    const float* xchg_other = xchg + (hf ^ 1) * 128 + row;
+    float* xchg_other = xchg + (hf ^ 1) * 128 + row;
+    int row_g = row / G, row_h = row % G;   // token of the tile and query head of this row
     const float scale = s.scale_log2;
     int sx = 0;                 // blocks of this tile in earlier work units: barrier phases follow it
     for (int k = 0;; ++k) {
       PfUnit u;
-      if (!get_work(k, u)) break;
+      bool more = false;
+      if (hf == 0) {
+        more = get_work(k, u);
+        *xchg_other = more ? 1.f : 0.f;      // the other thread's own slot: it reads it before it writes it again
+      }
+      pair_sync();
+      if (hf == 1) more = *xchg_mine != 0.f;
+      if (!more) break;
+      if (hf == 1) read_unit(k, u);
       const int nbx = x ? u.nb_b : u.nb_a;
       const int cnt = x ? u.cnt_b : u.cnt_a;
-      const int tok = u.q_begin + x * tile_tokens + row / G;   // token inside the request row
-      const bool real = row / G < cnt && row < tile_tokens * G;
+      const int tok = u.q_begin + x * tile_tokens + row_g;     // token inside the request row
+      const bool real = row_g < cnt && row < tile_tokens * G;
       const int lim = real ? u.ctx + tok + 1 : (x ? u.k_end_b : u.k_end_a);   // keys at positions >= lim are masked
       const int tok0 = u.tok0;
       float m_ref = -CUDART_INF_F, l = 0.f;
@@ -547,7 +550,10 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
         pair_sync();
         const float inv = 1.f / (l + *xchg_other);
         pair_sync();                      // both have read: the slots may be written again
-        uint16_t* orow = s.out + ((size_t)(tok0 + tok) * s.Hq + u.kv_head * G + row % G) * kD + hf * 64;
+        // A row's 64 columns are one thread's; stored as they are, every 16-byte store of a warp would touch
+        // 32 rows. The four lanes of a quad swap 16-byte chunks first, so that they write 64 bytes of a
+        // row together.
+        const uint32_t orow = real ? (uint32_t)(tok0 + tok) * s.Hq + u.kv_head * G + row_h : 0xffffffffu;
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
           float ov[32];
@@ -557,19 +563,34 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
             tc_fence_before();
             mbar_arrive(bar(BAR_O_EMPTY + x));   // O is in registers: the next unit may overwrite it
           }
-          if (real) {
+          uint32_t w[4][4];                      // [chunk of 8 columns][bf16 pair]
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) w[i][e] = pack_bf16(ov[8 * i + 2 * e] * inv, ov[8 * i + 2 * e + 1] * inv);
+#pragma unroll
+          for (int bit = 1; bit < 4; bit <<= 1) {          // 4 x 4 transpose over the quad: w[i] becomes chunk lane % 4 of row i
+            const bool up = lane & bit;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-              uint4 wv;
-              wv.x = pack_bf16(ov[8 * i] * inv, ov[8 * i + 1] * inv);
-              wv.y = pack_bf16(ov[8 * i + 2] * inv, ov[8 * i + 3] * inv);
-              wv.z = pack_bf16(ov[8 * i + 4] * inv, ov[8 * i + 5] * inv);
-              wv.w = pack_bf16(ov[8 * i + 6] * inv, ov[8 * i + 7] * inv);
-              *reinterpret_cast<uint4*>(orow + c * 32 + i * 8) = wv;
+              if (i & bit) continue;
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? w[i][e] : w[i | bit][e], bit);
+                if (up) w[i][e] = got; else w[i | bit][e] = got;
+              }
             }
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint32_t r = __shfl_sync(0xffffffffu, orow, (lane & ~3) + i);
+            if (r != 0xffffffffu)
+              *reinterpret_cast<uint4*>(s.out + (size_t)r * kD + hf * 64 + c * 32 + (lane & 3) * 8) =
+                  make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
           }
         }
       }
+      if (nbx == 0) pair_sync();             // hf 1 has read the slot
       sx += nbx;
     }
     // -------------------------------------------------------------- merge of the decode splits
@@ -667,7 +688,8 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
       // hides the round trip), and publishes each to the other roles through a small ring.
       int fetched = 0;
       auto fetch_one = [&]() {
-        const int w = atomicAdd(s.pf_queue, 1);
+        // a CTA that starts on prefill work has its first unit without asking; the queue hands out the rest
+        const int w = fetched == 0 && !decode_first ? (int)blockIdx.x : n_prefill_ctas + atomicAdd(s.pf_queue, 1);
         UnitRec r = {};
         r.w = -1;
         if (w < n_units) {
@@ -882,7 +904,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
         };
         for (int k = 0;; ++k) {
           PfUnit u;
-          append_until([&]() { return (int)misc[2] > k; });
+          if (k > 0) append_until([&]() { return (int)misc[2] > k; });   // the first Q tiles wait for nothing
           if (!get_work(k, u)) break;
           const int ta = u.tok0 + u.q_begin;
           if (k > 0) {
