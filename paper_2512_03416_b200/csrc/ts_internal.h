@@ -165,6 +165,19 @@ cudaError_t launch_gemm(const GemmArgs& g, const CUtensorMap& a_map, const CUten
 // out[row] = x[row] / sqrt(mean(x[row]^2) + eps) * gain, bf16 in and out, fp32 inside; width % 8 == 0
 cudaError_t launch_rmsnorm(const uint16_t* x, const uint16_t* gain, uint16_t* out, int rows, int width, float eps,
                            cudaStream_t stream);
+// The same, and pos[t] = position of token t: row r holds tokens tok0[r] .. tok0[r + 1] - 1 at positions
+// from ctx[r] on.
+constexpr int kPosRows = 400;           // 3.2 KB of launch parameters
+template <bool POS>
+struct PosRows {};
+template <>
+struct PosRows<true> {
+  int32_t* pos;
+  int32_t n_rows;
+  int32_t tok0[kPosRows], ctx[kPosRows];
+};
+cudaError_t launch_rmsnorm_pos(const uint16_t* x, const uint16_t* gain, uint16_t* out, int rows, int width, float eps,
+                               const PosRows<true>& pos, cudaStream_t stream);
 // table[p][i] = (cos, sin)(p * theta^(-2 i / 128)), p < max_position, i < 64 (computed in fp64)
 cudaError_t launch_rope_table(float2* table, int max_position, float theta, cudaStream_t stream);
 // dst row 256 b + r = gate row 128 b + r, dst row 256 b + 128 + r = up row 128 b + r (r < 128)

@@ -191,21 +191,36 @@ int ts_layer_step(ts_layer* l, const ts_step* st, const void* x_in, void* x_out,
   const ts_config* c = l->view.cfg;
   TSL_CUDA(l, cudaSetDevice(c->device));
   char* ws = (char*)l->cfg.workspace;
-  // positions of the new tokens: row r's token i sits at ctx_len[r] + i
-  const int slot = l->pos_next;
-  l->pos_next = (l->pos_next + 1) % kPosRing;
-  if (l->pos_busy[slot]) {
-    TSL_CUDA(l, cudaEventSynchronize(l->pos_ev[slot]));
-    l->pos_busy[slot] = false;
+  // positions of the new tokens (row r's token i sits at ctx_len[r] + i): written by the first RMSNorm
+  // launch from row arrays in its parameters, or, for more rows than those hold, uploaded
+  int32_t* pos_dev = (int32_t*)(ws + l->L.off_pos);
+  const bool pos_inline = st->n_rows <= ts::kPosRows;
+  ts::PosRows<true> pr;
+  if (pos_inline) {
+    pr.pos = pos_dev;
+    pr.n_rows = st->n_rows;
+    int32_t at = 0;
+    for (int r = 0; r < st->n_rows; ++r) {
+      pr.tok0[r] = at;
+      pr.ctx[r] = st->ctx_len[r];
+      at += st->q_len[r];
+    }
+  } else {
+    const int slot = l->pos_next;
+    l->pos_next = (l->pos_next + 1) % kPosRing;
+    if (l->pos_busy[slot]) {
+      TSL_CUDA(l, cudaEventSynchronize(l->pos_ev[slot]));
+      l->pos_busy[slot] = false;
+    }
+    int32_t* ph = (int32_t*)l->pos_host[slot];
+    int64_t at = 0;
+    for (int r = 0; r < st->n_rows; ++r)
+      for (int i = 0; i < st->q_len[r]; ++i) ph[at++] = st->ctx_len[r] + i;
+    pos_dev += (size_t)slot * l->max_tokens;
+    TSL_CUDA(l, cudaMemcpyAsync(pos_dev, ph, (size_t)n * sizeof(int32_t), cudaMemcpyHostToDevice, stream));
+    TSL_CUDA(l, cudaEventRecord(l->pos_ev[slot], stream));
+    l->pos_busy[slot] = true;
   }
-  int32_t* ph = (int32_t*)l->pos_host[slot];
-  int64_t at = 0;
-  for (int r = 0; r < st->n_rows; ++r)
-    for (int i = 0; i < st->q_len[r]; ++i) ph[at++] = st->ctx_len[r] + i;
-  int32_t* pos_dev = (int32_t*)(ws + l->L.off_pos) + (size_t)slot * l->max_tokens;
-  TSL_CUDA(l, cudaMemcpyAsync(pos_dev, ph, (size_t)n * sizeof(int32_t), cudaMemcpyHostToDevice, stream));
-  TSL_CUDA(l, cudaEventRecord(l->pos_ev[slot], stream));
-  l->pos_busy[slot] = true;
 
   const int N = (int)n, hidden = l->cfg.hidden, inter = l->cfg.intermediate;
   const int qd = c->n_q_heads * c->head_dim, kvd = c->n_kv_heads * c->head_dim;
@@ -223,7 +238,10 @@ int ts_layer_step(ts_layer* l, const ts_step* st, const void* x_in, void* x_out,
   g.M = N;
 
   // h = rmsnorm(x); (q, k, v) = rope(h . W_qkv^T)
-  TSL_CUDA(l, ts::launch_rmsnorm((const uint16_t*)x_in, (const uint16_t*)l->cfg.w_norm1, h, N, hidden, l->eps, stream));
+  if (pos_inline)
+    TSL_CUDA(l, ts::launch_rmsnorm_pos((const uint16_t*)x_in, (const uint16_t*)l->cfg.w_norm1, h, N, hidden, l->eps, pr, stream));
+  else
+    TSL_CUDA(l, ts::launch_rmsnorm((const uint16_t*)x_in, (const uint16_t*)l->cfg.w_norm1, h, N, hidden, l->eps, stream));
   g.N = qd + 2 * kvd; g.K = hidden; g.epi = ts::GEMM_EPI_ROPE; g.B = (const uint16_t*)l->cfg.w_qkv;
   g.C = q; g.C2 = k; g.C3 = v; g.q_cols = qd; g.kv_cols = kvd; g.pos = pos_dev;
   g.rope_table = (const float2*)(ws + l->L.off_table);

@@ -14,12 +14,26 @@ constexpr int kNormThreads = 256;
 
 // One CTA per row: every thread keeps its 16-byte chunks of the row in registers between the
 // sum of squares and the scaling (up to four chunks: widths up to 8192; wider rows read twice).
+// With POS the CTA also writes its token's position (row r's token i sits at ctx[r] + i), which the
+// rotary epilogue of the projection behind this launch reads; the row arrays are launch parameters.
+template <bool POS>
 __global__ void __launch_bounds__(kNormThreads) rmsnorm_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ gain,
-                                                               uint16_t* __restrict__ out, int width, float eps) {
+                                                               uint16_t* __restrict__ out, int width, float eps,
+                                                               const __grid_constant__ PosRows<POS> pr) {
   __shared__ float partial[kNormThreads / 32];
   pdl_launch_dependents();
   pdl_wait();
   const int tid = threadIdx.x, n_chunks = width / 8;
+  if constexpr (POS) {
+    if (tid == 0) {
+      int lo = 0, hi = pr.n_rows;                // last row that starts at or before this token
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (pr.tok0[mid] <= (int)blockIdx.x) lo = mid; else hi = mid;
+      }
+      pr.pos[blockIdx.x] = pr.ctx[lo] + (int)blockIdx.x - pr.tok0[lo];
+    }
+  }
   const uint16_t* row = x + (size_t)blockIdx.x * width;
   uint4 keep[4];
   float ss = 0.f;
@@ -82,7 +96,13 @@ __global__ void pack_gate_up_kernel(const uint16_t* __restrict__ gate, const uin
 cudaError_t launch_rmsnorm(const uint16_t* x, const uint16_t* gain, uint16_t* out, int rows, int width, float eps,
                            cudaStream_t stream) {
   if (rows <= 0) return cudaSuccess;
-  return launch_pdl(rmsnorm_kernel, dim3(rows), dim3(kNormThreads), 0, stream, x, gain, out, width, eps);
+  return launch_pdl(rmsnorm_kernel<false>, dim3(rows), dim3(kNormThreads), 0, stream, x, gain, out, width, eps, PosRows<false>{});
+}
+
+cudaError_t launch_rmsnorm_pos(const uint16_t* x, const uint16_t* gain, uint16_t* out, int rows, int width, float eps,
+                               const PosRows<true>& pos, cudaStream_t stream) {
+  if (rows <= 0) return cudaSuccess;
+  return launch_pdl(rmsnorm_kernel<true>, dim3(rows), dim3(kNormThreads), 0, stream, x, gain, out, width, eps, pos);
 }
 
 cudaError_t launch_rope_table(float2* table, int max_position, float theta, cudaStream_t stream) {

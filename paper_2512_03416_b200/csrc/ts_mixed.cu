@@ -21,11 +21,10 @@
 // head_dim columns 0-63 / 64-127 of O), warps 4-7 / 12-15 the same for tile B (thread = TMEM lane =
 // query row; a warp can only reach the 32 lanes its index modulo 4 selects, so a row is split by
 // columns). The two threads of a row agree on the row maximum through shared memory and a
-// 64-thread mbarrier per block. Two softmax warps per tile and SM sub-partition hide each
+// barrier of their two warps per block. Two softmax warps per tile and SM sub-partition hide each
 // other's instruction latencies: one warp per row quarter left the tensor pipe idle more than
-// half of the time although no unit was saturated. Warp 16 K loader, warp 17 V loader (16-byte
-// cp.async through the block table into the swizzled operand layout; the K loader's first thread
-// also claims the work units), warp 18 MMA issuer and TMEM owner, warp 19 Q loader (TMA).
+// half of the time although no unit was saturated. Warp 16 K loader, warp 17 V loader (TMA copies of
+// pages and of the chunk's own tokens; the K loader's first thread also claims the work units), warp 18 MMA issuer and TMEM owner, warp 19 Q loader (TMA).
 // All barrier phases follow running block counters, so the roles flow from one work unit into the
 // next without a CTA-wide stop: the loaders run ahead into the next unit's K/V, its Q tiles land
 // as soon as the last Q K^T of the current unit has been issued, and its first Q K^T overlaps

@@ -12,6 +12,7 @@ from paper_2512_03416_b200 import binding as B
 from paper_2512_03416_b200 import workloads as wl
 from paper_2512_03416_b200.harness import LoadedBatch, from_dev, to_dev
 from paper_2512_03416_b200.layer import DecoderLayer
+from tests.helpers import oracle_pool_with_context
 
 pytestmark = pytest.mark.gpu
 
@@ -173,4 +174,45 @@ def test_layer_step_validation_launches_nothing():
     assert B.ts_layer_step(layer.handle, st2, x.data_ptr(), out.data_ptr(), stream) == B.TS_ERR_INVALID
     after = lb.dec.velocity()
     assert after["kernel_launches"] == before["kernel_launches"] and after["steps"] == before["steps"]
+    layer.close()
+
+
+@pytest.mark.parametrize("rows", [1, 399, 400, 401])
+def test_layer_step_positions_for_any_number_of_rows(rows):
+    """The new tokens' positions come from row arrays in the launch parameters, or, past 400 rows, are
+    uploaded: output and rotated keys in the pages against the oracle's, the step issued twice."""
+    s, hidden, inter = wl.Shape(2, 2, 128), 128, 128
+    rng = np.random.default_rng(rows)
+    ctx, ql = [(7 * r) % 40 for r in range(rows)], [1 + (r % 3 == 1) * (r % 5) for r in range(rows)]
+    b = wl.make_batch("pos", s, ctx, ql, seed=rows, profile="peaked", chunk_size=sum(ql))
+    wt = make_weights(rng, s, hidden, inter)
+    for k in ("w_norm1", "w_norm2"):
+        wt[k] = wl.f32_to_bf16_bits((1.0 + wl.bf16_bits_to_f32(wt[k])).astype(np.float32))
+    x = bits(rng, (b.n_tokens, hidden), 1.0)
+    pool, tm = oracle_pool_with_context(b), b.table_matrix()
+
+    def attention(q, k, v):
+        return oracle.mixed_step(pool, s.Hq, s.Hkv, s.D, s.P, 1.0 / math.sqrt(s.D), tm, b.ctx_len, b.q_len, q, k, v)
+
+    want_bits, _ = OL.layer_step(attention, x, wt, OL.positions(b.ctx_len, b.q_len), s.Hq, s.Hkv, s.D, eps=1e-5, theta=500000.0)
+    want = OL.bits_to_f64(want_bits)
+    lb = LoadedBatch(b)
+    dev = {k: to_dev(v) for k, v in wt.items()}
+    layer = DecoderLayer(lb.dec, dev["w_norm1"], dev["w_qkv"], dev["w_o"], dev["w_norm2"], dev["w_gate"], dev["w_up"],
+                         dev["w_down"], max_position=64, rms_eps=1e-5, rope_theta=500000.0)
+    x_in, x_out = to_dev(x), torch.full((b.n_tokens, hidden), 0x7FC0, dtype=torch.int16, device="cuda")
+    for _ in range(2):
+        layer.step(lb.slots, b.q_len.tolist(), b.ctx_len.tolist(), x_in, x_out, keep_len=True)
+    torch.cuda.synchronize()
+    assert lb.dec.device_status() == 0
+    got = OL.bits_to_f64(from_dev(x_out))
+    assert np.abs(got - want).max() <= 2.0 ** -6 * np.abs(want).max()          # as in test_layer_step_matches_the_oracle
+    got_pool = lb.pool()
+    same = got_pool == pool
+    gp, wp = OL.bits_to_f64(got_pool[~same]), OL.bits_to_f64(pool[~same])
+    assert np.isfinite(wp).all() and np.isfinite(gp).all()
+    # One spacing of the stored value, and what one normalised input that rounds the other way moves a sum
+    # of 128 terms by: 2^-8 |h| |w| with |h| <= 4 and |w| <= 4 / sqrt(128), 5.5e-3 (a rotated value may
+    # cancel down to that). A wrong position turns the pair by a radian: differences of order one.
+    assert (np.abs(gp - wp) <= 2.0 ** -7 * np.abs(wp) + 6e-3).all()
     layer.close()
