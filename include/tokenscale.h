@@ -232,7 +232,8 @@ int ts_mixed_step(ts_ctx* ctx, const ts_step* step, void* cuda_stream);
  * the copies asynchronous). Copies the inputs into a staging set of the workspace on the
  * context's own upload stream, runs the step on cuda_stream, copies out back on the context's
  * download stream, makes cuda_stream wait for that copy, and waits for cuda_stream: on return
- * out is valid. N <= chunk_size required (the staging sets are sized by chunk_size; chunk_size
+ * out is valid. A large step goes in up to eight pieces of consecutive tokens, so that the copies
+ * in both directions and the kernels overlap. N <= chunk_size required (the staging sets are sized by chunk_size; chunk_size
  * must be > 0). The paper's decoder receives its inputs from the layers before attention, on the
  * device; this entry point serves callers and measurements that start from host memory.
  * With TS_STEP_HOST_ASYNC the call returns once everything is enqueued and cuda_stream does not

@@ -310,3 +310,27 @@ def test_metadata_inside_and_outside_the_launch_parameters(rows, shape):
         lens = [c + 1 for c in lens]
     assert lb.dec.device_status() == 0
     assert np.array_equal(lb.pool(), pool)
+
+
+@pytest.mark.parametrize("ctx,ql", [([300] * 8 + [0], [1] * 8 + [2048]), ([77, 40, 900], [1100, 1, 947]), ([0, 5, 6], [1536, 1, 1])],
+                         ids=["burst", "two-chunks", "chunk-first"])
+def test_host_step_in_pieces_equals_the_device_step(ctx, ql):
+    """A waiting host-buffer step that is large enough to go in pieces: result, pages, lengths and
+    counters are those of the same step on device buffers, bit for bit (a cut falls between work items)."""
+    b = wl.make_batch("pieces", wl.LLAMA8B, ctx, ql, seed=len(ctx), profile="peaked", chunk_size=sum(ql))
+    one, two = LoadedBatch(b), LoadedBatch(b)
+    one.step()
+    host = [torch.from_numpy(a.view(np.int16)).pin_memory() for a in (b.q, b.k_new, b.v_new)]
+    out = torch.full(host[0].shape, 0x7FC0, dtype=torch.int16).pin_memory()
+    two.dec.mixed_step_host(two.slots, b.q_len.tolist(), b.ctx_len.tolist(), *host, out)
+    assert np.array_equal(wl.bf16_bits_to_f32(out.numpy().view(np.uint16)), one.output())
+    assert np.array_equal(two.pool(), one.pool())
+    assert one.dec.device_status() == 0 and two.dec.device_status() == 0
+    a, c = one.dec.velocity(), two.dec.velocity()
+    assert all(a[k] == c[k] for k in ("steps", "prefill_tokens", "decode_tokens"))
+    assert [two.dec.block_table(s)[1] for s in two.slots] == [x + t for x, t in zip(ctx, ql)]
+    # and again, out in the place of q: not in pieces, the same result
+    buf = host[0].clone().pin_memory()
+    three = LoadedBatch(b)
+    three.dec.mixed_step_host(three.slots, b.q_len.tolist(), b.ctx_len.tolist(), buf, host[1], host[2], buf)
+    assert np.array_equal(wl.bf16_bits_to_f32(buf.numpy().view(np.uint16)), one.output())
