@@ -1,4 +1,6 @@
 """GPU parity: ts_mixed_step / ts_kv_append through the C ABI against the CPU oracle."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -260,3 +262,39 @@ def test_default_splits_of_small_batches(rows):
         run = GpuRun(b, chunk_size=0)
         assert_parity(run.step(), want, "peaked", f"{rows} {extra}")
         assert np.array_equal(run.pool(), pool_want)
+
+
+@pytest.mark.parametrize("shape", [wl.LLAMA8B, wl.Shape(16, 1, 128), wl.Shape(8, 2, 64)], ids=["32-8", "16-1", "8-2"])
+@pytest.mark.parametrize("chunk", [0, 40], ids=["decode", "mixed"])
+def test_a_decode_rows_largest_weight_is_exact(shape, chunk):
+    """A row whose softmax is carried by a late key, a little above a key of an earlier page of the same
+    warp, everything else far below. The largest weight of a page that brings a new maximum is 1 and thus exact
+    in bf16, and earlier sums are rescaled in fp32: what is left is the rounding of the result, 2^-8 of it.
+    A weight taken against a reference that lags behind the maximum would be rounded as well: another
+    2^-8 of nearly the whole result."""
+    ctx = [300, 1100, 131] + [0] * (chunk > 0)
+    b = wl.make_batch("late", shape, ctx, [1] * 3 + [chunk] * (chunk > 0), seed=shape.Hq + chunk, profile="peaked")
+    G, D = shape.Hq // shape.Hkv, shape.D
+    first, late = 5, 130                                   # pages 0 and 8: the same warp of a unit
+    starts = np.concatenate([[0], np.cumsum(ctx)])[:3]
+    coef = np.full(len(b.context_k), -1000.0)
+    for at in starts:
+        coef[at + first], coef[at + late] = 1.0, 2.0
+    b.context_k[:] = 0
+    b.context_k[:, :, 0] = wl.f32_to_bf16_bits(coef.astype(np.float32))[:, None]
+    b.k_new[:3] = 0
+    b.k_new[:3, :, 0] = wl.f32_to_bf16_bits(np.array([-1000.0], np.float32))[0]
+    gap = np.linspace(0.3, 7.6, 3 * shape.Hq).reshape(3, shape.Hq)          # log2(weight of late / of first)
+    b.q[:3] = 0
+    b.q[:3, :, 0] = wl.f32_to_bf16_bits((gap * math.log(2.0) * math.sqrt(D)).astype(np.float32))
+    gap = wl.bf16_bits_to_f32(b.q[:3, :, 0]).astype(np.float64) / (math.log(2.0) * math.sqrt(D))
+    v = wl.bf16_bits_to_f32(b.context_v).astype(np.float64)
+    run = GpuRun(b, chunk_size=0)
+    got = run.step()[:3].astype(np.float64)
+    for r, at in enumerate(starts):
+        w_first = (1.0 / (1.0 + 2.0 ** gap[r]))[:, None]
+        v_first, v_late = (np.repeat(v[at + t], G, axis=0) for t in (first, late))
+        want = w_first * v_first + (1.0 - w_first) * v_late
+        bound = 2.0 ** -8 * np.abs(want) + 1e-5 * (np.abs(v_first) + np.abs(v_late))
+        worst = float((np.abs(got[r] - want) / bound).max())
+        assert worst <= 1.0, f"row {r}: error {worst} times its bound"
