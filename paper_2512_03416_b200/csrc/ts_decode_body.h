@@ -40,6 +40,7 @@ namespace dec {
 constexpr int kDecWarps = 8;
 constexpr int kDecThreads = kDecWarps * 32;          // streaming threads; the scheduler warp comes on top
 constexpr int kDecRing = 3;                          // units of a CTA that are described at a time
+constexpr long long kDrainCycles = 20000000;         // about 10 ms: limit of the wait for copies in flight after a failure
 
 // Barrier of the kDecThreads decode threads (id 1; id 0 stays with the whole block).
 __device__ __forceinline__ void block_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(kDecThreads) : "memory"); }
@@ -75,7 +76,7 @@ struct UnitInfo {
 };
 static_assert(sizeof(UnitInfo) == 48, "UnitInfo is three 16-byte chunks");
 
-// Shared memory: page stages, partial results of the warps, unit descriptions, mbarriers.
+// Shared memory: page stages, partial results of the warps, unit descriptions, mbarriers, failure flag.
 template <int D, int STAGES>
 struct DecSmem {
   static constexpr int kStageBytes = 2 * kPageSize * D * 2;   // K + V of one page and KV head
@@ -86,13 +87,34 @@ struct DecSmem {
   // partial results written, partial results added up, unit nearly fetched
   static constexpr int kBarDesc = kDecWarps * STAGES, kBarDone = kBarDesc + kDecRing, kBarWritten = kBarDone + kDecRing,
                        kBarAdded = kBarWritten + 1, kBarNear = kBarAdded + 1, kBars = kBarNear + 1;
+  __host__ __device__ static constexpr int off_failed(int G) { return off_bars(G) + kBars * 8; }
 };
 template <int D, int STAGES>
 __host__ __device__ constexpr size_t decode_smem_bytes(int G) {
-  return (size_t)DecSmem<D, STAGES>::off_bars(G) + DecSmem<D, STAGES>::kBars * 8;
+  return (size_t)DecSmem<D, STAGES>::off_failed(G) + 4;
 }
-// The streaming threads and the scheduler warp meet once, when the barriers are set up.
-__device__ __forceinline__ void decode_ready() { asm volatile("bar.sync 3, %0;\n" ::"n"(kDecThreads + 32) : "memory"); }
+// The streaming threads and the scheduler warp meet when the barriers are set up and before they are given back.
+__device__ __forceinline__ void decode_meet() { asm volatile("bar.sync 3, %0;\n" ::"n"(kDecThreads + 32) : "memory"); }
+
+// Every wait of the path is bounded. The copy of a page has the step's limit; a wait for other warps of the
+// CTA may span many of their pages and has a limit of its own (unit_wait_cycles). A wait that runs out raises
+// the CTA's failure flag, which ends the other waits and with them the path.
+// Called by whole warps; true, for all lanes, when the phase has completed.
+__device__ __forceinline__ bool wait_for_warps(uint32_t bar, uint32_t parity, const volatile int* failed, long long limit) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const long long t0 = clock64();
+  for (;;) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (__any_sync(0xffffffffu, *failed != 0 || clock64() - t0 > limit)) return false;
+  }
+}
+__device__ __forceinline__ void give_up(const StepDevice& s, volatile int* failed) {
+  if ((threadIdx.x & 31) == 0) {
+    atomicOr(s.status, TS_DEV_TIMEOUT);
+    *failed = 1;
+  }
+  __syncwarp();
+}
 
 // Scheduler warp of CTA `cta` of `n_ctas`: its first unit is unit `cta`, the others come off the queue
 // s.pf_queue[4], which the launch leaves at zero.
@@ -103,14 +125,16 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
   const uint32_t bars = base + L::off_bars(G);
   UnitInfo* ring = reinterpret_cast<UnitInfo*>(smem + L::off_units(G));
   const int n_units = (s.n_items - s.n_prefill_items) * s.Hkv;
-  decode_ready();
+  volatile int* failed = reinterpret_cast<volatile int*>(smem + L::off_failed(G));
+  decode_meet();
   bool ok = true;
   for (int k = 0;; ++k) {
     const int e = k % kDecRing;
     int unit = cta;
     if (k > 0) {
       // not earlier: units taken ahead of need are units that a faster CTA cannot take
-      ok = mbar_wait(bars + L::kBarNear * 8, (k - 1) & 1, s.wait_cycles);
+      ok = wait_for_warps(bars + L::kBarNear * 8, (k - 1) & 1, failed, s.unit_wait_cycles);
+      if (!ok) break;
       if (lane == 0) unit = n_ctas + atomicAdd(s.pf_queue + 4, 1);
       unit = __shfl_sync(0xffffffffu, unit, 0);
     }
@@ -128,11 +152,8 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
       u.new_pos = s.row_ctx(it.row);
       u.table_row = s.table + (size_t)s.row_slot(it.row) * s.max_pages_per_req;
     }
-    if (k >= kDecRing) ok = ok && mbar_wait(bars + (L::kBarDone + e) * 8, ((k / kDecRing) & 1) ^ 1, s.wait_cycles);
-    if (!ok) {
-      if (lane == 0) atomicOr(s.status, TS_DEV_TIMEOUT);
-      u.n_pg = -1;
-    }
+    if (k >= kDecRing) ok = wait_for_warps(bars + (L::kBarDone + e) * 8, ((k / kDecRing) & 1) ^ 1, failed, s.unit_wait_cycles);
+    if (!ok) break;              // the entry may still be read: the streaming warps end by the failure flag
     if (lane == 0) {
       ring[e] = u;
       mbar_arrive(bars + (L::kBarDesc + e) * 8);
@@ -148,6 +169,8 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
     asm volatile("" ::"r"(touched));
     if (u.n_pg < 0) break;
   }
+  if (!ok) give_up(s, failed);
+  decode_meet();                 // from here on nobody looks at a barrier of the path
 }
 
 // Streams the units that decode_schedule describes, on the first kDecThreads threads of the block
@@ -171,19 +194,18 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
   const uint32_t bars = base + L::off_bars(G);
   auto bar = [&](int i) { return bars + (uint32_t)i * 8u; };
   const uint32_t my_bars = bars + warp * STAGES * 8;
+  volatile int* failed = reinterpret_cast<volatile int*>(smem + L::off_failed(G));
 
   if (tid == 0) {
     for (int i = 0; i < L::kBars; ++i) mbar_init(bar(i), i >= L::kBarDone && i != L::kBarNear ? W : 1);
+    *failed = 0;
     mbar_init_fence();
   }
-  decode_ready();
+  decode_meet();
 
-  bool dead = false;           // a wait ran out: stop issuing copies, keep the control flow
-  auto wait = [&](uint32_t b, uint32_t parity) {
-    if (!mbar_wait(b, parity, dead ? 1000 : s.wait_cycles)) {
-      if (!dead && lane == 0) atomicOr(s.status, TS_DEV_TIMEOUT);
-      dead = true;
-    }
+  bool dead = false;           // a wait of this warp ran out (all lanes agree): it starts no copy and no page any more
+  auto wait = [&](int i, uint32_t parity) {
+    dead = dead || !wait_for_warps(bar(i), parity, failed, s.unit_wait_cycles);
   };
   // ---------------------------------------------------------------- producer side (this warp)
   // Never blocks: where the next unit is not described yet, the free stages stay free until the next call.
@@ -197,7 +219,7 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
   bool near_sent = false;      // warp 0 tells the scheduler when it has three pages of the unit left to fetch
   auto fill = [&]() {
 #pragma unroll 1
-    while (n_issued - n_consumed < STAGES) {
+    while (n_issued - n_consumed < STAGES && !dead) {
       if (!p_have) {
         const int e = pk % kDecRing;
         if (!__all_sync(0xffffffffu, mbar_test(bar(L::kBarDesc + e), (pk / kDecRing) & 1))) return;
@@ -224,7 +246,7 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
         p_pages = j < pu.n_pg ? pu.table_row[pu.first_page + j] : 0;
       }
       int page = __shfl_sync(0xffffffffu, p_pages, idx & 31);
-      if (lane == 0 && !dead) {
+      if (lane == 0) {
         if ((unsigned)page >= (unsigned)s.n_pages) {
           atomicOr(s.status, TS_DEV_BAD_PAGE);
           page = s.n_pages;    // out of range on purpose: the copy then delivers zeros
@@ -281,7 +303,7 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
   bool owe = false;            // unit ck - 1 has not been added up by this warp yet
 #pragma unroll 1
   for (;; ++ck) {
-    wait(bar(L::kBarDesc + ck % kDecRing), (ck / kDecRing) & 1);
+    wait(L::kBarDesc + ck % kDecRing, (ck / kDecRing) & 1);
     if (dead) break;           // what the ring holds is not known to be this unit
     const UnitInfo cu = units[ck % kDecRing];
     if (cu.n_pg < 0) break;
@@ -315,7 +337,8 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
     for (int j = warp; j < cu.n_pg; j += W) {
       const int stage = n_consumed % STAGES;
       const uint32_t sp = ring + stage * STAGE_BYTES;
-      wait(my_bars + stage * 8, (n_consumed / STAGES) & 1);
+      dead = !__all_sync(0xffffffffu, mbar_wait(my_bars + stage * 8, (n_consumed / STAGES) & 1, s.wait_cycles));
+      if (dead) break;
       const int pos0 = cu.k_begin + j * kPageSize;   // position of the page's first slot
       if (new_pos >= pos0 && new_pos < pos0 + kPageSize) {
         // KV append (Sec. 2.1) without a launch of its own: this page holds the row's new token,
@@ -436,10 +459,13 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
 
     // ---- leave this warp's partial result, once everyone is done with the previous unit's
     if (owe) {
-      wait(bar(L::kBarWritten), (ck - 1) & 1);
+      wait(L::kBarWritten, (ck - 1) & 1);
+      if (dead) break;
       add_up(ck - 1);
+      owe = false;
     }
-    if (ck > 0) wait(bar(L::kBarAdded), (ck - 1) & 1);
+    if (ck > 0) wait(L::kBarAdded, (ck - 1) & 1);
+    if (dead) break;
 #pragma unroll
     for (int nh = 0; nh < NH; ++nh) {
 #pragma unroll
@@ -477,12 +503,13 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
     owe = true;
   }
   if (owe) {
-    wait(bar(L::kBarWritten), (ck - 1) & 1);
-    add_up(ck - 1);
+    wait(L::kBarWritten, (ck - 1) & 1);
+    if (!dead) add_up(ck - 1);
   }
-  // no copy stays in flight (only after a failure are there any left); give the barriers' shared memory back
-  for (; n_consumed < n_issued; ++n_consumed) mbar_wait(my_bars + (n_consumed % STAGES) * 8, (n_consumed / STAGES) & 1, 100000);
-  block_sync();
+  // no copy stays in flight (only after a failure are there any left)
+  if (dead) give_up(s, failed);
+  for (; n_consumed < n_issued; ++n_consumed) mbar_wait(my_bars + (n_consumed % STAGES) * 8, (n_consumed / STAGES) & 1, kDrainCycles);
+  decode_meet();               // the scheduler included: then the barriers' shared memory can be given back
   if (tid == 0) {
     for (int i = 0; i < L::kBars; ++i) asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(bar(i)) : "memory");
   }

@@ -557,6 +557,7 @@ void fill_device(ts_ctx* c, const ts_step* st, int64_t n_tokens, ts::StepDevice*
   d->max_requests = c->cfg.max_requests;
   d->scale_log2 = c->scale * 1.4426950408889634f;
   d->wait_cycles = c->cfg.wait_limit_cycles > 0 ? (long long)c->cfg.wait_limit_cycles : ts::kWaitCycles;
+  d->unit_wait_cycles = d->wait_cycles;
   d->append_wide = 0;          // both set by the mixed launch
   d->debug_arrivals = 0;
 }
@@ -617,6 +618,15 @@ int choose_prefill_ctas(const ts_ctx* c, int n_ctas, double prefill_block_pairs,
   return ((lo + hi) / 2) & ~1;
 }
 
+// Limit of a wait that may span the pages of two decode units, of which `longest` is the longest of the
+// step: the eight warps of a CTA share a unit's pages, and the copy of each may take wait_cycles. Not above
+// two seconds (or wait_cycles itself): a lost copy ends all waits by its own limit.
+long long unit_wait_cycles(long long wait_cycles, const WorkItem& longest) {
+  const long long pages = ceil_div(longest.k_end - longest.k_begin, ts::kPageSize), cap = std::max(wait_cycles, 2 * ts::kWaitCycles);
+  const long long copies = 2 * ((pages + 7) / 8) + 8;
+  return wait_cycles > cap / copies ? cap : wait_cycles * copies;
+}
+
 // Enqueues a checked step (c->tok0 holds its prefix sums).
 int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefill, cudaStream_t stream, bool attention) {
   if (attention) plan(c, st);
@@ -655,6 +665,7 @@ int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefi
     ++c->cnt.kernel_launches;
   }
   if (attention) {
+    if (n_items > c->n_prefill_items) d.unit_wait_cycles = unit_wait_cycles(d.wait_cycles, c->items[c->n_prefill_items]);
     if (pe) TS_CUDA(c, cudaEventRecord(pe[1], stream));
     d.n_prefill_items = c->n_prefill_items;
     bool decode_launched = false;

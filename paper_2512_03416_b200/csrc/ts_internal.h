@@ -68,7 +68,9 @@ struct StepDevice {
   int32_t n_prefill_items;  // items[0, n_prefill_items) are prefill tiles, the rest decode splits
   int32_t Hq, Hkv, D, n_pages, max_pages_per_req, max_requests;
   float scale_log2;        // softmax scale * log2(e)
-  long long wait_cycles;   // limit of every bounded wait of the step's kernels, in clock cycles
+  long long wait_cycles;   // limit of every bounded wait of the step's kernels, in clock cycles, but for those
+                           // that may span the pages of a whole decode unit:
+  long long unit_wait_cycles;
   int32_t append_wide;     // mixed kernel: CTAs that start on prefill units append with their softmax warps first
   int32_t debug_arrivals;  // > 0: the mixed kernel waits for that many arrivals, which nothing sends (TS_DEBUG_LOSE_APPEND_ARRIVAL)
   // The step's row arrays and work list: word offsets from `meta`, a device address, or, where they

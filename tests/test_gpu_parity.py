@@ -298,3 +298,15 @@ def test_a_decode_rows_largest_weight_is_exact(shape, chunk):
         bound = 2.0 ** -8 * np.abs(want) + 1e-5 * (np.abs(v_first) + np.abs(v_late))
         worst = float((np.abs(got[r] - want) / bound).max())
         assert worst <= 1.0, f"row {r}: error {worst} times its bound"
+
+
+@pytest.mark.parametrize("chunk", [0, 40], ids=["decode", "mixed"])
+def test_a_wait_limit_need_not_cover_a_whole_unit(chunk):
+    """The limit of a wait covers the copy of one page. A unit of 6251 pages is streamed by one thread block
+    for several times the 300,000 cycles (about 0.15 ms) allowed here, while its scheduler warp, and the
+    streaming warps among one another, wait for it: those waits go on as long as pages come in."""
+    b = wl.make_batch("limit", wl.Shape(4, 1, 128), [100000] + [0] * (chunk > 0), [1] + [chunk] * (chunk > 0), seed=chunk, profile="peaked")
+    want, pool_want = oracle_step(b)
+    run = GpuRun(b, chunk_size=0, decode_split_tokens=1 << 20, wait_limit_cycles=300_000)
+    assert_parity(run.step(), want, "peaked", "one long unit under a short limit")
+    assert np.array_equal(run.pool(), pool_want)
