@@ -45,6 +45,7 @@
 #include "ts_ptx.h"
 #include "ts_tc.h"
 #include "ts_tma.h"
+#include "ts_units.h"
 
 namespace ts {
 namespace {
@@ -61,7 +62,6 @@ static_assert(4 * 128 * kRegsSoftmax + 128 * kRegsAux <= kPfThreads * kRegsLaunc
 static_assert(2 * 128 * kRegsDecode + 2 * 128 * kRegsParked + 128 * kRegsAux <= kPfThreads * kRegsLaunch,
               "register split of the decode phase exceeds the launch's total");
 constexpr int kWarpLoader0 = 16, kWarpMma = 18, kWarpSched = 19;
-constexpr int kBlockKeys = 128;
 constexpr int kD = 128;
 constexpr int kTileBytes = 128 * kD * 2;        // one 128 x 128 bf16 operand tile: 32 KB
 constexpr int kHalfBytes = kTileBytes / 2;      // 64 head_dim columns of it
@@ -92,7 +92,6 @@ enum {
 // then a ring of the published units' records (8 words each)
 constexpr int kOffMisc = kOffBar + BAR_COUNT * 8;
 constexpr int kOffRing = kOffMisc + 16;
-constexpr int kSchedRing = 8;
 // row statistics the two threads of a query row exchange: [tile][half][row] floats
 constexpr int kOffXchg = kOffRing + kSchedRing * 32;
 constexpr int kSmemBytes = kOffXchg + 2 * 2 * 128 * 4;
@@ -173,42 +172,6 @@ __device__ __forceinline__ float max64(const float (&v)[64]) {
   m1 = max3(m1, v[62], v[63]);
   return fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
 }
-// One prefill work unit as its claimer publishes it in shared memory (8 words), and the shape
-// every role derives from it.
-struct UnitRec {
-  int32_t w;                 // work unit index, -1 = the queue is empty
-  int32_t table_slot;        // request slot: row of the block table
-  int32_t kv_head, q_begin, q_count;
-  int32_t ctx;               // tokens cached before the chunk
-  int32_t tok0;              // first token of the request row in the step's tensors
-  int32_t pad;
-};
-static_assert(sizeof(UnitRec) == 32, "UnitRec is 8 words");
-struct PfUnit {
-  int table_slot, kv_head, q_begin, ctx, tok0;
-  int cnt_a, cnt_b;          // tokens of tile A / tile B (tile B may be empty)
-  int k_end_a, k_end_b;      // one past the last key any row of the tile may see
-  int nb_a, nb_b, nb;        // key blocks per tile, and of the unit
-  int k_end;
-};
-__device__ __forceinline__ PfUnit unit_shape(const UnitRec& r, int tile_tokens) {
-  PfUnit u;
-  u.table_slot = r.table_slot;
-  u.kv_head = r.kv_head;
-  u.q_begin = r.q_begin;
-  u.ctx = r.ctx;
-  u.tok0 = r.tok0;
-  u.cnt_a = min(r.q_count, tile_tokens);
-  u.cnt_b = r.q_count - u.cnt_a;
-  u.k_end_a = u.ctx + r.q_begin + u.cnt_a;
-  u.k_end_b = u.k_end_a + u.cnt_b;
-  u.nb_a = (u.k_end_a + kBlockKeys - 1) / kBlockKeys;
-  u.nb_b = u.cnt_b > 0 ? (u.k_end_b + kBlockKeys - 1) / kBlockKeys : 0;
-  u.nb = max(u.nb_a, u.nb_b);
-  u.k_end = max(u.k_end_a, u.k_end_b);
-  return u;
-}
-
 // The append of the prefill rows' new tokens (Sec. 2.1). The prefill work items cover those tokens
 // exactly once, `per_item` at most each; warp i of n appends tokens i, i + n, ... of that list. A lane
 // looks up one of the warp's next 32 tokens (item -> row -> block table: three dependent loads, paid
@@ -312,7 +275,11 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
   auto wait = [&](int i, uint32_t parity) {
     if (!mbar_wait(bar(i), parity, misc[1] ? 2000 : s.wait_cycles)) give_up();
   };
-  // k-th work unit of this CTA (w = -1 after the last one), published by the K loaders' first thread
+  // k-th work unit of this CTA (w = -1 after the last one), published by the K loader. An entry of the
+  // ring stays while it is read: the K loader is at most three units in front of the softmax warps (it is
+  // two key blocks in front of the MMAs, and those need the P of all blocks before), and after a failure,
+  // when its waits end early, it publishes no further unit. (A tile without rows in a unit is not waited
+  // for; its warps only read the record, and have the whole unit's time for it.)
   volatile int4* ring = reinterpret_cast<volatile int4*>(smem + kOffRing);
   auto read_unit = [&](int k, PfUnit& u) -> bool {           // of a published unit
     UnitRec r;
@@ -325,11 +292,13 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
     u = unit_shape(r, tile_tokens);
     return true;
   };
+  // Called by whole warps; all lanes get the same answer (a warp that left its loop in part would never
+  // meet its partner, or itself, again).
   auto get_work = [&](int k, PfUnit& u) -> bool {
-    if ((int)misc[2] <= k) {
+    if (__any_sync(0xffffffffu, (int)misc[2] <= k)) {
       const long long t0 = clock64();
-      while ((int)misc[2] <= k) {
-        if (clock64() - t0 > (misc[1] ? 2000 : s.wait_cycles)) {
+      while (__any_sync(0xffffffffu, (int)misc[2] <= k)) {
+        if (__any_sync(0xffffffffu, clock64() - t0 > (misc[1] ? 2000 : s.wait_cycles))) {
           give_up();
           return false;
         }
@@ -442,7 +411,8 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
     // each exchange through shared memory; it wakes them sooner than an mbarrier (8192-token chunk
     // next to 190 rows 1274 -> 1238 us, 2048 tokens alone 50.7 -> 48.4 us). It has no time limit, so
     // the two must never disagree about how often they meet: all their other waits are limited and end
-    // in the same control flow, and whether there is another work unit is for the first of them to say.
+    // in the same control flow, and how many blocks of a unit the tile has (-1: there is no further unit)
+    // is for the first of them to say, one number for all lanes of both.
     auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;\n" ::"r"(4 + x * 4 + (warp & 3)) : "memory"); };
     float* xchg = reinterpret_cast<float*>(smem + kOffXchg) + x * 256;   // [half][row] of my tile
     float* xchg_mine = xchg + hf * 128 + row;
@@ -451,17 +421,16 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
     const float scale = s.scale_log2;
     int sx = 0;                 // blocks of this tile in earlier work units: barrier phases follow it
     for (int k = 0;; ++k) {
-      PfUnit u;
-      bool more = false;
+      PfUnit u = {};
+      int nbx = -1;
       if (hf == 0) {
-        more = get_work(k, u);
-        *xchg_other = more ? 1.f : 0.f;      // the other thread's own slot: it reads it before it writes it again
+        nbx = __shfl_sync(0xffffffffu, posted_blocks(get_work(k, u), u, x), 0);
+        *xchg_other = __int_as_float(nbx);   // the other thread's own slot: it reads it before it writes it again
       }
       pair_sync();
-      if (hf == 1) more = *xchg_mine != 0.f;
-      if (!more) break;
+      if (hf == 1) nbx = __shfl_sync(0xffffffffu, __float_as_int(*xchg_mine), 0);
+      if (nbx < 0) break;
       if (hf == 1) read_unit(k, u);
-      const int nbx = x ? u.nb_b : u.nb_a;
       const int cnt = x ? u.cnt_b : u.cnt_a;
       const int tok = u.q_begin + x * tile_tokens + row_g;     // token inside the request row
       const bool real = row_g < cnt && row < tile_tokens * G;
@@ -688,7 +657,8 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
       int fetched = 0;
       auto fetch_one = [&]() {
         // a CTA that starts on prefill work has its first unit without asking; the queue hands out the rest
-        const int w = fetched == 0 && !decode_first ? (int)blockIdx.x : n_prefill_ctas + atomicAdd(s.pf_queue, 1);
+        const int w = next_unit(misc[1] != 0, fetched == 0 && !decode_first, (int)blockIdx.x, n_units,
+                                [&]() { return n_prefill_ctas + atomicAdd(s.pf_queue, 1); });
         UnitRec r = {};
         r.w = -1;
         if (w < n_units) {
@@ -772,7 +742,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
           if (g >= stages) wait(empty + st, ((g / stages) & 1) ^ 1);
           const bool touch = kv == 0 && j == start_tile;
           const uint32_t landed = bar(kv ? BAR_V_LANDED + st : touch ? BAR_K_LANDED : full + st);
-          if (misc[1] == 0) {                                  // after a failure no new copies are started
+          if (__all_sync(0xffffffffu, misc[1] == 0)) {         // after a failure no new copies are started
             if (lane == 0) mbar_expect_tx(landed, kTileBytes);
             __syncwarp();
             const uint32_t dst = tile0 + st * kTileBytes;
