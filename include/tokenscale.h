@@ -104,10 +104,11 @@ typedef struct {
 } ts_config;
 
 /*
- * Debug flags (the paper has no counterpart). TS_DEBUG_LOSE_APPEND_ARRIVAL makes every thread block
- * of a head_dim 128 step with prefill rows wait, before its first prefill work, for an arrival that
- * nothing sends: every block then raises TS_DEV_TIMEOUT after wait_limit_cycles and carries on
- * (nothing depends on that arrival, so the step's output is still valid).
+ * Debug flags (the paper has no counterpart). TS_DEBUG_LOSE_APPEND_ARRIVAL makes the
+ * thread blocks of a head_dim 128 step with prefill rows, before they merge the splits of its decode
+ * rows, wait for one block more than there are: every block then raises TS_DEV_TIMEOUT after
+ * wait_limit_cycles and carries on (all blocks do arrive long before, so the step's output is still
+ * valid). Steps without prefill rows or without a split decode row have no such wait and take no notice.
  * It exists so that the time-out path can be exercised without a fault: ts_create refuses it
  * (TS_ERR_INVALID) unless 0 < wait_limit_cycles <= 50,000,000 (about 25 ms), so it can never spin
  * for the default second.

@@ -24,9 +24,9 @@ decode_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUte
     if (threadIdx.x == kDecThreads) {
       // the last scheduler to get here puts the queue back to zero for the next launch
       __threadfence();
-      if (atomicAdd(s.pf_queue + 5, 1) == (int)gridDim.x - 1) {
+      if (atomicAdd(s.pf_queue + 4, 1) == (int)gridDim.x - 1) {
+        s.pf_queue[3] = 0;
         s.pf_queue[4] = 0;
-        s.pf_queue[5] = 0;
       }
     }
   }

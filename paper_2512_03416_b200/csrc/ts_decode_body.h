@@ -117,7 +117,7 @@ __device__ __forceinline__ void give_up(const StepDevice& s, volatile int* faile
 }
 
 // Scheduler warp of CTA `cta` of `n_ctas`: its first unit is unit `cta`, the others come off the queue
-// s.pf_queue[4], which the launch leaves at zero.
+// s.pf_queue[3], which the launch leaves at zero.
 template <int D, int STAGES>
 __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned char* smem, uint32_t base, int cta, int n_ctas) {
   using L = DecSmem<D, STAGES>;
@@ -135,7 +135,7 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
       // not earlier: units taken ahead of need are units that a faster CTA cannot take
       ok = wait_for_warps(bars + L::kBarNear * 8, (k - 1) & 1, failed, s.unit_wait_cycles);
       if (!ok) break;
-      if (lane == 0) unit = n_ctas + atomicAdd(s.pf_queue + 4, 1);
+      if (lane == 0) unit = n_ctas + atomicAdd(s.pf_queue + 3, 1);
       unit = __shfl_sync(0xffffffffu, unit, 0);
     }
     UnitInfo u = {};

@@ -710,7 +710,7 @@ int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefi
         const double append_us = 2.0 * (double)n_prefill / (p + 4.0 * (n_ctas - p)) *
                                  ceil_div(4 * c->cfg.n_kv_heads * c->cfg.head_dim, 4096);
         d.append_wide = append_us > 2.0 * pairs / n_ctas;
-        d.debug_arrivals = (c->cfg.debug_flags & TS_DEBUG_LOSE_APPEND_ARRIVAL) ? n_ctas + 1 : 0;
+        d.debug_arrivals = (c->cfg.debug_flags & TS_DEBUG_LOSE_APPEND_ARRIVAL) ? 1 : 0;
         TS_CUDA(c, ts::launch_mixed(d, q_map, c->kv_map, c->kv_tile_map, new_maps, n_ctas, p, stream));
       } else {
         ts::StepDevice dp = d;

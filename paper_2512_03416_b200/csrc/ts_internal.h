@@ -54,8 +54,8 @@ struct StepDevice {
   int32_t* status;         // device status word
   int32_t* pf_queue;       // counters, all zero between launches (the last CTA to leave resets them):
                            // mixed kernel [0] next prefill work unit, [1] decode CTAs that have finished
-                           // their units, [2] see debug_arrivals, [3] CTAs that have left; [4] decode
-                           // units taken besides the CTAs' first ones; decode kernel [5] CTAs that are done
+                           // their units, [2] CTAs that have left; [3] decode units taken besides the
+                           // CTAs' first ones; decode kernel [4] CTAs that are done
   float* part_acc;         // [max_partials][Hq][D]
   float* part_ml;          // [max_partials][Hq][2]  (running max in log2 units, sum)
   // step tensors
@@ -72,7 +72,7 @@ struct StepDevice {
                            // that may span the pages of a whole decode unit:
   long long unit_wait_cycles;
   int32_t append_wide;     // mixed kernel: CTAs that start on prefill units append with their softmax warps first
-  int32_t debug_arrivals;  // > 0: the mixed kernel waits for that many arrivals, which nothing sends (TS_DEBUG_LOSE_APPEND_ARRIVAL)
+  int32_t debug_arrivals;  // decode CTAs besides the launch's own that the mixed kernel's merge waits for (TS_DEBUG_LOSE_APPEND_ARRIVAL)
   // The step's row arrays and work list: word offsets from `meta`, a device address, or, where they
   // are small, from `words`: they then travel as launch parameters, without an upload of their own (a copy
   // on another stream, two event records and two waits: ~6 us of host time and a dependency per step).

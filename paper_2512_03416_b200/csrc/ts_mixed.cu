@@ -311,16 +311,6 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
     if (tid == 0) {
       misc[1] = 0;
       misc[2] = 0;
-      if (s.debug_arrivals > 0) {   // a wait that nothing ends, asked for by ts_config.debug_flags
-        const volatile int32_t* arrived = s.pf_queue + 2;
-        const long long t0 = clock64();
-        while (*arrived < s.debug_arrivals) {
-          if (clock64() - t0 > s.wait_cycles) {
-            atomicOr(s.status, TS_DEV_TIMEOUT);
-            break;
-          }
-        }
-      }
       for (int i = 0; i < BAR_COUNT; ++i) {
         const bool softmax_arrives = (i >= BAR_P_FULL && i < BAR_P_FULL + 2) || (i >= BAR_O_EMPTY && i < BAR_O_EMPTY + 2);
         mbar_init(bar(i), softmax_arrives ? 256 : 1);
@@ -569,7 +559,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
       if (tid == 0) {
         const volatile int32_t* done = s.pf_queue + 1;
         const long long t0 = clock64();
-        while (*done < n_decode_ctas) {
+        while (*done < n_decode_ctas + s.debug_arrivals) {
           if (clock64() - t0 > (misc[1] ? 2000 : s.wait_cycles)) {
             give_up();
             break;
@@ -903,12 +893,11 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
   if (tid == 0) {
     // the last CTA to leave puts the launch's counters back to zero for the next launch
     __threadfence();
-    if (atomicAdd(s.pf_queue + 3, 1) == (int)gridDim.x - 1) {
+    if (atomicAdd(s.pf_queue + 2, 1) == (int)gridDim.x - 1) {
       s.pf_queue[0] = 0;
       s.pf_queue[1] = 0;
       s.pf_queue[2] = 0;
       s.pf_queue[3] = 0;
-      s.pf_queue[4] = 0;
     }
   }
 }

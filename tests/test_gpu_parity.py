@@ -169,8 +169,8 @@ def test_maximum_sizes_sampled():
 
 
 def test_a_wait_that_runs_out_is_reported_and_the_next_step_is_clean():
-    """Failure path without a fault: with TS_DEBUG_LOSE_APPEND_ARRIVAL the barrier after the KV
-    append of a mixed step waits for one thread block more than the launch has, under a limit of
+    """Failure path without a fault: with TS_DEBUG_LOSE_APPEND_ARRIVAL the wait in front of the merge of
+    a mixed step's decode splits is for one thread block more than stream them, under a limit of
     2 million clock cycles (about a millisecond; never the library's default second). Every block
     then gives that wait up, raises TS_DEV_TIMEOUT and carries on. The step must return, the status
     call must report TS_ERR_DEVICE_TIMEOUT once and then be clean, and a normal context's next
@@ -178,20 +178,23 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_step_is_clean():
     from paper_2512_03416_b200 import binding as B
     b = wl.make_batch("tmo", wl.LLAMA8B, [300, 40, 0], [1, 1, 300], seed=41, profile="peaked")
     want, pool_want = oracle_step(b)
-    run = GpuRun(b, chunk_size=0, wait_limit_cycles=2_000_000, debug_flags=B.TS_DEBUG_LOSE_APPEND_ARRIVAL)
+    run = GpuRun(b, chunk_size=0, decode_split_tokens=64, wait_limit_cycles=2_000_000, debug_flags=B.TS_DEBUG_LOSE_APPEND_ARRIVAL)
     run.lb.step(keep_len=True)
     rc, bits = B.ts_last_device_status(run.dec.ctx, torch.cuda.current_stream().cuda_stream)
     assert rc == B.TS_ERR_DEVICE_TIMEOUT and bits & B.TS_DEV_TIMEOUT
     # all blocks had in fact arrived, so even this step's result is complete
-    assert_parity(run.lb.output(), want, "peaked", "step whose append barrier gave up")
+    assert_parity(run.lb.output(), want, "peaked", "step whose merge gave up its wait")
     rc, bits = B.ts_last_device_status(run.dec.ctx, torch.cuda.current_stream().cuda_stream)
     assert rc == B.TS_OK and bits == 0, "the status word was not cleared"
     # the launch's counters are back at zero: the same context runs the step again, still flagged
     run.lb.step(keep_len=True)
     assert run.dec.device_status() == B.TS_DEV_TIMEOUT
     run.dec.close()
+    # without a split row nothing waits for the blocks that stream decode rows: the flag changes nothing
+    whole = GpuRun(b, chunk_size=0, wait_limit_cycles=2_000_000, debug_flags=B.TS_DEBUG_LOSE_APPEND_ARRIVAL)
+    assert_parity(whole.step(), want, "peaked", "flagged step without split rows")
     # and a context without the flag is clean
-    ok = GpuRun(b, chunk_size=0)
+    ok = GpuRun(b, chunk_size=0, decode_split_tokens=64)
     got = ok.step()
     assert_parity(got, want, "peaked", "step after a timed-out one")
     assert np.array_equal(ok.pool(), pool_want)
