@@ -35,7 +35,9 @@
 // every CTA copies a share of the prefill rows' tokens next to its other work, and nothing waits for
 // the copies, because the tiles take a chunk's own tokens from the step's tensors; the decode units
 // write their rows' own tokens.
-// Every wait is bounded; a wait that runs out raises TS_DEV_TIMEOUT and the CTA drains.
+// Every wait is bounded; a wait that runs out raises TS_DEV_TIMEOUT and the CTA drains: nothing new is
+// started, the other waits end early, and before the CTA leaves, the copies and MMAs it did start are
+// waited for (with a limit of their own).
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
@@ -66,6 +68,7 @@ constexpr int kD = 128;
 constexpr int kTileBytes = 128 * kD * 2;        // one 128 x 128 bf16 operand tile: 32 KB
 constexpr int kHalfBytes = kTileBytes / 2;      // 64 head_dim columns of it
 constexpr int kKStages = 2, kVStages = 3;       // measured: a third V stage is worth more than a third K stage (3%)
+constexpr long long kDrainCycles = 20000000;    // about 10 ms: limit of the waits for copies and MMAs in flight after a failure
 constexpr float kRescaleThreshold = 8.0f;       // log2 units
 
 // shared-memory map (offsets from the 1024-aligned base)
@@ -86,7 +89,8 @@ enum {
   BAR_Q_EMPTY = BAR_O_EMPTY + 2,          // the last Q K^T of a work unit has consumed the Q tiles
   BAR_V_LANDED = BAR_Q_EMPTY + 1,         // [kVStages] the copies of a V tile are in shared memory
   BAR_K_LANDED = BAR_V_LANDED + kVStages, // the same for a K tile that needs a touch-up before it is announced
-  BAR_COUNT = BAR_K_LANDED + 1
+  BAR_DRAIN = BAR_K_LANDED + 1,           // after a failure: the MMAs issued before it are done
+  BAR_COUNT = BAR_DRAIN + 1
 };
 // misc words: [0] TMEM base address, [1] failure flag, [2] work units published so far;
 // then a ring of the published units' records (8 words each)
@@ -672,6 +676,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
         misc[2] = (uint32_t)++fetched;
       };
       int g0 = 0;                                              // key blocks of earlier work units
+      int n_copied = 0;                                        // tiles whose copies were started: the first n_copied ones
       for (int k = 0;; ++k) {
         if (kv == 0 && lane == 0) fetch_one();
         __syncwarp();
@@ -733,6 +738,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
           const bool touch = kv == 0 && j == start_tile;
           const uint32_t landed = bar(kv ? BAR_V_LANDED + st : touch ? BAR_K_LANDED : full + st);
           if (__all_sync(0xffffffffu, misc[1] == 0)) {         // after a failure no new copies are started
+            n_copied = g + 1;
             if (lane == 0) mbar_expect_tx(landed, kTileBytes);
             __syncwarp();
             const uint32_t dst = tile0 + st * kTileBytes;
@@ -752,15 +758,20 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
               fence_proxy_async();
               __syncwarp();
               if (lane == 0) mbar_arrive(bar(full + st));
+              ++n_touched;
             }
           }
-          n_touched += touch;
           page = page_next;
         }
         // the last `lag` V tiles (fewer when the unit is short) have not been announced yet
         if (kv)
           for (int tile = max(0, u.nb - lag); tile < u.nb; ++tile) announce(tile);
         g0 += u.nb;
+      }
+      if (misc[1]) {
+        if (n_touched > 0) mbar_wait(bar(BAR_K_LANDED), (n_touched - 1) & 1, kDrainCycles);
+        for (int g = max(0, n_copied - stages); g < n_copied; ++g)
+          mbar_wait(bar((kv ? BAR_V_LANDED : full) + g % stages), (g / stages) & 1, kDrainCycles);
       }
     } else {
       // ------------------------------------------------------------------- MMA issuer
@@ -851,6 +862,10 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
             used[x] += nbx > 0;
           }
         }
+        if (__any_sync(0xffffffffu, misc[1] != 0)) {
+          tc_commit(bar(BAR_DRAIN), issue);
+          mbar_wait(bar(BAR_DRAIN), 0, kDrainCycles);
+        }
       }
       if (warp == kWarpSched) {
         // ------------------------------------------------------------------ Q loader
@@ -861,6 +876,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
         auto append_until = [&](auto&& ready) {
           while (!app.done() && !__any_sync(0xffffffffu, ready())) app.step<4>(s, 2 * tile_tokens, lane);   // 4: 64 registers here
         };
+        int n_loaded = 0;
         for (int k = 0;; ++k) {
           PfUnit u;
           if (k > 0) append_until([&]() { return (int)misc[2] > k; });   // the first Q tiles wait for nothing
@@ -870,6 +886,8 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
             append_until([&]() { return mbar_test(bar(BAR_Q_EMPTY), (k - 1) & 1); });
             wait(BAR_Q_EMPTY, (k - 1) & 1);
           }
+          if (__any_sync(0xffffffffu, misc[1] != 0)) break;    // after a failure no new copies are started
+          n_loaded = k + 1;
           // a box delivers 64 columns of tile_tokens * G packed rows (all 128 only when G divides 128)
           if (lane == 0) {
             mbar_expect_tx(bar(BAR_Q), (u.cnt_b > 0 ? 2 : 1) * 2 * (tile_tokens * G * 128));
@@ -883,6 +901,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
           __syncwarp();
         }
         append_until([]() { return false; });
+        if (misc[1] && n_loaded > 0) mbar_wait(bar(BAR_Q), (n_loaded - 1) & 1, kDrainCycles);
       }
       __syncwarp();
     }
