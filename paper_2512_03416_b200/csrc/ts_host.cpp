@@ -342,9 +342,15 @@ int validate(ts_ctx* c, const ts_step* st, bool attention, bool need_tensors, in
   return TS_OK;
 }
 
-// Builds c->items / c->combines for a validated step.
-void plan(ts_ctx* c, const ts_step* st) {
-  const int G = c->G;
+// A decode row of n keys in pieces of at most `split` keys: keys per piece (whole key tiles) and pieces.
+void cut_row(int n, int split, int* per, int* pieces) {
+  const int wanted = ceil_div(n, split);
+  *per = wanted <= 1 ? n : ceil_div(ceil_div(n, wanted), ts::kKeysPerTile) * ts::kKeysPerTile;
+  *pieces = ceil_div(n, *per);
+}
+
+// Keys per split of a step's decode rows.
+int decode_split(const ts_ctx* c, const ts_step* st) {
   int split = c->cfg.decode_split_tokens;
   if (split <= 0) {
     // An SM's share of the step's (key, KV head) pairs, so that a small batch's long rows spread over
@@ -360,37 +366,47 @@ void plan(ts_ctx* c, const ts_step* st) {
     split = (int)std::min<int64_t>(std::max<int64_t>(share, kMinDefaultSplit), kMaxDefaultSplit);
   }
   split = ceil_div(split, ts::kKeysPerTile) * ts::kKeysPerTile;
-  for (;;) {
-    c->items.clear();
-    c->combines.clear();
-    int partial = 0;
+  for (;; split *= 2) {
+    int64_t partials = 0;
     for (int r = 0; r < st->n_rows; ++r) {
-      const int ql = st->q_len[r], ctx = st->ctx_len[r];
-      if (ql > 1) {
-        // head_dim 128: two query tiles of 128 packed rows per item (128/G whole tokens each);
-        // head_dim 64: one tile of 64 packed rows
-        const int tt = c->cfg.head_dim == 128 ? 2 * (ts::kPackedRowsTc / G) : ts::kPackedRowsPerTile / G;
-        for (int t0 = 0; t0 < ql; t0 += tt) {
-          const int cnt = std::min(tt, ql - t0);
-          c->items.push_back(WorkItem{r, 1, t0, cnt, 0, ctx + t0 + cnt, -1, 0});
-        }
-      } else {
-        const int n = ctx + 1;
-        int ns = ceil_div(n, split);
-        if (ns <= 1) {
-          c->items.push_back(WorkItem{r, 0, 0, 1, 0, n, -1, 0});
-        } else {
-          const int per = ceil_div(ceil_div(n, ns), ts::kKeysPerTile) * ts::kKeysPerTile;
-          ns = ceil_div(n, per);
-          c->combines.push_back(CombineItem{c->tok0[r], partial, ns, 0});
-          for (int s = 0; s < ns; ++s) {
-            c->items.push_back(WorkItem{r, 0, 0, 1, s * per, std::min(n, (s + 1) * per), partial++, 0});
-          }
-        }
-      }
+      if (st->q_len[r] != 1) continue;
+      int per, pieces;
+      cut_row(st->ctx_len[r] + 1, split, &per, &pieces);
+      if (pieces > 1) partials += pieces;
     }
-    if (partial <= c->L.max_partials) break;
-    split *= 2;
+    if (partials <= c->L.max_partials) return split;
+  }
+}
+
+// Builds c->items / c->combines for a validated step whose decode rows are split by `split` keys
+// (decode_split of the step, or of the step that it is a piece of).
+void plan(ts_ctx* c, const ts_step* st, int split) {
+  const int G = c->G;
+  c->items.clear();
+  c->combines.clear();
+  int partial = 0;
+  for (int r = 0; r < st->n_rows; ++r) {
+    const int ql = st->q_len[r], ctx = st->ctx_len[r];
+    if (ql > 1) {
+      // head_dim 128: two query tiles of 128 packed rows per item (128/G whole tokens each);
+      // head_dim 64: one tile of 64 packed rows
+      const int tt = c->cfg.head_dim == 128 ? 2 * (ts::kPackedRowsTc / G) : ts::kPackedRowsPerTile / G;
+      for (int t0 = 0; t0 < ql; t0 += tt) {
+        const int cnt = std::min(tt, ql - t0);
+        c->items.push_back(WorkItem{r, 1, t0, cnt, 0, ctx + t0 + cnt, -1, 0});
+      }
+      continue;
+    }
+    const int n = ctx + 1;
+    int per, pieces;
+    cut_row(n, split, &per, &pieces);
+    if (pieces == 1) {
+      c->items.push_back(WorkItem{r, 0, 0, 1, 0, n, -1, 0});
+      continue;
+    }
+    c->combines.push_back(CombineItem{c->tok0[r], partial, pieces, 0});
+    for (int i = 0; i < pieces; ++i)
+      c->items.push_back(WorkItem{r, 0, 0, 1, i * per, std::min(n, (i + 1) * per), partial++, 0});
   }
   // Prefill tiles first, then decode splits; inside each group heaviest first, so that the tail
   // of each launch is made of short items.
@@ -627,9 +643,9 @@ long long unit_wait_cycles(long long wait_cycles, const WorkItem& longest) {
   return wait_cycles > cap / copies ? cap : wait_cycles * copies;
 }
 
-// Enqueues a checked step (c->tok0 holds its prefix sums).
-int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefill, cudaStream_t stream, bool attention) {
-  if (attention) plan(c, st);
+// Enqueues a checked step (c->tok0 holds its prefix sums); `split`: see plan (not read without attention).
+int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefill, int split, cudaStream_t stream, bool attention) {
+  if (attention) plan(c, st, split);
   int rc = ensure_cuda(c, stream);
   if (rc != TS_OK) return rc;
   int n_slot_deltas = 0;
@@ -750,7 +766,8 @@ void finish_step(ts_ctx* c, const ts_step* st, int n_decode, int64_t n_prefill, 
 // takes upload + kernels + download one after the other; in pieces the download of one overlaps the
 // kernels and uploads of the next (the copies run both ways at once). A piece still fills half of the
 // chip with prefill units and moves 4 MB up, so that neither its kernels nor its copies are bound by
-// latency; calls that do not wait overlap with one another already. Measured on 64 rows + 2048 tokens
+// latency; calls that do not wait overlap with one another already. Every piece has tokens of a chunk: rows
+// without one would run in the decode kernel, whose splits are merged by a launch that rounds differently. Measured on 64 rows + 2048 tokens
 // of the 8B shape (26 MB up, 17 MB down): one piece 988 us,
 // two 843, three (the rule) 815, four 830, six 875.
 int host_pieces(const ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefill, int64_t* cut) {
@@ -766,6 +783,11 @@ int host_pieces(const ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_
     const int64_t by_bytes = n_tokens * (int64_t)(tq + 2 * tk) >> 22;
     pieces = std::max<int64_t>(1, std::min<int64_t>({by_units, by_bytes, kMaxPieces}));
   }
+  auto has_chunk = [&](int64_t from, int64_t to) {
+    for (int r = 0; r < st->n_rows; ++r)
+      if (st->q_len[r] > 1 && c->tok0[r] < to && c->tok0[r + 1] > from) return true;
+    return false;
+  };
   int n = 0;
   cut[0] = 0;
   for (int64_t i = 1; i < pieces; ++i) {
@@ -775,7 +797,7 @@ int host_pieces(const ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_
     t = a + (t - a) / unit * unit;                                        // whole work items in front of the cut
     if (t - a == 1) t = a;                                                // no row is cut down to one token
     if (e - t == 1) t = e;
-    if (t > cut[n] && t < n_tokens) cut[++n] = t;
+    if (t > cut[n] && t < n_tokens && has_chunk(cut[n], t) && has_chunk(t, n_tokens)) cut[++n] = t;
   }
   cut[++n] = n_tokens;
   return n;
@@ -789,7 +811,7 @@ int run_step(ts_ctx* c, const ts_step* st, void* cuda_stream, bool attention) {
   if (st->n_rows == 0) return TS_OK;
   if (!aligned16(st->k_new) || !aligned16(st->v_new)) return TS_ERR_INVALID;
   if (attention && (!aligned16(st->q) || !aligned16(st->out))) return TS_ERR_INVALID;
-  rc = enqueue_step(c, st, n_tokens, n_prefill, (cudaStream_t)cuda_stream, attention);
+  rc = enqueue_step(c, st, n_tokens, n_prefill, attention ? decode_split(c, st) : 0, (cudaStream_t)cuda_stream, attention);
   if (rc != TS_OK) return rc;
   finish_step(c, st, n_decode, n_prefill, attention);
   return TS_OK;
@@ -1062,6 +1084,7 @@ int ts_mixed_step_host(ts_ctx* c, const ts_step* st, void* cuda_stream) {
   void* dv = ws + 2 * c->L.stage_q_bytes + c->L.stage_kv_bytes;
   int64_t cut[kMaxPieces + 1];
   const int n_pieces = host_pieces(c, st, n_tokens, n_prefill, cut);
+  const int split = decode_split(c, st);           // of the whole step: a row's result does not depend on the cuts
   const std::vector<int32_t> tok0 = c->tok0;       // of the whole step; a piece has its own in c->tok0
   const size_t tq = (size_t)c->cfg.n_q_heads * c->cfg.head_dim * 2, tk = (size_t)c->cfg.n_kv_heads * c->cfg.head_dim * 2;
   if (c->stage_used[b]) TS_CUDA(c, cudaStreamWaitEvent(c->up_stream, c->down_done[b], 0));
@@ -1098,7 +1121,7 @@ int ts_mixed_step_host(ts_ctx* c, const ts_step* st, void* cuda_stream) {
     dev.v_new = (char*)dv + t * tk;
     dev.out = (char*)dout + t * tq;
     TS_CUDA(c, cudaStreamWaitEvent(stream, c->up_done[b][i], 0));
-    const int rc = enqueue_step(c, &dev, (int64_t)len, piece_prefill, stream, true);
+    const int rc = enqueue_step(c, &dev, (int64_t)len, piece_prefill, split, stream, true);
     if (rc != TS_OK) {
       cudaStreamSynchronize(c->up_stream);  // the input copies may still be reading the caller's buffers
       return rc;
@@ -1275,7 +1298,7 @@ int ts_plan_step(ts_ctx* c, const ts_step* st, int32_t* items, int32_t items_cap
   if (rc != TS_OK) return rc;
   if (c->cfg.chunk_size > 0 && n_prefill + n_decode > c->cfg.chunk_size) return TS_ERR_BUDGET;
   if (n_tokens > c->L.max_tokens) return TS_ERR_BUDGET;
-  plan(c, st);
+  plan(c, st, decode_split(c, st));
   *n_items_out = (int32_t)c->items.size();
   if (items) {
     if (items_capacity < (int32_t)c->items.size()) return TS_ERR_INVALID;

@@ -312,17 +312,22 @@ def test_metadata_inside_and_outside_the_launch_parameters(rows, shape):
     assert np.array_equal(lb.pool(), pool)
 
 
-@pytest.mark.parametrize("ctx,ql", [([300] * 8 + [0], [1] * 8 + [2048]), ([77, 40, 900], [1100, 1, 947]), ([0, 5, 6], [1536, 1, 1])],
-                         ids=["burst", "two-chunks", "chunk-first"])
+@pytest.mark.parametrize("ctx,ql", [([300] * 8 + [0], [1] * 8 + [2048]), ([77, 40, 900], [1100, 1, 947]), ([0, 5, 6], [1536, 1, 1]),
+                                    ([2000] * 4 + [0] + [4000] * 60, [1] * 4 + [2048] + [1] * 60),
+                                    ([4200] * 60 + [20] * 1100 + [0], [1] * 1160 + [2048])],
+                         ids=["burst", "two-chunks", "chunk-first", "long-rows-around-a-chunk", "a-third-of-rows"])
 def test_host_step_in_pieces_equals_the_device_step(ctx, ql):
     """A waiting host-buffer step that is large enough to go in pieces: result, pages, lengths and
-    counters are those of the same step on device buffers, bit for bit (a cut falls between work items)."""
+    counters are those of the same step on device buffers, bit for bit (a cut falls between work items,
+    rows are split as the whole step would split them, and merged by the same kernel)."""
     b = wl.make_batch("pieces", wl.LLAMA8B, ctx, ql, seed=len(ctx), profile="peaked", chunk_size=sum(ql))
     one, two = LoadedBatch(b), LoadedBatch(b)
     one.step()
     host = [torch.from_numpy(a.view(np.int16)).pin_memory() for a in (b.q, b.k_new, b.v_new)]
     out = torch.full(host[0].shape, 0x7FC0, dtype=torch.int16).pin_memory()
     two.dec.mixed_step_host(two.slots, b.q_len.tolist(), b.ctx_len.tolist(), *host, out)
+    # both loaded their context with the same launches, so more of them are more pieces
+    assert two.dec.velocity()["kernel_launches"] > one.dec.velocity()["kernel_launches"], "it went in one piece"
     assert np.array_equal(wl.bf16_bits_to_f32(out.numpy().view(np.uint16)), one.output())
     assert np.array_equal(two.pool(), one.pool())
     assert one.dec.device_status() == 0 and two.dec.device_status() == 0
