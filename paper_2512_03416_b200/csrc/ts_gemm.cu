@@ -57,6 +57,15 @@ __device__ __forceinline__ void prefetch_weights(const GemmArgs& g, int row, int
 // bf16 x bf16 -> fp32, M = 128, N = 256, both operands K-major
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
 
+// After a time-out a role starts nothing any more, but the copies and MMAs of the last K blocks may still be
+// under way. They are done within microseconds; the thread that calls this gives them a millisecond before
+// its CTA leaves and gives shared memory and TMEM back.
+__device__ __forceinline__ void settle(bool failed) {
+  if (!failed) return;
+  const long long t0 = clock64();
+  while (clock64() - t0 < 2000000) {}
+}
+
 __device__ __forceinline__ uint4 pack8(const float* v) {
   uint4 w;
   w.x = pack_bf16(v[0], v[1]);
@@ -310,6 +319,7 @@ gemm_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, const _
       });
     }
   }
+  settle(misc[1] != 0);
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, 512);
@@ -474,6 +484,7 @@ gemm_pair_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, co
       });
     }
   }
+  settle(misc[1] != 0);
   tc_fence_before();
   __syncwarp();
   cluster_sync();                  // no CTA leaves while the other one's copies, commits or arrivals may still reach it
@@ -597,6 +608,7 @@ gemm_split_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, c
       }
     }
   }
+  settle(misc[1] != 0);
   __syncwarp();
   cluster_sync();                  // the images are complete
   pdl_wait();                      // every thread reads the residual or the positions below
