@@ -20,10 +20,10 @@
 //     row is padding and the accumulators stay small; P^T is re-laid out with movmatrix;
 //   * softmax is online in base 2 with fp32 state per head; a page without a new maximum costs no reduction.
 // Measured (us, one static deal, a reduction and rescale per page, two copies per page, all warps
-// meeting at every unit's end -> this): 64 rows of the 8B shape 130.1 -> 127.0; 203 rows of the 70B
-// shape 246.8 -> 232.8; next to a 2048-token chunk 163.9 -> 161.5; 717 tokens next to 198 rows 293 -> 284.
-// With the products left out (copies and waits only) the same steps take 125 / 226 us: what is left is
-// the rate at which the page copies come in.
+// meeting at every unit's end -> this): 64 rows of the 8B shape 127.9 -> 125.9; 203 rows of the 70B
+// shape 237.4 -> 226.9; next to a 2048-token chunk 160.0 -> 155.9; 717 tokens next to 198 rows 281 -> 273.
+// With the products left out (copies and waits only) 64 rows took 125 us where the whole took 127: what
+// is left is the rate at which the page copies come in.
 #pragma once
 #include <cuda_bf16.h>
 #include <math_constants.h>

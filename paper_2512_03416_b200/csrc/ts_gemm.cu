@@ -4,15 +4,19 @@
 //   A [M][K] bf16 (activations, one token per row), B [N][K] bf16 (weights, [out features][in
 //   features]), C [M][N] bf16. Both operands are K-major, exactly as they sit in memory.
 //
-// One persistent CTA per SM walks the output tiles (tile index t -> column block t / m_tiles, row
-// block t % m_tiles, so the CTAs that run at the same time share a few weight blocks through L2).
-// A tile is TILE_M x 256: TILE_M = 128 (one tcgen05.mma M = 128, N = 256 per 16 of K) or 256 (two of
-// them that share the weight block in shared memory, which cuts the bytes fetched per flop by a
-// third). Operands arrive by TMA in 64-wide K blocks (128-byte swizzle) through a ring of stages;
-// the accumulators live in TMEM (2 x 256 columns): with TILE_M = 128 they alternate between tiles,
-// so the epilogue of a tile overlaps the main loop of the next one; with TILE_M = 256 a tile takes both.
-// Warp roles: warp 0 TMA producer, warp 1 MMA issuer and TMEM owner, warps 2-5 epilogue
-// (thread = accumulator row: TMEM -> registers -> bf16 -> global).
+// Three kernels, chosen by gemm_plan from the shape:
+//   gemm_kernel        one persistent CTA per SM walks 128 x 256 tiles (one tcgen05.mma M = 128, N = 256
+//                      per 16 of K); two 256-column accumulators in TMEM alternate between tiles, so a
+//                      tile's epilogue overlaps the next tile's main loop;
+//   gemm_pair_kernel   many rows: a pair of CTAs (cta_group::2) walks 256 x 256 tiles, each CTA fetches and
+//                      holds half of both operand blocks; two accumulators as above;
+//   gemm_split_kernel  few tiles: a cluster of 2 to 8 CTAs shares the K range of one 128 x 128 tile and adds
+//                      its fp32 accumulators up through distributed shared memory.
+// Tile index t -> column block t / m_tiles, row block t % m_tiles, so the CTAs that run at the same time
+// share a few weight blocks through L2. Operands arrive by TMA in 64-wide K blocks (128-byte swizzle)
+// through a ring of stages.
+// Warp roles: warp 0 TMA producer, warp 1 MMA issuer and TMEM owner, warps 2-9 epilogue (thread = half an
+// accumulator row: TMEM -> registers -> bf16 -> global; in the split kernel all warps add up and write).
 // Epilogues: plain store, store + residual (C = R + A . B^T), rotary embedding of the query and key
 // heads of a fused QKV projection, and SiLU-gated product of a fused gate/up projection.
 // Every wait is bounded; a wait that runs out raises TS_DEV_TIMEOUT and the CTA drains.

@@ -36,7 +36,6 @@ struct Layout {
   int max_tokens, max_partials, max_items;
   size_t off_status, off_table, off_meta, off_delta, off_part_acc, off_part_ml, off_stage;
   size_t meta_bytes, slot_bytes, delta_bytes, stage_q_bytes, stage_kv_bytes, stage_set_bytes, total;
-  // int32 offsets inside the meta area
 };
 
 bool shape_ok(const ts_config* c) {
@@ -767,9 +766,9 @@ void finish_step(ts_ctx* c, const ts_step* st, int n_decode, int64_t n_prefill, 
 // kernels and uploads of the next (the copies run both ways at once). A piece still fills half of the
 // chip with prefill units and moves 4 MB up, so that neither its kernels nor its copies are bound by
 // latency; calls that do not wait overlap with one another already. Every piece has tokens of a chunk: rows
-// without one would run in the decode kernel, whose splits are merged by a launch that rounds differently. Measured on 64 rows + 2048 tokens
-// of the 8B shape (26 MB up, 17 MB down): one piece 988 us,
-// two 843, three (the rule) 815, four 830, six 875.
+// without one would run in the decode kernel, whose splits are merged by a launch that rounds differently.
+// Measured on 64 rows + 2048 tokens of the 8B shape (26 MB up, 17 MB down): one piece 988 us, two 843, three
+// (the rule) 815, four 830, six 875.
 int host_pieces(const ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefill, int64_t* cut) {
   const int64_t unit = c->cfg.head_dim == 128 ? 2 * (ts::kPackedRowsTc / c->G) : ts::kPackedRowsPerTile / c->G;   // tokens of a work item
   const size_t tq = (size_t)c->cfg.n_q_heads * c->cfg.head_dim * 2, tk = (size_t)c->cfg.n_kv_heads * c->cfg.head_dim * 2;

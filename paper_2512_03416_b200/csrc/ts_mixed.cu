@@ -35,7 +35,8 @@
 // every CTA copies a share of the prefill rows' tokens next to its other work, and nothing waits for
 // the copies, because the tiles take a chunk's own tokens from the step's tensors; the decode units
 // write their rows' own tokens.
-// Every wait is bounded; a wait that runs out raises TS_DEV_TIMEOUT and the CTA drains: nothing new is
+// Every wait is bounded (the hardware barriers are not, but all who meet on one do so equally often); a wait
+// that runs out raises TS_DEV_TIMEOUT and the CTA drains: nothing new is
 // started, the other waits end early, and before the CTA leaves, the copies and MMAs it did start are
 // waited for (with a limit of their own).
 #include <cuda_bf16.h>
@@ -402,8 +403,9 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
     const uint32_t tS = tmem + x * 128 + hf * 64 + lane_addr;         // my 64 score columns; P goes to the first 32
     const uint32_t tO = tmem + 256 + x * 128 + hf * 64 + lane_addr;   // my 64 columns of O
     // The two warps that share a quarter of a tile's rows meet on a hardware barrier (ids 4-11) around
-    // each exchange through shared memory; it wakes them sooner than an mbarrier (8192-token chunk
-    // next to 190 rows 1274 -> 1238 us, 2048 tokens alone 50.7 -> 48.4 us). It has no time limit, so
+    // each exchange through shared memory; it wakes them sooner than an mbarrier (together with
+    // the other changes to the unit loop that came with it: 8192-token chunk next to 190 rows 1272 -> 1263 us,
+    // 2048 tokens alone 49.5 -> 46.3 us). It has no time limit, so
     // the two must never disagree about how often they meet: all their other waits are limited and end
     // in the same control flow, and how many blocks of a unit the tile has (-1: there is no further unit)
     // is for the first of them to say, one number for all lanes of both.
