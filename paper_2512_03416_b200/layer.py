@@ -55,7 +55,7 @@ class DecoderLayer:
 
     def step_prepared(self, st, x_in, x_out) -> None:
         _check(B.ts_layer_step(self.handle, st, x_in.data_ptr(), x_out.data_ptr(),
-                               torch.cuda.current_stream(self.dec.device).cuda_stream), "ts_layer_step")
+                               self.dec._stream()), "ts_layer_step")
 
     def step(self, slots, q_len, ctx_len, x_in, x_out, keep_len: bool = False) -> None:
         st, _keep = self.make_step(slots, q_len, ctx_len, keep_len)
