@@ -500,7 +500,7 @@ int ts_layer_last_cuda_error(const ts_layer* layer);
  * ts_gemm_bf16: the layer's projection kernel by itself (for measurements and tests):
  * C[M][N] = (R ? R : 0) + A[M][K] . B[N][K]^T, all DEVICE bf16 row-major and 16-byte aligned, fp32
  * accumulation, bf16 result. N and K multiples of 8. tile_m: 128 = tiles of 128 x 256, one thread block
- * each; 256 = tiles of 256 x 256, a pair of thread blocks each; 0 = chosen from the shape (clusters that
+ * each; 256 = tiles of up to 256 rows of A x 256 of B, a pair of thread blocks each; 0 = chosen from the shape (clusters that
  * split K included), as ts_layer_step does. device_status: DEVICE int32 the caller has zeroed;
  * a bounded wait that runs out sets TS_DEV_TIMEOUT there. Asynchronous on cuda_stream.
  */

@@ -8,8 +8,8 @@
 //   gemm_kernel        one persistent CTA per SM walks 128 x 256 tiles (one tcgen05.mma M = 128, N = 256
 //                      per 16 of K); two 256-column accumulators in TMEM alternate between tiles, so a
 //                      tile's epilogue overlaps the next tile's main loop;
-//   gemm_pair_kernel   many rows: a pair of CTAs (cta_group::2) walks 256 x 256 tiles, each CTA fetches and
-//                      holds half of both operand blocks; two accumulators as above;
+//   gemm_pair_kernel   many rows: a pair of CTAs (cta_group::2) walks tiles of 256 features x 16 to 256 tokens,
+//                      each CTA fetches and holds half of both operand blocks; two accumulators as above;
 //   gemm_split_kernel  few tiles: a cluster of 2 to 8 CTAs shares the K range of one 128 x 128 tile and adds
 //                      its fp32 accumulators up through distributed shared memory.
 // Tile index t -> column block t / m_tiles, row block t % m_tiles, so the CTAs that run at the same time
@@ -107,13 +107,14 @@ __device__ __forceinline__ void rope8(const GemmArgs& g, int row, int col0, int 
   *reinterpret_cast<uint4*>(dst + c) = pack8(lo);
   *reinterpret_cast<uint4*>(dst + 64 + c) = pack8(hi);
 }
-// gate <- silu(gate) * up, both rounded to bf16 first (they are bf16 tensors of the layer's definition)
+// silu(gate) * up, both rounded to bf16 first (they are bf16 tensors of the layer's definition)
+__device__ __forceinline__ float silu_mul(float gate, float up) {
+  const float a = __bfloat162float(__float2bfloat16_rn(gate)), b = __bfloat162float(__float2bfloat16_rn(up));
+  return a / (1.f + __expf(-a)) * b;
+}
 __device__ __forceinline__ void silu_mul8(float* gate, const float* up) {
 #pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    const float a = __bfloat162float(__float2bfloat16_rn(gate[e])), b = __bfloat162float(__float2bfloat16_rn(up[e]));
-    gate[e] = a / (1.f + __expf(-a)) * b;
-  }
+  for (int e = 0; e < 8; ++e) gate[e] = silu_mul(gate[e], up[e]);
 }
 
 // Epilogue of one accumulator (TMEM lanes = 128 rows, 256 columns): half `hf` of this thread's row of
@@ -330,13 +331,18 @@ gemm_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, const _
 }
 
 // ------------------------------------------------------------------------------------ pair kernel
-// For products with many rows. Two CTAs of a cluster share a 256 x 256 tile (cta_group::2): CTA r
-// fetches rows [128 r, 128 r + 128) of both operand blocks and holds that half of the accumulator's
-// rows; one MMA of M = 256, N = 256 reads the B halves of both CTAs. Per CTA and 64 of K that is 32 KB
-// fetched and 32 KB read for 512 cycles of tensor work, where a CTA on its own moves 48 KB + 48 KB
-// for a 128 x 256 tile (shared memory gives 128 bytes per clock: its limit, not the tensor pipe's).
+// For products with many rows. Two CTAs of a cluster share a tile of 256 features x `nt` tokens
+// (cta_group::2), computed transposed: the weights are the MMA's M (always 256), the tokens its N, which may be
+// any multiple of 16 up to 256, so that the tokens divide into tiles of nearly equal size and little is
+// computed for padding. (With the tokens as M = 256, 2112 of them took nine tiles of 256: 8 % padding, and 300
+// took 512.) CTA r fetches 128 weight rows and nt / 2 token rows per 64 of K and holds the accumulator of its
+// weight rows: TMEM lane = feature, column = token. One MMA reads the token halves of both CTAs. Per CTA and
+// 64 of K that is at most 32 KB fetched and 32 KB read for 512 cycles of tensor work, where a CTA on its own moves
+// 48 KB + 48 KB for a 128 x 256 tile (shared memory gives 128 bytes per clock: its limit, not the tensor pipe's).
 // CTA 0 issues all MMAs. Every CTA's copies complete CTA 0's "full" barrier; the commits arrive at
 // both CTAs' "empty" and "accumulator full" barriers; both epilogues release the accumulator to CTA 0.
+// Features that the epilogue brings together (the two of a rotary pair, 64 apart; a gate and its up
+// feature, 128 apart) sit sixteen lanes apart: the weights' tensor map has those rows as a dimension of its own.
 __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
@@ -350,6 +356,13 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
   asm volatile(
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_5d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3, int c4) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%3, %4, %5, %6, %7}], [%2];\n" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
       : "memory");
 }
 __device__ __forceinline__ void mma_ss_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate, uint32_t issue) {
@@ -374,11 +387,90 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
 constexpr int kPairStages = 6, kPairStageBytes = 2 * kABytes;
 constexpr int kPairBars = 2 * kPairStages + 4;
 constexpr int kPairSmem = kPairStages * kPairStageBytes + kPairBars * 8 + 16 + 1024;
-constexpr uint32_t kIdescPair = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3) << 17) | ((256u >> 4) << 24);
+constexpr uint32_t kIdescPair = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 4) << 24);   // M = 256; N is added
+
+// 32 tokens (t0 .. t0 + 31, those below `end`) of this lane's feature of a 128-feature accumulator: quarter q of
+// the features, feature n0 + q * 32 + lane of the product (STORE) or the order of the permuted weight rows.
+// Neighbouring lanes swap values first, so that a lane writes two features of one token: 64 bytes
+// (STORE) or 32 bytes (the others) of a token's row together.
+template <int EPI>
+__device__ __forceinline__ void epilogue_tokens(const GemmArgs& g, float (&v)[32], int t0, int end, int n0, int q, int lane) {
+  const bool odd = lane & 1, upper = lane & 16;
+  auto swap_pair = [&](float mine_even, float mine_odd, float& lo, float& hi) {   // even lanes keep the first token, odd ones the second
+    const float got = __shfl_xor_sync(0xffffffffu, odd ? mine_even : mine_odd, 1);
+    lo = odd ? got : mine_even;
+    hi = odd ? mine_odd : got;
+  };
+  if (EPI == GEMM_EPI_STORE) {
+    const int col = n0 + q * 32 + (lane & ~1);
+    if (n0 + q * 32 >= g.N) return;                        // N is a multiple of 8: checked per lane below
+    uint32_t r[16];
+    if (g.R) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int t = t0 + 2 * i + odd;
+        r[i] = t < end && col < g.N ? *reinterpret_cast<const uint32_t*>(g.R + (size_t)t * g.ldc + col) : 0u;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      float lo, hi;
+      swap_pair(v[2 * i], v[2 * i + 1], lo, hi);
+      const int t = t0 + 2 * i + odd;
+      if (g.R) {
+        lo += __uint_as_float(r[i] << 16);
+        hi += __uint_as_float(r[i] & 0xFFFF0000u);
+      }
+      if (t < end && col < g.N) *reinterpret_cast<uint32_t*>(g.C + (size_t)t * g.ldc + col) = pack_bf16(lo, hi);
+    }
+  } else if (EPI == GEMM_EPI_ROPE) {
+    // lanes 0-15: features 16 q + lane of the head, lanes 16-31: their partners 64 further on
+    if (n0 >= g.N) return;
+    const bool rotate = n0 < g.q_cols + g.kv_cols;
+    uint16_t* dst = n0 < g.q_cols ? g.C + n0 : rotate ? g.C2 + (n0 - g.q_cols) : g.C3 + (n0 - g.q_cols - g.kv_cols);
+    const int ld = n0 < g.q_cols ? g.q_cols : g.kv_cols, f = q * 16 + (lane & 15);
+    if (rotate) {
+      const int pos = t0 + lane < end ? g.pos[t0 + lane] : 0;
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const float2 cs = g.rope_table[(size_t)__shfl_sync(0xffffffffu, pos, i) * 64 + f];   // (cos, sin)
+        const float other = __shfl_xor_sync(0xffffffffu, v[i], 16);
+        const float a = upper ? other : v[i], b = upper ? v[i] : other;
+        v[i] = upper ? b * cs.x + a * cs.y : a * cs.x - b * cs.y;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      float lo, hi;
+      swap_pair(v[2 * i], v[2 * i + 1], lo, hi);
+      const int t = t0 + 2 * i + odd;
+      if (t < end) *reinterpret_cast<uint32_t*>(dst + (size_t)t * ld + (upper ? 64 : 0) + (f & ~1)) = pack_bf16(lo, hi);
+    }
+  } else {
+    // lanes 0-15: gate features, lanes 16-31: the up features that belong to them. Of two tokens the lower lanes
+    // take the first, the upper ones the second. out[token][n0 / 2 + i] = silu(gate_i) * up_i.
+    if (n0 >= g.N) return;
+    uint16_t* dst = g.C + n0 / 2 + q * 16 + (lane & 14);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {                          // four tokens at a time
+      float h[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float first = v[4 * i + 2 * e], second = v[4 * i + 2 * e + 1];
+        const float got = __shfl_xor_sync(0xffffffffu, upper ? first : second, 16);
+        h[e] = silu_mul(upper ? got : first, upper ? second : got);
+      }
+      float lo, hi;
+      swap_pair(h[0], h[1], lo, hi);
+      const int t = t0 + 4 * i + (odd ? 2 : 0) + (upper ? 1 : 0);
+      if (t < end) *reinterpret_cast<uint32_t*>(dst + (size_t)t * g.ldc) = pack_bf16(lo, hi);
+    }
+  }
+}
 
 template <int EPI>
 __global__ void __launch_bounds__(kGemmThreads, 1)
-gemm_pair_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, const __grid_constant__ CUtensorMap b_map) {
+gemm_pair_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap w_map, const int nt) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
@@ -414,26 +506,32 @@ gemm_pair_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, co
   auto wait = [&](int i, uint32_t parity) {
     if (!mbar_wait(bar(i), parity, misc[1] ? 2000 : g.wait_cycles)) give_up();
   };
-  const int m_tiles = (g.M + 255) / 256, n_tiles = (g.N + kBN - 1) / kBN;
+  const int m_tiles = (g.M + nt - 1) / nt, n_tiles = (g.N + kBN - 1) / kBN;
   const int n_work = m_tiles * n_tiles, first = blockIdx.x >> 1, stride = gridDim.x >> 1;
   const int k_blocks = (g.K + kBK - 1) / kBK;
 
   if (warp == 0) {
     if (lane == 0) {
-      tma_prefetch_desc(&a_map);
-      tma_prefetch_desc(&b_map);
+      tma_prefetch_desc(&x_map);
+      tma_prefetch_desc(&w_map);
       pdl_wait();
+      const uint32_t bytes = 2u * (kABytes + (uint32_t)nt * (kBK * 2 / 2));
       int it = 0;
       for (int t = first; t < n_work; t += stride) {
-        const int m0 = (t % m_tiles) * 256 + (int)rank * 128, n0 = (t / m_tiles) * kBN + (int)rank * 128;
+        const int m0 = (t % m_tiles) * nt + (int)rank * (nt / 2), nb = t / m_tiles;
         for (int kb = 0; kb < k_blocks; ++kb, ++it) {
           const int st = it % kPairStages;
           if (it >= kPairStages) wait(BAR_EMPTY + st, ((it / kPairStages) & 1) ^ 1);
           if (misc[1]) continue;                           // after a failure no new copies are started
           const uint32_t dst = base + st * kPairStageBytes, full = mapa(bar(BAR_FULL + st), 0);
-          if (rank == 0) mbar_expect_tx(bar(BAR_FULL + st), 2 * kPairStageBytes);
-          tma_load_2d_pair(dst, &a_map, full, kb * kBK, m0);
-          tma_load_2d_pair(dst + kABytes, &b_map, full, kb * kBK, n0);
+          if (rank == 0) mbar_expect_tx(bar(BAR_FULL + st), bytes);
+          if (EPI == GEMM_EPI_STORE)
+            tma_load_2d_pair(dst, &w_map, full, kb * kBK, nb * kBN + (int)rank * 128);
+          else if (EPI == GEMM_EPI_ROPE)                   // sixteen rows, half of a head, quarter of its half, head
+            tma_load_5d_pair(dst, &w_map, full, kb * kBK, 0, 0, 0, nb * 2 + (int)rank);
+          else                                             // sixteen rows, gate | up, sixteenth of the block, block of 256 rows
+            tma_load_5d_pair(dst, &w_map, full, kb * kBK, 0, 0, (int)rank * 4, nb);
+          tma_load_2d_pair(dst + kABytes, &x_map, full, kb * kBK, m0);
         }
       }
       // the commits that free the last stages arrive here too: they must have before this CTA may leave
@@ -449,6 +547,7 @@ gemm_pair_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, co
           give_up();
         }
       };
+      const uint32_t idesc = kIdescPair | ((uint32_t)(nt >> 3) << 17);
       int it = 0, n_done = 0;
       for (int t = first; t < n_work; t += stride, ++n_done) {
         const int buf = n_done & 1, uses = n_done >> 1;
@@ -463,7 +562,7 @@ gemm_pair_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, co
             const uint64_t b_desc = smem_desc(base + st * kPairStageBytes + kABytes, 0, 1024);
 #pragma unroll
             for (int ks = 0; ks < kBK / 16; ++ks)
-              mma_ss_pair(tmem + buf * 256, a_desc + (uint64_t)(ks * 2), b_desc + (uint64_t)(ks * 2), kIdescPair,
+              mma_ss_pair(tmem + buf * 256, a_desc + (uint64_t)(ks * 2), b_desc + (uint64_t)(ks * 2), idesc,
                           (kb > 0 || ks > 0) ? 1u : 0u, issue);
             tc_commit_pair(bar(BAR_EMPTY + st), issue);
           }
@@ -477,15 +576,28 @@ gemm_pair_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, co
     const int q = warp & 3, hf = (warp - 2) >> 2;
     int n_done = 0;
     for (int t = first; t < n_work; t += stride, ++n_done) {
-      const int m0 = (t % m_tiles) * 256 + (int)rank * 128, n0 = (t / m_tiles) * kBN;
+      const int m0 = (t % m_tiles) * nt, end = min(g.M, m0 + nt);
+      // first feature of this CTA's half of the tile; SILU_MUL: gate and up features of half a block
+      const int n0 = (t / m_tiles) * kBN + (int)rank * 128;
       const int buf = n_done & 1;
       wait(BAR_ACC_FULL + buf, (n_done >> 1) & 1);
       tc_fence_after();
-      epilogue_row<EPI>(g, tmem + buf * 256 + ((uint32_t)(q * 32) << 16), m0 + q * 32 + lane, n0, hf, [&]() {
-        tc_fence_before();
+      const int chunks = (nt + 31) / 32, last = ((chunks - 1 - hf) & ~1) + hf;   // this warp: chunks hf, hf + 2, ...
+      for (int c = hf; c < chunks; c += 2) {
+        float v[32];
+        tmem_ld32(v, tmem + buf * 256 + ((uint32_t)(q * 32) << 16) + c * 32);
+        tmem_ld_wait();
+        if (c == last) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(mapa(bar(BAR_ACC_EMPTY + buf), 0));
+        }
+        if (m0 + c * 32 < end) epilogue_tokens<EPI>(g, v, m0 + c * 32, end, n0, q, lane);
+      }
+      if (hf >= chunks) {                                  // a narrow tile: nothing for this warp
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(mapa(bar(BAR_ACC_EMPTY + buf), 0));
-      });
+      }
     }
   }
   settle(misc[1] != 0);
@@ -731,34 +843,35 @@ cudaError_t launch_tile_t(const GemmArgs& g, const CUtensorMap& a_map, const CUt
 }
 
 template <int EPI>
-cudaError_t launch_pair_t(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, int n_sms, cudaStream_t stream) {
+cudaError_t launch_pair_t(const GemmArgs& g, const CUtensorMap& x_map, const CUtensorMap& w_map, int nt, int n_sms, cudaStream_t stream) {
   cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
   if (e != cudaSuccess) return e;
-  const int tiles = ((g.M + 255) / 256) * ((g.N + kBN - 1) / kBN);
-  return launch_cluster(gemm_pair_kernel<EPI>, 2 * std::min(n_sms / 2, tiles), 2, kPairSmem, stream, g, a_map, b_map);
+  const int tiles = ((g.M + nt - 1) / nt) * ((g.N + kBN - 1) / kBN);
+  return launch_cluster(gemm_pair_kernel<EPI>, 2 * std::min(n_sms / 2, tiles), 2, kPairSmem, stream, g, x_map, w_map, nt);
 }
 
 template <int EPI>
-cudaError_t launch_epi(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, GemmPlan plan, int n_sms,
-                       cudaStream_t stream) {
+cudaError_t launch_epi(const GemmArgs& g, const GemmMaps& maps, GemmPlan plan, int n_sms, cudaStream_t stream) {
   if constexpr (EPI != GEMM_EPI_SILU_MUL)                // a gate and its up column are 128 columns apart: no tile of 128 holds both
-    if (plan.split > 0) return launch_split_t<EPI>(g, a_map, b_map, plan.split, stream);
-  if (plan.tile_m == 256) return launch_pair_t<EPI>(g, a_map, b_map, n_sms, stream);
-  return launch_tile_t<EPI>(g, a_map, b_map, n_sms, stream);
+    if (plan.split > 0) return launch_split_t<EPI>(g, *maps.x, *maps.w, plan.split, stream);
+  if (plan.tile_m == 256) return launch_pair_t<EPI>(g, *maps.x_pair, *maps.w_pair, plan.pair_tokens, n_sms, stream);
+  return launch_tile_t<EPI>(g, *maps.x, *maps.w, n_sms, stream);
 }
 
 }  // namespace
 
 // Cost of a launch in us besides what every launch pays: waves x K blocks x the time of a K block, which
-// is what the tensor pipe and shared memory take (0.37 us for a CTA's 128 x 256 tile, 0.30 us for a
-// pair's 256 x 256 tile, 0.33 us for a 128 x 128 tile) or what HBM needs for the weight blocks in flight
+// is what the tensor pipe and shared memory take (0.45 us for a CTA's 128 x 256 tile, 0.2 us + 0.65 ns per token
+// for a pair's tile, 0.33 us for a 128 x 128 tile), what an SM needs to get a pair's weights from HBM (0.285 us), or
+// what HBM needs for the weight blocks in flight
 // at that moment; for the split kernel also the merge, and only where all clusters run at once.
-// Measured (8B-shaped projections, weights not in L2, us; 128 x 256 tile / pair / split kernel): 64 rows
-// QKV 30.4 / 26.8 / 15.3, output 29.7 / 26.3 / 11.6, down 88.8 / 71.8 / 25.5; 256 rows output 32.0 /
-// 29.1 / 17.3, down 90.9 / 75.0 / 40.3; 1024 rows (tile / pair) QKV 58.6 / 50.9, gate/up 212 / 180, down
-// 106 / 90; 2112 rows 89.3 / 82.5, output 60.5 / 56.1, gate/up 390 / 360, down 199 / 181.
+// Measured (8B-shaped projections, weights not in L2, us; 128 x 256 tile / pair with tiles of 256 tokens, as it
+// was / pair / split kernel): 64 rows QKV 29.4 / 25.9 / 22.3 / 15.2, output 27.5 / 24.7 / 22.0 / 11.9, gate/up 43.1 /
+// 51.6 / 47.8, down 86.2 / 70.4 / 64.1 / 25.4; 256 rows output 28.6 / 25.9 / 23.0 / 16.0, down 87.6 / 72.2 / 67.7 /
+// 38.2; gate/up with 130 rows 61.3 / 55.0 / 50.3, 297 88.0 / 93.1 / 79.8, 514 119 / 124 / 107, 800 169 / 167 / 150, 2112
+// 393 / 346 / 319; 2112 rows QKV 106 / 81.5 / 82.8, output 63.8 / 54.7 / 55.2, down 223 / 187 / 178.
 GemmPlan gemm_plan(const GemmArgs& g, int n_sms) {
-  constexpr double kTileUs = 0.37, kPairUs = 0.30, kSplitUs = 0.33, kHbmBytesPerUs = 6.2e6;
+  constexpr double kTileUs = 0.45, kPairUs = 0.2, kPairTokenUs = 0.00065, kPairMinUs = 0.285, kSplitUs = 0.33, kHbmBytesPerUs = 6.2e6;
   const double merge_us = 2.5 + 0.03 * std::min(g.M, 128);
   const int n_tiles = (g.N + kBN - 1) / kBN, m128 = (g.M + 127) / 128, m256 = (g.M + 255) / 256;
   const int kb = (g.K + kBK - 1) / kBK;
@@ -767,12 +880,16 @@ GemmPlan gemm_plan(const GemmArgs& g, int n_sms) {
     const double hbm = (double)std::min(tiles, workers) / m_tiles * width * kBK * 2 / kHbmBytesPerUs;
     return (double)((tiles + workers - 1) / workers) * blocks * std::max(us, hbm);
   };
-  GemmPlan best = {128, 0};
+  GemmPlan best = {128, 0, 0};
   double cost = cost_of(kTileUs, m128 * n_tiles, n_sms, m128, kBN, kb);
-  const double pair_cost = cost_of(kPairUs, m256 * n_tiles, n_sms / 2, m256, kBN, kb);
-  if (pair_cost < cost) {
-    cost = pair_cost;
-    best = {256, 0};
+  // tokens of a pair's tile: as many tiles as need be, or a few more where they fill the pairs' last wave better
+  for (int m = m256; m <= m256 + 3; ++m) {
+    const int nt = pair_tokens(g.M, m), tiles = (g.M + nt - 1) / nt;
+    const double c = cost_of(std::max(kPairUs + kPairTokenUs * nt, kPairMinUs), tiles * n_tiles, n_sms / 2, tiles, kBN, kb);
+    if (c < cost) {
+      cost = c;
+      best = {256, 0, nt};
+    }
   }
   const int split_tiles = m128 * ((g.N + kSplitN - 1) / kSplitN);
   for (int s = 2; s <= std::min(kMaxSplit, kb) && g.epi != GEMM_EPI_SILU_MUL; ++s) {
@@ -780,19 +897,18 @@ GemmPlan gemm_plan(const GemmArgs& g, int n_sms) {
     const double c = cost_of(kSplitUs, split_tiles * s, split_tiles * s, m128, kSplitN, (kb + s - 1) / s) + merge_us;
     if (c < cost * 0.98) {
       cost = c;
-      best = {128, s};
+      best = {128, s, 0};
     }
   }
   return best;
 }
 
-cudaError_t launch_gemm(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, GemmPlan plan, int n_sms,
-                        cudaStream_t stream) {
+cudaError_t launch_gemm(const GemmArgs& g, const GemmMaps& maps, GemmPlan plan, int n_sms, cudaStream_t stream) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
   switch (g.epi) {
-    case GEMM_EPI_ROPE: return launch_epi<GEMM_EPI_ROPE>(g, a_map, b_map, plan, n_sms, stream);
-    case GEMM_EPI_SILU_MUL: return launch_epi<GEMM_EPI_SILU_MUL>(g, a_map, b_map, plan, n_sms, stream);
-    default: return launch_epi<GEMM_EPI_STORE>(g, a_map, b_map, plan, n_sms, stream);
+    case GEMM_EPI_ROPE: return launch_epi<GEMM_EPI_ROPE>(g, maps, plan, n_sms, stream);
+    case GEMM_EPI_SILU_MUL: return launch_epi<GEMM_EPI_SILU_MUL>(g, maps, plan, n_sms, stream);
+    default: return launch_epi<GEMM_EPI_STORE>(g, maps, plan, n_sms, stream);
   }
 }
 

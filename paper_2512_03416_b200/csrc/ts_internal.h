@@ -154,16 +154,22 @@ struct CtxView {
 };
 int ctx_view(ts_ctx* c, cudaStream_t stream, CtxView* out);
 // How a product is laid over the chip. split = 0: 128 x 256 tiles, one CTA each, or (tile_m = 256)
-// 256 x 256 tiles, a pair of CTAs each; split > 0: 128 x 128 tiles whose K range a cluster of `split`
-// CTAs shares.
+// tiles of pair_tokens tokens x 256 features, a pair of CTAs each; split > 0: 128 x 128 tiles whose K range a
+// cluster of `split` CTAs shares.
 struct GemmPlan {
-  int tile_m, split;
+  int tile_m, split, pair_tokens;
 };
+// Smallest number of tokens, a multiple of 16, with which `tiles` tiles hold M tokens.
+inline int pair_tokens(int M, int tiles) { return ((M + tiles - 1) / tiles + 15) / 16 * 16; }
 // The plan for a product (M, N, K and epi are read). The device is the current one.
 GemmPlan gemm_plan(const GemmArgs& g, int n_sms);
-// Both maps view an operand as (K, row), box 64 x 128.
-cudaError_t launch_gemm(const GemmArgs& g, const CUtensorMap& a_map, const CUtensorMap& b_map, GemmPlan plan, int n_sms,
-                        cudaStream_t stream);
+// Views of the operands as (K, row). x, w: boxes of 64 x 128. The pair kernel's: x_pair, a box of 64 x
+// pair_tokens / 2; w_pair, for STORE the same as w, else boxes of 64 x 128 whose rows come in the order the epilogue
+// pairs them in (make_paired_map). Those that the plan does not use may be null.
+struct GemmMaps {
+  const CUtensorMap *x, *x_pair, *w, *w_pair;
+};
+cudaError_t launch_gemm(const GemmArgs& g, const GemmMaps& maps, GemmPlan plan, int n_sms, cudaStream_t stream);
 // out[row] = x[row] / sqrt(mean(x[row]^2) + eps) * gain, bf16 in and out, fp32 inside; width % 8 == 0
 cudaError_t launch_rmsnorm(const uint16_t* x, const uint16_t* gain, uint16_t* out, int rows, int width, float eps,
                            cudaStream_t stream);

@@ -20,15 +20,38 @@ typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void
                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// 2-D view of a K-major bf16 matrix [rows][k]: box = 64 of K (128 bytes, the swizzle span) x 128 rows.
-bool make_operand_map(void* encode_fn, const void* ptr, int64_t rows, int64_t k, CUtensorMap* out) {
+// 2-D view of a K-major bf16 matrix [rows][k]: box = 64 of K (128 bytes, the swizzle span) x box_rows rows.
+bool make_operand_map(void* encode_fn, const void* ptr, int64_t rows, int64_t k, CUtensorMap* out, int box_rows = 128) {
   const cuuint64_t dims[2] = {(cuuint64_t)k, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)k * 2};
-  const cuuint32_t box[2] = {64, 128};
+  const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return ((EncodeFn)encode_fn)(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// 5-D view of weights whose rows belong together in twos, `apart` rows from one another, in blocks of 2 * apart:
+// (K, sixteen rows, the two, sixteens of the block's half, block). Box = 64 of K x 128 rows: four times sixteen
+// rows and the sixteen that belong to them, in turn.
+bool make_paired_map(void* encode_fn, const void* ptr, int64_t rows, int64_t k, int apart, CUtensorMap* out) {
+  const cuuint64_t row = (cuuint64_t)k * 2;
+  const cuuint64_t dims[5] = {(cuuint64_t)k, 16, 2, (cuuint64_t)apart / 16, (cuuint64_t)rows / (2 * apart)};
+  const cuuint64_t strides[4] = {row, row * apart, row * 16, row * 2 * apart};
+  const cuuint32_t box[5] = {64, 16, 2, 4, 1};
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  return ((EncodeFn)encode_fn)(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(ptr), dims, strides, box, estr,
+                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+// An activation matrix as the projections read it: boxes of 128 rows, and of 8, 16 .. 128 rows for the pair kernel.
+struct Activations {
+  CUtensorMap full, pair[16];
+};
+bool make_activation_maps(void* encode_fn, const void* ptr, int64_t rows, int64_t k, Activations* out) {
+  bool ok = make_operand_map(encode_fn, ptr, rows, k, &out->full);
+  for (int i = 0; i < 16; ++i) ok = ok && make_operand_map(encode_fn, ptr, rows, k, &out->pair[i], 8 * (i + 1));
+  return ok;
 }
 
 struct LayerLayout {
@@ -68,7 +91,8 @@ struct ts_layer {
   int max_tokens = 0;
   float eps = 0.f, theta = 0.f;
   CUtensorMap w_qkv, w_o, w_gu, w_down;        // weights
-  CUtensorMap a_h, a_attn, a_z;                // activations in the workspace
+  CUtensorMap w_qkv_pair, w_gu_pair;           // rotary pairs, gates and ups together
+  Activations a_h, a_attn, a_z;                // in the workspace
   void* pos_host[kPosRing] = {};
   cudaEvent_t pos_ev[kPosRing] = {};
   bool pos_busy[kPosRing] = {};
@@ -140,9 +164,11 @@ int ts_layer_create(ts_ctx* ctx, const ts_layer_config* cfg, void* cuda_stream, 
             make_operand_map(view.encode_fn, cfg->w_o, cfg->hidden, qd, &l->w_o) &&
             make_operand_map(view.encode_fn, cfg->w_gate_up, 2 * (int64_t)cfg->intermediate, cfg->hidden, &l->w_gu) &&
             make_operand_map(view.encode_fn, cfg->w_down, cfg->hidden, cfg->intermediate, &l->w_down) &&
-            make_operand_map(view.encode_fn, ws + l->L.off_h, l->max_tokens, cfg->hidden, &l->a_h) &&
-            make_operand_map(view.encode_fn, ws + l->L.off_attn, l->max_tokens, qd, &l->a_attn) &&
-            make_operand_map(view.encode_fn, ws + l->L.off_z, l->max_tokens, cfg->intermediate, &l->a_z);
+            make_paired_map(view.encode_fn, cfg->w_qkv, qd + 2 * kvd, cfg->hidden, 64, &l->w_qkv_pair) &&
+            make_paired_map(view.encode_fn, cfg->w_gate_up, 2 * (int64_t)cfg->intermediate, cfg->hidden, 128, &l->w_gu_pair) &&
+            make_activation_maps(view.encode_fn, ws + l->L.off_h, l->max_tokens, cfg->hidden, &l->a_h) &&
+            make_activation_maps(view.encode_fn, ws + l->L.off_attn, l->max_tokens, qd, &l->a_attn) &&
+            make_activation_maps(view.encode_fn, ws + l->L.off_z, l->max_tokens, cfg->intermediate, &l->a_z);
   if (!ok) {
     delete l;
     return TS_ERR_CUDA;
@@ -236,6 +262,11 @@ int ts_layer_step(ts_layer* l, const ts_step* st, const void* x_in, void* x_out,
   g.status = l->view.status;
   g.wait_cycles = l->view.wait_cycles;
   g.M = N;
+  auto project = [&](const Activations& x, const CUtensorMap& w, const CUtensorMap& w_pair) {
+    const ts::GemmPlan plan = ts::gemm_plan(g, l->view.n_sms);
+    const CUtensorMap* x_pair = plan.pair_tokens > 0 ? &x.pair[plan.pair_tokens / 16 - 1] : nullptr;
+    return ts::launch_gemm(g, ts::GemmMaps{&x.full, x_pair, &w, &w_pair}, plan, l->view.n_sms, stream);
+  };
 
   // h = rmsnorm(x); (q, k, v) = rope(h . W_qkv^T)
   if (pos_inline)
@@ -245,7 +276,7 @@ int ts_layer_step(ts_layer* l, const ts_step* st, const void* x_in, void* x_out,
   g.N = qd + 2 * kvd; g.K = hidden; g.epi = ts::GEMM_EPI_ROPE; g.B = (const uint16_t*)l->cfg.w_qkv;
   g.C = q; g.C2 = k; g.C3 = v; g.q_cols = qd; g.kv_cols = kvd; g.pos = pos_dev;
   g.rope_table = (const float2*)(ws + l->L.off_table);
-  TSL_CUDA(l, ts::launch_gemm(g, l->a_h, l->w_qkv, ts::gemm_plan(g, l->view.n_sms), l->view.n_sms, stream));
+  TSL_CUDA(l, project(l->a_h, l->w_qkv, l->w_qkv_pair));
   // attention over the paged KV cache, with the append of the new K/V
   ts_step inner = *st;
   inner.q = q; inner.k_new = k; inner.v_new = v; inner.out = attn;
@@ -253,14 +284,14 @@ int ts_layer_step(ts_layer* l, const ts_step* st, const void* x_in, void* x_out,
   if (rc != TS_OK) return rc;
   // y = x + attn . W_o^T
   g.N = hidden; g.K = qd; g.epi = ts::GEMM_EPI_STORE; g.B = (const uint16_t*)l->cfg.w_o; g.C = y; g.R = (const uint16_t*)x_in; g.ldc = hidden;
-  TSL_CUDA(l, ts::launch_gemm(g, l->a_attn, l->w_o, ts::gemm_plan(g, l->view.n_sms), l->view.n_sms, stream));
+  TSL_CUDA(l, project(l->a_attn, l->w_o, l->w_o));
   // h2 = rmsnorm(y); z = silu(h2 . W_gate^T) * (h2 . W_up^T)
   TSL_CUDA(l, ts::launch_rmsnorm(y, (const uint16_t*)l->cfg.w_norm2, h, N, hidden, l->eps, stream));
   g.N = 2 * inter; g.K = hidden; g.epi = ts::GEMM_EPI_SILU_MUL; g.B = (const uint16_t*)l->cfg.w_gate_up; g.C = z; g.R = nullptr; g.ldc = inter;
-  TSL_CUDA(l, ts::launch_gemm(g, l->a_h, l->w_gu, ts::gemm_plan(g, l->view.n_sms), l->view.n_sms, stream));
+  TSL_CUDA(l, project(l->a_h, l->w_gu, l->w_gu_pair));
   // out = y + z . W_down^T
   g.N = hidden; g.K = inter; g.epi = ts::GEMM_EPI_STORE; g.B = (const uint16_t*)l->cfg.w_down; g.C = (uint16_t*)x_out; g.R = y; g.ldc = hidden;
-  TSL_CUDA(l, ts::launch_gemm(g, l->a_z, l->w_down, ts::gemm_plan(g, l->view.n_sms), l->view.n_sms, stream));
+  TSL_CUDA(l, project(l->a_z, l->w_down, l->w_down));
   return TS_OK;
 }
 
@@ -278,16 +309,18 @@ int ts_gemm_bf16(int32_t device, int32_t M, int32_t N, int32_t K, const void* A,
     return TS_ERR_CUDA;
   int n_sms = 0;
   if (cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return TS_ERR_CUDA;
-  CUtensorMap a_map, b_map;
-  if (!make_operand_map(encode_fn, A, M, K, &a_map) || !make_operand_map(encode_fn, B, N, K, &b_map)) return TS_ERR_CUDA;
   ts::GemmArgs g;
   std::memset(&g, 0, sizeof g);
   g.M = M; g.N = N; g.K = K; g.epi = ts::GEMM_EPI_STORE; g.B = (const uint16_t*)B;
   g.C = (uint16_t*)C; g.R = (const uint16_t*)R; g.ldc = N;
   g.status = device_status;
   g.wait_cycles = ts::kWaitCycles;
-  const ts::GemmPlan plan = tile_m ? ts::GemmPlan{tile_m, 0} : ts::gemm_plan(g, n_sms);
-  return ts::launch_gemm(g, a_map, b_map, plan, n_sms, (cudaStream_t)cuda_stream) == cudaSuccess ? TS_OK : TS_ERR_CUDA;
+  const ts::GemmPlan plan = tile_m ? ts::GemmPlan{tile_m, 0, tile_m == 256 ? ts::pair_tokens(M, (M + 255) / 256) : 0} : ts::gemm_plan(g, n_sms);
+  CUtensorMap x, x_pair, w;
+  if (!make_operand_map(encode_fn, A, M, K, &x) || !make_operand_map(encode_fn, B, N, K, &w) ||
+      (plan.pair_tokens > 0 && !make_operand_map(encode_fn, A, M, K, &x_pair, plan.pair_tokens / 2)))
+    return TS_ERR_CUDA;
+  return ts::launch_gemm(g, ts::GemmMaps{&x, &x_pair, &w, &w}, plan, n_sms, (cudaStream_t)cuda_stream) == cudaSuccess ? TS_OK : TS_ERR_CUDA;
 }
 
 int ts_layer_last_cuda_error(const ts_layer* l) { return l ? l->last_cuda_error : 0; }
