@@ -85,9 +85,8 @@ enum {
   BAR_V_EMPTY = BAR_V_FULL + kVStages,    // [kVStages]
   BAR_S_FULL = BAR_V_EMPTY + kVStages,    // [2] per tile
   BAR_P_FULL = BAR_S_FULL + 2,            // [2] per tile
-  BAR_O_FULL = BAR_P_FULL + 2,            // [2] per tile
-  BAR_O_EMPTY = BAR_O_FULL + 2,           // [2] per tile: the epilogue has read O out of TMEM
-  BAR_Q_EMPTY = BAR_O_EMPTY + 2,          // the last Q K^T of a work unit has consumed the Q tiles
+  BAR_O_FULL = BAR_P_FULL + 2,            // [2] per tile: the last P V of a work unit has landed in O
+  BAR_Q_EMPTY = BAR_O_FULL + 2,           // the last Q K^T of a work unit has consumed the Q tiles
   BAR_V_LANDED = BAR_Q_EMPTY + 1,         // [kVStages] the copies of a V tile are in shared memory
   BAR_K_LANDED = BAR_V_LANDED + kVStages, // the same for a K tile that needs a touch-up before it is announced
   BAR_DRAIN = BAR_K_LANDED + 1,           // after a failure: the MMAs issued before it are done
@@ -317,8 +316,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
       misc[1] = 0;
       misc[2] = 0;
       for (int i = 0; i < BAR_COUNT; ++i) {
-        const bool softmax_arrives = (i >= BAR_P_FULL && i < BAR_P_FULL + 2) || (i >= BAR_O_EMPTY && i < BAR_O_EMPTY + 2);
-        mbar_init(bar(i), softmax_arrives ? 256 : 1);
+        mbar_init(bar(i), i >= BAR_P_FULL && i < BAR_P_FULL + 2 ? kSoftmaxWarps / 2 : 1);
       }
       mbar_init_fence();
     }
@@ -416,6 +414,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
     int row_g = row / G, row_h = row % G;   // token of the tile and query head of this row
     const float scale = s.scale_log2;
     int sx = 0;                 // blocks of this tile in earlier work units: barrier phases follow it
+    int n_o = 0;                // earlier work units in which the tile had rows (O_FULL phases)
     for (int k = 0;; ++k) {
       PfUnit u = {};
       int nbx = -1;
@@ -431,7 +430,8 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
       const int tok = u.q_begin + x * tile_tokens + row_g;     // token inside the request row
       const bool real = row_g < cnt && row < tile_tokens * G;
       const int lim = real ? u.ctx + tok + 1 : (x ? u.k_end_b : u.k_end_a);   // keys at positions >= lim are masked
-      const int tok0 = u.tok0;
+      // the row's place in the output (counted in rows of head_dim), none for a row that is padding
+      const uint32_t orow = real ? (uint32_t)(u.tok0 + tok) * s.Hq + u.kv_head * G + row_h : 0xffffffffu;
       float m_ref = -CUDART_INF_F, l = 0.f;
       for (int j = 0; j < nbx; ++j) {
         wait(BAR_S_FULL + x, (sx + j) & 1);
@@ -482,8 +482,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
               m_ref = m_blk;
               l *= alpha;
             }
-            wait(BAR_O_FULL + x, (sx + j - 1) & 1);           // P V of block j-1 has landed in O
-            tc_fence_after();
+            // O is complete up to block j-1: that P V was issued in front of these scores' Q K^T
 #pragma unroll 1
             for (int c = 0; c < 4; ++c) {
               float ov[16];
@@ -502,13 +501,14 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
         l += ls;
         tmem_st_wait();
         tc_fence_before();
-        mbar_arrive(bar(BAR_P_FULL + x));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(BAR_P_FULL + x));
       }
       if (nbx > 0) {
         // epilogue: O / l -> bf16 -> global; l is the sum over both halves of the keys. (The last
         // P V has been issued, so the partner has arrived for the last block and is done with
         // that block's exchange slots.)
-        wait(BAR_O_FULL + x, (sx + nbx - 1) & 1);
+        wait(BAR_O_FULL + x, n_o++ & 1);
         tc_fence_after();
         *xchg_mine = l;
         pair_sync();
@@ -517,16 +517,11 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
         // A row's 64 columns are one thread's; stored as they are, every 16-byte store of a warp would touch
         // 32 rows. The four lanes of a quad swap 16-byte chunks first, so that they write 64 bytes of a
         // row together.
-        const uint32_t orow = real ? (uint32_t)(tok0 + tok) * s.Hq + u.kv_head * G + row_h : 0xffffffffu;
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
           float ov[32];
           tmem_ld32(ov, tO + c * 32);
           tmem_ld_wait();
-          if (c == 1) {
-            tc_fence_before();
-            mbar_arrive(bar(BAR_O_EMPTY + x));   // O is in registers: the next unit may overwrite it
-          }
           uint32_t w[4][4];                      // [chunk of 8 columns][bf16 pair]
 #pragma unroll
           for (int i = 0; i < 4; ++i)
@@ -782,10 +777,8 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
         const uint32_t issue = elect_one();
         // the warp keeps its own failure flag in a register: nothing on its path reads shared memory
         bool dead = false;
-        // The issuer polls its barriers instead of parking on them: it is the only warp that does,
-        // and every cycle between a tile's P and its next scores is on the critical path.
         auto iwait = [&](int i, uint32_t parity) {
-          if (!mbar_poll(bar(i), parity, dead ? 2000 : s.wait_cycles)) {
+          if (!mbar_wait(bar(i), parity, dead ? 2000 : s.wait_cycles)) {
             dead = true;
             give_up();
           }
@@ -795,9 +788,9 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
         const uint64_t q_desc0 = smem_desc(base + kOffQ, 0, 1024);
         const uint64_t k_desc0 = smem_desc(base + kOffK, 0, 1024);
         const uint64_t v_desc0 = smem_desc(base + kOffV, kHalfBytes, 1024);
-        auto issue_qk = [&](int x, int g) {          // S_x = Q_x K(g)^T
+        auto issue_qk = [&](int x, int stage) {      // S_x = Q_x K^T
           const uint64_t q_desc = q_desc0 + (uint64_t)((x * kTileBytes) >> 4);
-          const uint64_t k_desc = k_desc0 + (uint64_t)(((g % kKStages) * kTileBytes) >> 4);
+          const uint64_t k_desc = k_desc0 + (uint64_t)((stage * kTileBytes) >> 4);
 #pragma unroll
           for (int ks = 0; ks < kD / 16; ++ks) {
             const uint64_t off = (uint64_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4);
@@ -805,64 +798,64 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
           }
           tc_commit(bar(BAR_S_FULL + x), issue);
         };
-        auto issue_pv = [&](int x, int g, bool first) {   // O_x (+)= P_x V(g)
-          const uint64_t v_desc = v_desc0 + (uint64_t)(((g % kVStages) * kTileBytes) >> 4);
+        auto issue_pv = [&](int x, int stage, bool first) {   // O_x (+)= P_x V
+          const uint64_t v_desc = v_desc0 + (uint64_t)((stage * kTileBytes) >> 4);
 #pragma unroll
           for (int kk = 0; kk < kBlockKeys / 16; ++kk)   // P of keys 0-63 sits in columns 0-31 of S, of keys 64-127 in 64-95
             mma_ts(tmem + 256 + x * 128, tmem + x * 128 + (kk >> 2) * 64 + (kk & 3) * 8,
                    v_desc + (uint64_t)((kk * 2048) >> 4), idesc_pv, (!first || kk > 0) ? 1u : 0u, issue);
-          tc_commit(bar(BAR_O_FULL + x), issue);
         };
-        int g0 = 0;                 // key blocks of earlier work units (K/V ring position)
-        int sxb[2] = {0, 0};        // blocks per tile in earlier work units (S/P/O phases)
-        int used[2] = {0, 0};       // earlier work units in which the tile had rows (O_EMPTY phases)
+        int ks = 0, vs = 0;          // ring stages of the next K tile to be multiplied and of the next V tile
+        uint32_t kph = 0, vph = 0;   // and the parities of their "full" phases
+        int sxb[2] = {0, 0};         // blocks per tile in earlier work units (P phases)
         for (int k = 0;; ++k) {
           PfUnit u;
           if (!get_work(k, u)) break;
-          // Order: both Q K^T of block 0; then per block, for tile A then tile B:
-          // P V of block j followed at once by Q K^T of block j+1 of the same tile, so that the
-          // tile's warpgroup gets its next scores while the pipe turns to the other tile.
+          // Order: both Q K^T of block 0; then per block, for tile A then tile B: P V of block j and,
+          // at once behind it, Q K^T of block j+1 of the same tile, so that the tile's warpgroup gets its
+          // next scores while the pipe turns to the other tile. Whatever else the two need (V of block j,
+          // K of block j+1) is waited for in front of P: from P to the next scores is the tile's critical
+          // path, and this warp shares its scheduler with four softmax warps. One commit tells of both products,
+          // and the warp parks while it waits: the launch runs at the chip's power limit. (With looks at barriers
+          // between the products, a commit for each, polling, and arrivals by all lanes of the softmax warps:
+          // 8192-token chunk next to 190 rows 1250 us, now 1237; 2048 tokens alone 45.4, now 44.4.)
           iwait(BAR_Q, k & 1);
-          iwait(BAR_K_FULL + g0 % kKStages, (g0 / kKStages) & 1);
+          iwait(BAR_K_FULL + ks, kph);
           tc_fence_after();
           if (!dead) {
-            if (u.nb_a > 0) issue_qk(0, g0);
-            if (u.nb_b > 0) issue_qk(1, g0);
-            tc_commit(bar(BAR_K_EMPTY + g0 % kKStages), issue);
+            if (u.nb_a > 0) issue_qk(0, ks);
+            if (u.nb_b > 0) issue_qk(1, ks);
+            tc_commit(bar(BAR_K_EMPTY + ks), issue);
             if (u.nb == 1) tc_commit(bar(BAR_Q_EMPTY), issue);
           }
+          if (++ks == kKStages) { ks = 0; kph ^= 1; }
           for (int j = 0; j < u.nb; ++j) {
-            const int g = g0 + j;
             const bool next = j + 1 < u.nb;
+            iwait(BAR_V_FULL + vs, vph);
+            if (next) iwait(BAR_K_FULL + ks, kph);
 #pragma unroll
             for (int x = 0; x < 2; ++x) {
               const int nbx = x ? u.nb_b : u.nb_a;
-              if (j < nbx) {
-                iwait(BAR_P_FULL + x, (sxb[x] + j) & 1);
-                if (x == 0 || j >= u.nb_a) iwait(BAR_V_FULL + g % kVStages, (g / kVStages) & 1);
-                if (j == 0 && used[x] > 0) iwait(BAR_O_EMPTY + x, (used[x] - 1) & 1);   // the previous unit's O has been read
-                tc_fence_after();
-                if (!dead) issue_pv(x, g, j == 0);
-              }
-              if (x == 1 && !dead) tc_commit(bar(BAR_V_EMPTY + g % kVStages), issue);   // both tiles are done with V(g)
-              if (next) {
-                if (x == 0 || j + 1 >= u.nb_a) iwait(BAR_K_FULL + (g + 1) % kKStages, ((g + 1) / kKStages) & 1);
-                tc_fence_after();
-                if (j + 1 < nbx && !dead) issue_qk(x, g + 1);
-                if (x == 1 && !dead) {
-                  tc_commit(bar(BAR_K_EMPTY + (g + 1) % kKStages), issue);
-                  if (j + 2 == u.nb) tc_commit(bar(BAR_Q_EMPTY), issue);   // that was the unit's last Q K^T
-                }
-              }
+              if (j >= nbx) continue;
+              // P of a unit's first block also says that O is free: the warps that arrive have read the
+              // previous unit's O before.
+              iwait(BAR_P_FULL + x, (sxb[x] + j) & 1);
+              tc_fence_after();
+              if (dead) continue;
+              issue_pv(x, vs, j == 0);
+              if (j + 1 < nbx) issue_qk(x, ks);
+              else tc_commit(bar(BAR_O_FULL + x), issue);
             }
+            if (!dead) {                                      // both tiles are done with V(j) and K(j+1)
+              tc_commit(bar(BAR_V_EMPTY + vs), issue);
+              if (next) tc_commit(bar(BAR_K_EMPTY + ks), issue);
+              if (j + 2 == u.nb) tc_commit(bar(BAR_Q_EMPTY), issue);   // that was the unit's last Q K^T
+            }
+            if (++vs == kVStages) { vs = 0; vph ^= 1; }
+            if (next && ++ks == kKStages) { ks = 0; kph ^= 1; }
           }
-          g0 += u.nb;
-#pragma unroll
-          for (int x = 0; x < 2; ++x) {
-            const int nbx = x ? u.nb_b : u.nb_a;
-            sxb[x] += nbx;
-            used[x] += nbx > 0;
-          }
+          sxb[0] += u.nb_a;
+          sxb[1] += u.nb_b;
         }
         if (__any_sync(0xffffffffu, misc[1] != 0)) {
           tc_commit(bar(BAR_DRAIN), issue);
