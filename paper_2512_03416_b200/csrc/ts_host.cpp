@@ -497,6 +497,7 @@ int send_meta(ts_ctx* c, const ts_step* st, int n_items, int n_combines, int n_s
   char* ws = (char*)c->cfg.workspace;
   c->meta_cur = -1;
   d->meta = nullptr;
+  d->meta_in_place = 1;
   if (inline_meta) pack_meta(c, st, *d, n_items, n_combines, d->words);
   if (!inline_meta || !inline_deltas) {
     const int slot = c->meta_next;

