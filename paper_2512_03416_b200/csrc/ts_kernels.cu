@@ -539,6 +539,7 @@ extern "C" int ts_decode_attention_static(int32_t device, int32_t n_q_heads, int
   d.part_acc = sc->part_acc;
   d.part_ml = sc->part_ml;
   d.meta = (const int32_t*)sc;
+  d.meta_in_place = 0;                    // static_plan_kernel writes them in front of the attention kernel
   d.o_slot = offsetof(StaticScratch, row_slot) / 4;
   d.o_ctx = offsetof(StaticScratch, row_ctx) / 4;
   d.o_tok0 = offsetof(StaticScratch, row_tok0) / 4;
