@@ -118,8 +118,9 @@ __device__ __forceinline__ void give_up(const StepDevice& s, volatile int* faile
 
 // Scheduler warp of CTA `cta` of `n_ctas`: its first unit is unit `cta`, the others come off the queue
 // s.pf_queue[3], which the launch leaves at zero.
-template <int D, int STAGES>
-__device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned char* smem, uint32_t base, int cta, int n_ctas) {
+// `ready` waits for the launch in front of this one: called once the first unit is described.
+template <int D, int STAGES, typename Ready>
+__device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned char* smem, uint32_t base, int cta, int n_ctas, Ready&& ready) {
   using L = DecSmem<D, STAGES>;
   const int lane = threadIdx.x & 31, G = s.Hq / s.Hkv;
   const uint32_t bars = base + L::off_bars(G);
@@ -159,6 +160,7 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
       mbar_arrive(bars + (L::kBarDesc + e) * 8);
     }
     __syncwarp();
+    if (k == 0) ready();
     // one word of every 32-byte sector of the queries and of the page ids, for what it leaves in L1
     uint32_t touched = 0;
     if (u.n_pg > 0) {
@@ -175,11 +177,11 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
 
 // Streams the units that decode_schedule describes, on the first kDecThreads threads of the block
 // (the scheduler runs on another warp at the same time). `smem` is the 1024-byte-aligned shared-memory
-// window (decode_smem_bytes<D, STAGES>(G) bytes), `base` its shared-space address. The caller has
-// executed griddepcontrol.wait; the function leaves no copy in flight when it returns.
-template <int D, int NH, int STAGES>
+// window (decode_smem_bytes<D, STAGES>(G) bytes), `base` its shared-space address. `ready` waits for the launch
+// in front of this one, once the barriers are set up. The function leaves no copy in flight when it returns.
+template <int D, int NH, int STAGES, typename Ready>
 __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensorMap* kv_map, unsigned char* smem,
-                                             uint32_t base) {
+                                             uint32_t base, Ready&& ready) {
   using L = DecSmem<D, STAGES>;
   constexpr int W = kDecWarps;
   constexpr int STAGE_BYTES = L::kStageBytes;
@@ -202,6 +204,7 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
     mbar_init_fence();
   }
   decode_meet();
+  ready();
 
   bool dead = false;           // a wait of this warp ran out (all lanes agree): it starts no copy and no page any more
   auto wait = [&](int i, uint32_t parity) {
