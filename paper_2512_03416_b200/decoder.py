@@ -9,6 +9,11 @@ import torch
 from . import binding as B
 
 
+# The handle of a device's current stream. torch.cuda.current_stream() builds an object first (2.3 us of a small
+# step's call); the direct call is not a public name of torch, so a torch without it takes that way all the same.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
 class TsError(RuntimeError):
     def __init__(self, code: int, what: str):
         super().__init__(f"{what}: {B.ts_strerror(code)} ({code})")
@@ -94,7 +99,7 @@ class Decoder:
 
     # ------------------------------------------------------------------------------- steps
     def _stream(self) -> int:
-        return torch._C._cuda_getCurrentRawStream(self.device.index)     # current_stream() builds an object first: 2.3 us
+        return _raw_stream(self.device.index)
 
     def make_step(self, slots, q_len, ctx_len, q=None, k_new=None, v_new=None, out=None,
                   keep_len: bool = False, flags: int = 0):
