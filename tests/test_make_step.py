@@ -26,6 +26,13 @@ def test_a_step_outlives_its_second_result():
 
 
 def test_rows_of_unequal_length_are_not_mixed_up():
+    """The first array says how many rows there are: an array with more is refused, one with fewer is zero
+    from there on, and no number moves into another array or row."""
     with pytest.raises(IndexError):
         B.make_step([1, 2], [3, 4, 5], [6])          # six numbers for two rows all the same
-    assert rows_of(B.make_step([1, 2], [3, 4], [6])[0])[2][0] == 6
+    assert rows_of(B.make_step([1, 2], [3, 4], [6])[0]) == [[1, 2], [3, 4], [6, 0]]
+    assert rows_of(B.make_step([1, 2], [3], [5, 6])[0]) == [[1, 2], [3, 0], [5, 6]]
+
+
+def test_values_beyond_32_bits_keep_their_low_bits():
+    assert rows_of(B.make_step([(1 << 32) + 7, 1], [1, 2], [-(1 << 31) - 1, 4])[0]) == [[7, 1], [1, 2], [(1 << 31) - 1, 4]]
