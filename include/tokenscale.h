@@ -507,6 +507,15 @@ int ts_layer_last_cuda_error(const ts_layer* layer);
 int ts_gemm_bf16(int32_t device, int32_t M, int32_t N, int32_t K, const void* A, const void* B, const void* R,
                  void* C, int32_t tile_m, int32_t* device_status, void* cuda_stream);
 
+/*
+ * ts_gemm_plan: how ts_layer_step lays a projection of M tokens over the device, for measurements and tests.
+ * epilogue: 0 = plain store (output and down projection, ts_gemm_bf16 with tile_m 0), 1 = rotary (QKV), 2 = SiLU
+ * gate (gate/up, N = 2 * intermediate). *tile_m: 128 or 256 as above; *split: thread blocks that share a tile's K
+ * range, 0 = K is not split; *pair_tokens: rows of A in a pair's tile, 0 where tile_m is 128. Launches nothing.
+ */
+int ts_gemm_plan(int32_t device, int32_t M, int32_t N, int32_t K, int32_t epilogue, int32_t* tile_m, int32_t* split,
+                 int32_t* pair_tokens);
+
 /* The cudaError_t of the most recent failed CUDA call of this context (0 if none). */
 int ts_last_cuda_error(const ts_ctx* ctx);
 

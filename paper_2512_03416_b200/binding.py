@@ -84,7 +84,7 @@ EXPORTS = ["ts_pool_bytes", "ts_workspace_bytes", "ts_create", "ts_destroy", "ts
            "ts_convertible_prefill_velocity", "ts_reserved_memory", "ts_reserved_pages",
            "ts_prefiller_instances", "ts_decoder_demand", "ts_regular_decoders", "ts_route_prefill",
            "ts_layer_workspace_bytes", "ts_pack_gate_up", "ts_layer_create", "ts_layer_destroy", "ts_layer_step",
-           "ts_layer_last_cuda_error", "ts_gemm_bf16"]
+           "ts_layer_last_cuda_error", "ts_gemm_bf16", "ts_gemm_plan"]
 
 _lib = None
 
@@ -161,6 +161,7 @@ def lib() -> ctypes.CDLL:
         L.ts_layer_last_cuda_error.argtypes = [vp]
         L.ts_gemm_bf16.argtypes = [ctypes.c_int32, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32, vp, vp, vp, vp,
                                    ctypes.c_int32, vp, vp]
+        L.ts_gemm_plan.argtypes = [ctypes.c_int32] * 5 + [_i32p] * 3
         L.ts_strerror.restype = ctypes.c_char_p
         L.ts_strerror.argtypes = [ctypes.c_int]
         for name in EXPORTS:
@@ -424,3 +425,10 @@ def ts_layer_step(layer, step: ts_step, x_in: int, x_out: int, stream: int) -> i
 def ts_gemm_bf16(device: int, M: int, N: int, K: int, A: int, B: int, R: int, C: int, tile_m: int, status: int,
                  stream: int) -> int:
     return lib().ts_gemm_bf16(device, M, N, K, A, B, R or None, C, tile_m, status, stream)
+
+
+def ts_gemm_plan(device: int, M: int, N: int, K: int, epilogue: int):
+    """Returns (code, (tile_m, split, pair_tokens))."""
+    out = [ctypes.c_int32() for _ in range(3)]
+    rc = lib().ts_gemm_plan(device, M, N, K, epilogue, *[ctypes.byref(x) for x in out])
+    return rc, tuple(x.value for x in out)

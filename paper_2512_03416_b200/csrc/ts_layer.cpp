@@ -323,6 +323,24 @@ int ts_gemm_bf16(int32_t device, int32_t M, int32_t N, int32_t K, const void* A,
   return ts::launch_gemm(g, ts::GemmMaps{&x, &x_pair, &w, &w}, plan, n_sms, (cudaStream_t)cuda_stream) == cudaSuccess ? TS_OK : TS_ERR_CUDA;
 }
 
+int ts_gemm_plan(int32_t device, int32_t M, int32_t N, int32_t K, int32_t epilogue, int32_t* tile_m, int32_t* split,
+                 int32_t* pair_tokens) {
+  if (M <= 0 || N <= 0 || K <= 0 || epilogue < ts::GEMM_EPI_STORE || epilogue > ts::GEMM_EPI_SILU_MUL || !tile_m || !split ||
+      !pair_tokens)
+    return TS_ERR_INVALID;
+  int n_sms = 0;
+  if (cudaSetDevice(device) != cudaSuccess || cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+    return TS_ERR_CUDA;
+  ts::GemmArgs g;
+  std::memset(&g, 0, sizeof g);
+  g.M = M; g.N = N; g.K = K; g.epi = epilogue;
+  const ts::GemmPlan plan = ts::gemm_plan(g, n_sms);
+  *tile_m = plan.tile_m;
+  *split = plan.split;
+  *pair_tokens = plan.pair_tokens;
+  return TS_OK;
+}
+
 int ts_layer_last_cuda_error(const ts_layer* l) { return l ? l->last_cuda_error : 0; }
 
 }  // extern "C"
