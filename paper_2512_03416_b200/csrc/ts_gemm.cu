@@ -107,14 +107,12 @@ __device__ __forceinline__ void rope8(const GemmArgs& g, int row, int col0, int 
   *reinterpret_cast<uint4*>(dst + c) = pack8(lo);
   *reinterpret_cast<uint4*>(dst + 64 + c) = pack8(hi);
 }
-// silu(gate) * up, both rounded to bf16 first (they are bf16 tensors of the layer's definition)
-__device__ __forceinline__ float silu_mul(float gate, float up) {
-  const float a = __bfloat162float(__float2bfloat16_rn(gate)), b = __bfloat162float(__float2bfloat16_rn(up));
-  return a / (1.f + __expf(-a)) * b;
-}
+// silu(gate) * up of two bf16 values (they are bf16 tensors of the layer's definition)
+__device__ __forceinline__ float silu_mul(float gate, float up) { return gate / (1.f + __expf(-gate)) * up; }
 __device__ __forceinline__ void silu_mul8(float* gate, const float* up) {
 #pragma unroll
-  for (int e = 0; e < 8; ++e) gate[e] = silu_mul(gate[e], up[e]);
+  for (int e = 0; e < 8; ++e)
+    gate[e] = silu_mul(__bfloat162float(__float2bfloat16_rn(gate[e])), __bfloat162float(__float2bfloat16_rn(up[e])));
 }
 
 // Epilogue of one accumulator (TMEM lanes = 128 rows, 256 columns): half `hf` of this thread's row of
@@ -334,8 +332,7 @@ gemm_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, const _
 // For products with many rows. Two CTAs of a cluster share a tile of 256 features x `nt` tokens
 // (cta_group::2), computed transposed: the weights are the MMA's M (always 256), the tokens its N, which may be
 // any multiple of 16 up to 256, so that the tokens divide into tiles of nearly equal size and little is
-// computed for padding. (With the tokens as M = 256, 2112 of them took nine tiles of 256: 8 % padding, and 300
-// took 512.) CTA r fetches 128 weight rows and nt / 2 token rows per 64 of K and holds the accumulator of its
+// computed for padding: 2112 of them are nine tiles of 240, 300 two of 160 (as M they would take 256 each). CTA r fetches 128 weight rows and nt / 2 token rows per 64 of K and holds the accumulator of its
 // weight rows: TMEM lane = feature, column = token. One MMA reads the token halves of both CTAs. Per CTA and
 // 64 of K that is at most 32 KB fetched and 32 KB read for 512 cycles of tensor work, where a CTA on its own moves
 // 48 KB + 48 KB for a 128 x 256 tile (shared memory gives 128 bytes per clock: its limit, not the tensor pipe's).
@@ -389,46 +386,60 @@ constexpr int kPairBars = 2 * kPairStages + 4;
 constexpr int kPairSmem = kPairStages * kPairStageBytes + kPairBars * 8 + 16 + 1024;
 constexpr uint32_t kIdescPair = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 4) << 24);   // M = 256; N is added
 
+// One word of a token's row, read or written where at < n, by a predicate: with a branch around each, the sixteen
+// stores of 32 tokens take a warp 1640 cycles instead of 1050, and the sixteen loads of their residual 1100 instead of
+// 500, which the last tiles' epilogue adds to the launch.
+__device__ __forceinline__ uint32_t ld_below(const uint16_t* p, int at, int n) {
+  uint32_t w;
+  asm volatile("{\n.reg .pred p;\nsetp.lt.s32 p, %2, %3;\n@p ld.global.b32 %0, [%1];\n@!p mov.b32 %0, 0;\n}\n" : "=r"(w) : "l"(p), "r"(at), "r"(n) : "memory");
+  return w;
+}
+__device__ __forceinline__ void st_below(uint16_t* p, uint32_t w, int at, int n) {
+  asm volatile("{\n.reg .pred p;\nsetp.lt.s32 p, %2, %3;\n@p st.global.b32 [%0], %1;\n}\n" ::"l"(p), "r"(w), "r"(at), "r"(n) : "memory");
+}
+
+// The residual's words of 32 tokens x a warp's 32 features, as epilogue_tokens<STORE> adds them: r[i] = features
+// n0 + q * 32 + (lane & ~1) and the next one of token t0 + 2 i + (lane & 1). Zero outside the product.
+__device__ __forceinline__ void load_residual(const GemmArgs& g, uint32_t (&r)[16], int t0, int end, int n0, int q, int lane) {
+  const int col = n0 + q * 32 + (lane & ~1), n = col < g.N ? end - t0 - (lane & 1) : 0;
+  const uint16_t* src = g.R + (size_t)(t0 + (lane & 1)) * g.ldc + col;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) r[i] = ld_below(src + (size_t)(2 * i) * g.ldc, 2 * i, n);
+}
+
 // 32 tokens (t0 .. t0 + 31, those below `end`) of this lane's feature of a 128-feature accumulator: quarter q of
 // the features, feature n0 + q * 32 + lane of the product (STORE) or the order of the permuted weight rows.
 // Neighbouring lanes swap values first, so that a lane writes two features of one token: 64 bytes
-// (STORE) or 32 bytes (the others) of a token's row together.
+// (STORE) or 32 bytes (the others) of a token's row together. r: the residual (STORE with g.R).
 template <int EPI>
-__device__ __forceinline__ void epilogue_tokens(const GemmArgs& g, float (&v)[32], int t0, int end, int n0, int q, int lane) {
+__device__ __forceinline__ void epilogue_tokens(const GemmArgs& g, float (&v)[32], const uint32_t (&r)[16], int t0, int end, int n0, int q, int lane) {
   const bool odd = lane & 1, upper = lane & 16;
+  const int rest = end - t0 - odd;                         // tokens from this lane's first one on
   auto swap_pair = [&](float mine_even, float mine_odd, float& lo, float& hi) {   // even lanes keep the first token, odd ones the second
     const float got = __shfl_xor_sync(0xffffffffu, odd ? mine_even : mine_odd, 1);
     lo = odd ? got : mine_even;
     hi = odd ? mine_odd : got;
   };
   if (EPI == GEMM_EPI_STORE) {
-    const int col = n0 + q * 32 + (lane & ~1);
-    if (n0 + q * 32 >= g.N) return;                        // N is a multiple of 8: checked per lane below
-    uint32_t r[16];
-    if (g.R) {
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int t = t0 + 2 * i + odd;
-        r[i] = t < end && col < g.N ? *reinterpret_cast<const uint32_t*>(g.R + (size_t)t * g.ldc + col) : 0u;
-      }
-    }
+    const int col = n0 + q * 32 + (lane & ~1), n = col < g.N ? rest : 0;
+    uint16_t* dst = g.C + (size_t)(t0 + odd) * g.ldc + col;
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       float lo, hi;
       swap_pair(v[2 * i], v[2 * i + 1], lo, hi);
-      const int t = t0 + 2 * i + odd;
       if (g.R) {
         lo += __uint_as_float(r[i] << 16);
         hi += __uint_as_float(r[i] & 0xFFFF0000u);
       }
-      if (t < end && col < g.N) *reinterpret_cast<uint32_t*>(g.C + (size_t)t * g.ldc + col) = pack_bf16(lo, hi);
+      st_below(dst + (size_t)(2 * i) * g.ldc, pack_bf16(lo, hi), 2 * i, n);
     }
   } else if (EPI == GEMM_EPI_ROPE) {
     // lanes 0-15: features 16 q + lane of the head, lanes 16-31: their partners 64 further on
     if (n0 >= g.N) return;
     const bool rotate = n0 < g.q_cols + g.kv_cols;
-    uint16_t* dst = n0 < g.q_cols ? g.C + n0 : rotate ? g.C2 + (n0 - g.q_cols) : g.C3 + (n0 - g.q_cols - g.kv_cols);
     const int ld = n0 < g.q_cols ? g.q_cols : g.kv_cols, f = q * 16 + (lane & 15);
+    uint16_t* dst = n0 < g.q_cols ? g.C + n0 : rotate ? g.C2 + (n0 - g.q_cols) : g.C3 + (n0 - g.q_cols - g.kv_cols);
+    dst += (size_t)(t0 + odd) * ld + (upper ? 64 : 0) + (f & ~1);
     if (rotate) {
       const int pos = t0 + lane < end ? g.pos[t0 + lane] : 0;
 #pragma unroll
@@ -443,27 +454,25 @@ __device__ __forceinline__ void epilogue_tokens(const GemmArgs& g, float (&v)[32
     for (int i = 0; i < 16; ++i) {
       float lo, hi;
       swap_pair(v[2 * i], v[2 * i + 1], lo, hi);
-      const int t = t0 + 2 * i + odd;
-      if (t < end) *reinterpret_cast<uint32_t*>(dst + (size_t)t * ld + (upper ? 64 : 0) + (f & ~1)) = pack_bf16(lo, hi);
+      st_below(dst + (size_t)(2 * i) * ld, pack_bf16(lo, hi), 2 * i, rest);
     }
   } else {
-    // lanes 0-15: gate features, lanes 16-31: the up features that belong to them. Of two tokens the lower lanes
-    // take the first, the upper ones the second. out[token][n0 / 2 + i] = silu(gate_i) * up_i.
+    // lanes 0-15: gate features, lanes 16-31: the up features that belong to them. Of four tokens the lower lanes
+    // take the first two, the upper ones the others: bf16 values of two tokens change lanes in one word (one fp32 value
+    // of a token each: 1024 x 22528 x 2048 44.9 us instead of 42.0).
+    // out[token][n0 / 2 + i] = silu(gate_i) * up_i.
     if (n0 >= g.N) return;
-    uint16_t* dst = g.C + n0 / 2 + q * 16 + (lane & 14);
+    const int first = odd + (upper ? 2 : 0);
+    uint16_t* dst = g.C + (size_t)(t0 + first) * g.ldc + n0 / 2 + q * 16 + (lane & 14);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {                          // four tokens at a time
-      float h[2];
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const float first = v[4 * i + 2 * e], second = v[4 * i + 2 * e + 1];
-        const float got = __shfl_xor_sync(0xffffffffu, upper ? first : second, 16);
-        h[e] = silu_mul(upper ? got : first, upper ? second : got);
-      }
+      const uint32_t front = pack_bf16(v[4 * i], v[4 * i + 1]), back = pack_bf16(v[4 * i + 2], v[4 * i + 3]);
+      const uint32_t got = __shfl_xor_sync(0xffffffffu, upper ? front : back, 16);
+      const uint32_t gate = upper ? got : front, up = upper ? back : got;
       float lo, hi;
-      swap_pair(h[0], h[1], lo, hi);
-      const int t = t0 + 4 * i + (odd ? 2 : 0) + (upper ? 1 : 0);
-      if (t < end) *reinterpret_cast<uint32_t*>(dst + (size_t)t * g.ldc) = pack_bf16(lo, hi);
+      swap_pair(silu_mul(__uint_as_float(gate << 16), __uint_as_float(up << 16)),
+                silu_mul(__uint_as_float(gate & 0xFFFF0000u), __uint_as_float(up & 0xFFFF0000u)), lo, hi);
+      st_below(dst + (size_t)(4 * i) * g.ldc, pack_bf16(lo, hi), 4 * i, end - t0 - first);
     }
   }
 }
@@ -580,19 +589,31 @@ gemm_pair_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap x_map, co
       // first feature of this CTA's half of the tile; SILU_MUL: gate and up features of half a block
       const int n0 = (t / m_tiles) * kBN + (int)rank * 128;
       const int buf = n_done & 1;
+      const int chunks = (nt + 31) / 32, last = ((chunks - 1 - hf) & ~1) + hf;   // this warp: chunks hf, hf + 2, ...
+      // The residual is fetched a chunk ahead, the first one's before the sums are there: the epilogue of a launch's
+      // last tiles is not hidden behind anything. (1024 x 4096 x 4096, both with branches around the stores: 33.2 us
+      // with the residual fetched where it is added, 31.1 so.)
+      const bool with_r = EPI == GEMM_EPI_STORE && g.R != nullptr;
+      uint32_t next_r[16];
+      if (with_r) load_residual(g, next_r, m0 + hf * 32, end, n0, q, lane);
       wait(BAR_ACC_FULL + buf, (n_done >> 1) & 1);
       tc_fence_after();
-      const int chunks = (nt + 31) / 32, last = ((chunks - 1 - hf) & ~1) + hf;   // this warp: chunks hf, hf + 2, ...
       for (int c = hf; c < chunks; c += 2) {
         float v[32];
+        uint32_t r[16];
         tmem_ld32(v, tmem + buf * 256 + ((uint32_t)(q * 32) << 16) + c * 32);
+        if (with_r) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) r[i] = next_r[i];
+          load_residual(g, next_r, m0 + (c + 2) * 32, end, n0, q, lane);
+        }
         tmem_ld_wait();
         if (c == last) {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(mapa(bar(BAR_ACC_EMPTY + buf), 0));
         }
-        if (m0 + c * 32 < end) epilogue_tokens<EPI>(g, v, m0 + c * 32, end, n0, q, lane);
+        if (m0 + c * 32 < end) epilogue_tokens<EPI>(g, v, r, m0 + c * 32, end, n0, q, lane);
       }
       if (hf >= chunks) {                                  // a narrow tile: nothing for this warp
         __syncwarp();
