@@ -885,15 +885,16 @@ cudaError_t launch_epi(const GemmArgs& g, const GemmMaps& maps, GemmPlan plan, i
 // is what the tensor pipe and shared memory take (0.45 us for a CTA's 128 x 256 tile, 0.2 us + 0.65 ns per token
 // for a pair's tile, 0.33 us for a 128 x 128 tile), what an SM needs to get a pair's weights from HBM (0.285 us), or
 // what HBM needs for the weight blocks in flight
-// at that moment; for the split kernel also the merge, and only where all clusters run at once.
-// Measured (8B-shaped projections, weights not in L2, us; 128 x 256 tile / pair with tiles of 256 tokens, as it
-// was / pair / split kernel): 64 rows QKV 29.4 / 25.9 / 22.3 / 15.2, output 27.5 / 24.7 / 22.0 / 11.9, gate/up 43.1 /
-// 51.6 / 47.8, down 86.2 / 70.4 / 64.1 / 25.4; 256 rows output 28.6 / 25.9 / 23.0 / 16.0, down 87.6 / 72.2 / 67.7 /
-// 38.2; gate/up with 130 rows 61.3 / 55.0 / 50.3, 297 88.0 / 93.1 / 79.8, 514 119 / 124 / 107, 800 169 / 167 / 150, 2112
-// 393 / 346 / 319; 2112 rows QKV 106 / 81.5 / 82.8, output 63.8 / 54.7 / 55.2, down 223 / 187 / 178.
+// at that moment; for the split kernel also what its merge takes longer than another kernel's last epilogue, and only
+// where all clusters run at once.
+// Measured (bursts too short for the power cap, weights not in L2, us; 128 x 256 tile / pair / split kernel, the latter two
+// with their best tokens and split): 64 rows QKV 32.3 / 21.5 / 15.9, output 29.7 / 20.6 / 12.2, gate/up 46.5 / 47.7, down 88.8 / 62.9 /
+// 25.7; 256 rows output 32.3 / 22.2 / 17.8, down 92.4 / 66.9 / 42.0; gate/up with 130 rows 63.8 / 54.0, 300 86.4 / 84.5, 512 111 /
+// 94.3, 800 161 / 150, 2112 342 / 319; 2112 rows QKV 94.9 / 76.8, output 60.6 / 50.6, down 192 / 160. 2048 x 2048, where a pair's main
+// loop is short: 130 rows 19.7 / 12.5 / 10.7, 256 rows 19.8 / 12.7 / 11.0.
 GemmPlan gemm_plan(const GemmArgs& g, int n_sms) {
   constexpr double kTileUs = 0.45, kPairUs = 0.2, kPairTokenUs = 0.00065, kPairMinUs = 0.285, kSplitUs = 0.33, kHbmBytesPerUs = 6.2e6;
-  const double merge_us = 2.5 + 0.03 * std::min(g.M, 128);
+  const double merge_us = 2.0 + 0.03 * std::min(g.M, 128);
   const int n_tiles = (g.N + kBN - 1) / kBN, m128 = (g.M + 127) / 128, m256 = (g.M + 255) / 256;
   const int kb = (g.K + kBK - 1) / kBK;
   // `at_once` workers on weight blocks of `width` rows, each on another one unless m_tiles row blocks share it

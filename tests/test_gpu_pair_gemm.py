@@ -119,6 +119,13 @@ def test_layer_with_fused_epilogues_on_single_ctas(rows, tokens):
     _check_layer(s, inter, rows, tokens)
 
 
+@pytest.mark.parametrize("M", [129, 130, 192, 256])
+def test_products_of_few_tiles_split_k(M):
+    """A 2048 x 2048 product of a few hundred tokens: four CTAs on a tile's K range (10.6 us) and not pairs (13 us)."""
+    assert B.ts_gemm_plan(0, M, 2048, 2048, 0) == (B.TS_OK, (128, 4, 0))
+    gemm_matches((M, 2048, 2048, True), 0)
+
+
 def test_plan_refuses_what_is_no_product():
     for args in ((0, 256, 64, 0), (1, 0, 64, 0), (1, 256, 0, 0), (1, 256, 64, 3), (1, 256, 64, -1)):
         assert B.ts_gemm_plan(0, *args)[0] == B.TS_ERR_INVALID
