@@ -16,10 +16,12 @@ decode_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUte
   unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
   pdl_launch_dependents();
   if (threadIdx.x == 0) tma_prefetch_desc(&kv_map);
-  // Barriers and, where the step's metadata are launch parameters, each CTA's first unit are set up before the
-  // wait; the pool, the tables and Q are read behind it.
-  // (Latency of small batches, us before -> after: four rows of ~1500 keys 10.6 -> 9.85, one row of 4000 13.1 -> 12.4,
-  // eight of ~1500 21.9 -> 21.05.)
+  // Where the step's metadata are launch parameters, the barriers and each CTA's first unit are set up before the
+  // wait, and only the pool, the tables and Q are read behind it. Uploaded metadata (larger steps) and those of
+  // a planning kernel are read behind the wait, and all of the set-up stays there too.
+  // (Device time of a step, prepared steps back to back, with everything behind the wait and so, us: four rows of ~1500
+  // keys 10.50 / 9.74, one row of 4000 10.31 / 9.46, eight of ~1500 17.5 / 16.8, 64 rows 126.7 / 126.8. A call that
+  // marshals its rows and waits is bound by the host for so few.)
   auto ready = [&]() { pdl_wait(); };
   if (s.meta) ready();
   if (threadIdx.x < kDecThreads) {

@@ -459,7 +459,7 @@ __device__ __forceinline__ void epilogue_tokens(const GemmArgs& g, float (&v)[32
   } else {
     // lanes 0-15: gate features, lanes 16-31: the up features that belong to them. Of four tokens the lower lanes
     // take the first two, the upper ones the others: bf16 values of two tokens change lanes in one word (one fp32 value
-    // of a token each: 1024 x 22528 x 2048 44.9 us instead of 42.0).
+    // of a token each: 1024 x 11264 x 2048 44.9 us instead of 42.0).
     // out[token][n0 / 2 + i] = silu(gate_i) * up_i.
     if (n0 >= g.N) return;
     const int first = odd + (upper ? 2 : 0);

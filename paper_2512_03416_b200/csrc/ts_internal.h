@@ -77,7 +77,9 @@ struct StepDevice {
   // are small, from `words`: they then travel as launch parameters, without an upload of their own (a copy
   // on another stream, two event records and two waits: ~6 us of host time and a dependency per step).
   const int32_t* meta;     // null: `words`
-  int32_t meta_in_place;   // they were complete before the step's first kernel started (not where a kernel in front plans the step)
+  // Whether a launch behind the step's first reading one may read them before it waits for the launch in front: they are
+  // launch parameters, or the stream waited for their upload before the first launch that reads them. Not where a kernel plans the step.
+  int32_t meta_in_place;
   uint32_t o_slot, o_ctx, o_tok0, o_items, o_combines;
   int32_t words[kInlineWords];
 #ifdef __CUDACC__

@@ -67,7 +67,8 @@ __global__ void kv_append_kernel(const __grid_constant__ StepDevice s) {
 __global__ void combine_kernel(const __grid_constant__ StepDevice s) {
   pdl_launch_dependents();
   // Metadata that were in place before the decode launch started are read before the wait for its end: one round
-  // trip less behind it (four rows 10.8 -> 10.6 us, 64 rows 129.0 -> 128.6).
+  // trip less behind it (device time of a step, prepared steps back to back, read behind the wait and so, us: four
+  // rows of ~1500 keys 10.69 / 10.50, 64 rows 127.0 / 126.7).
   CombineItem c;
   if (s.meta_in_place) c = s.combine(blockIdx.x);
   pdl_wait();

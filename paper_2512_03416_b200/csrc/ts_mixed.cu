@@ -816,9 +816,9 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
           // next scores while the pipe turns to the other tile. Whatever else the two need (V of block j,
           // K of block j+1) is waited for in front of P: from P to the next scores is the tile's critical
           // path, and this warp shares its scheduler with four softmax warps. One commit tells of both products,
-          // and the warp parks while it waits: the launch runs at the chip's power limit. (With looks at barriers
-          // between the products, a commit for each, polling, and arrivals by all lanes of the softmax warps:
-          // 8192-token chunk next to 190 rows 1250 us, now 1237; 2048 tokens alone 45.4, now 44.4.)
+          // and the warp parks while it waits: the launch runs at the chip's power limit. (Looks at barriers between
+          // the products, a commit for each, polling, and arrivals by all lanes of the softmax warps, all together: 8192-token
+          // chunk next to 190 rows 1250 us instead of 1237; 2048 tokens alone 45.4 instead of 44.4.)
           iwait(BAR_Q, k & 1);
           iwait(BAR_K_FULL + ks, kph);
           tc_fence_after();
