@@ -20,8 +20,7 @@
 // Warp roles: warps 0-3 / 8-11 softmax and epilogue of tile A (keys 0-63 / 64-127 of each block,
 // head_dim columns 0-63 / 64-127 of O), warps 4-7 / 12-15 the same for tile B (thread = TMEM lane =
 // query row; a warp can only reach the 32 lanes its index modulo 4 selects, so a row is split by
-// columns). The two threads of a row agree on the row maximum through shared memory and a
-// barrier of their two warps per block. Two softmax warps per tile and SM sub-partition hide each
+// columns). The two threads of a row agree on a new row maximum by a vote of their two warps per block. Two softmax warps per tile and SM sub-partition hide each
 // other's instruction latencies: one warp per row quarter left the tensor pipe idle more than
 // half of the time although no unit was saturated. Warp 16 K loader, warp 17 V loader (TMA copies of
 // pages and of the chunk's own tokens; the K loader's first thread also claims the work units), warp 18 MMA issuer and TMEM owner, warp 19 Q loader (TMA).
@@ -70,6 +69,13 @@ constexpr int kTileBytes = 128 * kD * 2;        // one 128 x 128 bf16 operand ti
 constexpr int kHalfBytes = kTileBytes / 2;      // 64 head_dim columns of it
 constexpr int kKStages = 2, kVStages = 3;       // measured: a third V stage is worth more than a third K stage (3%)
 constexpr long long kDrainCycles = 20000000;    // about 10 ms: limit of the waits for copies and MMAs in flight after a failure
+// Keys of each half row whose P is announced, and multiplied by V, before the other ones' exponentials are taken: the
+// P V of these 48 and the exponentials of the last 16 take about the same time (six MMAs 384 cycles, 16 exponentials
+// of two warps 256 and the announcement), so that only two MMAs and the next Q K^T are left behind the last P.
+// 8192 tokens alone, 70B shape / 2048 tokens alone, 8B shape (us, launches too short for the power cap): all 64 at once 879 / 40.0,
+// 32 and 32 856 / 39.4, 48 and 16 837 / 38.4, three parts (32, 16, 16) no better than one; back to back, at the power cap
+// 1023 / 41.6, 993 / 41.2, 979 / 40.7.
+constexpr int kFirst = 48;
 constexpr float kRescaleThreshold = 8.0f;       // log2 units
 
 // shared-memory map (offsets from the 1024-aligned base)
@@ -84,8 +90,8 @@ enum {
   BAR_V_FULL = BAR_K_EMPTY + kKStages,    // [kVStages]
   BAR_V_EMPTY = BAR_V_FULL + kVStages,    // [kVStages]
   BAR_S_FULL = BAR_V_EMPTY + kVStages,    // [2] per tile
-  BAR_P_FULL = BAR_S_FULL + 2,            // [2] per tile
-  BAR_O_FULL = BAR_P_FULL + 2,            // [2] per tile: the last P V of a work unit has landed in O
+  BAR_P_FULL = BAR_S_FULL + 2,            // [2][2] per tile: the first kFirst keys of both halves of P, the others
+  BAR_O_FULL = BAR_P_FULL + 4,            // [2] per tile: the last P V of a work unit has landed in O
   BAR_Q_EMPTY = BAR_O_FULL + 2,           // the last Q K^T of a work unit has consumed the Q tiles
   BAR_V_LANDED = BAR_Q_EMPTY + 1,         // [kVStages] the copies of a V tile are in shared memory
   BAR_K_LANDED = BAR_V_LANDED + kVStages, // the same for a K tile that needs a touch-up before it is announced
@@ -138,28 +144,32 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
-// Half a row of a score block: p_i = 2^(x_i), x_i = v_i * scale + neg_m, for the 64 scores in v,
-// as bf16 pairs in pk (the scores are not needed afterwards, so their registers come free as
-// the loop advances); returns the sum of the unrounded p_i and, in x_max, the largest x_i (it
-// rides along in issue slots the exponentials leave free).
-__device__ __forceinline__ float exp_pack(const float (&v)[64], float scale, float neg_m, uint32_t (&pk)[32], float& x_max) {
-  const uint64_t scale2 = pack_f2(scale, scale), negm2 = pack_f2(neg_m, neg_m);
-  uint64_t sum_a = pack_f2(0.f, 0.f), sum_b = sum_a;
-  float xm0 = -CUDART_INF_F, xm1 = xm0;
+// N scores of a row: p_i = 2^(v_i * scale + neg_m) as bf16 pairs in pk (the scores are not needed
+// afterwards, so their registers come free as the loop advances); adds the unrounded p_i to sum. The largest of
+// these and of the NW scores in w rides along, in issue slots the exponentials leave free.
+template <int N, int NW = 0>
+__device__ __forceinline__ void exp_pack(const float* v, const float* w, uint64_t scale2, uint64_t negm2, uint32_t* pk, uint64_t (&sum)[2], float (&mx)[2]) {
 #pragma unroll
-  for (int i = 0; i < 32; ++i) {
+  for (int i = 0; i < N / 2; ++i) {
     float x0, x1, p0, p1;
     unpack_f2(fma2(pack_f2(v[2 * i], v[2 * i + 1]), scale2, negm2), x0, x1);
-    if (i & 1) xm1 = max3(xm1, x0, x1); else xm0 = max3(xm0, x0, x1);
+    if (NW > 0) mx[0] = max3(mx[0], v[2 * i], v[2 * i + 1]);
+    if (i < NW / 2) mx[1] = max3(mx[1], w[2 * i], w[2 * i + 1]);
     p0 = ex2(x0);
     p1 = ex2(x1);
-    if (i & 1) sum_b = add2(sum_b, pack_f2(p0, p1)); else sum_a = add2(sum_a, pack_f2(p0, p1));
+    sum[i & 1] = add2(sum[i & 1], pack_f2(p0, p1));
     pk[i] = pack_bf16(p0, p1);
   }
-  x_max = fmaxf(xm0, xm1);
-  float a0, a1;
-  unpack_f2(add2(sum_a, sum_b), a0, a1);
-  return a0 + a1;
+}
+// `mine` of any of the 64 threads of two warps, which meet on barrier `id`.
+__device__ __forceinline__ bool pair_any(int id, bool mine) {
+  int r;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.s32 p, %2, 0;\nbarrier.cta.red.or.pred q, %1, 64, p;\nselp.s32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"(id), "r"((int)mine)
+      : "memory");
+  return r != 0;
 }
 // Largest of the 64 raw scores of a half row.
 __device__ __forceinline__ float max64(const float (&v)[64]) {
@@ -316,7 +326,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
       misc[1] = 0;
       misc[2] = 0;
       for (int i = 0; i < BAR_COUNT; ++i) {
-        mbar_init(bar(i), i >= BAR_P_FULL && i < BAR_P_FULL + 2 ? kSoftmaxWarps / 2 : 1);
+        mbar_init(bar(i), i >= BAR_P_FULL && i < BAR_P_FULL + 4 ? kSoftmaxWarps / 2 : 1);
       }
       mbar_init_fence();
     }
@@ -413,6 +423,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
     float* xchg_other = xchg + (hf ^ 1) * 128 + row;
     int row_g = row / G, row_h = row % G;   // token of the tile and query head of this row
     const float scale = s.scale_log2;
+    const uint64_t scale2 = pack_f2(scale, scale);
     int sx = 0;                 // blocks of this tile in earlier work units: barrier phases follow it
     int n_o = 0;                // earlier work units in which the tile had rows (O_FULL phases)
     for (int k = 0;; ++k) {
@@ -432,6 +443,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
       const int lim = real ? u.ctx + tok + 1 : (x ? u.k_end_b : u.k_end_a);   // keys at positions >= lim are masked
       // the row's place in the output (counted in rows of head_dim), none for a row that is padding
       const uint32_t orow = real ? (uint32_t)(u.tok0 + tok) * s.Hq + u.kv_head * G + row_h : 0xffffffffu;
+      const int lim_min = (int)__reduce_min_sync(0xffffffffu, (unsigned)lim);
       float m_ref = -CUDART_INF_F, l = 0.f;
       for (int j = 0; j < nbx; ++j) {
         wait(BAR_S_FULL + x, (sx + j) & 1);
@@ -439,43 +451,43 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
         // my half of the score row comes into registers: one trip to TMEM per block
         float v[64];
         const int nvalid = lim - j * kBlockKeys - hf * 64;     // keys of my half the row may see
-        auto load_scores = [&]() {
-          tmem_ld32(&v[0], tS);
-          tmem_ld32(&v[32], tS + 32);
-          tmem_ld_wait();
-          if (__any_sync(0xffffffffu, nvalid < 64)) {          // only the blocks on the diagonal
+        tmem_ld32(&v[0], tS);
+        tmem_ld32(&v[32], tS + 32);
+        tmem_ld_wait();
+        if (lim_min - j * kBlockKeys - hf * 64 < 64) {         // only the blocks on the diagonal
 #pragma unroll
-            for (int i = 0; i < 64; ++i)
-              if (i >= nvalid) v[i] = -CUDART_INF_F;           // 2^(-inf) = 0 exactly
-          }
-        };
-        load_scores();
+          for (int i = 0; i < 64; ++i)
+            if (i >= nvalid) v[i] = -CUDART_INF_F;             // 2^(-inf) = 0 exactly
+        }
         // p = 2^(s*scale - m_ref) as bf16, to go over the first 32 columns of my half of S. Any
         // common reference is exact; p <= 2^threshold keeps the bf16 P and the fp32 sums
         // comfortable, so the reference only moves (and O is only rescaled) when the block maximum
-        // exceeds it by more than the threshold. The two threads of a row post the maxima of their
-        // halves (the scale is positive, so it commutes with max) and read the same two numbers,
-        // so they take the same decision. After the first block of a unit the exponentials are
-        // taken at once against the reference the row already has, and the maximum rides along
-        // with them: that is nearly always the final answer. P stays in registers until the
-        // decision is known, so the scores are still in TMEM for a warp with a row that does
-        // move: it fetches them again and takes the exponentials once more. A row of the last,
-        // diagonal block may be masked completely; it keeps its reference (block 0 always holds
-        // key 0, which every row sees).
+        // exceeds it by more than the threshold. After the first block of a unit the first exponentials are
+        // taken at once against the reference the row already has, and the maximum of all 64 scores rides along
+        // with them: that is nearly always the final answer, and one vote of the two warps says so. Where some
+        // row has to move, the two threads of each row post the maxima of their halves (the scale is positive, so it
+        // commutes with max) and see the same two numbers, so they take the same decision; no P has been stored by then,
+        // so the scores are still in TMEM and are fetched once more. A row of the last, diagonal block may be masked
+        // completely; it keeps its reference (block 0 always holds key 0, which every row sees).
         uint32_t pk[32];
-        float ls, x_max;
+        float mx[2] = {-CUDART_INF_F, -CUDART_INF_F};
+        uint64_t sum[2] = {0, 0};
+        uint64_t negm2;
         if (j == 0) {
-          *xchg_mine = max64(v) * scale;                       // first block of a unit: the maximum itself
+          *xchg_mine = max64(v) * scale;
           pair_sync();
           m_ref = fmaxf(*xchg_mine, *xchg_other);
-          ls = exp_pack(v, scale, -m_ref, pk, x_max);
+          negm2 = pack_f2(-m_ref, -m_ref);
+          exp_pack<kFirst>(&v[0], nullptr, scale2, negm2, pk, sum, mx);
         } else {
-          ls = exp_pack(v, scale, -m_ref, pk, x_max);
-          *xchg_mine = x_max + m_ref;                          // largest s*scale of my half
-          pair_sync();
-          const float m_blk = fmaxf(*xchg_mine, *xchg_other);
-          const bool move = m_blk > m_ref + kRescaleThreshold;
-          if (__any_sync(0xffffffffu, move)) {
+          negm2 = pack_f2(-m_ref, -m_ref);
+          exp_pack<kFirst, 64 - kFirst>(&v[0], &v[kFirst], scale2, negm2, pk, sum, mx);
+          const float mine = fmaxf(mx[0], mx[1]) * scale;
+          if (pair_any(4 + x * 4 + (warp & 3), mine > m_ref + kRescaleThreshold)) {
+            *xchg_mine = mine;
+            pair_sync();
+            const float m_blk = fmaxf(mine, *xchg_other);
+            const bool move = m_blk > m_ref + kRescaleThreshold;
             float alpha = 1.f;
             if (move) {
               alpha = ex2(m_ref - m_blk);
@@ -492,17 +504,36 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
               for (int i = 0; i < 16; ++i) ov[i] *= alpha;
               tmem_st16(tO + c * 16, *reinterpret_cast<const uint32_t(*)[16]>(ov));
             }
-            load_scores();
-            ls = exp_pack(v, scale, -m_ref, pk, x_max);
+            tmem_ld32(&v[0], tS);
+            if (kFirst > 32) tmem_ld16(&v[32], tS + 32);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < kFirst; ++i)
+              if (i >= nvalid) v[i] = -CUDART_INF_F;
+            negm2 = pack_f2(-m_ref, -m_ref);
+            sum[0] = sum[1] = 0;
+            exp_pack<kFirst>(&v[0], nullptr, scale2, negm2, pk, sum, mx);
           }
         }
+        // The exponentials of half of the rest hide the time the stores of the first part take.
+        auto announce = [&](int part) {
+          tmem_st_wait();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(BAR_P_FULL + x * 2 + part));
+        };
+        constexpr int kHalfRest = (64 - kFirst) / 2;
         tmem_st16(tS, *reinterpret_cast<const uint32_t(*)[16]>(&pk[0]));
-        tmem_st16(tS + 16, *reinterpret_cast<const uint32_t(*)[16]>(&pk[16]));
-        l += ls;
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(BAR_P_FULL + x));
+        if (kFirst > 32) tmem_st8(tS + 16, &pk[16]);
+        exp_pack<kHalfRest>(&v[kFirst], nullptr, scale2, negm2, pk + kFirst / 2, sum, mx);
+        announce(0);
+        exp_pack<kHalfRest>(&v[kFirst + kHalfRest], nullptr, scale2, negm2, pk + kFirst / 2 + kHalfRest / 2, sum, mx);
+        if (kFirst > 32) tmem_st8(tS + 24, &pk[24]);
+        else tmem_st16(tS + 16, *reinterpret_cast<const uint32_t(*)[16]>(&pk[16]));
+        float s0, s1;
+        unpack_f2(add2(sum[0], sum[1]), s0, s1);
+        l += s0 + s1;
+        announce(1);
       }
       if (nbx > 0) {
         // epilogue: O / l -> bf16 -> global; l is the sum over both halves of the keys. (The last
@@ -798,12 +829,14 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
           }
           tc_commit(bar(BAR_S_FULL + x), issue);
         };
-        auto issue_pv = [&](int x, int stage, bool first) {   // O_x (+)= P_x V
+        auto issue_pv = [&](int x, int stage, int part, bool first) {   // O_x (+)= P_x V, half of the keys
           const uint64_t v_desc = v_desc0 + (uint64_t)((stage * kTileBytes) >> 4);
 #pragma unroll
-          for (int kk = 0; kk < kBlockKeys / 16; ++kk)   // P of keys 0-63 sits in columns 0-31 of S, of keys 64-127 in 64-95
+          for (int kk = 0; kk < kBlockKeys / 16; ++kk) {       // P of keys 0-63 sits in columns 0-31 of S, of keys 64-127 in 64-95
+            if (((kk & 3) < kFirst / 16) != (part == 0)) continue;
             mma_ts(tmem + 256 + x * 128, tmem + x * 128 + (kk >> 2) * 64 + (kk & 3) * 8,
                    v_desc + (uint64_t)((kk * 2048) >> 4), idesc_pv, (!first || kk > 0) ? 1u : 0u, issue);
+          }
         };
         int ks = 0, vs = 0;          // ring stages of the next K tile to be multiplied and of the next V tile
         uint32_t kph = 0, vph = 0;   // and the parities of their "full" phases
@@ -815,7 +848,8 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
           // at once behind it, Q K^T of block j+1 of the same tile, so that the tile's warpgroup gets its
           // next scores while the pipe turns to the other tile. Whatever else the two need (V of block j,
           // K of block j+1) is waited for in front of P: from P to the next scores is the tile's critical
-          // path, and this warp shares its scheduler with four softmax warps. One commit tells of both products,
+          // path, and this warp shares its scheduler with four softmax warps. P comes in two parts, the first of which
+          // is multiplied while the softmax warps take the exponentials of the second. One commit tells of both products,
           // and the warp parks while it waits: the launch runs at the chip's power limit. (Looks at barriers between
           // the products, a commit for each, polling, and arrivals by all lanes of the softmax warps, all together: 8192-token
           // chunk next to 190 rows 1250 us instead of 1237; 2048 tokens alone 45.4 instead of 44.4.)
@@ -839,10 +873,13 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
               if (j >= nbx) continue;
               // P of a unit's first block also says that O is free: the warps that arrive have read the
               // previous unit's O before.
-              iwait(BAR_P_FULL + x, (sxb[x] + j) & 1);
+              iwait(BAR_P_FULL + x * 2, (sxb[x] + j) & 1);
+              tc_fence_after();
+              if (!dead) issue_pv(x, vs, 0, j == 0);
+              iwait(BAR_P_FULL + x * 2 + 1, (sxb[x] + j) & 1);
               tc_fence_after();
               if (dead) continue;
-              issue_pv(x, vs, j == 0);
+              issue_pv(x, vs, 1, j == 0);
               if (j + 1 < nbx) issue_qk(x, ks);
               else tc_commit(bar(BAR_O_FULL + x), issue);
             }
