@@ -320,6 +320,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
     }
     return read_unit(k, u);
   };
+  auto ready = []() { pdl_wait(); };
   // The set-up every warp class runs between the decode phase and the prefill phase.
   auto prefill_setup = [&]() {
     if (tid == 0) {
@@ -366,17 +367,28 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
     reg_dec<kRegsAux>();
     if (decode_first) {
       if (warp == kSoftmaxWarps)
-        dec::decode_schedule<128, 3>(s, smem, base, (int)blockIdx.x - n_prefill_ctas, (int)gridDim.x - n_prefill_ctas, []() {});
-      else
+        dec::decode_schedule<128, 3>(s, smem, base, (int)blockIdx.x - n_prefill_ctas, (int)gridDim.x - n_prefill_ctas, ready);
+      else {
+        ready();
         AppendCursor{n_prefill_ctas * warps_first + ((int)blockIdx.x - n_prefill_ctas) * kWarpsAux + (warp - kSoftmaxWarps - 1),
                      append_end, append_warps}
             .run<8>(s, 2 * tile_tokens, lane);
+      }
       cta_sync();
     }
     prefill_setup();
   };
 
-  pdl_wait();                  // the previous step's kernels are done with the pool and the counters
+  // The launch in front of this one (the previous step's kernels, which must be done with the pool and the counters) is
+  // waited for as late as can be: a CTA's barriers, TMEM and, where the step's metadata are launch parameters, its
+  // first decode unit are set up before.
+  if (decode_first && s.meta) ready();
+  if (tid == kSoftmaxWarps * 32) {
+    tma_prefetch_desc(&q_map);
+    tma_prefetch_desc(&kv_tile_map);
+    tma_prefetch_desc(&new_maps.k);
+    tma_prefetch_desc(&new_maps.v);
+  }
 
   if (warp < kSoftmaxWarps) {
     // ------------------ softmax + epilogue: thread = half of a query row of tile x (64 of the 128
@@ -384,7 +396,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
     if (decode_first) {
       if (warp < 8) {
         reg_inc<kRegsDecode>();       // waits until the parked warpgroups have given their registers up
-        dec::decode_units<128, 1, 3>(s, &kv_map, smem, base, []() {});
+        dec::decode_units<128, 1, 3>(s, &kv_map, smem, base, ready);
         if (tid == 0) {          // this CTA's split partials are written: count it as done
           __threadfence();
           atomicAdd(s.pf_queue + 1, 1);
@@ -401,6 +413,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
       reg_inc<kRegsSoftmax>();
     }
     prefill_setup();
+    ready();
     if (!decode_first && s.append_wide)
       AppendCursor{(int)blockIdx.x * kSoftmaxWarps + warp, append_end, append_warps}.run<8>(s, 2 * tile_tokens, lane);
     const uint32_t tmem = misc[0];
@@ -668,10 +681,6 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
       const int full = kv ? BAR_V_FULL : BAR_K_FULL, empty = kv ? BAR_V_EMPTY : BAR_K_EMPTY;
       const uint32_t tile0 = base + (kv ? kOffV : kOffK);
       const CUtensorMap* new_map = kv ? &new_maps.v : &new_maps.k;
-      if (lane == 0) {
-        tma_prefetch_desc(new_map);
-        tma_prefetch_desc(&kv_tile_map);
-      }
       int n_touched = 0;                                       // K tiles that went through BAR_K_LANDED
       // The K loader's first thread takes work units off the global queue, one at a time and only
       // when the K loader is ready for it (it runs a few key blocks ahead of the tensor pipe, which
@@ -703,10 +712,15 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
         __threadfence_block();
         misc[2] = (uint32_t)++fetched;
       };
+      // A first unit that the launch parameters tell is published before the wait: the reads that describe it
+      // are a chain, and cold (1.1 us in front of the first copies of 2048 tokens alone).
+      const bool first_early = !decode_first && !s.meta;
+      if (first_early && kv == 0 && lane == 0) fetch_one();
+      ready();
       int g0 = 0;                                              // key blocks of earlier work units
       int n_copied = 0;                                        // tiles whose copies were started: the first n_copied ones
       for (int k = 0;; ++k) {
-        if (kv == 0 && lane == 0) fetch_one();
+        if (kv == 0 && lane == 0 && !(first_early && k == 0)) fetch_one();
         __syncwarp();
         PfUnit u;
         if (!get_work(k, u)) break;
@@ -903,7 +917,7 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
         // ------------------------------------------------------------------ Q loader
         // Brings in each work unit's Q tiles by TMA once the previous unit's last Q K^T is done.
         // Between two units it appends, a token at a time, this CTA's share of the new K/V.
-        if (lane == 0) tma_prefetch_desc(&q_map);
+        ready();
         AppendCursor app{decode_first || s.append_wide ? append_end : (int)blockIdx.x, append_end, append_warps};
         auto append_until = [&](auto&& ready) {
           while (!app.done() && !__any_sync(0xffffffffu, ready())) app.step<4>(s, 2 * tile_tokens, lane);   // 4: 64 registers here
