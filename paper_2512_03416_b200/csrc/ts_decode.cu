@@ -8,9 +8,10 @@ namespace {
 
 using dec::kDecThreads;
 
-template <int D, int NH, int STAGES>
+template <int D, int NH, int STAGES, int W>
 __global__ void __launch_bounds__(kDecThreads + 32, 1)
-decode_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUtensorMap kv_map) {
+decode_kernel(const __grid_constant__ StepParams<W> params, const __grid_constant__ CUtensorMap kv_map) {
+  const StepDevice& s = params.s;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
@@ -39,16 +40,26 @@ decode_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUte
   }
 }
 
-template <int D, int NH, int STAGES>
-cudaError_t launch_decode_t(const StepDevice& s, const CUtensorMap& map, int n_sms, cudaStream_t stream) {
+template <int D, int NH, int STAGES, int W>
+cudaError_t launch_decode_w(const StepDevice& s, const CUtensorMap& map, int n_sms, cudaStream_t stream) {
   const int G = s.Hq / s.Hkv;
   const size_t smem = 1024 + dec::decode_smem_bytes<D, STAGES>(G);
-  cudaError_t e = cudaFuncSetAttribute(decode_kernel<D, NH, STAGES>,
+  cudaError_t e = cudaFuncSetAttribute(decode_kernel<D, NH, STAGES, W>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const long long units = (long long)(s.n_items - s.n_prefill_items) * s.Hkv;
   const int grid = (int)(units < n_sms ? units : n_sms);
-  return launch_pdl(decode_kernel<D, NH, STAGES>, dim3(grid), dim3(kDecThreads + 32), smem, stream, s, map);
+  StepParams<W> params;
+  fill_params(s, &params);
+  return launch_pdl(decode_kernel<D, NH, STAGES, W>, dim3(grid), dim3(kDecThreads + 32), smem, stream, params, map);
+}
+template <int D, int NH, int STAGES>
+cudaError_t launch_decode_t(const StepDevice& s, const CUtensorMap& map, int n_sms, cudaStream_t stream) {
+  if (s.n_words <= kInlineWords) return launch_decode_w<D, NH, STAGES, kInlineWords>(s, map, n_sms, stream);
+  if constexpr (D == 128 && NH == 1)
+    return s.n_words <= kInlineWordsMid ? launch_decode_w<D, NH, STAGES, kInlineWordsMid>(s, map, n_sms, stream)
+                                        : launch_decode_w<D, NH, STAGES, kInlineWordsMax>(s, map, n_sms, stream);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace

@@ -128,6 +128,7 @@ struct ts_ctx {
   int ring_next = 0;
   size_t ring_bytes = 0;
   MetaSlot meta[kRing];             // step metadata
+  std::vector<int32_t> words;       // the metadata of the step that is being enqueued, where it travels with its launches
   int meta_next = 0;
   int meta_cur = 0;                 // slot of the step being issued
   cudaStream_t copy_stream = nullptr;
@@ -484,21 +485,31 @@ void pack_meta(const ts_ctx* c, const ts_step* st, const ts::StepDevice& d, int 
   if (n_combines > 0) std::memcpy(dst + d.o_combines, c->combines.data(), sizeof(CombineItem) * n_combines);
 }
 
-// Brings the step's metadata and its block-table entries to the kernels. Small metadata (at most
-// ts::kInlineWords words) travels inside the step's launch parameters, few table entries inside the
+// Brings the step's metadata and its block-table entries to the kernels. The metadata of most steps
+// travels inside the launch parameters (as many words as the step's kernels take), few table entries inside the
 // parameters of the launch that applies them; what is larger goes to the next device slot over the
 // context's copy stream: that copy only has to wait for the step that last read the slot (kRing steps
 // ago), so it runs while the previous step's kernels are still busy, and the caller's stream just
 // waits for its event.
 int send_meta(ts_ctx* c, const ts_step* st, int n_items, int n_combines, int n_slot_deltas, cudaStream_t stream, ts::StepDevice* d) {
   const size_t used = meta_offsets(st->n_rows, n_items, n_combines, d);
-  const bool inline_meta = used <= (size_t)ts::kInlineWords;
+  // the decode and mixed kernels are there for larger parameters, the merge's list has to fit into the smaller ones
+  const bool large = n_items > 0 && c->cfg.head_dim == 128 && c->G <= 8 &&
+                     n_combines * (int)(sizeof(CombineItem) / sizeof(int32_t)) <= ts::kInlineWords;
+  const bool inline_meta = used <= (size_t)(large ? ts::kInlineWordsMax : ts::kInlineWords);
   const bool inline_deltas = n_slot_deltas <= ts::kInlineDeltas;
   char* ws = (char*)c->cfg.workspace;
   c->meta_cur = -1;
   d->meta = nullptr;
   d->meta_in_place = 1;
-  if (inline_meta) pack_meta(c, st, *d, n_items, n_combines, d->words);
+  d->n_words = 0;
+  d->host_words = nullptr;
+  if (inline_meta) {
+    c->words.resize(ts::kInlineWordsMax);
+    pack_meta(c, st, *d, n_items, n_combines, c->words.data());
+    d->n_words = (int32_t)used;
+    d->host_words = c->words.data();
+  }
   if (!inline_meta || !inline_deltas) {
     const int slot = c->meta_next;
     c->meta_next = (c->meta_next + 1) % kRing;

@@ -7,6 +7,8 @@
 
 #include "../../include/tokenscale.h"
 
+#include <cstddef>
+#include <cstring>
 #include <utility>
 
 namespace ts {
@@ -45,7 +47,13 @@ struct TableDelta {
   int32_t slot, index, page;
 };
 
-constexpr int kInlineWords = 768;   // 3 KB: with the tensor maps the mixed kernel's parameters stay within 4 KB
+// Words of row arrays and work list that travel as launch parameters. Every kernel takes up to kInlineWords (3 KB: with
+// its other parameters that stays within 4 KB), the mixed kernel and the decode kernel of head_dim 128 with up to eight
+// heads per KV head are there for larger steps as well (parameters end at 32764 bytes). A launch with 3 KB of
+// parameters costs the host 2.4 us, with 8 KB 2.7, 16 KB 3.7, 30 KB 5 to 11; an upload on the copy stream, its event and the
+// wait for it 4.8 with the launch. The wait also ends the overlap with the launch in front: next to a 2048-token chunk a
+// step's first thread blocks started 5.7 us after the last one of the step before had left, 1.7 without.
+constexpr int kInlineWords = 768, kInlineWordsMid = 3072, kInlineWordsMax = 7680;
 // One step as its kernels see it; device pointers lie in the caller's workspace unless noted.
 struct StepDevice {
   // static
@@ -73,17 +81,18 @@ struct StepDevice {
   long long unit_wait_cycles;
   int32_t append_wide;     // mixed kernel: CTAs that start on prefill units append with their softmax warps first
   int32_t debug_arrivals;  // decode CTAs besides the launch's own that the mixed kernel's merge waits for (TS_DEBUG_LOSE_APPEND_ARRIVAL)
-  // The step's row arrays and work list: word offsets from `meta`, a device address, or, where they
-  // are small, from `words`: they then travel as launch parameters, without an upload of their own (a copy
+  // The step's row arrays and work list: word offsets from `meta`, a device address, or, unless they
+  // are large, from the words behind this struct in the launch parameters (StepParams): no upload of their own (a copy
   // on another stream, two event records and two waits: ~6 us of host time and a dependency per step).
-  const int32_t* meta;     // null: `words`
+  const int32_t* meta;     // null: the words behind this struct
   // Whether a launch behind the step's first reading one may read them before it waits for the launch in front: they are
   // launch parameters, or the stream waited for their upload before the first launch that reads them. Not where a kernel plans the step.
   int32_t meta_in_place;
   uint32_t o_slot, o_ctx, o_tok0, o_items, o_combines;
-  int32_t words[kInlineWords];
+  int32_t n_words;             // for the launchers: words in host memory that travel with the launch (none where meta is set)
+  const int32_t* host_words;
 #ifdef __CUDACC__
-  __device__ __forceinline__ const int32_t* at(uint32_t o) const { return (meta ? meta : words) + o; }
+  __device__ __forceinline__ const int32_t* at(uint32_t o) const { return (meta ? meta : reinterpret_cast<const int32_t*>(this + 1)) + o; }
   __device__ __forceinline__ int32_t row_slot(int r) const { return at(o_slot)[r]; }
   __device__ __forceinline__ int32_t row_ctx(int r) const { return at(o_ctx)[r]; }
   __device__ __forceinline__ int32_t row_tok0(int r) const { return at(o_tok0)[r]; }   // [n_rows + 1] prefix sums of the new tokens
@@ -91,6 +100,19 @@ struct StepDevice {
   __device__ __forceinline__ CombineItem combine(int i) const { return reinterpret_cast<const CombineItem*>(at(o_combines))[i]; }
 #endif
 };
+
+// A step as a launch parameter.
+template <int W>
+struct StepParams {
+  StepDevice s;
+  int32_t words[W];
+};
+static_assert(offsetof(StepParams<kInlineWords>, words) == sizeof(StepDevice), "the words follow the step");
+template <int W>
+inline void fill_params(const StepDevice& s, StepParams<W>* p) {
+  p->s = s;
+  if (s.n_words > 0) std::memcpy(p->words, s.host_words, sizeof(int32_t) * (size_t)s.n_words);
+}
 
 // Launchers. Each enqueues on `stream` and returns the launch's cudaError_t.
 cudaError_t launch_table_update(int32_t* table, int max_pages_per_req, int max_requests, int32_t* status,

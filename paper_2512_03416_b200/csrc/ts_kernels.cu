@@ -53,7 +53,8 @@ __global__ void table_update_inline_kernel(int32_t* table, int width, int max_re
 }
 
 // KV append as a launch of its own (ts_kv_append): one warp per new token at a time, see append_tokens.
-__global__ void kv_append_kernel(const __grid_constant__ StepDevice s) {
+__global__ void kv_append_kernel(const __grid_constant__ StepParams<kInlineWords> params) {
+  const StepDevice& s = params.s;
   extern __shared__ int32_t rows[];             // staged row arrays, see stage_rows
   pdl_launch_dependents();
   pdl_wait();
@@ -64,7 +65,8 @@ __global__ void kv_append_kernel(const __grid_constant__ StepDevice s) {
 }
 
 // Merge of the splits of one token: grid (n_combines, Hq), block D threads.
-__global__ void combine_kernel(const __grid_constant__ StepDevice s) {
+__global__ void combine_kernel(const __grid_constant__ StepParams<kInlineWords> params) {
+  const StepDevice& s = params.s;
   pdl_launch_dependents();
   // Metadata that were in place before the decode launch started are read before the wait for its end: one round
   // trip less behind it (device time of a step, prepared steps back to back, read behind the wait and so, us: four
@@ -204,7 +206,8 @@ __device__ __forceinline__ void warp_tile(uint32_t sK, uint32_t sV, int key_row0
 }
 
 template <int D>
-__global__ void __launch_bounds__(kThreads, 2) attention_kernel(const __grid_constant__ StepDevice s) {
+__global__ void __launch_bounds__(kThreads, 2) attention_kernel(const __grid_constant__ StepParams<kInlineWords> params) {
+  const StepDevice& s = params.s;
   extern __shared__ __align__(128) unsigned char smem[];
   pdl_launch_dependents();
   pdl_wait();
@@ -378,7 +381,9 @@ cudaError_t launch_attention_d(const StepDevice& s, cudaStream_t stream) {
   constexpr int smem = smem_pipe > smem_merge ? smem_pipe : smem_merge;
   cudaError_t e = cudaFuncSetAttribute(attention_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(attention_kernel<D>, dim3(s.n_items, s.Hkv), dim3(kThreads), smem, stream, s);
+  StepParams<kInlineWords> params;
+  fill_params(s, &params);
+  return launch_pdl(attention_kernel<D>, dim3(s.n_items, s.Hkv), dim3(kThreads), smem, stream, params);
 }
 
 }  // namespace
@@ -402,7 +407,9 @@ cudaError_t launch_kv_append(const StepDevice& s, cudaStream_t stream) {
   const int threads = 256;                                    // eight warps = eight tokens per block at a time
   const int blocks = (s.n_tokens + 7) / 8;
   const int grid = blocks < 148 * 8 ? blocks : 148 * 8;
-  return launch_pdl(kv_append_kernel, dim3(grid), dim3(threads), staged_rows_bytes(s.n_rows), stream, s);
+  StepParams<kInlineWords> params;
+  fill_params(s, &params);
+  return launch_pdl(kv_append_kernel, dim3(grid), dim3(threads), staged_rows_bytes(s.n_rows), stream, params);
 }
 
 cudaError_t launch_attention(const StepDevice& s, cudaStream_t stream) {
@@ -412,7 +419,18 @@ cudaError_t launch_attention(const StepDevice& s, cudaStream_t stream) {
 
 cudaError_t launch_combine(const StepDevice& s, cudaStream_t stream) {
   if (s.n_combines <= 0) return cudaSuccess;
-  return launch_pdl(combine_kernel, dim3(s.n_combines, s.Hq), dim3(s.D), 0, stream, s);
+  StepParams<kInlineWords> params;
+  if (s.meta) {
+    fill_params(s, &params);
+  } else {                                                    // of the words it reads the merge list alone
+    StepDevice c = s;
+    c.host_words = s.host_words + s.o_combines;
+    c.n_words = s.n_combines * (int)(sizeof(CombineItem) / sizeof(int32_t));
+    c.o_combines = 0;
+    if (c.n_words > kInlineWords) return cudaErrorInvalidValue;
+    fill_params(c, &params);
+  }
+  return launch_pdl(combine_kernel, dim3(s.n_combines, s.Hq), dim3(s.D), 0, stream, params);
 }
 
 }  // namespace ts
@@ -540,6 +558,8 @@ extern "C" int ts_decode_attention_static(int32_t device, int32_t n_q_heads, int
   d.part_acc = sc->part_acc;
   d.part_ml = sc->part_ml;
   d.meta = (const int32_t*)sc;
+  d.n_words = 0;
+  d.host_words = nullptr;
   d.meta_in_place = 0;                    // static_plan_kernel writes them in front of the attention kernel
   d.o_slot = offsetof(StaticScratch, row_slot) / 4;
   d.o_ctx = offsetof(StaticScratch, row_ctx) / 4;

@@ -259,10 +259,12 @@ struct AppendCursor {
 
 __device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 0;\n" ::: "memory"); }
 
+template <int W>
 __global__ void __launch_bounds__(kPfThreads, 1)
-mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUtensorMap q_map,
+mixed_kernel(const __grid_constant__ StepParams<W> params, const __grid_constant__ CUtensorMap q_map,
              const __grid_constant__ CUtensorMap kv_map, const __grid_constant__ CUtensorMap kv_tile_map,
              const __grid_constant__ NewKvMaps new_maps, const int n_prefill_ctas) {
+  const StepDevice& s = params.s;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
@@ -967,10 +969,9 @@ mixed_kernel(const __grid_constant__ StepDevice s, const __grid_constant__ CUten
   }
 }
 
-}  // namespace
-
-cudaError_t launch_mixed(const StepDevice& s, const CUtensorMap& q_map, const CUtensorMap& kv_map,
-                         const CUtensorMap& kv_tile_map, const NewKvMaps& new_maps, int n_ctas, int n_prefill_ctas, cudaStream_t stream) {
+template <int W>
+cudaError_t launch_mixed_w(const StepDevice& s, const CUtensorMap& q_map, const CUtensorMap& kv_map,
+                           const CUtensorMap& kv_tile_map, const NewKvMaps& new_maps, int n_ctas, int n_prefill_ctas, cudaStream_t stream) {
   if (s.n_prefill_items <= 0 || n_ctas <= 0) return cudaSuccess;
   const int G = s.Hq / s.Hkv;
   size_t smem = kSmemBytes;
@@ -978,9 +979,21 @@ cudaError_t launch_mixed(const StepDevice& s, const CUtensorMap& q_map, const CU
     const size_t dec_smem = 1024 + dec::decode_smem_bytes<128, 3>(G);
     if (dec_smem > smem) smem = dec_smem;
   }
-  cudaError_t e = cudaFuncSetAttribute(mixed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(mixed_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(mixed_kernel, dim3(n_ctas), dim3(kPfThreads), smem, stream, s, q_map, kv_map, kv_tile_map, new_maps, n_prefill_ctas);
+  StepParams<W> params;
+  fill_params(s, &params);
+  return launch_pdl(mixed_kernel<W>, dim3(n_ctas), dim3(kPfThreads), smem, stream, params, q_map, kv_map, kv_tile_map, new_maps, n_prefill_ctas);
+}
+
+}  // namespace
+
+cudaError_t launch_mixed(const StepDevice& s, const CUtensorMap& q_map, const CUtensorMap& kv_map,
+                         const CUtensorMap& kv_tile_map, const NewKvMaps& new_maps, int n_ctas, int n_prefill_ctas, cudaStream_t stream) {
+  const auto launch = s.n_words <= kInlineWords      ? launch_mixed_w<kInlineWords>
+                      : s.n_words <= kInlineWordsMid ? launch_mixed_w<kInlineWordsMid>
+                                                     : launch_mixed_w<kInlineWordsMax>;
+  return launch(s, q_map, kv_map, kv_tile_map, new_maps, n_ctas, n_prefill_ctas, stream);
 }
 
 }  // namespace ts
