@@ -1,5 +1,6 @@
 // Stand-alone split-KV flash-decode kernel for the 1-token rows (sm_100a): one persistent CTA
-// per SM running dec::decode_units and its scheduler (ts_decode_body.h) over all decode units of the step.
+// per SM running dec::decode_units and its scheduler (ts_decode_body.h) over all decode units of the step. The schedulers
+// also merge the rows that were split.
 // The units also append the rows' new K/V.
 #include "ts_decode_body.h"
 
@@ -26,9 +27,9 @@ decode_kernel(const __grid_constant__ StepParams<W> params, const __grid_constan
   auto ready = [&]() { pdl_wait(); };
   if (s.meta) ready();
   if (threadIdx.x < kDecThreads) {
-    dec::decode_units<D, NH, STAGES>(s, &kv_map, smem, base, ready);
+    dec::decode_units<D, NH, STAGES, true>(s, &kv_map, smem, base, ready);
   } else {
-    dec::decode_schedule<D, STAGES>(s, smem, base, blockIdx.x, gridDim.x, ready);
+    dec::decode_schedule<D, STAGES, true>(s, smem, base, blockIdx.x, gridDim.x, ready);
     if (threadIdx.x == kDecThreads) {
       // the last scheduler to get here puts the queue back to zero for the next launch
       __threadfence();

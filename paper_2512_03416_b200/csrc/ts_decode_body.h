@@ -72,9 +72,11 @@ struct UnitInfo {
   int partial_slot;
   int tok, new_pos;       // token of the row in the step's tensors, position of the row's new token
   const int32_t* table_row;
-  int64_t pad;
+  int combine;            // of a split row: its CombineItem, and what that says
+  CombineItem merge;
+  int pad;
 };
-static_assert(sizeof(UnitInfo) == 48, "UnitInfo is three 16-byte chunks");
+static_assert(sizeof(UnitInfo) == 64, "UnitInfo is four 16-byte chunks");
 
 // Shared memory: page stages, partial results of the warps, unit descriptions, mbarriers, failure flag.
 template <int D, int STAGES>
@@ -87,7 +89,8 @@ struct DecSmem {
   // partial results written, partial results added up, unit nearly fetched
   static constexpr int kBarDesc = kDecWarps * STAGES, kBarDone = kBarDesc + kDecRing, kBarWritten = kBarDone + kDecRing,
                        kBarAdded = kBarWritten + 1, kBarNear = kBarAdded + 1, kBars = kBarNear + 1;
-  __host__ __device__ static constexpr int off_failed(int G) { return off_bars(G) + kBars * 8; }
+  __host__ __device__ static constexpr int off_merges(int G) { return off_bars(G) + kBars * 8; }   // entries of the ring for merge_by_all
+  __host__ __device__ static constexpr int off_failed(int G) { return off_merges(G) + kDecRing * 4; }
 };
 template <int D, int STAGES>
 __host__ __device__ constexpr size_t decode_smem_bytes(int G) {
@@ -116,10 +119,114 @@ __device__ __forceinline__ void give_up(const StepDevice& s, volatile int* faile
   __syncwarp();
 }
 
+// Merge of a row's splits, by one warp: the log-sum-exp merge of merge_splits for `n_heads` heads from head0 on, 32 * E of
+// their columns from col0 on. The loads of HEADS heads x SPLITS splits fly at a time.
+template <int D, int E, int HEADS, int SPLITS>
+__device__ __forceinline__ void merge_heads(const StepDevice& s, const CombineItem& c, int head0, int n_heads, int col0, int lane) {
+  const int col = col0 + lane * E;
+  const float* ml = s.part_ml + ((size_t)c.first_partial * s.Hq + head0) * 2;
+  const float* pa = s.part_acc + ((size_t)c.first_partial * s.Hq + head0) * D + col;
+  const size_t ml_stride = (size_t)s.Hq * 2, pa_stride = (size_t)s.Hq * D;
+#pragma unroll 1
+  for (int h0 = 0; h0 < n_heads; h0 += HEADS) {
+    float m[HEADS], l[HEADS], acc[HEADS][E];
+#pragma unroll
+    for (int h = 0; h < HEADS; ++h) {
+      m[h] = -CUDART_INF_F;
+      l[h] = 0.f;
+#pragma unroll
+      for (int e = 0; e < E; ++e) acc[h][e] = 0.f;
+    }
+#pragma unroll 1
+    for (int b0 = 0; b0 < c.n_splits; b0 += SPLITS) {
+      float2 st[HEADS][SPLITS];
+      float a[HEADS][SPLITS][E];
+#pragma unroll
+      for (int h = 0; h < HEADS; ++h)
+#pragma unroll
+        for (int j = 0; j < SPLITS; ++j) {
+          const bool on = b0 + j < c.n_splits && h0 + h < n_heads;
+          const float* src = pa + (b0 + j) * pa_stride + (h0 + h) * D;
+          st[h][j] = on ? __ldcg(reinterpret_cast<const float2*>(ml + (b0 + j) * ml_stride + (h0 + h) * 2)) : make_float2(-CUDART_INF_F, 0.f);
+          if constexpr (E == 4) {
+            const float4 v = on ? __ldcg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            a[h][j][0] = v.x; a[h][j][1] = v.y; a[h][j][2] = v.z; a[h][j][3] = v.w;
+          } else {
+            const float2 v = on ? __ldcg(reinterpret_cast<const float2*>(src)) : make_float2(0.f, 0.f);
+            a[h][j][0] = v.x; a[h][j][1] = v.y;
+          }
+        }
+#pragma unroll
+      for (int h = 0; h < HEADS; ++h) {
+        if (h0 + h >= n_heads) continue;               // no arithmetic on the infinities of heads that are not there
+        float mn = m[h];
+#pragma unroll
+        for (int j = 0; j < SPLITS; ++j) mn = fmaxf(mn, st[h][j].x);
+        const float keep = exp2f(m[h] - mn);           // 0 on the first group (m = -inf)
+        l[h] *= keep;
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[h][e] *= keep;
+#pragma unroll
+        for (int j = 0; j < SPLITS; ++j) {
+          const float w = exp2f(st[h][j].x - mn);      // absent split: exp2(-inf) = 0
+          l[h] += w * st[h][j].y;
+#pragma unroll
+          for (int e = 0; e < E; ++e) acc[h][e] += w * a[h][j][e];
+        }
+        m[h] = mn;
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < HEADS; ++h) {
+      if (h0 + h >= n_heads) continue;
+      uint32_t* dst = reinterpret_cast<uint32_t*>(s.out + ((size_t)c.token * s.Hq + head0 + h0 + h) * D + col);
+#pragma unroll
+      for (int e = 0; e < E; e += 2) dst[e / 2] = pack_bf16(acc[h][e] / l[h], acc[h][e + 1] / l[h]);
+    }
+  }
+}
+// Rows that were split. A unit whose eight warps have all written their shares is counted by the scheduler warp; whoever
+// counts the last split of a (row, KV head) merges it: the scheduler warp itself while its CTA still streams, all
+// streaming warps for the CTA's last units, where the merge is what the launch ends with. (Counted and merged by the
+// streaming warps, the fence and the counter's round trip stopped the page stream.) A launch with one unit per CTA at
+// most leaves the merge to a launch of its own, whose blocks merge a head each. Device time of a step, merged by that
+// launch / here, us: 64 rows 122.7 / 120.5, 203 rows of the 70B shape 224.3 / 221.1, but four rows of ~1500 keys 9.9 / 10.4:
+// fence, count and merge are one behind the other at the end of the only unit.
+// True, for the whole warp, when this was the last split.
+__device__ __forceinline__ bool count_split(const StepDevice& s, int combine, int n_splits, int kv_head, int lane) {
+  int last = 0;
+  if (lane == 0) {
+    int32_t* count = s.merge_count + (size_t)combine * s.Hkv + kv_head;
+    int before;
+    // releases the unit's results, which this warp has seen through the unit's barrier, and acquires the other splits'
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;\n" : "=r"(before) : "l"(count) : "memory");
+    last = before == n_splits - 1;
+    if (last) *count = 0;                              // for the next launch
+  }
+  return __shfl_sync(0xffffffffu, last, 0);
+}
+template <int D>
+__device__ __forceinline__ void merge_by_scheduler(const StepDevice& s, const CombineItem& c, int kv_head, int lane) {
+  const int G = s.Hq / s.Hkv;
+  merge_heads<D, D / 32, 2, 4>(s, c, kv_head * G, G, 0, lane);
+}
+// Warp `warp` of the kDecWarps streaming warps: a head or half a head at a time, so that all have something to do.
+template <int D>
+__device__ __forceinline__ void merge_by_all(const StepDevice& s, const CombineItem& c, int kv_head, int warp, int lane) {
+  const int G = s.Hq / s.Hkv;
+  if (D == 64 || G <= kDecWarps / 2) {
+    for (int i = warp; i < G * (D / 64); i += kDecWarps)
+      merge_heads<D, 2, 1, 16>(s, c, kv_head * G + i / (D / 64), 1, i % (D / 64) * 64, lane);
+  } else {
+    for (int i = warp; i < G; i += kDecWarps) merge_heads<D, D / 32, 1, 8>(s, c, kv_head * G + i, 1, 0, lane);
+  }
+}
+
 // Scheduler warp of CTA `cta` of `n_ctas`: its first unit is unit `cta`, the others come off the queue
 // s.pf_queue[3], which the launch leaves at zero.
-// `ready` waits for the launch in front of this one: called once the first unit is described.
-template <int D, int STAGES, typename Ready>
+// `ready` waits for the launch in front of this one: called once the first unit is described. MERGE: the warp also merges
+// the rows that were split (count_split), a unit once the entry of the ring it was described in is free.
+template <int D, int STAGES, bool MERGE, typename Ready>
 __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned char* smem, uint32_t base, int cta, int n_ctas, Ready&& ready) {
   using L = DecSmem<D, STAGES>;
   const int lane = threadIdx.x & 31, G = s.Hq / s.Hkv;
@@ -129,6 +236,8 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
   volatile int* failed = reinterpret_cast<volatile int*>(smem + L::off_failed(G));
   decode_meet();
   bool ok = true;
+  const bool merging = MERGE && merges_splits(n_units, n_ctas);
+  int n_described = 0, n_finished = 0;
   for (int k = 0;; ++k) {
     const int e = k % kDecRing;
     int unit = cta;
@@ -147,6 +256,10 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
       u.k_begin = it.k_begin;
       u.k_end = it.k_end;
       u.partial_slot = it.partial_slot;
+      if (merging && it.partial_slot >= 0) {
+        u.combine = it.combine;
+        u.merge = s.combine(it.combine);
+      }
       u.first_page = it.k_begin >> 4;
       u.n_pg = (it.k_end - it.k_begin + kPageSize - 1) >> 4;
       u.tok = s.row_tok0(it.row);
@@ -155,6 +268,17 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
     }
     if (k >= kDecRing) ok = wait_for_warps(bars + (L::kBarDone + e) * 8, ((k / kDecRing) & 1) ^ 1, failed, s.unit_wait_cycles);
     if (!ok) break;              // the entry may still be read: the streaming warps end by the failure flag
+    bool split_done = false;                           // the unit whose entry this is going to be was a split: it is counted below
+    int done_combine = 0, done_head = 0;
+    CombineItem done_merge = {};
+    if (merging && k >= kDecRing) {
+      split_done = ring[e].partial_slot >= 0;
+      done_combine = ring[e].combine;
+      done_head = ring[e].head;
+      done_merge = ring[e].merge;
+      n_finished = k - kDecRing + 1;
+    }
+    __syncwarp();
     if (lane == 0) {
       ring[e] = u;
       mbar_arrive(bars + (L::kBarDesc + e) * 8);
@@ -169,7 +293,21 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
       for (int i = lane * 8; i < G * D / 2; i += 256) touched ^= __ldca(q + i);
     }
     asm volatile("" ::"r"(touched));
+    if (split_done && count_split(s, done_combine, done_merge.n_splits, done_head, lane))
+      merge_by_scheduler<D>(s, done_merge, done_head, lane);
     if (u.n_pg < 0) break;
+    n_described = k + 1;
+  }
+  if (merging) {
+    int* merges = reinterpret_cast<int*>(smem + L::off_merges(G));
+    if (lane < kDecRing) merges[lane] = -1;
+    __syncwarp();
+    for (int k = n_finished; ok && k < n_described; ++k) {
+      const int e = k % kDecRing;
+      ok = wait_for_warps(bars + (L::kBarDone + e) * 8, (k / kDecRing) & 1, failed, s.unit_wait_cycles);
+      if (ok && ring[e].partial_slot >= 0 && count_split(s, ring[e].combine, ring[e].merge.n_splits, ring[e].head, lane))
+        merges[k - n_finished] = e;
+    }
   }
   if (!ok) give_up(s, failed);
   decode_meet();                 // from here on nobody looks at a barrier of the path
@@ -179,7 +317,7 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
 // (the scheduler runs on another warp at the same time). `smem` is the 1024-byte-aligned shared-memory
 // window (decode_smem_bytes<D, STAGES>(G) bytes), `base` its shared-space address. `ready` waits for the launch
 // in front of this one, once the barriers are set up. The function leaves no copy in flight when it returns.
-template <int D, int NH, int STAGES, typename Ready>
+template <int D, int NH, int STAGES, bool MERGE, typename Ready>
 __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensorMap* kv_map, unsigned char* smem,
                                              uint32_t base, Ready&& ready) {
   using L = DecSmem<D, STAGES>;
@@ -513,6 +651,11 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
   if (dead) give_up(s, failed);
   for (; n_consumed < n_issued; ++n_consumed) mbar_wait(my_bars + (n_consumed % STAGES) * 8, (n_consumed / STAGES) & 1, kDrainCycles);
   decode_meet();               // the scheduler included: then the barriers' shared memory can be given back
+  if (MERGE && merges_splits((s.n_items - s.n_prefill_items) * s.Hkv, (int)gridDim.x)) {
+    const int* merges = reinterpret_cast<const int*>(smem + L::off_merges(G));
+    for (int i = 0; i < kDecRing; ++i)
+      if (merges[i] >= 0) merge_by_all<D>(s, units[merges[i]].merge, units[merges[i]].head, warp, lane);
+  }
   if (tid == 0) {
     for (int i = 0; i < L::kBars; ++i) asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(bar(i)) : "memory");
   }

@@ -35,7 +35,7 @@ constexpr int kStageSets = 3;   // staging sets of ts_mixed_step_host: one step 
 struct Layout {
   int max_tokens, max_partials, max_items;
   size_t off_status, off_table, off_meta, off_delta, off_part_acc, off_part_ml, off_stage;
-  size_t meta_bytes, slot_bytes, delta_bytes, stage_q_bytes, stage_kv_bytes, stage_set_bytes, total;
+  size_t status_bytes, meta_bytes, slot_bytes, delta_bytes, stage_q_bytes, stage_kv_bytes, stage_set_bytes, total;
 };
 
 bool shape_ok(const ts_config* c) {
@@ -61,7 +61,8 @@ void compute_layout(const ts_config* c, Layout* L) {
   L->meta_bytes = align_up(m * sizeof(int32_t));
   L->delta_bytes = align_up((size_t)kDeltaCapacity * sizeof(TableDelta));
   size_t off = 0;
-  L->off_status = off; off += kAlign;
+  L->status_bytes = kAlign + align_up((size_t)R * c->n_kv_heads * sizeof(int32_t));   // and the kernels' counters
+  L->off_status = off; off += L->status_bytes;
   L->off_table = off; off += align_up((size_t)R * c->max_pages_per_req * sizeof(int32_t));
   // one slot per step in flight: the step's metadata, then up to kSlotDeltas block-table entries
   L->slot_bytes = L->meta_bytes + align_up((size_t)kSlotDeltas * sizeof(TableDelta));
@@ -150,6 +151,7 @@ struct ts_ctx {
   // scratch reused across steps
   std::vector<WorkItem> items;
   std::vector<CombineItem> combines;
+  std::vector<int32_t> combine_of;                       // index into combines, by partial slot
   std::vector<int32_t> tok0;
   std::vector<TableDelta> deltas;
   std::vector<std::pair<int32_t, int32_t>> sync_marks;   // (slot, table entries the device will hold)
@@ -273,7 +275,7 @@ int ensure_cuda(ts_ctx* c, cudaStream_t stream) {
     c->cuda_ready = true;
   }
   if (!c->status_cleared) {
-    TS_CUDA(c, cudaMemsetAsync((char*)c->cfg.workspace + c->L.off_status, 0, kAlign, stream));
+    TS_CUDA(c, cudaMemsetAsync((char*)c->cfg.workspace + c->L.off_status, 0, c->L.status_bytes, stream));
     c->status_cleared = true;
   }
   return TS_OK;
@@ -384,6 +386,7 @@ void plan(ts_ctx* c, const ts_step* st, int split) {
   const int G = c->G;
   c->items.clear();
   c->combines.clear();
+  c->combine_of.clear();
   int partial = 0;
   for (int r = 0; r < st->n_rows; ++r) {
     const int ql = st->q_len[r], ctx = st->ctx_len[r];
@@ -404,6 +407,7 @@ void plan(ts_ctx* c, const ts_step* st, int split) {
       c->items.push_back(WorkItem{r, 0, 0, 1, 0, n, -1, 0});
       continue;
     }
+    c->combine_of.resize(partial + pieces, (int32_t)c->combines.size());
     c->combines.push_back(CombineItem{c->tok0[r], partial, pieces, 0});
     for (int i = 0; i < pieces; ++i)
       c->items.push_back(WorkItem{r, 0, 0, 1, i * per, std::min(n, (i + 1) * per), partial++, 0});
@@ -481,7 +485,13 @@ void pack_meta(const ts_ctx* c, const ts_step* st, const ts::StepDevice& d, int 
   std::memcpy(dst + d.o_slot, st->slot, sizeof(int32_t) * R);
   std::memcpy(dst + d.o_ctx, st->ctx_len, sizeof(int32_t) * R);
   std::memcpy(dst + d.o_tok0, c->tok0.data(), sizeof(int32_t) * (R + 1));
-  if (n_items > 0) std::memcpy(dst + d.o_items, c->items.data(), sizeof(WorkItem) * n_items);
+  if (n_items > 0) {
+    std::memcpy(dst + d.o_items, c->items.data(), sizeof(WorkItem) * n_items);
+    // a split row's items name its merge (the list holds the rows in the order of their partial slots)
+    WorkItem* items = (WorkItem*)(dst + d.o_items);
+    for (int i = 0; i < n_items; ++i)
+      if (items[i].partial_slot >= 0) items[i].combine = c->combine_of[items[i].partial_slot];
+  }
   if (n_combines > 0) std::memcpy(dst + d.o_combines, c->combines.data(), sizeof(CombineItem) * n_combines);
 }
 
@@ -493,9 +503,8 @@ void pack_meta(const ts_ctx* c, const ts_step* st, const ts::StepDevice& d, int 
 // waits for its event.
 int send_meta(ts_ctx* c, const ts_step* st, int n_items, int n_combines, int n_slot_deltas, cudaStream_t stream, ts::StepDevice* d) {
   const size_t used = meta_offsets(st->n_rows, n_items, n_combines, d);
-  // the decode and mixed kernels are there for larger parameters, the merge's list has to fit into the smaller ones
-  const bool large = n_items > 0 && c->cfg.head_dim == 128 && c->G <= 8 &&
-                     n_combines * (int)(sizeof(CombineItem) / sizeof(int32_t)) <= ts::kInlineWords;
+  // the decode and mixed kernels are there for larger parameters
+  const bool large = n_items > 0 && c->cfg.head_dim == 128 && c->G <= 8;
   const bool inline_meta = used <= (size_t)(large ? ts::kInlineWordsMax : ts::kInlineWords);
   const bool inline_deltas = n_slot_deltas <= ts::kInlineDeltas;
   char* ws = (char*)c->cfg.workspace;
@@ -565,6 +574,7 @@ void fill_device(ts_ctx* c, const ts_step* st, int64_t n_tokens, ts::StepDevice*
   d->table = (int32_t*)(ws + c->L.off_table);
   d->status = (int32_t*)(ws + c->L.off_status);
   d->pf_queue = d->status + 1;
+  d->merge_count = d->status + kAlign / sizeof(int32_t);
   d->part_acc = (float*)(ws + c->L.off_part_acc);
   d->part_ml = (float*)(ws + c->L.off_part_ml);
   d->q = (const uint16_t*)st->q;
@@ -752,8 +762,9 @@ int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefi
       ++c->cnt.kernel_launches;
     }
     if (pe) TS_CUDA(c, cudaEventRecord(pe[3], stream));
-    if (n_combines > 0 && !decode_launched) {      // the mixed launch merges its own splits
-      TS_CUDA(c, ts::launch_combine(d, stream));
+    const long long n_units = (long long)(n_items - c->n_prefill_items) * c->cfg.n_kv_heads;
+    if (n_combines > 0 && !decode_launched && !ts::merges_splits((int)n_units, std::min((int)n_units, c->n_sms))) {
+      TS_CUDA(c, ts::launch_combine(d, stream));   // else the launch has merged its own splits
       ++c->cnt.kernel_launches;
     }
     if (pe) TS_CUDA(c, cudaEventRecord(pe[4], stream));
@@ -1330,7 +1341,7 @@ int ts_last_device_status(ts_ctx* c, void* cuda_stream, int32_t* status_out) {
   TS_CUDA(c, cudaStreamSynchronize(stream));
   // a clean status clears only its word; after a failure the kernels' counters next to it may be
   // stale as well, so the whole block goes back to zero
-  TS_CUDA(c, cudaMemsetAsync(dev, 0, *status_out ? kAlign : sizeof(int32_t), stream));
+  TS_CUDA(c, cudaMemsetAsync(dev, 0, *status_out ? c->L.status_bytes : sizeof(int32_t), stream));
   TS_CUDA(c, cudaStreamSynchronize(stream));
   return (*status_out & TS_DEV_TIMEOUT) ? TS_ERR_DEVICE_TIMEOUT : TS_OK;
 }

@@ -31,7 +31,7 @@ struct WorkItem {
   int32_t k_begin;      // first key position (multiple of kKeysPerTile)
   int32_t k_end;        // one past the last key position any row of the item may see
   int32_t partial_slot; // >= 0: write (m, l, acc) partials there; -1: write out directly
-  int32_t reserved;
+  int32_t combine;      // of a partial_slot >= 0, as the kernels get it: index of the token's CombineItem
 };
 static_assert(sizeof(WorkItem) == 32, "WorkItem is 8 int32");
 
@@ -42,6 +42,12 @@ struct CombineItem {
   int32_t n_splits;
   int32_t reserved;
 };
+
+// Whether decode_kernel, as `n_ctas` CTAs over n_units units, merges the split rows itself (see count_split).
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline bool merges_splits(int n_units, int n_ctas) { return n_units > n_ctas; }
 
 struct TableDelta {
   int32_t slot, index, page;
@@ -64,6 +70,7 @@ struct StepDevice {
                            // mixed kernel [0] next prefill work unit, [1] decode CTAs that have finished
                            // their units, [2] CTAs that have left; [3] decode units taken besides the
                            // CTAs' first ones; decode kernel [4] CTAs that are done
+  int32_t* merge_count;    // [n_combines][Hkv] splits of a token that the decode kernel has finished, zero between launches
   float* part_acc;         // [max_partials][Hq][D]
   float* part_ml;          // [max_partials][Hq][2]  (running max in log2 units, sum)
   // step tensors
@@ -128,6 +135,7 @@ cudaError_t launch_table_update(int32_t* table, int max_pages_per_req, int max_r
 cudaError_t launch_kv_append(const StepDevice& s, cudaStream_t stream);
 // Work items [0, n_items); prefill items read their chunk's own K/V from the step's tensors and append them.
 cudaError_t launch_attention(const StepDevice& s, cudaStream_t stream);
+// Merges the splits that launch_attention left, or launch_decode where merges_splits says no (launch_mixed merges its own).
 cudaError_t launch_combine(const StepDevice& s, cudaStream_t stream);
 // Decode splits items[n_prefill_items, n_items): persistent kernel, one CTA per SM, K/V pages by TMA
 // through kv_map (5-D view of the pool: 64 columns, KV head x slot, half, K|V, page; box = one page of one head).

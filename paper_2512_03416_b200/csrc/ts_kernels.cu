@@ -69,8 +69,7 @@ __global__ void combine_kernel(const __grid_constant__ StepParams<kInlineWords> 
   const StepDevice& s = params.s;
   pdl_launch_dependents();
   // Metadata that were in place before the decode launch started are read before the wait for its end: one round
-  // trip less behind it (device time of a step, prepared steps back to back, read behind the wait and so, us: four
-  // rows of ~1500 keys 10.69 / 10.50, 64 rows 127.0 / 126.7).
+  // trip less behind it (device time of a step of four rows of ~1500 keys, prepared steps back to back: 10.69 / 10.50 us).
   CombineItem c;
   if (s.meta_in_place) c = s.combine(blockIdx.x);
   pdl_wait();
@@ -427,7 +426,7 @@ cudaError_t launch_combine(const StepDevice& s, cudaStream_t stream) {
     c.host_words = s.host_words + s.o_combines;
     c.n_words = s.n_combines * (int)(sizeof(CombineItem) / sizeof(int32_t));
     c.o_combines = 0;
-    if (c.n_words > kInlineWords) return cudaErrorInvalidValue;
+    if (c.n_words > kInlineWords) return cudaErrorInvalidValue;   // not with a unit per CTA at most
     fill_params(c, &params);
   }
   return launch_pdl(combine_kernel, dim3(s.n_combines, s.Hq), dim3(s.D), 0, stream, params);
@@ -482,7 +481,7 @@ __global__ void static_plan_kernel(StaticScratch* sc, const int32_t* kv_len, int
   it.row = r;
   it.kind = 0;
   it.q_begin = 0;
-  it.reserved = 0;
+  it.combine = 0;
   if (s < ns) {
     it.q_count = 1;
     it.k_begin = s * per;
@@ -555,6 +554,7 @@ extern "C" int ts_decode_attention_static(int32_t device, int32_t n_q_heads, int
   d.table = (int32_t*)block_tables;       // only read
   d.status = &sc->status;
   d.pf_queue = nullptr;
+  d.merge_count = nullptr;
   d.part_acc = sc->part_acc;
   d.part_ml = sc->part_ml;
   d.meta = (const int32_t*)sc;

@@ -369,7 +369,7 @@ mixed_kernel(const __grid_constant__ StepParams<W> params, const __grid_constant
     reg_dec<kRegsAux>();
     if (decode_first) {
       if (warp == kSoftmaxWarps)
-        dec::decode_schedule<128, 3>(s, smem, base, (int)blockIdx.x - n_prefill_ctas, (int)gridDim.x - n_prefill_ctas, ready);
+        dec::decode_schedule<128, 3, false>(s, smem, base, (int)blockIdx.x - n_prefill_ctas, (int)gridDim.x - n_prefill_ctas, ready);
       else {
         ready();
         AppendCursor{n_prefill_ctas * warps_first + ((int)blockIdx.x - n_prefill_ctas) * kWarpsAux + (warp - kSoftmaxWarps - 1),
@@ -398,7 +398,7 @@ mixed_kernel(const __grid_constant__ StepParams<W> params, const __grid_constant
     if (decode_first) {
       if (warp < 8) {
         reg_inc<kRegsDecode>();       // waits until the parked warpgroups have given their registers up
-        dec::decode_units<128, 1, 3>(s, &kv_map, smem, base, ready);
+        dec::decode_units<128, 1, 3, false>(s, &kv_map, smem, base, ready);
         if (tid == 0) {          // this CTA's split partials are written: count it as done
           __threadfence();
           atomicAdd(s.pf_queue + 1, 1);

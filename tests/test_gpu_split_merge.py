@@ -1,0 +1,51 @@
+"""GPU parity of decode steps around the size from which the decode launch merges split rows itself."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2512_03416_b200 import workloads as wl
+from tests.helpers import GpuRun, assert_parity, oracle_step
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _need_gpu():
+    if not torch.cuda.is_available():
+        pytest.fail("these tests need a CUDA device")
+
+
+def sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def check(b, launches, **kw):
+    want, pool_want = oracle_step(b)
+    run = GpuRun(b, chunk_size=0, **kw)
+    for i in range(3):                                     # the counters are back at zero after a step
+        before = run.dec.velocity()["kernel_launches"]
+        assert_parity(run.step(keep_len=True), want, "peaked", f"step {i}")
+        if i > 0:                                          # the first one may bring block-table entries along
+            assert run.dec.velocity()["kernel_launches"] - before == launches
+    assert np.array_equal(run.pool(), pool_want)
+
+
+@pytest.mark.parametrize("shape", [wl.Shape(32, 8, 128), wl.Shape(8, 1, 128), wl.Shape(3, 1, 128), wl.Shape(12, 1, 128), wl.Shape(16, 8, 64)],
+                         ids=["32-8", "8-1", "3-1", "12-1", "d64"])
+@pytest.mark.parametrize("over", [0, 1])
+def test_split_rows_are_merged_by_the_decode_launch(shape, over):
+    """Rows in 2 to 18 splits of 64 keys; as many units as SMs (merged by a launch of its own) and one item more."""
+    n, ctx = sms() // shape.Hkv + over, []
+    for pieces in [18, 9, 5, 4] + [2] * n:
+        left = n - sum(-(-(c + 1) // 64) for c in ctx)
+        if left <= 0:
+            break
+        ctx.append(64 * min(pieces, left) - 3)
+    b = wl.make_batch("merge", shape, ctx, [1] * len(ctx), seed=over + shape.Hq, profile="peaked")
+    check(b, 1 if over else 2, decode_split_tokens=64)
+
+
+def test_many_units_of_split_rows():
+    """Most units are finished, counted and merged while their thread block streams on."""
+    b = wl.make_batch("many", wl.Shape(32, 8, 128), [1000 + 37 * i for i in range(24)], [1] * 24, seed=5, profile="peaked")
+    check(b, 1, decode_split_tokens=128)
