@@ -705,7 +705,7 @@ int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefi
     if (n_items > c->n_prefill_items) d.unit_wait_cycles = unit_wait_cycles(d.wait_cycles, c->items[c->n_prefill_items]);
     if (pe) TS_CUDA(c, cudaEventRecord(pe[1], stream));
     d.n_prefill_items = c->n_prefill_items;
-    bool decode_launched = false;
+    bool decode_launched = false, merged = false;              // the decode splits have been launched; with the merge of the split rows
     if (c->n_prefill_items > 0) {
       if (c->cfg.head_dim == 128) {
         CUtensorMap q_map;
@@ -737,7 +737,7 @@ int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefi
           p = (int)std::min<long long>(p, pf_units);
           p = std::min(p, n_ctas - 1);                         // at least one CTA runs the decode splits
           p = std::max(p, n_ctas - (int)std::min<long long>(dec_units, n_ctas));   // no CTA without a decode unit
-          decode_launched = true;
+          decode_launched = merged = true;
         }
         if (pe) c->prof_mixed.back() = decode_launched;
         // A CTA that starts on prefill units appends its share of the new tokens with one warp next
@@ -749,6 +749,9 @@ int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefi
         d.append_wide = append_us > 2.0 * pairs / n_ctas;
         d.debug_arrivals = (c->cfg.debug_flags & TS_DEBUG_LOSE_APPEND_ARRIVAL) ? 1 : 0;
         TS_CUDA(c, ts::launch_mixed(d, q_map, c->kv_map, c->kv_tile_map, new_maps, n_ctas, p, stream));
+      } else if (n_items > c->n_prefill_items && (long long)n_items * c->cfg.n_kv_heads <= c->n_sms) {
+        TS_CUDA(c, ts::launch_small_step(d, c->kv_map, stream));
+        decode_launched = true;
       } else {
         ts::StepDevice dp = d;
         dp.n_items = c->n_prefill_items;
@@ -759,12 +762,13 @@ int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefi
     if (pe) TS_CUDA(c, cudaEventRecord(pe[2], stream));
     if (n_items > c->n_prefill_items && !decode_launched) {
       TS_CUDA(c, ts::launch_decode(d, c->kv_map, c->n_sms, stream));
+      const long long n_units = (long long)(n_items - c->n_prefill_items) * c->cfg.n_kv_heads;
+      merged = ts::merges_splits((int)n_units, (int)std::min<long long>(n_units, c->n_sms));
       ++c->cnt.kernel_launches;
     }
     if (pe) TS_CUDA(c, cudaEventRecord(pe[3], stream));
-    const long long n_units = (long long)(n_items - c->n_prefill_items) * c->cfg.n_kv_heads;
-    if (n_combines > 0 && !decode_launched && !ts::merges_splits((int)n_units, std::min((int)n_units, c->n_sms))) {
-      TS_CUDA(c, ts::launch_combine(d, stream));   // else the launch has merged its own splits
+    if (n_combines > 0 && !merged) {
+      TS_CUDA(c, ts::launch_combine(d, stream));
       ++c->cnt.kernel_launches;
     }
     if (pe) TS_CUDA(c, cudaEventRecord(pe[4], stream));

@@ -135,6 +135,9 @@ cudaError_t launch_table_update(int32_t* table, int max_pages_per_req, int max_r
 cudaError_t launch_kv_append(const StepDevice& s, cudaStream_t stream);
 // Work items [0, n_items); prefill items read their chunk's own K/V from the step's tensors and append them.
 cudaError_t launch_attention(const StepDevice& s, cudaStream_t stream);
+// Prefill items and decode splits of a head_dim 64 step in one launch, a block per (item, KV head): for steps that have
+// both and no more of these than the device has SMs. Split rows are left to launch_combine.
+cudaError_t launch_small_step(const StepDevice& s, const CUtensorMap& kv_map, cudaStream_t stream);
 // Merges the splits that launch_attention left, or launch_decode where merges_splits says no (launch_mixed merges its own).
 cudaError_t launch_combine(const StepDevice& s, cudaStream_t stream);
 // Decode splits items[n_prefill_items, n_items): persistent kernel, one CTA per SM, K/V pages by TMA
