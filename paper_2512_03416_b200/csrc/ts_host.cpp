@@ -609,7 +609,11 @@ bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 // than with four.
 //   G <= 4: an SM streams a decode unit at 70 GB/s plus ~2 us per unit, and all of them together
 //           at no more than 6.1 TB/s; the step time is flat over a range of splits, of which the
-//           middle is taken (its ends are the sensitive ones).
+//           middle is taken (its ends are the sensitive ones). Long steps run at the chip's power limit, where the
+//           clock and with it an SM's rate are lower: 62 GB/s from 120 us on, in between below that. (8B shape, steps
+//           back to back, us, at 70 GB/s / so / at 60 GB/s always: 64 rows + 2048 tokens 152.3 / 150.0 / 151.1, 128 rows +
+//           4 x 512 tokens 520 / 509 / 505, 60 rows + 3 x 300 tokens 217.5 / 209.4 / 226.7, 100 rows + 1000 tokens behind 6144
+//           199.0 / 197.0 / 201.4, 150 rows + 200 tokens 161.5 / 158.4 / 158.4, 8 rows + 300 tokens 22.2 / 22.2 / 23.9.)
 //   G >  4: measured fraction of the full-chip rate by SM count, linear in between:
 //           48 0.43, 64 0.62, 74 0.715, 84 0.78, 100 0.85, 116 0.92, 132 0.95, 148 1
 int choose_prefill_ctas(const ts_ctx* c, int n_ctas, double prefill_block_pairs, double prefill_units,
@@ -620,7 +624,7 @@ int choose_prefill_ctas(const ts_ctx* c, int n_ctas, double prefill_block_pairs,
   const double w_pf = prefill_block_pairs * 2.1 + prefill_units * 2.0;
   const double t_dec_full = decode_bytes / 6.1e6;   // us at 6.1 TB/s
   const double unit_bytes = decode_bytes / std::max(1.0, decode_units);
-  const double sm_rate = unit_bytes / (unit_bytes / 70e3 + 2.0);   // bytes per us and SM
+  double sm_rate = 0.0;                                  // bytes per us and SM
   auto step_time = [&](int p) {
     double td;
     if (wide) {
@@ -636,12 +640,17 @@ int choose_prefill_ctas(const ts_ctx* c, int n_ctas, double prefill_block_pairs,
     return std::max(td, (w_pf + (double)(n_ctas - p) * td) / n_ctas);
   };
   int best = 0;
-  double best_t = 1e30;
-  for (int p = 0; p < n_ctas; p += 2) {
-    const double t = step_time(p);
-    if (t < best_t - 1e-9) {
-      best_t = t;
-      best = p;
+  double best_t = 60.0;                                  // us; what the first pass finds sets the rate of the second
+  for (int pass = 0; pass < (wide ? 1 : 2); ++pass) {
+    const double rate = 70e3 - 8e3 * std::min(1.0, std::max(0.0, best_t - 60.0) / 60.0);
+    sm_rate = unit_bytes / (unit_bytes / rate + 2.0);
+    best_t = 1e30;
+    for (int p = 0; p < n_ctas; p += 2) {
+      const double t = step_time(p);
+      if (t < best_t - 1e-9) {
+        best_t = t;
+        best = p;
+      }
     }
   }
   if (wide) return best;
