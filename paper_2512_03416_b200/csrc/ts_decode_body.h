@@ -188,10 +188,8 @@ __device__ __forceinline__ void merge_heads(const StepDevice& s, const CombineIt
 // Rows that were split. A unit whose eight warps have all written their shares is counted by the scheduler warp; whoever
 // counts the last split of a (row, KV head) merges it: the scheduler warp itself while its CTA still streams, all
 // streaming warps for the CTA's last units, where the merge is what the launch ends with. (Counted and merged by the
-// streaming warps, the fence and the counter's round trip stopped the page stream.) A launch with one unit per CTA at
-// most leaves the merge to a launch of its own, whose blocks merge a head each. Device time of a step, merged by that
-// launch / here, us: 64 rows 122.7 / 120.5, 203 rows of the 70B shape 224.3 / 221.1, but four rows of ~1500 keys 9.9 / 10.4:
-// fence, count and merge are one behind the other at the end of the only unit.
+// streaming warps, the fence and the counter's round trip stopped the page stream.) A launch of few units leaves the
+// merge to a launch of its own, whose blocks merge a head each (merge_here, decided on the host).
 // True, for the whole warp, when this was the last split.
 __device__ __forceinline__ bool count_split(const StepDevice& s, int combine, int n_splits, int kv_head, int lane) {
   int last = 0;
@@ -236,7 +234,7 @@ __device__ __forceinline__ void decode_schedule(const StepDevice& s, unsigned ch
   volatile int* failed = reinterpret_cast<volatile int*>(smem + L::off_failed(G));
   decode_meet();
   bool ok = true;
-  const bool merging = MERGE && merges_splits(n_units, n_ctas);
+  const bool merging = MERGE && s.merge_here != 0;
   int n_described = 0, n_finished = 0;
   for (int k = 0;; ++k) {
     const int e = k % kDecRing;
@@ -651,7 +649,7 @@ __device__ __forceinline__ void decode_units(const StepDevice& s, const CUtensor
   if (dead) give_up(s, failed);
   for (; n_consumed < n_issued; ++n_consumed) mbar_wait(my_bars + (n_consumed % STAGES) * 8, (n_consumed / STAGES) & 1, kDrainCycles);
   decode_meet();               // the scheduler included: then the barriers' shared memory can be given back
-  if (MERGE && merges_splits((s.n_items - s.n_prefill_items) * s.Hkv, (int)gridDim.x)) {
+  if (MERGE && s.merge_here != 0) {
     const int* merges = reinterpret_cast<const int*>(smem + L::off_merges(G));
     for (int i = 0; i < kDecRing; ++i)
       if (merges[i] >= 0) merge_by_all<D>(s, units[merges[i]].merge, units[merges[i]].head, warp, lane);

@@ -20,7 +20,7 @@ using ts::WorkItem;
 constexpr int kRing = 4;                  // pinned metadata buffers in flight
 constexpr int kDeltaCapacity = 32768;     // table entries per upload batch (bulk loads)
 constexpr int kSlotDeltas = 4096;         // table entries that ride along with a step's metadata
-constexpr int kMinDefaultSplit = 512, kMaxDefaultSplit = 4096;   // keys per decode split, see plan()
+constexpr int kMinSmallSplit = 128, kMinOneWaveSplit = 256, kMinDefaultSplit = 512, kMaxDefaultSplit = 4096;   // keys per decode split, see plan()
 constexpr int kSmsB200 = 148;             // for plans made before the device is known
 constexpr int kDefaultMaxTokens = 16384;  // step size bound when chunk_size == 0
 constexpr size_t kAlign = 256;
@@ -362,10 +362,43 @@ int decode_split(const ts_ctx* c, const ts_step* st) {
     // (2234) 41.3 / 39.1 / 38.3 / 39.0; 64 rows (7864) 109 / 101.5 / 99.0 / 100.9; with G = 8, 203 rows
     // (16579) 248 / 209 / 201 / 196.
     int64_t keys = 0;
-    for (int r = 0; r < st->n_rows; ++r)
-      if (st->q_len[r] == 1) keys += st->ctx_len[r] + 1;
+    int longest = 0;
+    bool chunks = false;
+    for (int r = 0; r < st->n_rows; ++r) {
+      chunks = chunks || st->q_len[r] > 1;
+      if (st->q_len[r] == 1) {
+        keys += st->ctx_len[r] + 1;
+        longest = std::max(longest, st->ctx_len[r] + 1);
+      }
+    }
     const int64_t share = keys * c->cfg.n_kv_heads / (c->n_sms > 0 ? c->n_sms : kSmsB200);
     split = (int)std::min<int64_t>(std::max<int64_t>(share, kMinDefaultSplit), kMaxDefaultSplit);
+    // A step of few decode rows, some of which are split anyway, takes as long as the thread block with most to do: the
+    // shortest split, of 256 keys at least, with which every unit (but 3 % short ones) has an SM to itself, if that is near the
+    // share. Where at most two thirds of the SMs cost no more than 100 keys of 128 elements per unit in addition (0.7 us), or
+    // where the units are shorter yet, they are the better ones: the next step's thread blocks start on the other SMs, and the
+    // merge is a launch of its own (see merge_here). Device time of a step of the 8B shape, us, by the share and 512 alone / so:
+    // one row of 1014 keys 9.5 / 6.9, one of 2157 9.4 / 8.2, 4 rows of ~1300 9.9 / 9.3, 4 of ~2600 14.5 / 11.3, 8 of ~2350 19.8 /
+    // 15.8, 12 of ~970 15.0 / 12.7. Not for rows of 512 keys and less, which are not worth a merge.
+    const int n_sms = c->n_sms > 0 ? c->n_sms : kSmsB200;
+    if (!chunks && longest > kMinDefaultSplit && st->n_rows * c->cfg.n_kv_heads <= n_sms) {
+      const int64_t most = std::min<int64_t>(std::max<int64_t>(share * 29 / 20, kMinDefaultSplit), kMaxDefaultSplit);
+      int64_t one_wave = 0;                                // the shortest split that gives every unit an SM
+      for (int64_t s = std::max<int64_t>(kMinSmallSplit, ceil_div((int)share, ts::kKeysPerTile) * ts::kKeysPerTile); s <= most; s += ts::kKeysPerTile) {
+        if (one_wave > 0 && (s - one_wave) * c->cfg.head_dim > 100 * 128) break;
+        int units = 0;
+        for (int r = 0; r < st->n_rows; ++r) {
+          int per, pieces;
+          cut_row(st->ctx_len[r] + 1, (int)s, &per, &pieces);
+          units += pieces * c->cfg.n_kv_heads;
+        }
+        if (one_wave == 0 && s >= kMinOneWaveSplit && units <= n_sms + n_sms / 32) split = (int)(one_wave = s);
+        if (3 * units <= 2 * n_sms) {
+          split = (int)s;
+          break;
+        }
+      }
+    }
   }
   split = ceil_div(split, ts::kKeysPerTile) * ts::kKeysPerTile;
   for (;; split *= 2) {
@@ -595,6 +628,7 @@ void fill_device(ts_ctx* c, const ts_step* st, int64_t n_tokens, ts::StepDevice*
   d->scale_log2 = c->scale * 1.4426950408889634f;
   d->wait_cycles = c->cfg.wait_limit_cycles > 0 ? (long long)c->cfg.wait_limit_cycles : ts::kWaitCycles;
   d->unit_wait_cycles = d->wait_cycles;
+  d->merge_here = 0;           // set for the decode launch
   d->append_wide = 0;          // both set by the mixed launch
   d->debug_arrivals = 0;
 }
@@ -770,9 +804,13 @@ int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefi
     }
     if (pe) TS_CUDA(c, cudaEventRecord(pe[2], stream));
     if (n_items > c->n_prefill_items && !decode_launched) {
+      // Few units: a merge launch, whose blocks wait on the free SMs, is sooner done than the count and merge at the end of
+      // every thread block. (Device time of a step in us, merged by a launch / in place: 64 rows of the 8B shape 122.7 / 120.5, 203
+      // rows of the 70B shape 224.3 / 221.1; 4 rows of ~1300 keys as 96 units 9.9 / 10.4; between 100 units and one per SM a
+      // launch takes 1 to 1.5 us more than up to 96.)
+      merged = 3 * (long long)(n_items - c->n_prefill_items) * c->cfg.n_kv_heads > 2 * c->n_sms;
+      d.merge_here = merged;
       TS_CUDA(c, ts::launch_decode(d, c->kv_map, c->n_sms, stream));
-      const long long n_units = (long long)(n_items - c->n_prefill_items) * c->cfg.n_kv_heads;
-      merged = ts::merges_splits((int)n_units, (int)std::min<long long>(n_units, c->n_sms));
       ++c->cnt.kernel_launches;
     }
     if (pe) TS_CUDA(c, cudaEventRecord(pe[3], stream));

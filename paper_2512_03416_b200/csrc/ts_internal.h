@@ -43,12 +43,6 @@ struct CombineItem {
   int32_t reserved;
 };
 
-// Whether decode_kernel, as `n_ctas` CTAs over n_units units, merges the split rows itself (see count_split).
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline bool merges_splits(int n_units, int n_ctas) { return n_units > n_ctas; }
-
 struct TableDelta {
   int32_t slot, index, page;
 };
@@ -71,6 +65,7 @@ struct StepDevice {
                            // their units, [2] CTAs that have left; [3] decode units taken besides the
                            // CTAs' first ones; decode kernel [4] CTAs that are done
   int32_t* merge_count;    // [n_combines][Hkv] splits of a token that the decode kernel has finished, zero between launches
+  int32_t merge_here;      // the decode kernel merges the rows it split itself (see count_split)
   float* part_acc;         // [max_partials][Hq][D]
   float* part_ml;          // [max_partials][Hq][2]  (running max in log2 units, sum)
   // step tensors
@@ -138,7 +133,7 @@ cudaError_t launch_attention(const StepDevice& s, cudaStream_t stream);
 // Prefill items and decode splits of a head_dim 64 step in one launch, a block per (item, KV head): for steps that have
 // both and no more of these than the device has SMs. Split rows are left to launch_combine.
 cudaError_t launch_small_step(const StepDevice& s, const CUtensorMap& kv_map, cudaStream_t stream);
-// Merges the splits that launch_attention left, or launch_decode where merges_splits says no (launch_mixed merges its own).
+// Merges the splits that launch_attention left, or launch_decode without merge_here (launch_mixed merges its own).
 cudaError_t launch_combine(const StepDevice& s, cudaStream_t stream);
 // Decode splits items[n_prefill_items, n_items): persistent kernel, one CTA per SM, K/V pages by TMA
 // through kv_map (5-D view of the pool: 64 columns, KV head x slot, half, K|V, page; box = one page of one head).

@@ -491,7 +491,7 @@ cudaError_t launch_combine(const StepDevice& s, cudaStream_t stream) {
     c.host_words = s.host_words + s.o_combines;
     c.n_words = s.n_combines * (int)(sizeof(CombineItem) / sizeof(int32_t));
     c.o_combines = 0;
-    if (c.n_words > kInlineWords) return cudaErrorInvalidValue;   // not with a unit per CTA at most
+    if (c.n_words > kInlineWords) return cudaErrorInvalidValue;   // not with as few units as come here
     fill_params(c, &params);
   }
   return launch_pdl(combine_kernel, dim3(s.n_combines, s.Hq), dim3(s.D), 0, stream, params);
@@ -620,6 +620,7 @@ extern "C" int ts_decode_attention_static(int32_t device, int32_t n_q_heads, int
   d.status = &sc->status;
   d.pf_queue = nullptr;
   d.merge_count = nullptr;
+  d.merge_here = 0;
   d.part_acc = sc->part_acc;
   d.part_ml = sc->part_ml;
   d.meta = (const int32_t*)sc;

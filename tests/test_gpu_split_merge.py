@@ -32,10 +32,11 @@ def check(b, launches, **kw):
 
 @pytest.mark.parametrize("shape", [wl.Shape(32, 8, 128), wl.Shape(8, 1, 128), wl.Shape(3, 1, 128), wl.Shape(12, 1, 128), wl.Shape(16, 8, 64)],
                          ids=["32-8", "8-1", "3-1", "12-1", "d64"])
-@pytest.mark.parametrize("over", [0, 1])
+@pytest.mark.parametrize("over", [0, 1, 2])
 def test_split_rows_are_merged_by_the_decode_launch(shape, over):
-    """Rows in 2 to 18 splits of 64 keys; as many units as SMs (merged by a launch of its own) and one item more."""
-    n, ctx = sms() // shape.Hkv + over, []
+    """Rows in 2 to 18 splits of 64 keys; units on two thirds of the SMs (merged by a launch of its own), one item more, and
+    more units than SMs."""
+    n, ctx = (2 * sms() // (3 * shape.Hkv), 2 * sms() // (3 * shape.Hkv) + 1, sms() // shape.Hkv + 1)[over], []
     for pieces in [18, 9, 5, 4] + [2] * n:
         left = n - sum(-(-(c + 1) // 64) for c in ctx)
         if left <= 0:
@@ -43,6 +44,18 @@ def test_split_rows_are_merged_by_the_decode_launch(shape, over):
         ctx.append(64 * min(pieces, left) - 3)
     b = wl.make_batch("merge", shape, ctx, [1] * len(ctx), seed=over + shape.Hq, profile="peaked")
     check(b, 1 if over else 2, decode_split_tokens=64)
+
+
+@pytest.mark.parametrize("rows", [[521], [2157], [900] * 4 + [100], [2000, 1500, 1100, 600], [5400, 30, 4000, 300], [2300] * 8, [970] * 12, [16000] + [200] * 17],
+                         ids=lambda r: f"{len(r)}x{r[0]}")
+def test_default_splits_of_steps_around_one_unit_per_SM(rows):
+    """The split follows the number of units; the plan, and parity with it."""
+    b = wl.make_batch("few", wl.LLAMA8B, rows, [1] * len(rows), seed=len(rows), profile="peaked")
+    want, pool_want = oracle_step(b)
+    run = GpuRun(b, chunk_size=0)
+    for i in range(3):
+        assert_parity(run.step(keep_len=True), want, "peaked", f"{rows}, step {i}")
+    assert np.array_equal(run.pool(), pool_want)
 
 
 def test_many_units_of_split_rows():
