@@ -88,20 +88,19 @@ __device__ __forceinline__ void unpack8(const uint4& w, float* v) {
 }
 
 // Eight columns c .. c + 7 of a 128-column head that starts at column col0 of the fused projection,
-// and their partners 64 further on: rotated (query and key heads) and written to the head's tensor.
-__device__ __forceinline__ void rope8(const GemmArgs& g, int row, int col0, int c, float (&lo)[8], float (&hi)[8]) {
+// and their partners 64 further on: rotated by cs (query and key heads) and written to the head's tensor.
+__device__ __forceinline__ void rope8(const GemmArgs& g, int row, int col0, int c, float (&lo)[8], float (&hi)[8], const float4 (&cs)[4]) {
   const bool rotate = col0 < g.q_cols + g.kv_cols;
   uint16_t* dst = col0 < g.q_cols ? g.C + (size_t)row * g.q_cols + col0
                   : rotate        ? g.C2 + (size_t)row * g.kv_cols + (col0 - g.q_cols)
                                   : g.C3 + (size_t)row * g.kv_cols + (col0 - g.q_cols - g.kv_cols);
   if (rotate) {
-    const float2* cs = g.rope_table + (size_t)g.pos[row] * 64 + c;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const float2 t2 = cs[e];                             // (cos, sin)
+      const float co = e & 1 ? cs[e / 2].z : cs[e / 2].x, si = e & 1 ? cs[e / 2].w : cs[e / 2].y;
       const float a = lo[e], b = hi[e];
-      lo[e] = a * t2.x - b * t2.y;
-      hi[e] = b * t2.x + a * t2.y;
+      lo[e] = a * co - b * si;
+      hi[e] = b * co + a * si;
     }
   }
   *reinterpret_cast<uint4*>(dst + c) = pack8(lo);
@@ -708,11 +707,33 @@ gemm_split_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, c
   const int k_blocks = (g.K + kBK - 1) / kBK;
   const int kb0 = k_blocks * rank / split, kb1 = k_blocks * (rank + 1) / split;   // never empty: split <= k_blocks
 
+  // one item = 8 columns of a row, for ROPE with their partners 64 further on
+  constexpr int kItems = EPI == GEMM_EPI_STORE ? 16 : 8;
+  const int first_item = rank * kGemmThreads + tid, stride = split * kGemmThreads;
+  // What an item adds to the product: the residual's columns, or the angles' (cos, sin).
+  auto fetch = [&](int i, float4 (&extra)[EPI == GEMM_EPI_STORE ? 1 : 4]) {
+    const int r = i / kItems, ch = i % kItems, row = m0 + r;
+    if (i >= rows * kItems) return;
+    if constexpr (EPI == GEMM_EPI_STORE) {
+      if (g.R && n0 + ch * 8 < g.N) extra[0] = *reinterpret_cast<const float4*>(g.R + (size_t)row * g.ldc + n0 + ch * 8);
+    } else if (n0 < g.q_cols + g.kv_cols) {
+      const float4* cs = reinterpret_cast<const float4*>(g.rope_table + (size_t)g.pos[row] * 64 + ch * 8);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) extra[e] = cs[e];
+    }
+  };
+  // Each thread fetches its first item's (of a decode batch its only one) before the product: behind it, position and
+  // angles are two round trips in a row.
+  float4 extra[EPI == GEMM_EPI_STORE ? 1 : 4];
+  if (warp >= 2 && tid - 64 < kSplitN) prefetch_weights(g, n0 + tid - 64, kb0 * kBK, kb1 * kBK);
+  if (tid == 0) {
+    tma_prefetch_desc(&a_map);
+    tma_prefetch_desc(&b_map);
+  }
+  pdl_wait();                      // the activations, the residual and the positions come from the launches in front
+
   if (warp == 0) {
     if (lane == 0) {
-      tma_prefetch_desc(&a_map);
-      tma_prefetch_desc(&b_map);
-      pdl_wait();
       for (int kb = kb0, it = 0; kb < kb1; ++kb, ++it) {
         const int st = it % kSplitStages;
         if (it >= kSplitStages && !mbar_wait(bar(BAR_EMPTY + st), ((it / kSplitStages) & 1) ^ 1, misc[1] ? 2000 : g.wait_cycles)) give_up();
@@ -743,7 +764,7 @@ gemm_split_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, c
     }
     if (!dead) tc_commit(bar(BAR_ACC), issue);
   } else {
-    if (tid - 64 < kSplitN) prefetch_weights(g, n0 + tid - 64, kb0 * kBK, kb1 * kBK);
+    fetch(first_item, extra);
     // accumulator -> image in shared memory; every operand stage has been read once the barrier completes
     if (!mbar_wait(bar(BAR_ACC), 0, misc[1] ? 2000 : g.wait_cycles)) give_up();
     tc_fence_after();
@@ -765,10 +786,8 @@ gemm_split_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, c
   }
   settle(misc[1] != 0);
   __syncwarp();
+  if (warp < 2) fetch(first_item, extra);
   cluster_sync();                  // the images are complete
-  pdl_wait();                      // every thread reads the residual or the positions below
-  // one item = 8 columns of a row, for ROPE with their partners 64 further on
-  constexpr int kItems = EPI == GEMM_EPI_STORE ? 16 : 8;
   auto sum8 = [&](int row, int col, float (&v)[8]) {
     float4 x[kMaxSplit], y[kMaxSplit];                     // all loads fly at once
 #pragma unroll
@@ -788,18 +807,17 @@ gemm_split_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, c
       v[4] += y[r].x; v[5] += y[r].y; v[6] += y[r].z; v[7] += y[r].w;
     }
   };
-  for (int i = rank * kGemmThreads + tid; i < rows * kItems; i += split * kGemmThreads) {
+  for (int i = first_item; i < rows * kItems; i += stride) {
     const int r = i / kItems, ch = i % kItems, row = m0 + r;
-    if (EPI == GEMM_EPI_STORE) {
+    if (i != first_item) fetch(i, extra);
+    if constexpr (EPI == GEMM_EPI_STORE) {
       const int col = n0 + ch * 8;
       if (col >= g.N) continue;
       float v[8];
-      uint4 res;
-      if (g.R) res = *reinterpret_cast<const uint4*>(g.R + (size_t)row * g.ldc + col);
       sum8(r, ch * 8, v);
       if (g.R) {
         float x[8];
-        unpack8(res, x);
+        unpack8(*reinterpret_cast<const uint4*>(&extra[0]), x);
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] += x[e];
       }
@@ -808,7 +826,7 @@ gemm_split_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, c
       float lo[8], hi[8];
       sum8(r, ch * 8, lo);
       sum8(r, 64 + ch * 8, hi);
-      rope8(g, row, n0, ch * 8, lo, hi);
+      rope8(g, row, n0, ch * 8, lo, hi, extra);
     }
   }
   tc_fence_before();
