@@ -284,8 +284,8 @@ int ts_report_step_time(ts_ctx* ctx, double seconds);
 typedef struct {
   double append_ms;     /* table update + KV append kernels                  */
   double prefill_ms;    /* attention kernel of steps whose launch held prefill tiles only */
-  double decode_ms;     /* stand-alone split-KV decode attention kernel      */
-  double combine_ms;    /* split-combine kernel                              */
+  double decode_ms;     /* stand-alone split-KV decode attention kernel; with the merge of split rows where it does that itself */
+  double combine_ms;    /* split-combine kernel, where the merge is a launch of its own */
   int64_t steps;
   double mixed_ms;      /* attention kernel of steps where one launch ran the prefill tiles
                            and the decode rows together                       */

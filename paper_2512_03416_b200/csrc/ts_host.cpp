@@ -795,6 +795,7 @@ int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefi
       } else if (n_items > c->n_prefill_items && (long long)n_items * c->cfg.n_kv_heads <= c->n_sms) {
         TS_CUDA(c, ts::launch_small_step(d, c->kv_map, stream));
         decode_launched = true;
+        if (pe) c->prof_mixed.back() = 1;
       } else {
         ts::StepDevice dp = d;
         dp.n_items = c->n_prefill_items;

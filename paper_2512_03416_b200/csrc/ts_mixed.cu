@@ -425,8 +425,8 @@ mixed_kernel(const __grid_constant__ StepParams<W> params, const __grid_constant
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t tS = tmem + x * 128 + hf * 64 + lane_addr;         // my 64 score columns; P goes to the first 32
     const uint32_t tO = tmem + 256 + x * 128 + hf * 64 + lane_addr;   // my 64 columns of O
-    // The two warps that share a quarter of a tile's rows meet on a hardware barrier (ids 4-11) around
-    // each exchange through shared memory; it wakes them sooner than an mbarrier (together with
+    // The two warps that share a quarter of a tile's rows meet on a hardware barrier (ids 4-11): around
+    // each exchange through shared memory, and for the vote on a block's maxima; it wakes them sooner than an mbarrier (together with
     // the other changes to the unit loop that came with it: 8192-token chunk next to 190 rows 1272 -> 1263 us,
     // 2048 tokens alone 49.5 -> 46.3 us). It has no time limit, so
     // the two must never disagree about how often they meet: all their other waits are limited and end
