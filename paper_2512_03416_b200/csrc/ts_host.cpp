@@ -379,20 +379,22 @@ int decode_split(const ts_ctx* c, const ts_step* st) {
     // where the units are shorter yet, they are the better ones: the next step's thread blocks start on the other SMs, and the
     // merge is a launch of its own (see merge_here). Device time of a step of the 8B shape, us, by the share and 512 alone / so:
     // one row of 1014 keys 9.5 / 6.9, one of 2157 9.4 / 8.2, 4 rows of ~1300 9.9 / 9.3, 4 of ~2600 14.5 / 11.3, 8 of ~2350 19.8 /
-    // 15.8, 12 of ~970 15.0 / 12.7. Not for rows of 512 keys and less, which are not worth a merge.
+    // 15.8, 12 of ~970 15.0 / 12.7. Not for rows of 512 keys and less, which are not worth a merge (14 rows of up to 513 keys of 64
+    // elements, a call bound by the host: 10.8 / 11.2); keys of 64 elements count half.
     const int n_sms = c->n_sms > 0 ? c->n_sms : kSmsB200;
-    if (!chunks && longest > kMinDefaultSplit && st->n_rows * c->cfg.n_kv_heads <= n_sms) {
+    const int keys128 = 128 / c->cfg.head_dim;             // keys that are as long as one of 128 elements
+    if (!chunks && longest > kMinDefaultSplit * keys128 && st->n_rows * c->cfg.n_kv_heads <= n_sms) {
       const int64_t most = std::min<int64_t>(std::max<int64_t>(share * 29 / 20, kMinDefaultSplit), kMaxDefaultSplit);
       int64_t one_wave = 0;                                // the shortest split that gives every unit an SM
-      for (int64_t s = std::max<int64_t>(kMinSmallSplit, ceil_div((int)share, ts::kKeysPerTile) * ts::kKeysPerTile); s <= most; s += ts::kKeysPerTile) {
-        if (one_wave > 0 && (s - one_wave) * c->cfg.head_dim > 100 * 128) break;
+      for (int64_t s = std::max<int64_t>(kMinSmallSplit * keys128, ceil_div((int)share, ts::kKeysPerTile) * ts::kKeysPerTile); s <= most; s += ts::kKeysPerTile) {
+        if (one_wave > 0 && s - one_wave > 100 * keys128) break;
         int units = 0;
         for (int r = 0; r < st->n_rows; ++r) {
           int per, pieces;
           cut_row(st->ctx_len[r] + 1, (int)s, &per, &pieces);
           units += pieces * c->cfg.n_kv_heads;
         }
-        if (one_wave == 0 && s >= kMinOneWaveSplit && units <= n_sms + n_sms / 32) split = (int)(one_wave = s);
+        if (one_wave == 0 && s >= kMinOneWaveSplit * keys128 && units <= n_sms + n_sms / 32) split = (int)(one_wave = s);
         if (3 * units <= 2 * n_sms) {
           split = (int)s;
           break;
