@@ -524,7 +524,7 @@ void pack_meta(const ts_ctx* c, const ts_step* st, const ts::StepDevice& d, int 
     std::memcpy(dst + d.o_items, c->items.data(), sizeof(WorkItem) * n_items);
     // a split row's items name its merge (the list holds the rows in the order of their partial slots)
     WorkItem* items = (WorkItem*)(dst + d.o_items);
-    for (int i = 0; i < n_items; ++i)
+    for (int i = c->n_prefill_items; n_combines > 0 && i < n_items; ++i)
       if (items[i].partial_slot >= 0) items[i].combine = c->combine_of[items[i].partial_slot];
   }
   if (n_combines > 0) std::memcpy(dst + d.o_combines, c->combines.data(), sizeof(CombineItem) * n_combines);
