@@ -82,7 +82,8 @@ typedef struct {
   int32_t reserved_pages;     /* Eq. 6: pages only ts_alloc_pages(..., for_prefill=1) may take */
   int32_t decode_split_tokens;/* keys per split of a decode row, rounded up to a multiple of
                                  64; 0 = the library decides per step (512 to 4096, by how many
-                                 keys the step's decode rows have per SM)                      */
+                                 keys the step's decode rows have per SM; from 128 on in
+                                 decode-only steps of few rows)                                */
   int32_t mixed_prefill_ctas; /* CTAs of the mixed attention kernel that only take prefill tiles
                                  while the other CTAs stream the decode rows first (Sec. 3.4:
                                  the decoder absorbs prefill work next to its decode batch);
