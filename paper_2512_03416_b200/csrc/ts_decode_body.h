@@ -119,10 +119,11 @@ __device__ __forceinline__ void give_up(const StepDevice& s, volatile int* faile
   __syncwarp();
 }
 
-// Merge of a row's splits, by one warp: the log-sum-exp merge of merge_splits for `n_heads` heads from head0 on, 32 * E of
-// their columns from col0 on. The loads of HEADS heads x SPLITS splits fly at a time.
-template <int D, int E, int HEADS, int SPLITS>
+// Merge of a row's splits, by one warp: the merge of merge_splits, bit for bit, for `n_heads` heads from head0 on, 32 * E of
+// their columns from col0 on. The loads of HEADS heads x GROUPS groups of splits fly at a time.
+template <int D, int E, int HEADS, int GROUPS>
 __device__ __forceinline__ void merge_heads(const StepDevice& s, const CombineItem& c, int head0, int n_heads, int col0, int lane) {
+  constexpr int kGroup = kMergeGroup;
   const int col = col0 + lane * E;
   const float* ml = s.part_ml + ((size_t)c.first_partial * s.Hq + head0) * 2;
   const float* pa = s.part_acc + ((size_t)c.first_partial * s.Hq + head0) * D + col;
@@ -138,43 +139,33 @@ __device__ __forceinline__ void merge_heads(const StepDevice& s, const CombineIt
       for (int e = 0; e < E; ++e) acc[h][e] = 0.f;
     }
 #pragma unroll 1
-    for (int b0 = 0; b0 < c.n_splits; b0 += SPLITS) {
-      float2 st[HEADS][SPLITS];
-      float a[HEADS][SPLITS][E];
+    for (int b0 = 0; b0 < c.n_splits; b0 += GROUPS * kGroup) {
+      float mi[HEADS][GROUPS][kGroup], li[HEADS][GROUPS][kGroup], a[HEADS][GROUPS][kGroup][E];
 #pragma unroll
       for (int h = 0; h < HEADS; ++h)
 #pragma unroll
-        for (int j = 0; j < SPLITS; ++j) {
-          const bool on = b0 + j < c.n_splits && h0 + h < n_heads;
-          const float* src = pa + (b0 + j) * pa_stride + (h0 + h) * D;
-          st[h][j] = on ? __ldcg(reinterpret_cast<const float2*>(ml + (b0 + j) * ml_stride + (h0 + h) * 2)) : make_float2(-CUDART_INF_F, 0.f);
-          if constexpr (E == 4) {
-            const float4 v = on ? __ldcg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            a[h][j][0] = v.x; a[h][j][1] = v.y; a[h][j][2] = v.z; a[h][j][3] = v.w;
-          } else {
-            const float2 v = on ? __ldcg(reinterpret_cast<const float2*>(src)) : make_float2(0.f, 0.f);
-            a[h][j][0] = v.x; a[h][j][1] = v.y;
+        for (int g = 0; g < GROUPS; ++g)
+#pragma unroll
+          for (int j = 0; j < kGroup; ++j) {
+            const int i = b0 + g * kGroup + j;
+            const bool on = i < c.n_splits && h0 + h < n_heads;
+            const float* src = pa + i * pa_stride + (h0 + h) * D;
+            const float2 st = on ? __ldcg(reinterpret_cast<const float2*>(ml + i * ml_stride + (h0 + h) * 2)) : make_float2(-CUDART_INF_F, 0.f);
+            mi[h][g][j] = st.x;
+            li[h][g][j] = st.y;
+            if constexpr (E == 4) {
+              const float4 v = on ? __ldcg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+              a[h][g][j][0] = v.x; a[h][g][j][1] = v.y; a[h][g][j][2] = v.z; a[h][g][j][3] = v.w;
+            } else {
+              const float2 v = on ? __ldcg(reinterpret_cast<const float2*>(src)) : make_float2(0.f, 0.f);
+              a[h][g][j][0] = v.x; a[h][g][j][1] = v.y;
+            }
           }
-        }
 #pragma unroll
-      for (int h = 0; h < HEADS; ++h) {
-        if (h0 + h >= n_heads) continue;               // no arithmetic on the infinities of heads that are not there
-        float mn = m[h];
+      for (int h = 0; h < HEADS; ++h)
 #pragma unroll
-        for (int j = 0; j < SPLITS; ++j) mn = fmaxf(mn, st[h][j].x);
-        const float keep = exp2f(m[h] - mn);           // 0 on the first group (m = -inf)
-        l[h] *= keep;
-#pragma unroll
-        for (int e = 0; e < E; ++e) acc[h][e] *= keep;
-#pragma unroll
-        for (int j = 0; j < SPLITS; ++j) {
-          const float w = exp2f(st[h][j].x - mn);      // absent split: exp2(-inf) = 0
-          l[h] += w * st[h][j].y;
-#pragma unroll
-          for (int e = 0; e < E; ++e) acc[h][e] += w * a[h][j][e];
-        }
-        m[h] = mn;
-      }
+        for (int g = 0; g < GROUPS; ++g)               // no arithmetic on the infinities of heads and groups that are not there
+          if (h0 + h < n_heads && b0 + g * kGroup < c.n_splits) merge_group<E>(m[h], l[h], acc[h], mi[h][g], li[h][g], a[h][g]);
     }
 #pragma unroll
     for (int h = 0; h < HEADS; ++h) {
@@ -206,7 +197,7 @@ __device__ __forceinline__ bool count_split(const StepDevice& s, int combine, in
 template <int D>
 __device__ __forceinline__ void merge_by_scheduler(const StepDevice& s, const CombineItem& c, int kv_head, int lane) {
   const int G = s.Hq / s.Hkv;
-  merge_heads<D, D / 32, 2, 4>(s, c, kv_head * G, G, 0, lane);
+  merge_heads<D, D / 32, 2, 1>(s, c, kv_head * G, G, 0, lane);
 }
 // Warp `warp` of the kDecWarps streaming warps: a head or half a head at a time, so that all have something to do.
 template <int D>
@@ -214,9 +205,9 @@ __device__ __forceinline__ void merge_by_all(const StepDevice& s, const CombineI
   const int G = s.Hq / s.Hkv;
   if (D == 64 || G <= kDecWarps / 2) {
     for (int i = warp; i < G * (D / 64); i += kDecWarps)
-      merge_heads<D, 2, 1, 16>(s, c, kv_head * G + i / (D / 64), 1, i % (D / 64) * 64, lane);
+      merge_heads<D, 2, 1, 2>(s, c, kv_head * G + i / (D / 64), 1, i % (D / 64) * 64, lane);
   } else {
-    for (int i = warp; i < G; i += kDecWarps) merge_heads<D, D / 32, 1, 8>(s, c, kv_head * G + i, 1, 0, lane);
+    for (int i = warp; i < G; i += kDecWarps) merge_heads<D, D / 32, 1, 1>(s, c, kv_head * G + i, 1, 0, lane);
   }
 }
 

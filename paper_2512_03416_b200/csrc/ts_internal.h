@@ -316,40 +316,47 @@ __device__ __forceinline__ void append_tokens(const StepDevice& s, const int32_t
     append_one(s, tok, rows[n + lo] + (tok - row_start[lo]), rows[2 * n + lo], lane);
   }
 }
-// Log-sum-exp merge of the splits of one (token, head) for head_dim element d: the exact merge
-//   m = max m_i,  l = sum l_i 2^(m_i - m),  O = sum acc_i 2^(m_i - m) / l
-// over the partial slots [first_partial, first_partial + n_splits). Eight splits' loads are in
-// flight at a time. Reads bypass L1 (the partials may have been written by another SM of the
-// same launch).
+// Log-sum-exp merge of the splits of one (token, head),
+//   m = max m_i,  l = sum l_i 2^(m_i - m),  O = sum acc_i 2^(m_i - m) / l,
+// in groups of eight: one group added to the running (m, l, acc) of E head_dim elements. The groups and each rounding are
+// the same for whoever merges (the combine launch, or inside the decode launch whichever warps come last), so that a row's
+// result does not depend on the timing of its splits. Splits that are not there have m_i = -inf, l_i = acc_i = 0.
+constexpr int kMergeGroup = 8;
+template <int E>
+__device__ __forceinline__ void merge_group(float& m, float& l, float (&acc)[E], const float (&mi)[kMergeGroup],
+                                            const float (&li)[kMergeGroup], const float (&ai)[kMergeGroup][E]) {
+  float mn = m;
+#pragma unroll
+  for (int j = 0; j < kMergeGroup; ++j) mn = fmaxf(mn, mi[j]);
+  const float keep = exp2f(m - mn);            // 0 on the first group (m = -inf)
+#pragma unroll
+  for (int j = 0; j < kMergeGroup; ++j) {
+    const float w = exp2f(mi[j] - mn);         // absent split: exp2(-inf) = 0
+    l = j == 0 ? __fmaf_rn(l, keep, __fmul_rn(w, li[j])) : __fmaf_rn(w, li[j], l);
+#pragma unroll
+    for (int e = 0; e < E; ++e) acc[e] = j == 0 ? __fmaf_rn(acc[e], keep, __fmul_rn(w, ai[j][e])) : __fmaf_rn(w, ai[j][e], acc[e]);
+  }
+  m = mn;
+}
+// The merge for head_dim element d over the partial slots [first_partial, first_partial + n_splits). A group's
+// loads are in flight at a time. Reads bypass L1 (another SM wrote the partials).
 __device__ __forceinline__ float merge_splits(const StepDevice& s, int first_partial, int n_splits, int h, int d) {
   const float* ml = s.part_ml + ((size_t)first_partial * s.Hq + h) * 2;
   const float* pa = s.part_acc + ((size_t)first_partial * s.Hq + h) * s.D + d;
   const size_t ml_stride = (size_t)s.Hq * 2, pa_stride = (size_t)s.Hq * s.D;
-  float m = -__int_as_float(0x7f800000), l = 0.f, acc = 0.f;
-  for (int base = 0; base < n_splits; base += 8) {
-    float mi[8], li[8], ai[8];
+  float m = -__int_as_float(0x7f800000), l = 0.f, acc[1] = {0.f};
+  for (int base = 0; base < n_splits; base += kMergeGroup) {
+    float mi[kMergeGroup], li[kMergeGroup], ai[kMergeGroup][1];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int j = 0; j < kMergeGroup; ++j) {
       const bool on = base + j < n_splits;
       mi[j] = on ? __ldcg(ml + (base + j) * ml_stride) : -__int_as_float(0x7f800000);
       li[j] = on ? __ldcg(ml + (base + j) * ml_stride + 1) : 0.f;
-      ai[j] = on ? __ldcg(pa + (base + j) * pa_stride) : 0.f;
+      ai[j][0] = on ? __ldcg(pa + (base + j) * pa_stride) : 0.f;
     }
-    float mn = m;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) mn = fmaxf(mn, mi[j]);
-    const float keep = exp2f(m - mn);          // 0 on the first group (m = -inf)
-    l *= keep;
-    acc *= keep;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float w = exp2f(mi[j] - mn);       // absent split: exp2(-inf) = 0
-      l += w * li[j];
-      acc += w * ai[j];
-    }
-    m = mn;
+    merge_group<1>(m, l, acc, mi, li, ai);
   }
-  return acc / l;
+  return acc[0] / l;
 }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }

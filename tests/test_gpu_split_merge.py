@@ -62,3 +62,42 @@ def test_many_units_of_split_rows():
     """Most units are finished, counted and merged while their thread block streams on."""
     b = wl.make_batch("many", wl.Shape(32, 8, 128), [1000 + 37 * i for i in range(24)], [1] * 24, seed=5, profile="peaked")
     check(b, 1, decode_split_tokens=128)
+
+
+@pytest.mark.parametrize("shape", [wl.Shape(8, 2, 128), wl.Shape(16, 2, 128), wl.Shape(32, 2, 128), wl.Shape(8, 2, 64)], ids=["G4", "G8", "G16", "d64"])
+def test_a_rows_bits_do_not_depend_on_who_merges_it(shape):
+    """200 rows of 5 to 18 splits, merged inside the decode launch by whichever warps finish a row's last split, and one by
+    one, merged by a launch of their own: the same bits every time."""
+    ctx = [64 * (5 + i % 14) - 1 - i % 60 for i in range(200)]
+    b = wl.make_batch("bits", shape, ctx, [1] * 200, seed=shape.Hq, profile="peaked")
+    run = GpuRun(b, chunk_size=0, decode_split_tokens=64)
+    first = run.step(keep_len=True)
+    for i in range(6):
+        before = run.dec.velocity()["kernel_launches"]
+        assert np.array_equal(run.step(keep_len=True), first), f"step {i}"
+        assert run.dec.velocity()["kernel_launches"] - before == 1, "not merged inside the decode launch"
+    lb, before = run.lb, run.dec.velocity()["kernel_launches"]
+    for r in range(200):
+        run.dec.mixed_step([lb.slots[r]], [1], [ctx[r]], lb.q[r:r + 1], lb.k_new[r:r + 1], lb.v_new[r:r + 1], lb.out[r:r + 1], keep_len=True)
+    assert run.dec.velocity()["kernel_launches"] - before == 400, "not merged by a launch of their own"
+    alone = lb.output()
+    differ = np.flatnonzero((alone != first).any(axis=(1, 2)))
+    assert differ.size == 0, f"rows {differ[:8]} differ, {int((alone != first).sum())} of {alone.size} values"
+
+
+@pytest.mark.parametrize("shape", [wl.Shape(32, 2, 64), wl.Shape(32, 2, 128)], ids=["d64", "G16"])
+def test_host_step_in_pieces_whose_rows_are_merged_elsewhere(shape):
+    """Shapes whose decode rows never ride along with the tiles: the first piece's three rows are merged by a launch of their
+    own, in the whole step by the decode launch. Bit for bit the same."""
+    ctx = [1000, 990, 980, 0] + [64 * (5 + i % 14) - 9 for i in range(60)] + [0]
+    ql = [1, 1, 1, 1400] + [1] * 60 + [1400]
+    b = wl.make_batch("pieces", shape, ctx, ql, seed=shape.D, profile="peaked", chunk_size=sum(ql))
+    one, two = GpuRun(b, decode_split_tokens=64), GpuRun(b, decode_split_tokens=64)
+    want = one.step()
+    host = [torch.from_numpy(a.view(np.int16)).pin_memory() for a in (b.q, b.k_new, b.v_new)]
+    out = torch.full(host[0].shape, 0x7FC0, dtype=torch.int16).pin_memory()
+    two.dec.mixed_step_host(two.slots, ql, ctx, *host, out)
+    assert two.dec.velocity()["kernel_launches"] > one.dec.velocity()["kernel_launches"] + 2, "it went in one piece"
+    assert np.array_equal(wl.bf16_bits_to_f32(out.numpy().view(np.uint16)), want)
+    assert np.array_equal(two.pool(), one.pool())
+    assert two.dec.device_status() == 0
