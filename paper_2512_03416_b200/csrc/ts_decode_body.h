@@ -192,7 +192,9 @@ __device__ __forceinline__ bool count_split(const StepDevice& s, int combine, in
     last = before == n_splits - 1;
     if (last) *count = 0;                              // for the next launch
   }
-  return __shfl_sync(0xffffffffu, last, 0);
+  last = __shfl_sync(0xffffffffu, last, 0);
+  __syncwarp();                                        // what lane 0 acquired holds for the lanes that read the splits (a shuffle orders no memory)
+  return last;
 }
 template <int D>
 __device__ __forceinline__ void merge_by_scheduler(const StepDevice& s, const CombineItem& c, int kv_head, int lane) {
