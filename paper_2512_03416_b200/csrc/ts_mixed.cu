@@ -820,6 +820,7 @@ mixed_kernel(const __grid_constant__ StepParams<W> params, const __grid_constant
     } else {
       // ------------------------------------------------------------------- MMA issuer
       if (warp == kWarpMma) {
+        ready();                   // the time limits of its waits are for this launch, not for what the one in front still has to do
         const uint32_t tmem = misc[0];
         const uint32_t issue = elect_one();
         // the warp keeps its own failure flag in a register: nothing on its path reads shared memory
