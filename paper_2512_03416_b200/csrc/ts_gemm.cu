@@ -278,6 +278,7 @@ gemm_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap a_map, const _
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------------ MMA issuer
+    pdl_wait();                    // the time limits of its waits are for this launch, not for what the one in front still has to do
     const uint32_t issue = elect_one();
     bool dead = false;
     auto iwait = [&](int i, uint32_t parity) {
@@ -565,6 +566,7 @@ gemm_pair_kernel(const GemmArgs g, const __grid_constant__ CUtensorMap x_map, co
     }
   } else if (warp == 1) {
     if (rank == 0) {
+      pdl_wait();                  // as in gemm_kernel
       const uint32_t issue = elect_one();
       bool dead = false;
       auto iwait = [&](int i, uint32_t parity) {

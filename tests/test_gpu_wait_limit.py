@@ -5,7 +5,10 @@ import pytest
 import torch
 
 from paper_2512_03416_b200 import workloads as wl
+from paper_2512_03416_b200.harness import from_dev, to_dev
+from paper_2512_03416_b200.layer import DecoderLayer
 from tests.helpers import GpuRun
+from tests.test_gpu_layer import bits, make_weights
 
 pytestmark = pytest.mark.gpu
 
@@ -43,3 +46,23 @@ def test_tiles_behind_a_long_launch(long_launch, ctx, ql):
         assert run.dec.device_status() == 0
         assert np.array_equal(run.lb.output(), want)
     assert long_launch.dec.device_status() == 0
+
+
+@pytest.mark.parametrize("ctx,ql", [([40, 0, 7], [1, 33, 1]), ([40, 0], [1, 1100])], ids=["few-tokens", "many-tokens"])
+def test_projections_behind_a_long_launch(long_launch, ctx, ql):
+    """The norm's thread blocks, one per token, all start next to the long launch, so that the projection behind them does too."""
+    s, hidden, inter, n = wl.Shape(8, 2, 128), 512, 1024, sum(ql)
+    run = GpuRun(wl.make_batch("layer", s, ctx, ql, seed=n, profile="peaked"), chunk_size=n, wait_limit_cycles=LIMIT)
+    rng = np.random.default_rng(n)
+    dev = {k: to_dev(v) for k, v in make_weights(rng, s, hidden, inter).items()}
+    layer = DecoderLayer(run.dec, dev["w_norm1"], dev["w_qkv"], dev["w_o"], dev["w_norm2"], dev["w_gate"], dev["w_up"], dev["w_down"], max_position=4096)
+    x_in = to_dev(bits(rng, (n, hidden), 1.0))
+    x_out = torch.empty_like(x_in)
+    layer.step(run.slots, ql, ctx, x_in, x_out, keep_len=True)
+    want = from_dev(x_out)
+    for _ in range(3):
+        long_launch.lb.step(keep_len=True)
+        layer.step(run.slots, ql, ctx, x_in, x_out, keep_len=True)
+        assert run.dec.device_status() == 0
+        assert np.array_equal(from_dev(x_out), want)
+    layer.close()
