@@ -351,6 +351,27 @@ void cut_row(int n, int split, int* per, int* pieces) {
   *pieces = ceil_div(n, *per);
 }
 
+// Keys of a unit that take as long as the busiest of n_sms thread blocks has to do, in a step without chunks at a split of `split`
+// keys, whose units are dealt out longest first. Of more units than SMs a bound: at least (two of the longest n_sms + 1 units
+// share an SM and pay for a unit once more) or, `at_most`, at most (the k-th unit of a second wave finds an SM that is done
+// with the k-th shortest unit of the first; for less than n_sms units too many).
+int busiest_sm_keys(const ts_ctx* c, const ts_step* st, int split, int n_sms, bool at_most) {
+  std::vector<int> len;                                    // of the items: units of n_kv_heads heads each
+  for (int r = 0; r < st->n_rows; ++r) {
+    int per, pieces;
+    cut_row(st->ctx_len[r] + 1, split, &per, &pieces);
+    for (int i = 0; i < pieces; ++i) len.push_back(std::min(per, st->ctx_len[r] + 1 - i * per));
+  }
+  auto nth = [&](int unit) {                               // length of the unit-th longest unit
+    std::nth_element(len.begin(), len.begin() + unit / c->cfg.n_kv_heads, len.end(), [](int x, int y) { return x > y; });
+    return len[unit / c->cfg.n_kv_heads];
+  };
+  const int longest = nth(0), over = (int)len.size() * c->cfg.n_kv_heads - n_sms;
+  if (over <= 0) return longest;
+  const int unit_cost = 140000 / (4 * c->cfg.head_dim);    // 2 us at 70 GB/s, in keys
+  return std::max(longest, nth(n_sms - (at_most ? over : 1)) + nth(n_sms) + unit_cost);
+}
+
 // Keys per split of a step's decode rows.
 int decode_split(const ts_ctx* c, const ts_step* st) {
   int split = c->cfg.decode_split_tokens;
@@ -371,35 +392,52 @@ int decode_split(const ts_ctx* c, const ts_step* st) {
         longest = std::max(longest, st->ctx_len[r] + 1);
       }
     }
-    const int64_t share = keys * c->cfg.n_kv_heads / (c->n_sms > 0 ? c->n_sms : kSmsB200);
-    split = (int)std::min<int64_t>(std::max<int64_t>(share, kMinDefaultSplit), kMaxDefaultSplit);
-    // A step of few decode rows, some of which are split anyway, takes as long as the thread block with most to do: the
-    // shortest split, of 256 keys at least, with which every unit (but 3 % short ones) has an SM to itself, if that is near the
-    // share. Where at most two thirds of the SMs cost no more than 100 keys of 128 elements per unit in addition (0.7 us), or
-    // where the units are shorter yet, they are the better ones: the next step's thread blocks start on the other SMs, and the
-    // merge is a launch of its own (see merge_here). Device time of a step of the 8B shape, us, by the share and 512 alone / so:
-    // one row of 1014 keys 9.5 / 6.9, one of 2157 9.4 / 8.2, 4 rows of ~1300 9.9 / 9.3, 4 of ~2600 14.5 / 11.3, 8 of ~2350 19.8 /
-    // 15.8, 12 of ~970 15.0 / 12.7. Not for rows of 512 keys and less, which are not worth a merge (14 rows of up to 513 keys of 64
-    // elements, a call bound by the host: 10.8 / 11.2); keys of 64 elements count half.
     const int n_sms = c->n_sms > 0 ? c->n_sms : kSmsB200;
+    const int64_t share = keys * c->cfg.n_kv_heads / n_sms;
+    split = (int)std::min<int64_t>(std::max<int64_t>(share, kMinDefaultSplit), kMaxDefaultSplit);
+    split = ceil_div(split, ts::kKeysPerTile) * ts::kKeysPerTile;
+    // A step of few decode rows, some of which are split anyway, takes as long as the thread block with most to do. It gets
+    // the shortest split, of 256 keys at least, with which every unit has an SM to itself; or a shorter one with some units too
+    // many (19 items of eight KV heads are four more than 148 SMs), where two short ones on an SM are done before the longest.
+    // None is taken with which the busiest thread block has more to do than without this rule. Where at most two thirds of the
+    // SMs cost no more than 100 keys of 128 elements per unit in addition, or where the units are shorter yet, they are the
+    // better ones: the next step's thread blocks start on the other SMs, and the merge is a launch of its own (see merge_here),
+    // which together is worth 0.7 us, the time of 100 keys. Device time of a step of the 8B shape, us, by the share and 512 alone,
+    // with the shortest split of up to 152 units whatever their lengths, and so: one row of 1014 keys 9.5 / 7.0 / 7.0, of 2157
+    // 9.4 / 8.2 / 8.2, of 7104 10.6 / 15.7 / 10.6, of 7950 10.6 / 11.7 / 10.7, rows of 3042, 4371 and 751 keys 11.9 / 14.8 / 10.5, 4 rows of
+    // ~1300 9.8 / 9.3 / 9.2, 8 of 2350 20.3 / 15.2 / 15.1, 12 of 970 16.3 / 16.3 / 12.0. Not for rows of 512 keys and less, which are
+    // not worth a merge (14 rows of up to 513 keys of 64 elements, a call bound by the host: 10.8 / 11.2 us); keys of 64 elements
+    // count half.
     const int keys128 = 128 / c->cfg.head_dim;             // keys that are as long as one of 128 elements
-    if (!chunks && longest > kMinDefaultSplit * keys128 && st->n_rows * c->cfg.n_kv_heads <= n_sms) {
-      const int64_t most = std::min<int64_t>(std::max<int64_t>(share * 29 / 20, kMinDefaultSplit), kMaxDefaultSplit);
-      int64_t one_wave = 0;                                // the shortest split that gives every unit an SM
-      for (int64_t s = std::max<int64_t>(kMinSmallSplit * keys128, ceil_div((int)share, ts::kKeysPerTile) * ts::kKeysPerTile); s <= most; s += ts::kKeysPerTile) {
-        if (one_wave > 0 && s - one_wave > 100 * keys128) break;
-        int units = 0;
-        for (int r = 0; r < st->n_rows; ++r) {
-          int per, pieces;
-          cut_row(st->ctx_len[r] + 1, (int)s, &per, &pieces);
-          units += pieces * c->cfg.n_kv_heads;
+    if (!chunks && longest > kMinDefaultSplit * keys128 && (int64_t)st->n_rows * c->cfg.n_kv_heads <= n_sms) {
+      const int tile = ts::kKeysPerTile;
+      const int most = std::min(busiest_sm_keys(c, st, split, n_sms, false), kMaxDefaultSplit);
+      // the shortest split of `from` to `most` keys, in key tiles, with at most `units` units; 0: none
+      auto shortest = [&](int64_t from, int64_t units) -> int {
+        for (int64_t s = (from + tile - 1) / tile * tile; s <= most; s += tile) {
+          int64_t n = 0;
+          for (int r = 0; r < st->n_rows; ++r) {
+            int per, pieces;
+            cut_row(st->ctx_len[r] + 1, (int)s, &per, &pieces);
+            n += pieces;
+          }
+          if (n * c->cfg.n_kv_heads <= units) return (int)s;
         }
-        if (one_wave == 0 && s >= kMinOneWaveSplit * keys128 && units <= n_sms + n_sms / 32) split = (int)(one_wave = s);
-        if (3 * units <= 2 * n_sms) {
-          split = (int)s;
-          break;
-        }
-      }
+        return 0;
+      };
+      const int64_t from = std::max<int64_t>(share, kMinSmallSplit * keys128);
+      int one_wave = shortest(std::max<int64_t>(from, kMinOneWaveSplit * keys128), n_sms + n_sms / 32);
+      const int two_thirds = shortest(from, 2 * n_sms / 3);
+      const int exact = shortest(std::max<int64_t>(from, kMinOneWaveSplit * keys128), n_sms);
+      if (one_wave != exact && busiest_sm_keys(c, st, one_wave, n_sms, true) > (exact > 0 ? exact : most)) one_wave = exact;
+      if (one_wave > 0) split = one_wave;
+      // More than sixteen splits of a row are another round trip of the merge. The eight warps of a thread block take 128 keys at a
+      // time: up to a multiple of that a unit takes no longer.
+      int per, pieces;
+      cut_row(longest, split, &per, &pieces);
+      const int whole = ceil_div(split, 8 * ts::kPageSize) * 8 * ts::kPageSize;
+      if (one_wave > 0 && pieces > 16 && whole <= most) split = whole;
+      if (two_thirds > 0 && (one_wave == 0 || two_thirds - one_wave <= 100 * keys128)) split = two_thirds;
     }
   }
   split = ceil_div(split, ts::kKeysPerTile) * ts::kKeysPerTile;
