@@ -152,6 +152,7 @@ struct ts_ctx {
   std::vector<WorkItem> items;
   std::vector<CombineItem> combines;
   std::vector<int32_t> combine_of;                       // index into combines, by partial slot
+  std::vector<int> unit_keys;                            // see busiest_sm_keys
   std::vector<int32_t> tok0;
   std::vector<TableDelta> deltas;
   std::vector<std::pair<int32_t, int32_t>> sync_marks;   // (slot, table entries the device will hold)
@@ -355,25 +356,30 @@ void cut_row(int n, int split, int* per, int* pieces) {
 // keys, whose units are dealt out longest first. Of more units than SMs a bound: at least (two of the longest n_sms + 1 units
 // share an SM and pay for a unit once more) or, `at_most`, at most (the k-th unit of a second wave finds an SM that is done
 // with the k-th shortest unit of the first; for less than n_sms units too many).
-int busiest_sm_keys(const ts_ctx* c, const ts_step* st, int split, int n_sms, bool at_most) {
-  std::vector<int> len;                                    // of the items: units of n_kv_heads heads each
+int busiest_sm_keys(ts_ctx* c, const ts_step* st, int split, int n_sms, bool at_most) {
+  std::vector<int>& len = c->unit_keys;                    // of the items: units of n_kv_heads heads each
+  len.clear();
+  int longest = 0;
   for (int r = 0; r < st->n_rows; ++r) {
-    int per, pieces;
-    cut_row(st->ctx_len[r] + 1, split, &per, &pieces);
-    for (int i = 0; i < pieces; ++i) len.push_back(std::min(per, st->ctx_len[r] + 1 - i * per));
+    const int n = st->ctx_len[r] + 1;
+    int per = n, pieces = 1;
+    if (n > split) cut_row(n, split, &per, &pieces);
+    longest = std::max(longest, per);
+    for (; pieces > 1; --pieces) len.push_back(per);
+    len.push_back((n - 1) % per + 1);
   }
+  const int over = (int)len.size() * c->cfg.n_kv_heads - n_sms;
+  if (over <= 0) return longest;
   auto nth = [&](int unit) {                               // length of the unit-th longest unit
     std::nth_element(len.begin(), len.begin() + unit / c->cfg.n_kv_heads, len.end(), [](int x, int y) { return x > y; });
     return len[unit / c->cfg.n_kv_heads];
   };
-  const int longest = nth(0), over = (int)len.size() * c->cfg.n_kv_heads - n_sms;
-  if (over <= 0) return longest;
   const int unit_cost = 140000 / (4 * c->cfg.head_dim);    // 2 us at 70 GB/s, in keys
   return std::max(longest, nth(n_sms - (at_most ? over : 1)) + nth(n_sms) + unit_cost);
 }
 
 // Keys per split of a step's decode rows.
-int decode_split(const ts_ctx* c, const ts_step* st) {
+int decode_split(ts_ctx* c, const ts_step* st) {
   int split = c->cfg.decode_split_tokens;
   if (split <= 0) {
     // An SM's share of the step's (key, KV head) pairs, so that a small batch's long rows spread over
@@ -409,27 +415,40 @@ int decode_split(const ts_ctx* c, const ts_step* st) {
     // not worth a merge (14 rows of up to 513 keys of 64 elements, a call bound by the host: 10.8 / 11.2 us); keys of 64 elements
     // count half.
     const int keys128 = 128 / c->cfg.head_dim;             // keys that are as long as one of 128 elements
-    if (!chunks && longest > kMinDefaultSplit * keys128 && (int64_t)st->n_rows * c->cfg.n_kv_heads <= n_sms) {
+    // Whether the units are at most `units` many. A look at a row that stays whole costs nothing, and no more rows are cut than
+    // there may be pieces.
+    auto fits = [&](int s, int64_t units) {
+      int64_t left = units / c->cfg.n_kv_heads - st->n_rows;
+      for (int r = 0; r < st->n_rows && left >= 0; ++r) {
+        if (st->ctx_len[r] < s) continue;
+        int per, pieces;
+        cut_row(st->ctx_len[r] + 1, s, &per, &pieces);
+        left -= pieces - 1;
+      }
+      return left >= 0;
+    };
+    const int allowed = n_sms + n_sms / 32;
+    if (!chunks && longest > kMinDefaultSplit * keys128 && (int64_t)st->n_rows * c->cfg.n_kv_heads <= n_sms && fits(kMaxDefaultSplit, allowed)) {
       const int tile = ts::kKeysPerTile;
       const int most = std::min(busiest_sm_keys(c, st, split, n_sms, false), kMaxDefaultSplit);
-      // the shortest split of `from` to `most` keys, in key tiles, with at most `units` units; 0: none
+      // the shortest split of `from` to `most` keys, in key tiles, with at most `units` units (the pieces of a row never grow
+      // with the split); 0: none
       auto shortest = [&](int64_t from, int64_t units) -> int {
-        for (int64_t s = (from + tile - 1) / tile * tile; s <= most; s += tile) {
-          int64_t n = 0;
-          for (int r = 0; r < st->n_rows; ++r) {
-            int per, pieces;
-            cut_row(st->ctx_len[r] + 1, (int)s, &per, &pieces);
-            n += pieces;
-          }
-          if (n * c->cfg.n_kv_heads <= units) return (int)s;
+        int64_t lo = (from + tile - 1) / tile, hi = most / tile;
+        if (lo > hi || !fits((int)hi * tile, units)) return 0;
+        while (lo < hi) {
+          const int64_t mid = (lo + hi) / 2;
+          if (fits((int)mid * tile, units)) hi = mid; else lo = mid + 1;
         }
-        return 0;
+        return (int)lo * tile;
       };
       const int64_t from = std::max<int64_t>(share, kMinSmallSplit * keys128);
-      int one_wave = shortest(std::max<int64_t>(from, kMinOneWaveSplit * keys128), n_sms + n_sms / 32);
+      int one_wave = shortest(std::max<int64_t>(from, kMinOneWaveSplit * keys128), allowed);
       const int two_thirds = shortest(from, 2 * n_sms / 3);
-      const int exact = shortest(std::max<int64_t>(from, kMinOneWaveSplit * keys128), n_sms);
-      if (one_wave != exact && busiest_sm_keys(c, st, one_wave, n_sms, true) > (exact > 0 ? exact : most)) one_wave = exact;
+      if (one_wave > 0 && !fits(one_wave, n_sms)) {
+        const int exact = shortest(one_wave, n_sms);
+        if (busiest_sm_keys(c, st, one_wave, n_sms, true) > (exact > 0 ? exact : most)) one_wave = exact;
+      }
       if (one_wave > 0) split = one_wave;
       // More than sixteen splits of a row are another round trip of the merge. The eight warps of a thread block take 128 keys at a
       // time: up to a multiple of that a unit takes no longer.
@@ -444,10 +463,10 @@ int decode_split(const ts_ctx* c, const ts_step* st) {
   for (;; split *= 2) {
     int64_t partials = 0;
     for (int r = 0; r < st->n_rows; ++r) {
-      if (st->q_len[r] != 1) continue;
+      if (st->q_len[r] != 1 || st->ctx_len[r] < split) continue;
       int per, pieces;
       cut_row(st->ctx_len[r] + 1, split, &per, &pieces);
-      if (pieces > 1) partials += pieces;
+      partials += pieces;
     }
     if (partials <= c->L.max_partials) return split;
   }
