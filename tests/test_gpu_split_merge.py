@@ -46,15 +46,25 @@ def test_split_rows_are_merged_by_the_decode_launch(shape, over):
     check(b, 1 if over else 2, decode_split_tokens=64)
 
 
-@pytest.mark.parametrize("rows", [[521], [2157], [900] * 4 + [100], [2000, 1500, 1100, 600], [5400, 30, 4000, 300], [2300] * 8, [970] * 12, [16000] + [200] * 17],
-                         ids=lambda r: f"{len(r)}x{r[0]}")
-def test_default_splits_of_steps_around_one_unit_per_SM(rows):
-    """The split follows the number of units; the plan, and parity with it."""
+@pytest.mark.parametrize("rows,units,longest", [([521], 40, 128), ([2157], 96, 192), ([900] * 4 + [100], 136, 256), ([2000, 1500, 1100, 600], 144, 320),
+                                                ([5400, 30, 4000, 300], 152, 576), ([2300] * 8, 128, 1152), ([970] * 12, 96, 971),
+                                                ([3041, 4370, 750], 136, 512), ([16000] + [200] * 17, 256, 1088)],
+                         ids=lambda r: f"{len(r)}x{r[0]}" if isinstance(r, list) else str(r))
+def test_default_splits_of_steps_around_one_unit_per_SM(rows, units, longest):
+    """The planned units and the longest one's keys on 148 SMs (of the last batch no split fits: an SM's share), who merges, and
+    parity."""
     b = wl.make_batch("few", wl.LLAMA8B, rows, [1] * len(rows), seed=len(rows), profile="peaked")
     want, pool_want = oracle_step(b)
     run = GpuRun(b, chunk_size=0)
+    items = run.dec.plan_step(run.slots, [1] * len(rows), rows)
+    if sms() == 148:
+        assert (8 * len(items), max(i[5] - i[4] for i in items)) == (units, longest)
     for i in range(3):
+        before = run.dec.velocity()["kernel_launches"]
         assert_parity(run.step(keep_len=True), want, "peaked", f"{rows}, step {i}")
+        if i > 0:
+            own_merge = len(items) > len(rows) and 3 * 8 * len(items) <= 2 * sms()
+            assert run.dec.velocity()["kernel_launches"] - before == 1 + own_merge
     assert np.array_equal(run.pool(), pool_want)
 
 
