@@ -120,10 +120,13 @@ __device__ __forceinline__ void give_up(const StepDevice& s, volatile int* faile
 }
 
 // Merge of a row's splits, by one warp: the merge of merge_splits, bit for bit, for `n_heads` heads from head0 on, 32 * E of
-// their columns from col0 on. The loads of HEADS heads x GROUPS groups of splits fly at a time.
+// their columns from col0 on. The loads of HEADS heads x GROUPS groups of splits fly at a time. Lane i takes the weight of
+// split i of these and the others get it from there: this is the end of a launch, whose code comes in cold, and a weight per
+// lane and split is most of merge_group's.
 template <int D, int E, int HEADS, int GROUPS>
 __device__ __forceinline__ void merge_heads(const StepDevice& s, const CombineItem& c, int head0, int n_heads, int col0, int lane) {
-  constexpr int kGroup = kMergeGroup;
+  constexpr int kGroup = kMergeGroup, kSplits = GROUPS * kGroup;
+  static_assert(kSplits <= 32, "a lane per split");
   const int col = col0 + lane * E;
   const float* ml = s.part_ml + ((size_t)c.first_partial * s.Hq + head0) * 2;
   const float* pa = s.part_acc + ((size_t)c.first_partial * s.Hq + head0) * D + col;
@@ -139,33 +142,57 @@ __device__ __forceinline__ void merge_heads(const StepDevice& s, const CombineIt
       for (int e = 0; e < E; ++e) acc[h][e] = 0.f;
     }
 #pragma unroll 1
-    for (int b0 = 0; b0 < c.n_splits; b0 += GROUPS * kGroup) {
-      float mi[HEADS][GROUPS][kGroup], li[HEADS][GROUPS][kGroup], a[HEADS][GROUPS][kGroup][E];
+    for (int b0 = 0; b0 < c.n_splits; b0 += kSplits) {
+      float2 st[HEADS];                                // lane i: maximum and sum of split b0 + i
+      float a[HEADS][kSplits][E];
 #pragma unroll
-      for (int h = 0; h < HEADS; ++h)
+      for (int h = 0; h < HEADS; ++h) {
+        const bool head = h0 + h < n_heads;
+        st[h] = make_float2(-CUDART_INF_F, 0.f);
+        if (head && lane < kSplits && b0 + lane < c.n_splits)
+          st[h] = __ldcg(reinterpret_cast<const float2*>(ml + (b0 + lane) * ml_stride + (h0 + h) * 2));
 #pragma unroll
-        for (int g = 0; g < GROUPS; ++g)
+        for (int j = 0; j < kSplits; ++j) {
+          const bool on = head && b0 + j < c.n_splits;
+          const float* src = pa + (b0 + j) * pa_stride + (h0 + h) * D;
+          if constexpr (E == 4) {
+            const float4 v = on ? __ldcg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            a[h][j][0] = v.x; a[h][j][1] = v.y; a[h][j][2] = v.z; a[h][j][3] = v.w;
+          } else {
+            const float2 v = on ? __ldcg(reinterpret_cast<const float2*>(src)) : make_float2(0.f, 0.f);
+            a[h][j][0] = v.x; a[h][j][1] = v.y;
+          }
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < HEADS; ++h) {
+        float top = st[h].x;                           // the largest maximum of the lane's group
+#pragma unroll
+        for (int sh = 1; sh < kGroup; sh <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, sh));
+        float mn[GROUPS], keep[GROUPS], mine = 0.f;
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) {
+          const float before = g > 0 ? mn[g - 1] : m[h];
+          mn[g] = fmaxf(before, __shfl_sync(0xffffffffu, top, g * kGroup));
+          keep[g] = exp2f(before - mn[g]);             // 0 on the first group (m = -inf)
+          if (lane / kGroup == g) mine = mn[g];
+        }
+        const float w = exp2f(st[h].x - mine);         // absent split: exp2(-inf) = 0
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) {
+          if (b0 + g * kGroup >= c.n_splits) break;
 #pragma unroll
           for (int j = 0; j < kGroup; ++j) {
-            const int i = b0 + g * kGroup + j;
-            const bool on = i < c.n_splits && h0 + h < n_heads;
-            const float* src = pa + i * pa_stride + (h0 + h) * D;
-            const float2 st = on ? __ldcg(reinterpret_cast<const float2*>(ml + i * ml_stride + (h0 + h) * 2)) : make_float2(-CUDART_INF_F, 0.f);
-            mi[h][g][j] = st.x;
-            li[h][g][j] = st.y;
-            if constexpr (E == 4) {
-              const float4 v = on ? __ldcg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
-              a[h][g][j][0] = v.x; a[h][g][j][1] = v.y; a[h][g][j][2] = v.z; a[h][g][j][3] = v.w;
-            } else {
-              const float2 v = on ? __ldcg(reinterpret_cast<const float2*>(src)) : make_float2(0.f, 0.f);
-              a[h][g][j][0] = v.x; a[h][g][j][1] = v.y;
-            }
+            const int i = g * kGroup + j;
+            const float wj = __shfl_sync(0xffffffffu, w, i), lj = __shfl_sync(0xffffffffu, st[h].y, i);
+            l[h] = j == 0 ? __fmaf_rn(l[h], keep[g], __fmul_rn(wj, lj)) : __fmaf_rn(wj, lj, l[h]);
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+              acc[h][e] = j == 0 ? __fmaf_rn(acc[h][e], keep[g], __fmul_rn(wj, a[h][i][e])) : __fmaf_rn(wj, a[h][i][e], acc[h][e]);
           }
-#pragma unroll
-      for (int h = 0; h < HEADS; ++h)
-#pragma unroll
-        for (int g = 0; g < GROUPS; ++g)               // no arithmetic on the infinities of heads and groups that are not there
-          if (h0 + h < n_heads && b0 + g * kGroup < c.n_splits) merge_group<E>(m[h], l[h], acc[h], mi[h][g], li[h][g], a[h][g]);
+        }
+        m[h] = mn[GROUPS - 1];
+      }
     }
 #pragma unroll
     for (int h = 0; h < HEADS; ++h) {
