@@ -6,7 +6,7 @@
 //                   memory through a 3-stage cp.async ring, mma.sync bf16 MMAs with fp32 online
 //                   softmax (warp-shuffle reductions). head_dim 128 steps run ts_mixed.cu and
 //                   ts_decode.cu instead.
-//   small_step    - the same tiles and the decode units (ts_decode_body.h) of a small head_dim 64 step
+//                   With NH > 0 also the decode units (ts_decode_body.h) of a small head_dim 64 step.
 //   combine       - log-sum-exp merge of the decode splits
 #include <cuda_bf16.h>
 #include <math_constants.h>
@@ -207,12 +207,64 @@ __device__ __forceinline__ void warp_tile(uint32_t sK, uint32_t sV, int key_row0
   }
 }
 
-// Barrier of the kThreads threads that work on an item (the first of their block).
-__device__ __forceinline__ void item_sync() { asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory"); }
+// Decode units of a step in the blocks of the launch that runs its tiles (small_step_units), 0: tiles only.
+template <int NH>
+struct DecodeMap {
+  CUtensorMap kv;
+};
+template <>
+struct DecodeMap<0> {};
+// The decode units of a small head_dim 64 step: block `cta` of `n_ctas`.
+constexpr int kStages64 = 4;                    // page stages of a warp at head_dim 64, as in decode_kernel
+template <int NH>
+__device__ __forceinline__ void small_step_units(const StepDevice& s, const CUtensorMap* kv_map, unsigned char* smem_raw, int cta, int n_ctas) {
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
+  if (threadIdx.x == 0) tma_prefetch_desc(kv_map);
+  auto ready = [&]() { pdl_wait(); };
+  if (s.meta) ready();
+  if (threadIdx.x < dec::kDecThreads) {
+    dec::decode_units<64, NH, kStages64, false>(s, kv_map, smem, base, ready);
+  } else {
+    dec::decode_schedule<64, kStages64, false>(s, smem, base, cta, n_ctas, ready);
+    if (threadIdx.x == dec::kDecThreads) {
+      __threadfence();
+      if (atomicAdd(s.pf_queue + 4, 1) == n_ctas - 1) {          // as in decode_kernel
+        s.pf_queue[3] = 0;
+        s.pf_queue[4] = 0;
+      }
+    }
+  }
+}
 
-// One work item of one KV head, by kThreads threads.
-template <int D>
-__device__ __forceinline__ void attention_item(const StepDevice& s, int item, int kv_head, unsigned char* smem) {
+// One work item of one KV head per block, by kThreads threads: grid (items, KV heads). With NH > 0 the launch is a whole
+// head_dim 64 step of few prefill items and few decode units: blocks [0, n_prefill_items x Hkv) of the prefill items, then the
+// decode units'. Such a step is bound by launches: 4 rows and 64 tokens next to one another in one launch take 2.2 us less
+// of the host than in two, and on the device the decode units no longer wait for the tiles.
+// (The tiles' code stays in the kernel's body: as a function of its own with the step by reference, the same text ran 2 to 4 %
+// slower, 2048 tokens of 32 heads behind 8000 next to 64 rows 993 us instead of 975.)
+template <int D, int NH>
+__global__ void __launch_bounds__(NH > 0 ? dec::kDecThreads + 32 : kThreads, NH > 0 ? 1 : 2)
+attention_kernel(const __grid_constant__ StepParams<kInlineWords> params, const __grid_constant__ DecodeMap<NH> decode_map) {
+  const StepDevice& s = params.s;
+  extern __shared__ __align__(128) unsigned char smem[];
+  pdl_launch_dependents();
+  int item = blockIdx.x, kv_head = blockIdx.y;
+  if constexpr (NH > 0) {
+    const int n_blocks = s.n_prefill_items * s.Hkv;              // the prefill items'
+    if ((int)blockIdx.x >= n_blocks) {
+      small_step_units<NH>(s, &decode_map.kv, smem, (int)blockIdx.x - n_blocks, (int)gridDim.x - n_blocks);
+      return;
+    }
+    if (threadIdx.x >= kThreads) return;
+    item = blockIdx.x / s.Hkv;
+    kv_head = blockIdx.x % s.Hkv;
+  }
+  // barrier of the threads that work on the item
+  auto item_sync = []() {
+    if (NH == 0) __syncthreads();
+    else asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory");
+  };
   constexpr int kTileBytes = kKeysPerTile * D * 2;
   const uint32_t smem_base = smem_u32(smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -383,67 +435,25 @@ constexpr int item_smem_bytes() {
   return pipe > merge ? pipe : merge;
 }
 
-template <int D>
-__global__ void __launch_bounds__(kThreads, 2) attention_kernel(const __grid_constant__ StepParams<kInlineWords> params) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  pdl_launch_dependents();
-  attention_item<D>(params.s, blockIdx.x, blockIdx.y, smem);
-}
-
-// A head_dim 64 step with few prefill items and few decode units, one block each: blocks [0, n_items x Hkv) of the
-// prefill items, then the decode units'. It is bound by launches: a step of 4 rows and 64 tokens next to one another in
-// one launch takes 2.2 us less of the host than in two, and on the device the decode units no longer wait for the tiles.
-constexpr int kStages64 = 4;                    // page stages of a warp at head_dim 64, as in decode_kernel
-template <int NH>
-__global__ void __launch_bounds__(dec::kDecThreads + 32, 1)
-small_step_kernel(const __grid_constant__ StepParams<kInlineWords> params, const __grid_constant__ CUtensorMap kv_map) {
-  const StepDevice& s = params.s;
-  extern __shared__ unsigned char smem_raw[];
-  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  unsigned char* smem = smem_raw + (base - smem_u32(smem_raw));
-  pdl_launch_dependents();
-  const int n_tiles = s.n_prefill_items * s.Hkv;
-  if ((int)blockIdx.x < n_tiles) {
-    if (threadIdx.x < kThreads) attention_item<64>(s, blockIdx.x / s.Hkv, blockIdx.x % s.Hkv, smem);
-    return;
-  }
-  if (threadIdx.x == 0) tma_prefetch_desc(&kv_map);
-  auto ready = [&]() { pdl_wait(); };
-  if (s.meta) ready();
-  const int cta = (int)blockIdx.x - n_tiles, n_ctas = (int)gridDim.x - n_tiles;
-  if (threadIdx.x < dec::kDecThreads) {
-    dec::decode_units<64, NH, kStages64, false>(s, &kv_map, smem, base, ready);
-  } else {
-    dec::decode_schedule<64, kStages64, false>(s, smem, base, cta, n_ctas, ready);
-    if (threadIdx.x == dec::kDecThreads) {
-      __threadfence();
-      if (atomicAdd(s.pf_queue + 4, 1) == n_ctas - 1) {          // as in decode_kernel
-        s.pf_queue[3] = 0;
-        s.pf_queue[4] = 0;
-      }
-    }
-  }
-}
-
 template <int NH>
 cudaError_t launch_small_step_t(const StepDevice& s, const CUtensorMap& kv_map, cudaStream_t stream) {
   const int G = s.Hq / s.Hkv;
   const size_t smem = 1024 + std::max<size_t>(dec::decode_smem_bytes<64, kStages64>(G), item_smem_bytes<64>());
-  cudaError_t e = cudaFuncSetAttribute(small_step_kernel<NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(attention_kernel<64, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   StepParams<kInlineWords> params;
   fill_params(s, &params);
-  return launch_pdl(small_step_kernel<NH>, dim3(s.n_items * s.Hkv), dim3(dec::kDecThreads + 32), smem, stream, params, kv_map);
+  return launch_pdl(attention_kernel<64, NH>, dim3(s.n_items * s.Hkv), dim3(dec::kDecThreads + 32), smem, stream, params, DecodeMap<NH>{kv_map});
 }
 
 template <int D>
 cudaError_t launch_attention_d(const StepDevice& s, cudaStream_t stream) {
   constexpr int smem = item_smem_bytes<D>();
-  cudaError_t e = cudaFuncSetAttribute(attention_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = cudaFuncSetAttribute(attention_kernel<D, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   StepParams<kInlineWords> params;
   fill_params(s, &params);
-  return launch_pdl(attention_kernel<D>, dim3(s.n_items, s.Hkv), dim3(kThreads), smem, stream, params);
+  return launch_pdl(attention_kernel<D, 0>, dim3(s.n_items, s.Hkv), dim3(kThreads), smem, stream, params, DecodeMap<0>{});
 }
 
 }  // namespace
