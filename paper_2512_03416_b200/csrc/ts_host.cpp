@@ -21,6 +21,7 @@ constexpr int kRing = 4;                  // pinned metadata buffers in flight
 constexpr int kDeltaCapacity = 32768;     // table entries per upload batch (bulk loads)
 constexpr int kSlotDeltas = 4096;         // table entries that ride along with a step's metadata
 constexpr int kMinSmallSplit = 128, kMinOneWaveSplit = 256, kMinDefaultSplit = 512, kMaxDefaultSplit = 4096;   // keys per decode split, see plan()
+constexpr int kSmallStepKeys = 8192;      // most keys of a tile of a step in one launch, see enqueue_step
 constexpr int kSmsB200 = 148;             // for plans made before the device is known
 constexpr int kDefaultMaxTokens = 16384;  // step size bound when chunk_size == 0
 constexpr size_t kAlign = 256;
@@ -851,7 +852,11 @@ int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefi
         d.append_wide = append_us > 2.0 * pairs / n_ctas;
         d.debug_arrivals = (c->cfg.debug_flags & TS_DEBUG_LOSE_APPEND_ARRIVAL) ? 1 : 0;
         TS_CUDA(c, ts::launch_mixed(d, q_map, c->kv_map, c->kv_tile_map, new_maps, n_ctas, p, stream));
-      } else if (n_items > c->n_prefill_items && (long long)n_items * c->cfg.n_kv_heads <= c->n_sms) {
+      } else if (n_items > c->n_prefill_items && (long long)n_items * c->cfg.n_kv_heads <= c->n_sms && c->items[0].k_end <= kSmallStepKeys) {
+        // The tiles have 168 registers there instead of 203 (48 bytes of spills), which is 1 to 3 % of a long tile's time: beyond
+        // 8192 keys more than the 2 to 4 us that one launch saves. (us, two launches / one, next to 20 rows of 300 keys a chunk of
+        // 600 tokens of two heads behind 0 keys 20.1 / 14.7, 4000 101.6 / 100.6, 8000 183.6 / 185.3, 16000 347 / 356; next to 60 rows
+        // 120 tokens of 16 heads behind 4000 98.4 / 94.2, 8000 182.4 / 180.8, 16000 348 / 354.)
         TS_CUDA(c, ts::launch_small_step(d, c->kv_map, stream));
         decode_launched = true;
         if (pe) c->prof_mixed.back() = 1;

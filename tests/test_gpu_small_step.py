@@ -43,3 +43,10 @@ def test_tiles_and_decode_units_of_head_dim_64_in_one_launch(shape, over):
 def test_split_rows_of_a_small_step_are_merged():
     b = wl.make_batch("small", wl.Shape(4, 2, 64), [300, 64, 63, 150, 0], [1] * 4 + [70], seed=3, profile="peaked")
     check(b, 2, decode_split_tokens=64)
+
+
+@pytest.mark.parametrize("last", [8191, 8192])
+def test_long_tiles_have_a_launch_of_their_own(last):
+    """A tile that sees 8192 keys, and one more."""
+    b = wl.make_batch("small", wl.Shape(4, 2, 64), [300, 5, last - 39], [1, 1, 40], seed=last, profile="peaked")
+    check(b, 1 if last == 8191 else 2)
