@@ -873,7 +873,13 @@ int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefi
       // every thread block. (Device time of a step in us, merged by a launch / in place: 64 rows of the 8B shape 122.7 / 120.5, 203
       // rows of the 70B shape 224.3 / 221.1; 4 rows of ~1300 keys as 96 units 9.9 / 10.4; between 100 units and one per SM a
       // launch takes 1 to 1.5 us more than up to 96.)
-      merged = 3 * (long long)(n_items - c->n_prefill_items) * c->cfg.n_kv_heads > 2 * c->n_sms;
+      // With head_dim 64, whose units are half as long, the same goes for up to 1.8 units per SM, but not for one wave of them (and
+      // the few more that decode_split allows). Us, merged by a launch / in place, 16 query heads: 5 x 1200 keys as 120 units 8.4 / 8.6, 8 x
+      // 2000 as 128 11.8 / 11.7, 12 x 600 as 192 11.5 / 12.2, 18 rows of 64 to 16000 keys as 240 41.4 / 42.0, 22 rows as 264 35.6 /
+      // 36.4, 26 rows as 280 36.8 / 36.0, 32 as 344 44.8 / 43.0; with head_dim 128 18 rows as 240 63.3 / 62.0.
+      const long long units = (long long)(n_items - c->n_prefill_items) * c->cfg.n_kv_heads;
+      const bool short_second_wave = c->cfg.head_dim == 64 && units > c->n_sms + c->n_sms / 32 && 5 * units <= 9 * c->n_sms;
+      merged = 3 * units > 2 * c->n_sms && !short_second_wave;
       d.merge_here = merged;
       TS_CUDA(c, ts::launch_decode(d, c->kv_map, c->n_sms, stream));
       ++c->cnt.kernel_launches;

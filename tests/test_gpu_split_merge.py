@@ -111,3 +111,14 @@ def test_host_step_in_pieces_whose_rows_are_merged_elsewhere(shape):
     assert np.array_equal(wl.bf16_bits_to_f32(out.numpy().view(np.uint16)), want)
     assert np.array_equal(two.pool(), one.pool())
     assert two.dec.device_status() == 0
+
+
+@pytest.mark.parametrize("items,launches", [(152, 1), (153, 2), (266, 2), (267, 1)])
+def test_who_merges_short_units_of_head_dim_64(items, launches):
+    """One wave of units and four more, a second one of up to 1.8 units per SM, and more, on 148 SMs: the first and last are merged by the
+    decode launch."""
+    if sms() != 148:
+        pytest.skip("sizes are those of 148 SMs")
+    ctx = [64 * 3 - 5] * (items // 3) + [64 * (items % 3) - 7] * (items % 3 > 0)
+    b = wl.make_batch("wave", wl.Shape(4, 1, 64), ctx, [1] * len(ctx), seed=items, profile="peaked")
+    check(b, launches, decode_split_tokens=64)
