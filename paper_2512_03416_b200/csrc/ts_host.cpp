@@ -880,7 +880,7 @@ int enqueue_step(ts_ctx* c, const ts_step* st, int64_t n_tokens, int64_t n_prefi
       const long long units = (long long)(n_items - c->n_prefill_items) * c->cfg.n_kv_heads;
       const bool short_second_wave = c->cfg.head_dim == 64 && units > c->n_sms + c->n_sms / 32 && 5 * units <= 9 * c->n_sms;
       merged = 3 * units > 2 * c->n_sms && !short_second_wave;
-      d.merge_here = merged;
+      d.merge_here = merged && n_combines > 0;                 // without a split row the schedulers have nothing to wait for at the end
       TS_CUDA(c, ts::launch_decode(d, c->kv_map, c->n_sms, stream));
       ++c->cnt.kernel_launches;
     }
