@@ -20,7 +20,7 @@ using ts::WorkItem;
 constexpr int kRing = 4;                  // pinned metadata buffers in flight
 constexpr int kDeltaCapacity = 32768;     // table entries per upload batch (bulk loads)
 constexpr int kSlotDeltas = 4096;         // table entries that ride along with a step's metadata
-constexpr int kMinSmallSplit = 128, kMinOneWaveSplit = 256, kMinDefaultSplit = 512, kMaxDefaultSplit = 4096;   // keys per decode split, see plan()
+constexpr int kMinSmallSplit = 128, kMinOneWaveSplit = 256, kMinDefaultSplit = 512, kMaxDefaultSplit = 4096;   // keys per decode split, see decode_split()
 constexpr int kSmallStepKeys = 8192;      // most keys of a tile of a step in one launch, see enqueue_step
 constexpr int kSmsB200 = 148;             // for plans made before the device is known
 constexpr int kDefaultMaxTokens = 16384;  // step size bound when chunk_size == 0
